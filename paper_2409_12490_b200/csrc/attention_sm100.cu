@@ -1,17 +1,17 @@
 // K4 / K5: block-sparse (Algorithm 2, lines 6-13) and dense causal (Eq. 2) attention on the
-// sm_100a tensor cores.  bf16 or fp16 operands, fp32 accumulation in tensor memory, online softmax.
+// sm_100a tensor cores.  bf16 or fp16 operands, head_dim 128 or 64, fp32 accumulation in tensor memory, online softmax.
 //
 // Persistent CTAs (one per SM) walk over work units; a unit is 256 consecutive query rows of one
 // (batch, query head): two 128-row tiles "A" and "B" that share every K/V tile the producer brings in
 // (tile B is absent in the last unit of a segment with an odd number of 128-row tiles).  Roles (384 threads):
 //   warps 0-3  softmax for tile A (one thread per query row)
 //   warps 4-7  softmax for tile B
-//   warp  8    TMA producer: K/V tiles through a 5-slot ring of 32 KB buffers; a gathered
+//   warp  8    TMA producer: K/V tiles through a ring of 5 x 32 KB (head_dim 64: 8 x 16 KB); a gathered
 //              tile is assembled from 128/blk boxes addressed by the block list
 //   warp  9    MMA issuer (warps 10-11 idle; they complete the third warpgroup): S = Q K^T
 //              (operands in shared memory), O += P V (P read from tensor memory, where the
 //              softmax warps overwrite S with 16-bit probabilities)
-// Tensor memory (512 columns): S_A | S_B | O_A | O_B, 128 fp32 columns each.
+// Tensor memory (512 columns): S_A | S_B (128 fp32 columns each) | O_A | O_B (head_dim columns each).
 // The tile sequence of a unit is: gathered past tiles, contiguous unmasked tiles, then the
 // diagonal tiles; tile A stops one tile earlier than B.  Units are handed out by an atomic
 // counter (producer warp) and published to the other warps.  Every wait is bounded: on
@@ -21,17 +21,30 @@
 namespace cp {
 namespace {
 
-constexpr int kD = 128;
 constexpr int kTile = 128;
 constexpr int kHalfBytes = kTile * 64 * 2;   // [128 rows x 64 cols] of 16-bit elements, 128-byte swizzled
-constexpr int kTileBytes = 2 * kHalfBytes;   // both halves of head_dim
-constexpr int kSlots = 5;
 constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {producer, MMA, 2 idle}
-constexpr int kSmemQ = 0;
-constexpr int kSmemKV = 2 * kTileBytes;
-constexpr int kSmemBar = kSmemKV + kSlots * kTileBytes;
+constexpr int kMaxSlots = 8;
 constexpr int kBarBytes = 512;
-constexpr int kSmemTotal = kSmemBar + kBarBytes + 1024;   // + barrier block + slack to align the tiles to 1024 bytes
+// What head_dim decides.  Heads of 64 channels keep their probabilities to 32-bit accuracy: P is stored as the sum of two
+// 16-bit values (hi over the first 64 columns of S, lo over the other 64), and O += P V runs over both; O has 64 columns.
+// That costs 8 further N = 64 MMAs per tile, which hide under the softmax (the exponentials bound this shape: 128 per
+// row and tile against half the MMA work of 128 channels).  Measured on two sequences of 6001 tokens, 16 heads, segment 512,
+// block 64, budget 1024 (fp16): the whole layer 33.8 ms with the one-warp-per-row kernel of attention_simt.cu, 0.154 ms here;
+// error against fp64 the same to five digits (2.052e-4 relative at 4099 tokens in fp16, 1.645e-3 in bf16: the output's rounding).
+template <int D> struct Shape {
+  static constexpr bool kSplitP = D == 64;
+  static constexpr int kHalves = D / 64;
+  static constexpr int kTileBytes = kHalves * kHalfBytes;
+  static constexpr int kSlots = D == 128 ? 5 : kMaxSlots;           // 5 x 32 KB + 64 KB of Q; 8 x 16 KB + 32 KB
+  static constexpr int kSmemQ = 0;
+  static constexpr int kSmemKV = 2 * kTileBytes;
+  static constexpr int kSmemBar = kSmemKV + kSlots * kTileBytes;
+  static constexpr int kSmemTotal = kSmemBar + kBarBytes + 1024;    // + barrier block + slack to align the tiles to 1024 bytes
+};
+// fp16 halves of P are scaled by 2^7: the reference maximum is at most 2^8 behind (lazy rescale), so P stays below 2^15,
+// and the low halves of small probabilities stay out of the subnormals
+template <bool kF16, int D> constexpr float kPShift = (kF16 && Shape<D>::kSplitP) ? 7.f : 0.f;
 constexpr float kRescaleThreshold = 8.0f;           // in log2 units
 #ifndef CP_EMUL_EVERY
 #define CP_EMUL_EVERY 8
@@ -63,8 +76,8 @@ struct Unit {
 struct Bars {
   unsigned long long q_full;
   unsigned long long q_empty;
-  unsigned long long kv_full[kSlots];
-  unsigned long long kv_empty[kSlots];
+  unsigned long long kv_full[kMaxSlots];
+  unsigned long long kv_empty[kMaxSlots];
   unsigned long long s_full[2];
   unsigned long long p_full[2];
   unsigned long long o_done[2];
@@ -84,6 +97,8 @@ struct Args {
   DeviceStatus* st;
   int B, Hq, Hkv, g, n, seg, blk, k, r, n1, n2;
   int64_t osb, osh, ost;
+  const uint16_t *Q, *K, *V;    // only for rows that are recomputed one by one (recompute_row)
+  int64_t qs[3], ks[3], vs[3];
   float sm_scale;
   int dense;
   int n_units;
@@ -259,12 +274,58 @@ __device__ __forceinline__ bool receive_unit(const Args& a, Bars* bars, uint32_t
 // ---------------------------------------------------------------- softmax role
 constexpr int kMaskNone = 0, kMaskCausal = 1, kMaskCols = 2, kMaskGeneric = 3;
 
+__device__ __forceinline__ float elem_f32(uint16_t x, bool f16) {
+  return f16 ? __half2float(__ushort_as_half(x)) : __uint_as_float(uint32_t(x) << 16);
+}
+
+// One row of a 64-channel head in plain fp32, key by key, by one thread.  A tile's MMA multiplies the zero probability of a
+// key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row whose
+// output came out as NaN or infinite is therefore evaluated again over exactly the keys it sees.
 template <bool kF16>
+__device__ __noinline__ void recompute_row(const Args* ap, int b, int h, const int32_t* list, int cnt, int t) {
+  const Args& a = *ap;
+  const uint16_t* q = a.Q + b * a.qs[0] + h * a.qs[1] + int64_t(t) * a.qs[2];
+  const uint16_t* kb = a.K + b * a.ks[0] + (h / a.g) * a.ks[1];
+  const uint16_t* vb = a.V + b * a.vs[0] + (h / a.g) * a.vs[1];
+  uint16_t* o = a.O + b * a.osb + h * a.osh + int64_t(t) * a.ost;
+  const int n_ranges = a.dense ? 1 : cnt;
+  auto logit = [&](int key) {
+    float s = 0.f;
+    for (int c = 0; c < 64; ++c) s = fmaf(elem_f32(q[c], kF16), elem_f32(kb[int64_t(key) * a.ks[2] + c], kF16), s);
+    return s * a.sm_scale;
+  };
+  float m = -CUDART_INF_F;
+  for (int e = 0; e < n_ranges; ++e) {
+    const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
+    for (int key = u0; key < u1; ++key) m = fmaxf(m, logit(key));
+  }
+  float l = 0.f;
+  for (int c0 = 0; c0 < 64; c0 += 16) {
+    float acc[16];
+    for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+    l = 0.f;
+    for (int e = 0; e < n_ranges; ++e) {
+      const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
+      for (int key = u0; key < u1; ++key) {
+        const float p = expf(logit(key) - m);
+        l += p;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) acc[c] = fmaf(p, elem_f32(vb[int64_t(key) * a.vs[2] + c0 + c], kF16), acc[c]);
+      }
+    }
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    for (int c = 0; c < 16; ++c) o[c0 + c] = uint16_t(pack2<kF16>(acc[c] * inv, 0.f));
+  }
+  if (a.lse != nullptr) a.lse[((long long)b * a.Hq + h) * a.n + t] = m + logf(l);
+}
+
+template <bool kF16, int D>
 __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int which, int warp_in_wg, int lane) {
+  constexpr bool kSplitP = Shape<D>::kSplitP;
   const uint32_t tm = bars->tmem_base;
   const uint32_t lane_off = uint32_t(warp_in_wg * 32) << 16;
   const uint32_t tS = tm + lane_off + which * 128;
-  const uint32_t tO = tm + lane_off + 256 + which * 128;
+  const uint32_t tO = tm + lane_off + 256 + which * D;
   const int row = warp_in_wg * 32 + lane;
   const float c = a.sm_scale * 1.4426950408889634f;   // logits -> log2 units
   CP_EV_DECL;
@@ -282,7 +343,7 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
       if ((which == 0 || u.rowsB) && t < a.n) {
         uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + int64_t(t) * a.ost);
 #pragma unroll
-        for (int i = 0; i < kD * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = 0; i < D * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
         if (a.lse != nullptr) a.lse[((long long)u.b * a.Hq + u.h) * a.n + t] = -CUDART_INF;
       }
       continue;
@@ -351,7 +412,7 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
         const float f = need ? ex2((m_run - m_new) * c) : 1.f;
         if (need) { m_run = m_new; l_run *= f; }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < D / 32; ++q) {
           uint32_t ov[32];
           tmem_ld32(tO + q * 32, ov);
           tmem_wait_ld();
@@ -360,11 +421,26 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
           tmem_st32(tO + q * 32, ov);
         }
       }
-      const float neg_mc = (m_run == -CUDART_INF) ? 0.f : -m_run * c;   // a row that has not seen a key yet (generic lists only): exp2(-inf) = 0
+      const float neg_mc = (m_run == -CUDART_INF) ? 0.f : kPShift<kF16, D> - m_run * c;   // a row that has not seen a key yet (generic lists only): exp2(-inf) = 0
       const float2 c2 = make_float2(c, c), nm2 = make_float2(neg_mc, neg_mc);
       float2 sum2 = make_float2(0.f, 0.f);
       uint32_t pk[64];
-      if (kind == kMaskNone && a.emul) {
+      if constexpr (kSplitP) {
+        // P = hi + lo, each rounded to the operand type: 2^-22 (fp16) / 2^-17 (bf16) relative, far below the output's rounding
+        uint32_t lo[64];
+#pragma unroll
+        for (int i = 0; i < 128; i += 2) {
+          const float2 xx = __ffma2_rn(make_float2(s[i], s[i + 1]), c2, nm2);
+          float2 p;
+          p.x = ex2(xx.x); p.y = ex2(xx.y);
+          sum2 = __fadd2_rn(sum2, p);
+          const uint32_t hi = pack2<kF16>(p.x, p.y);
+          const float2 hf = unpack2<kF16>(hi);
+          pk[i >> 1] = hi;
+          lo[i >> 1] = pack2<kF16>(p.x - hf.x, p.y - hf.y);
+        }
+        tmem_st64(tS + 64, lo);
+      } else if (kind == kMaskNone && a.emul) {
         // unmasked tile of a long unit: every kEmulEvery-th pair takes the polynomial path, the rest the MUFU
 #pragma unroll
         for (int i = 0; i < 128; i += 2) {
@@ -402,14 +478,19 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
     const int t = u.q_tok + which * kTile + row;
     uint16_t* orow = a.O + u.b * a.osb + u.h * a.osh + int64_t(t) * a.ost;
     const float inv = l_run > 0.f ? 1.f / l_run : 0.f;   // a row without any visible key (generic lists only): zeros
+    float odd = 0.f;                                     // NaN as soon as one output of the row is NaN or infinite
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < D / 32; ++q) {
       uint32_t ov[32];
       tmem_ld32(tO + q * 32, ov);
       tmem_wait_ld();
       uint32_t w[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) w[i] = pack2<kF16>(__uint_as_float(ov[2 * i]) * inv, __uint_as_float(ov[2 * i + 1]) * inv);
+      if constexpr (kSplitP) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) odd = fmaf(__uint_as_float(ov[i]), 0.f, odd);
+      }
       if (t < a.n) {                                 // rows past the end of the sequence (ragged last tile) are dropped
         if (a.o_vec32) {
           // 32-byte stores: every store fills whole 32-byte sectors (a thread owns a row, so the lanes of a
@@ -424,15 +505,21 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
       }
     }
     if (a.lse != nullptr && t < a.n)
-      a.lse[((long long)u.b * a.Hq + u.h) * a.n + t] = m_run * a.sm_scale + __logf(l_run);
+      a.lse[((long long)u.b * a.Hq + u.h) * a.n + t] =
+          m_run * a.sm_scale + (kSplitP ? logf(l_run) - kPShift<kF16, D> * 0.693147180559945f : __logf(l_run));
+    if constexpr (kSplitP) {
+      if (!(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < a.n) recompute_row<kF16>(&a, u.b, u.h, u.list, u.cnt, t);
+    }
     CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 4);            // epilogue done
   }
 }
 
 // ---------------------------------------------------------------- producer role
+template <int D>
 __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_t smem_base, const CUtensorMap* tmQ,
                                               const CUtensorMap* tmKb, const CUtensorMap* tmVb,
                                               const CUtensorMap* tmKt, const CUtensorMap* tmVt, int lane) {
+  constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes, kHalves = Shape<D>::kHalves;
   const int bpt = kTile / a.blk;
   CP_EV_DECL;
   uint32_t item = 0;      // K/V tiles issued so far (all units): item i lives in slot i % kSlots
@@ -459,8 +546,8 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
       const int nq = u_cur.nB ? 2 : 1;
       mbar_expect_tx(&bars->q_full, nq * kTileBytes);
       for (int w = 0; w < nq; ++w)
-        for (int hf = 0; hf < 2; ++hf)
-          tma_load_4d(smem_base + kSmemQ + w * kTileBytes + hf * kHalfBytes, tmQ, &bars->q_full, hf * 64,
+        for (int hf = 0; hf < kHalves; ++hf)
+          tma_load_4d(smem_base + Shape<D>::kSmemQ + w * kTileBytes + hf * kHalfBytes, tmQ, &bars->q_full, hf * 64,
                       u_cur.q_tok + w * kTile, u_cur.h, u_cur.b);
     }
     ++n_units;
@@ -471,7 +558,7 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
       if (lane == 0 && !(a.withhold_v && (it & 1))) {
         const int jt = it >> 1;
         const bool is_v = it & 1;
-        const uint32_t dst = smem_base + kSmemKV + slot * kTileBytes;
+        const uint32_t dst = smem_base + Shape<D>::kSmemKV + slot * kTileBytes;
         unsigned long long* bar = &bars->kv_full[slot];
         mbar_expect_tx(bar, kTileBytes);
         if (jt < u_cur.n_past_tiles) {
@@ -480,14 +567,14 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
             const int li = jt * bpt + q;
             // boxes beyond the list read past the end of the tensor and arrive as zeros
             const int tok = li < u_cur.n_past ? u_cur.list[li] * a.blk : a.n;
-            for (int hf = 0; hf < 2; ++hf)
+            for (int hf = 0; hf < kHalves; ++hf)
               tma_load_4d(dst + hf * kHalfBytes + q * a.blk * 128, tm, bar, hf * 64, tok, u_cur.kvh, u_cur.b);
           }
         } else {
           const CUtensorMap* tm = is_v ? tmVt : tmKt;
           const int ci = jt - u_cur.n_past_tiles;
           const int tok = ci < u_cur.n_cont ? u_cur.c_tok + ci * kTile : u_cur.d_tok + (ci - u_cur.n_cont) * kTile;
-          for (int hf = 0; hf < 2; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, bar, hf * 64, tok, u_cur.kvh, u_cur.b);
+          for (int hf = 0; hf < kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, bar, hf * 64, tok, u_cur.kvh, u_cur.b);
         }
       }
       __syncwarp();
@@ -496,33 +583,39 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
 }
 
 // ---------------------------------------------------------------- MMA role
-template <bool kF16>
+template <bool kF16, int D>
 __device__ __forceinline__ void issue_qk(uint32_t d_tmem, uint32_t q_smem, uint32_t k_smem) {
   const uint64_t base = desc_base(16);
 #pragma unroll
-  for (int kk = 0; kk < kD / 16; ++kk) {
+  for (int kk = 0; kk < D / 16; ++kk) {
     const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
     umma_ss(d_tmem, desc_at(base, q_smem + off), desc_at(base, k_smem + off), Idesc<kF16>::qk, kk > 0);
   }
 }
-template <bool kF16>
+template <bool kF16, int D>
 __device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint32_t v_smem, bool acc) {
   const uint64_t base = desc_base(kHalfBytes);   // the two 64-column halves of head_dim are 16 KB apart
 #pragma unroll
   for (int kk = 0; kk < kTile / 16; ++kk)
-    umma_ts(d_tmem, p_tmem + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16>::pv, (acc || kk > 0) ? 1u : 0u);
+    umma_ts(d_tmem, p_tmem + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, (acc || kk > 0) ? 1u : 0u);
+  if constexpr (Shape<D>::kSplitP) {             // the low halves of P
+#pragma unroll
+    for (int kk = 0; kk < kTile / 16; ++kk)
+      umma_ts(d_tmem, p_tmem + 64 + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, 1u);
+  }
 }
 
-template <bool kF16>
+template <bool kF16, int D>
 __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t smem_base, int lane) {
+  constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes;
   const uint32_t tm = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
-  const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 384};
-  const uint32_t qA = smem_base + kSmemQ, qB = qA + kTileBytes;
+  const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 256 + D};
+  const uint32_t qA = smem_base + Shape<D>::kSmemQ, qB = qA + kTileBytes;
   CP_EV_DECL;
   uint32_t item0 = 0;                 // first K/V item of the current unit
   uint32_t nA = 0, nB = 0;            // P tiles consumed so far per query tile (all units)
   uint32_t n_units = 0;
-  auto slot_addr = [&](uint32_t item) { return smem_base + kSmemKV + (item % kSlots) * kTileBytes; };
+  auto slot_addr = [&](uint32_t item) { return smem_base + Shape<D>::kSmemKV + (item % kSlots) * kTileBytes; };
   auto full_wait = [&](uint32_t item) {
     return mbar_wait(&bars->kv_full[item % kSlots], (item / kSlots) & 1, bars, a.st, 40);
   };
@@ -540,8 +633,8 @@ __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t sme
     if (!full_wait(item0)) return;
     CP_EV(lane == 0, q, 202);                                                // K0 ready
     tc_fence_after();
-    issue_qk<kF16>(tS[0], qA, slot_addr(item0)); umma_commit(&bars->s_full[0]);
-    if (hasB) { issue_qk<kF16>(tS[1], qB, slot_addr(item0)); umma_commit(&bars->s_full[1]); }
+    issue_qk<kF16, D>(tS[0], qA, slot_addr(item0)); umma_commit(&bars->s_full[0]);
+    if (hasB) { issue_qk<kF16, D>(tS[1], qB, slot_addr(item0)); umma_commit(&bars->s_full[1]); }
     umma_commit(&bars->kv_empty[item0 % kSlots]);
     if (T == 1) umma_commit(&bars->q_empty);               // a one-tile unit has no further QK^T
     for (int jt = 0; jt < T; ++jt) {
@@ -555,8 +648,8 @@ __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t sme
         CP_EV(lane == 0, q, 210);                                            // P_A ready
         ++nA;
         tc_fence_after();
-        issue_pv<kF16>(tO[0], tS[0], v_smem, jt > 0);
-        if (jt + 1 < TA) { issue_qk<kF16>(tS[0], qA, kn_smem); umma_commit(&bars->s_full[0]); }
+        issue_pv<kF16, D>(tO[0], tS[0], v_smem, jt > 0);
+        if (jt + 1 < TA) { issue_qk<kF16, D>(tS[0], qA, kn_smem); umma_commit(&bars->s_full[0]); }
         else umma_commit(&bars->o_done[0]);
       }
       if (hasB) {
@@ -565,11 +658,11 @@ __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t sme
         CP_EV(lane == 0, q, 212);                                            // P_B ready
         ++nB;
         tc_fence_after();
-        issue_pv<kF16>(tO[1], tS[1], v_smem, jt > 0);
+        issue_pv<kF16, D>(tO[1], tS[1], v_smem, jt > 0);
       }
       umma_commit(&bars->kv_empty[iv % kSlots]);             // every PV that reads this V tile has been issued
       if (has_next) {
-        if (hasB) { issue_qk<kF16>(tS[1], qB, kn_smem); umma_commit(&bars->s_full[1]); }
+        if (hasB) { issue_qk<kF16, D>(tS[1], qB, kn_smem); umma_commit(&bars->s_full[1]); }
         umma_commit(&bars->kv_empty[ik % kSlots]);
         if (jt + 1 == T - 1) umma_commit(&bars->q_empty);   // that was the unit's last QK^T: Q may be replaced
       } else if (hasB) {
@@ -583,22 +676,22 @@ __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t sme
 }
 
 // ---------------------------------------------------------------- kernel
-template <bool kF16>
+template <bool kF16, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKb,
                        const __grid_constant__ CUtensorMap tmVb, const __grid_constant__ CUtensorMap tmKt,
-                       const __grid_constant__ CUtensorMap tmVt, const Args a) {
+                       const __grid_constant__ CUtensorMap tmVt, const __grid_constant__ Args a) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t smem_base = (raw + 1023u) & ~1023u;
   static_assert(sizeof(Bars) <= kBarBytes, "barrier block too small");
-  Bars* bars = reinterpret_cast<Bars*>(smem_raw + (smem_base - raw) + kSmemBar);
+  Bars* bars = reinterpret_cast<Bars*>(smem_raw + (smem_base - raw) + Shape<D>::kSmemBar);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     mbar_init(&bars->q_full, 1);
     mbar_init(&bars->q_empty, 1);
-    for (int i = 0; i < kSlots; ++i) { mbar_init(&bars->kv_full[i], 1); mbar_init(&bars->kv_empty[i], 1); }
+    for (int i = 0; i < Shape<D>::kSlots; ++i) { mbar_init(&bars->kv_full[i], 1); mbar_init(&bars->kv_empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->s_full[i], 1); mbar_init(&bars->p_full[i], 128); mbar_init(&bars->o_done[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->sched_full[i], 1); mbar_init(&bars->sched_empty[i], 9); }
     bars->abort_flag = 0;
@@ -618,11 +711,11 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   static_assert(kRegPoolNeeded <= kThreads * 168, "setmaxnreg budget exceeds the launch allocation");
   if (warp < 8) {
     reg_inc<216>();
-    softmax_role<kF16>(a, bars, warp >> 2, warp & 3, lane);
+    softmax_role<kF16, D>(a, bars, warp >> 2, warp & 3, lane);
   } else {
     reg_dec<64>();
-    if (warp == 8) producer_role(a, bars, smem_base, &tmQ, &tmKb, &tmVb, &tmKt, &tmVt, lane);
-    else if (warp == 9) mma_role<kF16>(a, bars, smem_base, lane);
+    if (warp == 8) producer_role<D>(a, bars, smem_base, &tmQ, &tmKb, &tmVb, &tmKt, &tmVt, lane);
+    else if (warp == 9) mma_role<kF16, D>(a, bars, smem_base, lane);
   }
   if (bars->abort_flag) {
     // give copies and MMAs still in flight time to land before the CTA's resources go away
@@ -634,11 +727,11 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 }
 
 // ---------------------------------------------------------------- host side
-// [B, H, n, 128] bf16 with element strides (sb, sh, st); box = 64 columns x `rows` tokens
-bool make_map(CUtensorMap* map, const void* base, int B, int H, int n, const int64_t* s, int rows, bool f16) {
+// [B, H, n, d] 16-bit with element strides (sb, sh, st); box = 64 columns x `rows` tokens
+bool make_map(CUtensorMap* map, const void* base, int B, int H, int n, int d, const int64_t* s, int rows, bool f16) {
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return false;
-  cuuint64_t dims[4] = {cuuint64_t(kD), cuuint64_t(n), cuuint64_t(H), cuuint64_t(B)};
+  cuuint64_t dims[4] = {cuuint64_t(d), cuuint64_t(n), cuuint64_t(H), cuuint64_t(B)};
   cuuint64_t strides[3] = {cuuint64_t(s[2]) * 2, cuuint64_t(s[1]) * 2, cuuint64_t(s[0]) * 2};
   cuuint32_t box[4] = {64, cuuint32_t(rows), 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -650,7 +743,7 @@ bool make_map(CUtensorMap* map, const void* base, int B, int H, int n, const int
 }  // namespace
 
 bool sm100_path_applies(const cp_params& p, const Dims& m) {
-  return (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 && m.seg % kTile == 0 && (m.blk == 32 || m.blk == 64 || m.blk == 128) &&
+  return (p.dtype == CP_BF16 || p.dtype == CP_F16) && (m.d == 128 || m.d == 64) && m.seg % kTile == 0 && (m.blk == 32 || m.blk == 64 || m.blk == 128) &&
          !(p.flags & CP_FLAG_FORCE_SIMT);
 }
 
@@ -659,32 +752,37 @@ int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, con
                            bool dense, cudaStream_t s) {
   CUtensorMap tmQ, tmKb, tmVb, tmKt, tmVt;
   const bool f16 = p.dtype == CP_F16;
-  if (!make_map(&tmQ, Q, m.B, m.Hq, m.n, p.q_stride, kTile, f16) || !make_map(&tmKb, K, m.B, m.Hkv, m.n, p.k_stride, m.blk, f16) ||
-      !make_map(&tmVb, V, m.B, m.Hkv, m.n, p.v_stride, m.blk, f16) || !make_map(&tmKt, K, m.B, m.Hkv, m.n, p.k_stride, kTile, f16) ||
-      !make_map(&tmVt, V, m.B, m.Hkv, m.n, p.v_stride, kTile, f16))
+  if (!make_map(&tmQ, Q, m.B, m.Hq, m.n, m.d, p.q_stride, kTile, f16) || !make_map(&tmKb, K, m.B, m.Hkv, m.n, m.d, p.k_stride, m.blk, f16) ||
+      !make_map(&tmVb, V, m.B, m.Hkv, m.n, m.d, p.v_stride, m.blk, f16) || !make_map(&tmKt, K, m.B, m.Hkv, m.n, m.d, p.k_stride, kTile, f16) ||
+      !make_map(&tmVt, V, m.B, m.Hkv, m.n, m.d, p.v_stride, kTile, f16))
     return CP_ERR_CUDA;
   Args a;
   a.idx = idx; a.cnt = cnt; a.O = static_cast<uint16_t*>(O); a.lse = lse; a.st = st;
   a.B = m.B; a.Hq = m.Hq; a.Hkv = m.Hkv; a.g = m.g; a.n = m.n; a.seg = m.seg; a.blk = m.blk; a.k = m.k;
   a.r = m.r; a.n1 = m.n1; a.n2 = m.n2;
   a.osb = p.o_stride[0]; a.osh = p.o_stride[1]; a.ost = p.o_stride[2];
+  a.Q = static_cast<const uint16_t*>(Q); a.K = static_cast<const uint16_t*>(K); a.V = static_cast<const uint16_t*>(V);
+  for (int i = 0; i < 3; ++i) { a.qs[i] = p.q_stride[i]; a.ks[i] = p.k_stride[i]; a.vs[i] = p.v_stride[i]; }
   a.sm_scale = p.sm_scale; a.dense = dense ? 1 : 0;
   // a unit is two 128-row query tiles (one when a segment, or the sequence, has an odd tile count)
   const long long units = dense ? (long long)m.B * m.Hq * (((m.n + kTile - 1) / kTile + 1) / 2)
                                 : (long long)m.B * m.Hq * m.n1 * ((m.seg / kTile + 1) / 2);
   if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  auto kern = f16 ? attention_sm100_kernel<true> : attention_sm100_kernel<false>;
+  const bool d64 = m.d == 64;
+  auto kern = d64 ? (f16 ? attention_sm100_kernel<true, 64> : attention_sm100_kernel<false, 64>)
+                  : (f16 ? attention_sm100_kernel<true, 128> : attention_sm100_kernel<false, 128>);
+  const int smem = d64 ? Shape<64>::kSmemTotal : Shape<128>::kSmemTotal, variant = (d64 ? 2 : 0) + (f16 ? 1 : 0);
   // setmaxnreg.inc blocks forever when the CTA's register pool (threads x registers the kernel was compiled
   // to) is smaller than what the roles ask for, and no bounded wait covers that: check the real allocation of
   // this build once per variant and refuse to launch instead.
-  static int regs_ok[2] = {0, 0};   // 0 = not checked yet, 1 = fits, -1 = does not fit
-  if (regs_ok[f16] == 0) {
+  static int regs_ok[4] = {0, 0, 0, 0};   // 0 = not checked yet, 1 = fits, -1 = does not fit
+  if (regs_ok[variant] == 0) {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return CP_ERR_CUDA;
-    regs_ok[f16] = (fa.numRegs * kThreads >= kRegPoolNeeded) ? 1 : -1;
+    regs_ok[variant] = (fa.numRegs * kThreads >= kRegPoolNeeded) ? 1 : -1;
   }
-  if (regs_ok[f16] < 0) return CP_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal) != cudaSuccess)
+  if (regs_ok[variant] < 0) return CP_ERR_UNSUPPORTED;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return CP_ERR_CUDA;
   a.n_units = int(units);
   a.withhold_v = (p.flags & CP_FLAG_TEST_WITHHOLD_V) ? 1 : 0;
@@ -700,7 +798,7 @@ int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, con
     return CP_ERR_CUDA;
   // persistent CTAs, one per SM (the kernel takes all of an SM's tensor memory and shared memory)
   const unsigned grid = unsigned(units < sms ? units : sms);
-  kern<<<grid, kThreads, kSmemTotal, s>>>(tmQ, tmKb, tmVb, tmKt, tmVt, a);
+  kern<<<grid, kThreads, smem, s>>>(tmQ, tmKb, tmVb, tmKt, tmVt, a);
   return check_launch();
 }
 

@@ -184,6 +184,12 @@ template <> __device__ __forceinline__ uint32_t pack2<false>(float lo, float hi)
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+template <bool kF16> __device__ __forceinline__ float2 unpack2(uint32_t v);
+template <> __device__ __forceinline__ float2 unpack2<true>(uint32_t v) { return __half22float2(*reinterpret_cast<__half2*>(&v)); }
+template <> __device__ __forceinline__ float2 unpack2<false>(uint32_t v) {   // a bf16 is the upper half of a float
+  return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+
 // Shared-memory matrix descriptors for 128-byte-swizzled tiles whose rows are 128 bytes
 // (64 bf16) and whose 8-row groups are 1024 bytes apart.
 __device__ __forceinline__ uint64_t desc_base(uint32_t lbo_bytes) {
@@ -193,11 +199,11 @@ __device__ __forceinline__ uint64_t desc_at(uint64_t base, uint32_t smem_addr) {
   return base | uint64_t((smem_addr & 0x3FFFFu) >> 4);
 }
 
-// instruction descriptors: D fp32, A/B bf16, M = 128, N = 128; B is K-major for Q K^T and
+// instruction descriptors: D fp32, A/B 16-bit, M = 128, N = 128 for Q K^T and head_dim for P V; B is K-major for Q K^T and
 // MN-major (head_dim contiguous) for P V
-template <bool kF16> struct Idesc {   // operand format field: 0 = fp16, 1 = bf16
+template <bool kF16, int D = 128> struct Idesc {   // operand format field: 0 = fp16, 1 = bf16
   static constexpr uint32_t qk = (1u << 4) | ((kF16 ? 0u : 1u) << 7) | ((kF16 ? 0u : 1u) << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-  static constexpr uint32_t pv = qk | (1u << 16);
+  static constexpr uint32_t pv = (qk & ~(0x3Fu << 17)) | ((uint32_t(D) >> 3) << 17) | (1u << 16);
 };
 
 // cuTensorMapEncodeTiled, fetched through the runtime so that the library loads on a machine without a driver

@@ -1,0 +1,71 @@
+"""The tensor-core attention kernel on heads of 64 channels (probabilities held as the sum of two 16-bit values) against
+the fp64 oracle: tile edges, ragged tails, odd tile counts, one-unit and long problems, and values that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2409_12490_b200 import binding as cp
+from paper_2409_12490_b200.inputs import make_uniform_qkv
+
+from helpers import f32
+
+pytestmark = pytest.mark.gpu
+
+SM = f32(1.0 / np.sqrt(64))
+TDT = {"bf16": torch.bfloat16, "f16": torch.float16}
+
+
+def layer(dtype, B, Hq, Hkv, n, seg, blk, k, seed=3):
+    Q, K, V = make_uniform_qkv(B, Hq, Hkv, n, 64, dtype=dtype, seed=seed)
+    prob = cp.Problem(B, Hq, Hkv, n, 64, seg, blk, k, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    Qd, Kd, Vd = Q.cuda(), K.cuda(), V.cuda()
+    idx, cnt = cp.select(prob, cp.estimate(prob, Qd, Kd, ws), ws)
+    return Q, K, V, prob, ws, Qd, Kd, Vd, idx, cnt
+
+
+def assert_close(O, O_ref, V, dtype):
+    """|O_gpu - O| <= u |O| + e max|V|: u is the unit roundoff of the one rounding of O; e covers the split of P (2^-17 for
+    bf16, 2^-22 for fp16), exponentials and logits in fp32 (2^-20 each) and fp32 accumulation over up to 2^11 keys (2^-16 at
+    most).  A single 16-bit rounding of P (2^-9 max|V| and 2^-12 max|V|) would not pass on averages of this length."""
+    u, e = {"bf16": (2.0 ** -8, 2.0 ** -15), "f16": (2.0 ** -11, 2.0 ** -15)}[dtype]
+    err = np.abs(O.float().cpu().numpy().astype(np.float64) - O_ref)
+    assert (err <= u * np.abs(O_ref) + e * float(V.float().abs().max())).all(), float(err.max())
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("B,Hq,Hkv,n,seg,blk,k", [
+    (1, 2, 1, 1, 128, 32, 4), (1, 4, 2, 127, 128, 32, 5), (2, 2, 2, 129, 128, 64, 3), (1, 4, 1, 640, 384, 128, 4),
+    (1, 2, 1, 1301, 512, 32, 19), (3, 4, 2, 2048, 256, 64, 9), (1, 2, 2, 4099, 1024, 128, 17)])
+def test_sparse_and_dense_match_the_oracle(dtype, B, Hq, Hkv, n, seg, blk, k):
+    Q, K, V, prob, ws, Qd, Kd, Vd, idx, cnt = layer(dtype, B, Hq, Hkv, n, seg, blk, k)
+    O, lse = cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws, want_lse=True)
+    Od = cp.dense_attention(prob, Qd, Kd, Vd, ws)
+    assert cp.device_status(ws) == 0
+    O_ref, lse_ref = oracle.sparse_attention(Q, K, V, idx.cpu().numpy(), cnt.cpu().numpy(), seg, blk, SM)
+    assert_close(O, O_ref, V, dtype)
+    assert np.abs(lse.cpu().numpy() - lse_ref).max() <= 1e-4
+    assert_close(Od, oracle.dense_attention(Q, K, V, SM)[0], V, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+def test_value_that_is_not_finite_reaches_only_the_rows_that_see_it(dtype):
+    n, seg, blk, k = 700, 256, 32, 12
+    Q, K, V, prob, ws, Qd, Kd, Vd, idx, cnt = layer(dtype, 1, 2, 1, n, seg, blk, k)
+    bad = 300
+    Vd[0, 0, bad, 5] = float("inf")
+    Vf = V.clone()
+    Vf[0, 0, bad, 5] = 0
+    for dense in (False, True):
+        O = cp.dense_attention(prob, Qd, Kd, Vd, ws) if dense else cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws)
+        assert cp.device_status(ws) == 0
+        O = O.float().cpu().numpy()
+        li = idx.cpu().numpy()
+        sees = np.zeros((2, n), dtype=bool)
+        for h in range(2):
+            for t in range(bad, n):
+                sees[h, t] = dense or bad // blk in li[0, h, t // seg]
+        assert np.isfinite(O[0][~sees]).all() and not np.isfinite(O[0][sees][:, 5]).any()
+        O_ref = oracle.dense_attention(Q, K, Vf, SM)[0] if dense else oracle.sparse_attention(Q, K, Vf, li, cnt.cpu().numpy(), seg, blk, SM)[0]
+        assert_close(torch.from_numpy(O[0][~sees]), O_ref[0][~sees], V, dtype)
