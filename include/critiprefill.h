@@ -14,7 +14,7 @@
  *   - Calls validate their arguments on the host, enqueue kernels on `cuda_stream`
  *     (a cudaStream_t passed as void*; NULL = the default stream) and return without
  *     synchronising.  Outputs are valid once the stream reaches that point.
- *     The calls (critiprefill_device_status excepted) only enqueue kernels and one small memset, so a stream
+ *     The calls (critiprefill_device_status excepted) only enqueue kernels (critiprefill_estimate_static also a small memset), so a stream
  *     that is being captured into a CUDA graph may carry them; the graph then refers to the buffers given at
  *     capture time (tensor maps are encoded on the host from those pointers).
  *   - Return value: a cp_status.  Conditions only the device can see (a block list that
@@ -234,8 +234,9 @@ int critiprefill_dense_attention(const cp_params* p, const void* Q, const void* 
  *   S_prev      in  device, nullable; S_out, idx, cnt  out device: the per-sequence arrays of critiprefill_estimate /
  *               critiprefill_select ([Hq,n1_i,n2_i] fp64, [Hq,n1_i,k] int32, [Hq,n1_i] int32 with n1_i, n2_i from
  *               len_i) stored one after another in sequence order; critiprefill_varlen_sizes gives the totals
- * The sequences run one after another on `cuda_stream` through the same kernels as the single-sequence calls, so each
- * sequence's results are those of critiprefill_estimate + _select + _attention on its slice, bit for bit.
+ * The sequences go through the same kernels as the single-sequence calls (where the tensor-core attention kernel applies, all
+ * of them in one launch), so each sequence's results are those of critiprefill_estimate + _select + _attention on its slice,
+ * bit for bit.
  * Errors: CP_ERR_SHAPE for a bad cu_seqlens or batch != 1; otherwise as the single-sequence calls. */
 int critiprefill_prefill_varlen(const cp_params* p, const int32_t* cu_seqlens, int32_t n_seqs, const void* Q,
                                 const void* K, const void* V, const double* S_prev, double* S_out, int32_t* idx,

@@ -164,18 +164,18 @@ int critiprefill_dense_attention(const cp_params* p, const void* Q, const void* 
 
 namespace {
 // cu_seqlens checked, and the packed offsets of sequence i's S / idx / cnt arrays (in elements)
-struct SeqSlot { int64_t s, idx, cnt; int len; };
 int varlen_walk(const cp_params* p, const int32_t* cu, int32_t n_seqs, std::vector<SeqSlot>* slots, SeqSlot* total) {
   if (p == nullptr || cu == nullptr) return CP_ERR_NULL;
   if (n_seqs <= 0 || cu[0] != 0 || p->batch != 1 || p->segment_size <= 0 || p->block_size <= 0 || p->budget_blocks <= 0 ||
       p->n_q_heads <= 0)
     return CP_ERR_SHAPE;
-  SeqSlot at{0, 0, 0, 0};
+  SeqSlot at{0, 0, 0, 0, 0};
   for (int i = 0; i < n_seqs; ++i) {
     const int64_t len = int64_t(cu[i + 1]) - cu[i];
     if (len <= 0 || len > p->seq_len) return CP_ERR_SHAPE;
     const int64_t n1 = (len + p->segment_size - 1) / p->segment_size, n2 = (len + p->block_size - 1) / p->block_size;
     at.len = int(len);
+    at.tok = cu[i];
     if (slots != nullptr) slots->push_back(at);
     at.s += int64_t(p->n_q_heads) * n1 * n2;
     at.idx += int64_t(p->n_q_heads) * n1 * p->budget_blocks;
@@ -211,6 +211,8 @@ int critiprefill_prefill_varlen(const cp_params* p, const int32_t* cu_seqlens, i
   auto at = [&](const void* base, int64_t token, const int64_t* stride) {
     return static_cast<const char*>(base) + token * stride[2] * m.es;
   };
+  // the tensor-core attention kernel takes all sequences in one launch
+  const bool one_launch = n_seqs > 1 && sm100_path_applies(*p, m) && aligned16(Q) && aligned16(K) && aligned16(V) && aligned16(O);
   for (int i = 0; i < n_seqs; ++i) {
     cp_params q = *p;
     q.seq_len = slots[i].len;
@@ -224,11 +226,14 @@ int critiprefill_prefill_varlen(const cp_params* p, const int32_t* cu_seqlens, i
     int32_t* cnt_i = cnt + slots[i].cnt;
     if ((rc = critiprefill_estimate(&q, Qi, Ki, S_prev ? S_prev + slots[i].s : nullptr, Si, ws, ws_bytes, cuda_stream)) != CP_OK) return rc;
     if ((rc = critiprefill_select(&q, Si, idx_i, cnt_i, ws, ws_bytes, cuda_stream)) != CP_OK) return rc;
-    if ((rc = critiprefill_attention(&q, Qi, Ki, Vi, idx_i, cnt_i, Oi, lse ? lse + int64_t(p->n_q_heads) * t0 : nullptr, ws, ws_bytes,
+    if (!one_launch &&
+        (rc = critiprefill_attention(&q, Qi, Ki, Vi, idx_i, cnt_i, Oi, lse ? lse + int64_t(p->n_q_heads) * t0 : nullptr, ws, ws_bytes,
                                      cuda_stream)) != CP_OK)
       return rc;
   }
-  return CP_OK;
+  if (!one_launch) return CP_OK;
+  return launch_attention_sm100_varlen(*p, m, slots.data(), n_seqs, Q, K, V, idx, cnt, O, lse, static_cast<DeviceStatus*>(ws),
+                                       static_cast<cudaStream_t>(cuda_stream));
 }
 
 int critiprefill_device_status(const void* ws, int32_t* status_out, void* cuda_stream) {

@@ -1,7 +1,7 @@
 // K4 / K5: block-sparse (Algorithm 2, lines 6-13) and dense causal (Eq. 2) attention on the
 // sm_100a tensor cores.  bf16 or fp16 operands, head_dim 128 or 64, fp32 accumulation in tensor memory, online softmax.
 //
-// Persistent CTAs (one per SM) walk over work units; a unit is 256 consecutive query rows of one
+// CTAs (one per SM) walk over work units; a unit is 256 consecutive query rows of one
 // (batch, query head): two 128-row tiles "A" and "B" that share every K/V tile the producer brings in
 // (tile B is absent in the last unit of a segment with an odd number of 128-row tiles).  Roles (384 threads):
 //   warps 0-3  softmax for tile A (one thread per query row)
@@ -13,9 +13,14 @@
 //              softmax warps overwrite S with 16-bit probabilities)
 // Tensor memory (512 columns): S_A | S_B (128 fp32 columns each) | O_A | O_B (head_dim columns each).
 // The tile sequence of a unit is: gathered past tiles, contiguous unmasked tiles, then the
-// diagonal tiles; tile A stops one tile earlier than B.  Units are handed out by an atomic
-// counter (producer warp) and published to the other warps.  Every wait is bounded: on
-// expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
+// diagonal tiles; tile A stops one tile earlier than B.  The grid has one CTA per unit; those that
+// are resident take over the units of those that have not started yet, one after another
+// (clusterlaunchcontrol.try_cancel, producer warp), and publish them to the other warps, so faster SMs
+// take more units without a counter in memory that a launch of its own would have to clear (and whose
+// round trip the producer had to wait out: 131072 tokens x 32 heads, segment 512, budget 1024: 2.03 -> 1.83 ms).  Every wait
+// is bounded: on expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
+// One launch serves one problem or a packed batch of up to kMaxSeqs sequences (each with tensor maps of
+// its own, so that reads past a sequence's end arrive as zeros and never as a neighbour's tokens).
 #include "sm100_ptx.cuh"
 
 namespace cp {
@@ -56,6 +61,8 @@ constexpr int kRegPoolNeeded = 256 * 216 + 128 * 64;   // registers the roles ho
 // the decoding is a chain of integer divisions that would otherwise sit at the start of every unit).
 struct Unit {
   int b, h, kvh;
+  int seq;          // sequence of a packed batch (0 for a single problem)
+  int n;            // its length
   int q_tok;        // first query row of tile A
   int n_past;       // listed blocks strictly before the segment
   int n_past_tiles; // gathered tiles
@@ -83,30 +90,47 @@ struct Bars {
   unsigned long long o_done[2];
   unsigned long long sched_full[2];
   unsigned long long sched_empty[2];
+  unsigned long long clc_full;
+  __align__(16) uint32_t clc_resp[4];  // the hardware's answer to the last request for a further unit
   int sched_unit[2];
   Unit sched_u[2];                   // the published unit, decoded; its cnt carries kBadList / kEmptyUnit
   uint32_t tmem_base;
   volatile int abort_flag;
 };
 
-struct Args {
+// One sequence: where its tokens, lists and rows of lse start in the arrays of the launch.
+struct Seq {
+  int n, n1, n2;
+  int seg0;                     // segments of the sequences before it
+  int64_t tok0, idx0, cnt0, lse0;
+};
+constexpr int kMaxSeqs = 16;
+constexpr int kMaxOrder = 1024;
+
+template <int NS> struct Args {
   const int32_t* idx;
   const int32_t* cnt;
   uint16_t* O;                  // bf16 or fp16 elements
   float* lse;
   DeviceStatus* st;
-  int B, Hq, Hkv, g, n, seg, blk, k, r, n1, n2;
+  int B, Hq, Hkv, g, seg, blk, k, r;
   int64_t osb, osh, ost;
   const uint16_t *Q, *K, *V;    // only for rows that are recomputed one by one (recompute_row)
   int64_t qs[3], ks[3], vs[3];
   float sm_scale;
   int dense;
   int n_units;
+  int n_seqs, n_segs;           // sequences, segments of all sequences
+  int long_first;               // order of the units: see decode_unit
+  Seq seq[NS];
+  uint16_t order[kMaxOrder];    // long_first, not dense: (segment * pairs per segment + pair), longest units first
   int o_vec32;                  // O rows are 32-byte aligned: the epilogue may use 32-byte stores
   int emul;                     // long units: part of the exponentials on the FMA pipes (see launch_attention_sm100)
   int withhold_v;               // test hook: the producer never issues V tiles, so a bounded wait must expire
-  unsigned int* work_counter;   // next unit to hand out (zeroed by the host before the launch)
 };
+// tensor maps of each sequence; the launch's tensors have up to 4 dimensions, kQ .. kVt name their boxes
+enum { kQ = 0, kKb = 1, kVb = 2, kKt = 3, kVt = 4, kMaps = 5 };   // query tile, K / V block, K / V tile
+template <int NS> struct Maps { CUtensorMap m[NS][kMaps]; };
 
 // Optional event trace (compiled only with -DCP_TRACE, never in the product build): in CTA 0 the first softmax warp of
 // each query tile, the producer and the MMA warp each append (clock, tag) pairs for units 4..7 to a region of their own
@@ -133,24 +157,38 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
 
 // ---------------------------------------------------------------- unit geometry
 
-// Units are ordered KV-head-major so that CTAs resident at the same time share K/V tiles in
-// L2; within a KV head the dense kernel takes the longest rows first.
+// Units of a segment or of a long sequence share K/V tiles with the other query heads of their KV head, so units are
+// ordered KV-head-major (within a KV head from the sequence's end, longest first for the dense kernel): the CTAs that are
+// resident together then read the same tiles through L2.  When all K and V (nearly) fit L2 together that does not matter
+// and the order is longest units first over all heads and sequences (long_first; the host sorts the (segment, pair)s by
+// the tiles they stream), which leaves the short ones to even out the ends of the CTAs: 8192 tokens x 32 heads, segment 512,
+// budget 1024: 133 -> 118 us; 32768 tokens (134 MB), budget 2048: 857 -> 836 us; dense 24576 tokens (101 MB): 3.95 -> 3.80 ms;
+// but 131072 tokens (537 MB), segment 1024, budget 4096: 6.4 -> 6.8 ms.
 // `cnt` is the unit's list length when the caller already has it, kLoadCnt to read it from global memory.
 constexpr int kLoadCnt = -2, kBadList = -1, kEmptyUnit = -3, kZeroUnit = -4;   // kEmptyUnit: no query row of the unit lies inside the sequence;
                                                                                 // kZeroUnit: an empty list -- the unit's rows are zeros
-__device__ __forceinline__ Unit decode_unit(const Args& a, int x, int cnt) {
+template <int NS>
+__device__ __forceinline__ Unit decode_unit(const Args<NS>& a, int x, int cnt) {
   Unit u;
   u.list = nullptr;
   u.cnt = 0;
+  u.seq = 0;
+  u.n = a.seq[0].n;
   if (a.dense) {
-    const int ntiles = (a.n + kTile - 1) / kTile;
+    const int ntiles = (u.n + kTile - 1) / kTile;
     const int np = (ntiles + 1) / 2;
-    const int per_kvh = a.g * np;
-    const int bkv = x / per_kvh;
-    const int rest = x - bkv * per_kvh;
-    const int pair = np - 1 - rest / a.g;
-    const int gi = rest % a.g;
-    u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + gi;
+    int pair;
+    if (a.long_first) {
+      const int heads = a.B * a.Hq, bh = x % heads;
+      pair = np - 1 - x / heads;
+      u.b = bh / a.Hq; u.h = bh % a.Hq; u.kvh = u.h / a.g;
+    } else {
+      const int per_kvh = a.g * np;
+      const int bkv = x / per_kvh;
+      const int rest = x - bkv * per_kvh;
+      pair = np - 1 - rest / a.g;
+      u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + rest % a.g;
+    }
     u.q_tok = pair * 256;
     u.n_past = 0; u.n_past_tiles = 0; u.last_cols = kTile;
     u.c_tok = 0; u.n_cont = 2 * pair; u.d_tok = pair * 256;
@@ -159,25 +197,39 @@ __device__ __forceinline__ Unit decode_unit(const Args& a, int x, int cnt) {
   } else {
     const int q_tiles = a.seg / kTile;
     const int pp = (q_tiles + 1) / 2;
-    const int gi_p = a.g * pp;
-    const int per_kvh = a.n1 * gi_p;
-    const int bkv = x / per_kvh;
-    const int rest = x - bkv * per_kvh;
-    const int j = a.n1 - 1 - rest / gi_p;
-    const int gi = (rest % gi_p) / pp;
-    const int p = rest % pp;
-    u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + gi;
+    int j, p;
+    if (a.long_first) {
+      const int heads = a.B * a.Hq, bh = x % heads;
+      const int y = a.order[x / heads];
+      j = y / pp;
+      p = y % pp;
+      if constexpr (NS > 1) {
+        while (u.seq + 1 < a.n_seqs && j >= a.seq[u.seq + 1].seg0) ++u.seq;
+        j -= a.seq[u.seq].seg0;
+        u.n = a.seq[u.seq].n;
+      }
+      u.b = bh / a.Hq; u.h = bh % a.Hq; u.kvh = u.h / a.g;
+    } else {
+      const int gi_p = a.g * pp;
+      const int per_kvh = a.n_segs * gi_p;
+      const int bkv = x / per_kvh;
+      const int rest = x - bkv * per_kvh;
+      j = a.n_segs - 1 - rest / gi_p;
+      p = rest % pp;
+      u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + (rest % gi_p) / pp;
+    }
+    const Seq& sq = a.seq[u.seq];
     u.seg_j = j;
     u.q_tok = j * a.seg + p * 256;
-    const long long unit = ((long long)u.b * a.Hq + u.h) * a.n1 + j;
-    u.list = a.idx + unit * a.k;
-    u.cnt = cnt == kLoadCnt ? a.cnt[unit] : cnt;
-    u.rj = min(a.n2, (j + 1) * a.r) - j * a.r;
+    const long long unit = ((long long)u.b * a.Hq + u.h) * sq.n1 + j;
+    u.list = a.idx + sq.idx0 + unit * a.k;
+    u.cnt = cnt == kLoadCnt ? a.cnt[sq.cnt0 + unit] : cnt;
+    u.rj = min(sq.n2, (j + 1) * a.r) - j * a.r;
     u.n_past = min(max(u.cnt - u.rj, 0), a.k);
     u.n_past_tiles = (u.n_past * a.blk + kTile - 1) / kTile;
     u.last_cols = u.n_past * a.blk - (u.n_past_tiles - 1) * kTile;
     u.c_tok = j * a.seg; u.n_cont = 2 * p; u.d_tok = u.q_tok;
-    u.nB = (2 * p + 1 < q_tiles && u.q_tok + kTile < a.n) ? 1 : 0;   // tile B exists and starts inside the sequence
+    u.nB = (2 * p + 1 < q_tiles && u.q_tok + kTile < u.n) ? 1 : 0;   // tile B exists and starts inside the sequence
   }
   u.generic = 0;
   u.rowsB = u.nB ? 1 : 0;
@@ -191,9 +243,10 @@ __device__ __forceinline__ Unit decode_unit(const Args& a, int x, int cnt) {
 // each a block the segment can see (0 <= b < (j+1)*r).  Returns 0 when the list has the form the selection emits
 // (past blocks, then exactly the diagonal blocks of the segment: the fast tile sequence applies), 1 for any other
 // valid list (generic tile sequence), -1 for a list that breaks the contract.
-__device__ __forceinline__ int classify_unit(const Args& a, const Unit& u, int lane) {
+template <int NS>
+__device__ __forceinline__ int classify_unit(const Args<NS>& a, const Unit& u, int lane) {
   if (a.dense) return 0;
-  const int vis = min(a.n2, (u.seg_j + 1) * a.r);
+  const int vis = min(a.seq[u.seq].n2, (u.seg_j + 1) * a.r);
   bool gen_ok = (u.cnt >= 0) && (u.cnt <= a.k);
   bool std_ok = gen_ok && (u.cnt >= u.rj);
   if (gen_ok) {
@@ -210,27 +263,49 @@ __device__ __forceinline__ int classify_unit(const Args& a, const Unit& u, int l
   return !gen_ok ? -1 : (std_ok ? 0 : 1);
 }
 
-__device__ __forceinline__ bool stop_requested(const Args& a, Bars* bars) {
+template <int NS>
+__device__ __forceinline__ bool stop_requested(const Args<NS>& a, Bars* bars) {
   return bars->abort_flag || (a.st != nullptr && *reinterpret_cast<volatile int32_t*>(&a.st->code) == CP_ERR_TIMEOUT);
 }
 
 // ---------------------------------------------------------------- unit scheduler
-// Units are handed out dynamically (an atomic counter in global memory) so that SMs that run
-// faster take more of them.  The producer warp draws the q-th unit of this CTA, reads and checks
+// The producer warp gets the q-th unit of this CTA (its own block index first, then those of CTAs that the hardware
+// lets it cancel; the request for the next one is on its way while the current one is served), reads and checks
 // its block list, and publishes (unit, list length) through a two-entry ring; the MMA warp and
 // the eight softmax warps take it from there and touch no global memory at a unit's start.
 // A list that breaks its contract is published with length kBadList and skipped by everyone.
-__device__ __forceinline__ bool publish_unit(const Args& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
+__device__ __forceinline__ void request_unit(Bars* bars) {
+  mbar_expect_tx(&bars->clc_full, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(smem_u32(bars->clc_resp)), "r"(smem_u32(&bars->clc_full)) : "memory");
+}
+// block index of the cancelled CTA, or `none` when every CTA has started (no further request may be made then)
+__device__ __forceinline__ int requested_unit(Bars* bars, int none) {
+  uint32_t ok, x;
+  asm volatile(
+      "{\n.reg .pred p;\n.reg .b128 r;\nld.shared.b128 r, [%2];\n"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\nselp.u32 %0, 1, 0, p;\nmov.u32 %1, 0;\n"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, _, _, _}, r;\n}"
+      : "=r"(ok), "=r"(x) : "r"(smem_u32(bars->clc_resp)) : "memory");
+  return ok ? int(x) : none;
+}
+template <int NS>
+__device__ __forceinline__ bool publish_unit(const Args<NS>& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
   const uint32_t slot = q & 1;
   if (q >= 2 && !mbar_wait(&bars->sched_empty[slot], ((q >> 1) - 1) & 1, bars, a.st, 50)) return false;
-  int x = 0;
-  if (lane == 0) x = int(min(atomicAdd(a.work_counter, 1u), 0x7fffffffu));
-  x = __shfl_sync(0xffffffffu, x, 0);
+  int x = int(blockIdx.x);
+  if (q > 0) {
+    if (!mbar_wait(&bars->clc_full, (q - 1) & 1, bars, a.st, 52)) return false;
+    x = requested_unit(bars, a.n_units);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one is written
+  }
+  __syncwarp();
+  if (lane == 0 && x < a.n_units) request_unit(bars);
   int cnt = 0;
   if (x < a.n_units) {
     *u_out = decode_unit(a, x, kLoadCnt);
     cnt = u_out->cnt;
-    if (u_out->q_tok >= a.n) {
+    if (u_out->q_tok >= u_out->n) {
       cnt = kEmptyUnit;                               // a short last segment has fewer units
     } else {
       const int cls = classify_unit(a, *u_out, lane);
@@ -260,7 +335,8 @@ __device__ __forceinline__ bool publish_unit(const Args& a, Bars* bars, uint32_t
   *x_out = x;
   return true;
 }
-__device__ __forceinline__ bool receive_unit(const Args& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
+template <int NS>
+__device__ __forceinline__ bool receive_unit(const Args<NS>& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
   const uint32_t slot = q & 1;
   if (!mbar_wait(&bars->sched_full[slot], (q >> 1) & 1, bars, a.st, 51)) return false;
   *x_out = *reinterpret_cast<volatile int*>(&bars->sched_unit[slot]);
@@ -281,13 +357,14 @@ __device__ __forceinline__ float elem_f32(uint16_t x, bool f16) {
 // One row of a 64-channel head in plain fp32, key by key, by one thread.  A tile's MMA multiplies the zero probability of a
 // key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row whose
 // output came out as NaN or infinite is therefore evaluated again over exactly the keys it sees.
-template <bool kF16>
-__device__ __noinline__ void recompute_row(const Args* ap, int b, int h, const int32_t* list, int cnt, int t) {
-  const Args& a = *ap;
-  const uint16_t* q = a.Q + b * a.qs[0] + h * a.qs[1] + int64_t(t) * a.qs[2];
-  const uint16_t* kb = a.K + b * a.ks[0] + (h / a.g) * a.ks[1];
-  const uint16_t* vb = a.V + b * a.vs[0] + (h / a.g) * a.vs[1];
-  uint16_t* o = a.O + b * a.osb + h * a.osh + int64_t(t) * a.ost;
+template <bool kF16, int NS>
+__device__ __noinline__ void recompute_row(const Args<NS>* ap, int seq, int b, int h, const int32_t* list, int cnt, int t) {
+  const Args<NS>& a = *ap;
+  const Seq& sq = a.seq[seq];
+  const uint16_t* q = a.Q + b * a.qs[0] + h * a.qs[1] + (sq.tok0 + t) * a.qs[2];
+  const uint16_t* kb = a.K + b * a.ks[0] + (h / a.g) * a.ks[1] + sq.tok0 * a.ks[2];
+  const uint16_t* vb = a.V + b * a.vs[0] + (h / a.g) * a.vs[1] + sq.tok0 * a.vs[2];
+  uint16_t* o = a.O + b * a.osb + h * a.osh + (sq.tok0 + t) * a.ost;
   const int n_ranges = a.dense ? 1 : cnt;
   auto logit = [&](int key) {
     float s = 0.f;
@@ -316,11 +393,11 @@ __device__ __noinline__ void recompute_row(const Args* ap, int b, int h, const i
     const float inv = l > 0.f ? 1.f / l : 0.f;
     for (int c = 0; c < 16; ++c) o[c0 + c] = uint16_t(pack2<kF16>(acc[c] * inv, 0.f));
   }
-  if (a.lse != nullptr) a.lse[((long long)b * a.Hq + h) * a.n + t] = m + logf(l);
+  if (a.lse != nullptr) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m + logf(l);
 }
 
-template <bool kF16, int D>
-__device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int which, int warp_in_wg, int lane) {
+template <bool kF16, int D, int NS>
+__device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int which, int warp_in_wg, int lane) {
   constexpr bool kSplitP = Shape<D>::kSplitP;
   const uint32_t tm = bars->tmem_base;
   const uint32_t lane_off = uint32_t(warp_in_wg * 32) << 16;
@@ -340,11 +417,11 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
     if (u.cnt == kZeroUnit) {
       // an empty list: no key is visible to any row of the unit -- zeros, and lse = ln 0
       const int t = u.q_tok + which * kTile + row;
-      if ((which == 0 || u.rowsB) && t < a.n) {
-        uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + int64_t(t) * a.ost);
+      if ((which == 0 || u.rowsB) && t < u.n) {
+        uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost);
 #pragma unroll
         for (int i = 0; i < D * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (a.lse != nullptr) a.lse[((long long)u.b * a.Hq + u.h) * a.n + t] = -CUDART_INF;
+        if (a.lse != nullptr) a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] = -CUDART_INF;
       }
       continue;
     }
@@ -476,7 +553,7 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
     ++n_units;
     tc_fence_after();
     const int t = u.q_tok + which * kTile + row;
-    uint16_t* orow = a.O + u.b * a.osb + u.h * a.osh + int64_t(t) * a.ost;
+    uint16_t* orow = a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost;
     const float inv = l_run > 0.f ? 1.f / l_run : 0.f;   // a row without any visible key (generic lists only): zeros
     float odd = 0.f;                                     // NaN as soon as one output of the row is NaN or infinite
 #pragma unroll
@@ -491,7 +568,7 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
 #pragma unroll
         for (int i = 0; i < 32; ++i) odd = fmaf(__uint_as_float(ov[i]), 0.f, odd);
       }
-      if (t < a.n) {                                 // rows past the end of the sequence (ragged last tile) are dropped
+      if (t < u.n) {                                 // rows past the end of the sequence (ragged last tile) are dropped
         if (a.o_vec32) {
           // 32-byte stores: every store fills whole 32-byte sectors (a thread owns a row, so the lanes of a
           // store instruction hit 32 different rows; 16-byte stores would touch every sector twice)
@@ -504,21 +581,19 @@ __device__ __forceinline__ void softmax_role(const Args& a, Bars* bars, int whic
         }
       }
     }
-    if (a.lse != nullptr && t < a.n)
-      a.lse[((long long)u.b * a.Hq + u.h) * a.n + t] =
+    if (a.lse != nullptr && t < u.n)
+      a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] =
           m_run * a.sm_scale + (kSplitP ? logf(l_run) - kPShift<kF16, D> * 0.693147180559945f : __logf(l_run));
     if constexpr (kSplitP) {
-      if (!(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < a.n) recompute_row<kF16>(&a, u.b, u.h, u.list, u.cnt, t);
+      if (!(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n) recompute_row<kF16>(&a, u.seq, u.b, u.h, u.list, u.cnt, t);
     }
     CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 4);            // epilogue done
   }
 }
 
 // ---------------------------------------------------------------- producer role
-template <int D>
-__device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_t smem_base, const CUtensorMap* tmQ,
-                                              const CUtensorMap* tmKb, const CUtensorMap* tmVb,
-                                              const CUtensorMap* tmKt, const CUtensorMap* tmVt, int lane) {
+template <int D, int NS>
+__device__ __forceinline__ void producer_role(const Args<NS>& a, Bars* bars, uint32_t smem_base, const Maps<NS>& maps, int lane) {
   constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes, kHalves = Shape<D>::kHalves;
   const int bpt = kTile / a.blk;
   CP_EV_DECL;
@@ -539,6 +614,7 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
     if (!publish_unit(a, bars, q + 1, lane, &x, &u)) return;
     CP_EV(lane == 0, q, 301);                                                // unit q+1 published
     if (u_cur.cnt == kBadList || u_cur.cnt == kEmptyUnit || u_cur.cnt == kZeroUnit) continue;
+    const CUtensorMap* tm = maps.m[NS > 1 ? u_cur.seq : 0];
     // Q tiles: the buffer is free once every QK^T of the previous unit has completed
     if (n_units > 0 && !mbar_wait(&bars->q_empty, (n_units - 1) & 1, bars, a.st, 31)) return;
     CP_EV(lane == 0, q, 302);                                                // Q buffer free: Q loads go out
@@ -547,7 +623,7 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
       mbar_expect_tx(&bars->q_full, nq * kTileBytes);
       for (int w = 0; w < nq; ++w)
         for (int hf = 0; hf < kHalves; ++hf)
-          tma_load_4d(smem_base + Shape<D>::kSmemQ + w * kTileBytes + hf * kHalfBytes, tmQ, &bars->q_full, hf * 64,
+          tma_load_4d(smem_base + Shape<D>::kSmemQ + w * kTileBytes + hf * kHalfBytes, tm + kQ, &bars->q_full, hf * 64,
                       u_cur.q_tok + w * kTile, u_cur.h, u_cur.b);
     }
     ++n_units;
@@ -562,19 +638,17 @@ __device__ __forceinline__ void producer_role(const Args& a, Bars* bars, uint32_
         unsigned long long* bar = &bars->kv_full[slot];
         mbar_expect_tx(bar, kTileBytes);
         if (jt < u_cur.n_past_tiles) {
-          const CUtensorMap* tm = is_v ? tmVb : tmKb;
           for (int q = 0; q < bpt; ++q) {
             const int li = jt * bpt + q;
             // boxes beyond the list read past the end of the tensor and arrive as zeros
-            const int tok = li < u_cur.n_past ? u_cur.list[li] * a.blk : a.n;
+            const int tok = li < u_cur.n_past ? u_cur.list[li] * a.blk : u_cur.n;
             for (int hf = 0; hf < kHalves; ++hf)
-              tma_load_4d(dst + hf * kHalfBytes + q * a.blk * 128, tm, bar, hf * 64, tok, u_cur.kvh, u_cur.b);
+              tma_load_4d(dst + hf * kHalfBytes + q * a.blk * 128, tm + (is_v ? kVb : kKb), bar, hf * 64, tok, u_cur.kvh, u_cur.b);
           }
         } else {
-          const CUtensorMap* tm = is_v ? tmVt : tmKt;
           const int ci = jt - u_cur.n_past_tiles;
           const int tok = ci < u_cur.n_cont ? u_cur.c_tok + ci * kTile : u_cur.d_tok + (ci - u_cur.n_cont) * kTile;
-          for (int hf = 0; hf < kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, bar, hf * 64, tok, u_cur.kvh, u_cur.b);
+          for (int hf = 0; hf < kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm + (is_v ? kVt : kKt), bar, hf * 64, tok, u_cur.kvh, u_cur.b);
         }
       }
       __syncwarp();
@@ -605,8 +679,8 @@ __device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint3
   }
 }
 
-template <bool kF16, int D>
-__device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t smem_base, int lane) {
+template <bool kF16, int D, int NS>
+__device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t smem_base, int lane) {
   constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes;
   const uint32_t tm = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 256 + D};
@@ -676,11 +750,9 @@ __device__ __forceinline__ void mma_role(const Args& a, Bars* bars, uint32_t sme
 }
 
 // ---------------------------------------------------------------- kernel
-template <bool kF16, int D>
+template <bool kF16, int D, int NS>
 __global__ void __launch_bounds__(kThreads, 1)
-attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKb,
-                       const __grid_constant__ CUtensorMap tmVb, const __grid_constant__ CUtensorMap tmKt,
-                       const __grid_constant__ CUtensorMap tmVt, const __grid_constant__ Args a) {
+attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_constant__ Args<NS> a) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t smem_base = (raw + 1023u) & ~1023u;
@@ -693,14 +765,13 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     mbar_init(&bars->q_empty, 1);
     for (int i = 0; i < Shape<D>::kSlots; ++i) { mbar_init(&bars->kv_full[i], 1); mbar_init(&bars->kv_empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->s_full[i], 1); mbar_init(&bars->p_full[i], 128); mbar_init(&bars->o_done[i], 1); }
+    mbar_init(&bars->clc_full, 1);
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->sched_full[i], 1); mbar_init(&bars->sched_empty[i], 9); }
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 8 && lane == 0) {
-    prefetch_tmap(&tmQ); prefetch_tmap(&tmKb); prefetch_tmap(&tmVb); prefetch_tmap(&tmKt); prefetch_tmap(&tmVt);
-  }
+  if (warp == 8 && lane < kMaps && NS == 1) prefetch_tmap(&maps.m[0][lane]);
   if (warp == 9) { tmem_alloc(&bars->tmem_base, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
@@ -711,11 +782,11 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   static_assert(kRegPoolNeeded <= kThreads * 168, "setmaxnreg budget exceeds the launch allocation");
   if (warp < 8) {
     reg_inc<216>();
-    softmax_role<kF16, D>(a, bars, warp >> 2, warp & 3, lane);
+    softmax_role<kF16, D, NS>(a, bars, warp >> 2, warp & 3, lane);
   } else {
     reg_dec<64>();
-    if (warp == 8) producer_role<D>(a, bars, smem_base, &tmQ, &tmKb, &tmVb, &tmKt, &tmVt, lane);
-    else if (warp == 9) mma_role<kF16, D>(a, bars, smem_base, lane);
+    if (warp == 8) producer_role<D, NS>(a, bars, smem_base, maps, lane);
+    else if (warp == 9) mma_role<kF16, D, NS>(a, bars, smem_base, lane);
   }
   if (bars->abort_flag) {
     // give copies and MMAs still in flight time to land before the CTA's resources go away
@@ -747,59 +818,138 @@ bool sm100_path_applies(const cp_params& p, const Dims& m) {
          !(p.flags & CP_FLAG_FORCE_SIMT);
 }
 
-int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, const void* K, const void* V,
-                           const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st,
-                           bool dense, cudaStream_t s) {
-  CUtensorMap tmQ, tmKb, tmVb, tmKt, tmVt;
-  const bool f16 = p.dtype == CP_F16;
-  if (!make_map(&tmQ, Q, m.B, m.Hq, m.n, m.d, p.q_stride, kTile, f16) || !make_map(&tmKb, K, m.B, m.Hkv, m.n, m.d, p.k_stride, m.blk, f16) ||
-      !make_map(&tmVb, V, m.B, m.Hkv, m.n, m.d, p.v_stride, m.blk, f16) || !make_map(&tmKt, K, m.B, m.Hkv, m.n, m.d, p.k_stride, kTile, f16) ||
-      !make_map(&tmVt, V, m.B, m.Hkv, m.n, m.d, p.v_stride, kTile, f16))
+namespace {
+
+template <bool kF16, int D, int NS>
+int launch_variant(const Maps<NS>& maps, const Args<NS>& a, cudaStream_t s) {
+  auto kern = attention_sm100_kernel<kF16, D, NS>;
+  // setmaxnreg.inc blocks forever when the CTA's register pool (threads x registers the kernel was compiled
+  // to) is smaller than what the roles ask for, and no bounded wait covers that: check the real allocation of
+  // this build once per variant and refuse to launch instead.
+  static int regs_ok = 0;   // 0 = not checked yet, 1 = fits, -1 = does not fit
+  if (regs_ok == 0) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return CP_ERR_CUDA;
+    regs_ok = (fa.numRegs * kThreads >= kRegPoolNeeded) ? 1 : -1;
+  }
+  if (regs_ok < 0) return CP_ERR_UNSUPPORTED;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<D>::kSmemTotal) != cudaSuccess)
     return CP_ERR_CUDA;
-  Args a;
+  kern<<<unsigned(a.n_units), kThreads, Shape<D>::kSmemTotal, s>>>(maps, a);
+  return check_launch();
+}
+
+// (segment, pair)s that have query rows, by the tiles they stream, longest first (counting sort; equal ones from the last
+// segment down).  Returns their number, 0 when there are more than the table holds.
+template <int NS>
+int order_units(Args<NS>& a, int pp) {
+  if ((long long)a.n_segs * pp > kMaxOrder) return 0;
+  constexpr int kCosts = 256;
+  uint16_t cost[kMaxOrder];
+  int start[kCosts + 1] = {0};
+  const int m = a.k - a.r;                          // blocks before the segment that a list can hold
+  int total = 0;
+  for (int i = 0; i < a.n_seqs; ++i)
+    for (int j = 0; j < a.seq[i].n1; ++j)
+      for (int p = 0; p < pp; ++p) {
+        const long long past = (long long)j * a.r < m ? (long long)j * a.r : m;
+        const long long c = j * a.seg + p * 256 < a.seq[i].n ? (past * a.blk + kTile - 1) / kTile + 2 * p + 2 : 0;
+        const int cc = int(c < kCosts ? c : kCosts - 1);
+        cost[(a.seq[i].seg0 + j) * pp + p] = uint16_t(cc);
+        if (cc > 0) { ++start[kCosts - cc]; ++total; }   // start[x]: units of the costs above x's
+      }
+  for (int c = 1; c <= kCosts; ++c) start[c] += start[c - 1];
+  for (int e = a.n_segs * pp - 1; e >= 0; --e)
+    if (cost[e] > 0) a.order[start[kCosts - cost[e] - 1]++] = uint16_t(e);
+  return total;
+}
+
+// slots[0..n_seqs): the sequences of one launch (a single problem is one sequence that starts at 0)
+template <int NS>
+int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const void* Q, const void* K, const void* V,
+                const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st, bool dense, cudaStream_t s) {
+  const bool f16 = p.dtype == CP_F16;
+  Maps<NS> maps;
+  Args<NS> a;
+  a.n_segs = 0;
+  long long kv_tokens = 0;
+  for (int i = 0; i < n_seqs; ++i) {
+    const SeqSlot& q = slots[i];
+    auto at = [&](const void* base, const int64_t* stride) { return static_cast<const char*>(base) + q.tok * stride[2] * m.es; };
+    CUtensorMap* t = maps.m[i];
+    if (!make_map(t + kQ, at(Q, p.q_stride), m.B, m.Hq, q.len, m.d, p.q_stride, kTile, f16) ||
+        !make_map(t + kKb, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, m.blk, f16) ||
+        !make_map(t + kVb, at(V, p.v_stride), m.B, m.Hkv, q.len, m.d, p.v_stride, m.blk, f16) ||
+        !make_map(t + kKt, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, kTile, f16) ||
+        !make_map(t + kVt, at(V, p.v_stride), m.B, m.Hkv, q.len, m.d, p.v_stride, kTile, f16))
+      return CP_ERR_CUDA;
+    Seq& x = a.seq[i];
+    x.n = q.len; x.n1 = (q.len + m.seg - 1) / m.seg; x.n2 = (q.len + m.blk - 1) / m.blk;
+    x.seg0 = a.n_segs;
+    x.tok0 = q.tok; x.idx0 = q.idx; x.cnt0 = q.cnt; x.lse0 = int64_t(m.Hq) * q.tok;
+    a.n_segs += x.n1;
+    kv_tokens += q.len;
+  }
+  a.n_seqs = n_seqs;
   a.idx = idx; a.cnt = cnt; a.O = static_cast<uint16_t*>(O); a.lse = lse; a.st = st;
-  a.B = m.B; a.Hq = m.Hq; a.Hkv = m.Hkv; a.g = m.g; a.n = m.n; a.seg = m.seg; a.blk = m.blk; a.k = m.k;
-  a.r = m.r; a.n1 = m.n1; a.n2 = m.n2;
+  a.B = m.B; a.Hq = m.Hq; a.Hkv = m.Hkv; a.g = m.g; a.seg = m.seg; a.blk = m.blk; a.k = m.k;
+  a.r = m.r;
   a.osb = p.o_stride[0]; a.osh = p.o_stride[1]; a.ost = p.o_stride[2];
   a.Q = static_cast<const uint16_t*>(Q); a.K = static_cast<const uint16_t*>(K); a.V = static_cast<const uint16_t*>(V);
   for (int i = 0; i < 3; ++i) { a.qs[i] = p.q_stride[i]; a.ks[i] = p.k_stride[i]; a.vs[i] = p.v_stride[i]; }
   a.sm_scale = p.sm_scale; a.dense = dense ? 1 : 0;
   // a unit is two 128-row query tiles (one when a segment, or the sequence, has an odd tile count)
   const long long units = dense ? (long long)m.B * m.Hq * (((m.n + kTile - 1) / kTile + 1) / 2)
-                                : (long long)m.B * m.Hq * m.n1 * ((m.seg / kTile + 1) / 2);
+                                : (long long)m.B * m.Hq * a.n_segs * ((m.seg / kTile + 1) / 2);
   if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  const bool d64 = m.d == 64;
-  auto kern = d64 ? (f16 ? attention_sm100_kernel<true, 64> : attention_sm100_kernel<false, 64>)
-                  : (f16 ? attention_sm100_kernel<true, 128> : attention_sm100_kernel<false, 128>);
-  const int smem = d64 ? Shape<64>::kSmemTotal : Shape<128>::kSmemTotal, variant = (d64 ? 2 : 0) + (f16 ? 1 : 0);
-  // setmaxnreg.inc blocks forever when the CTA's register pool (threads x registers the kernel was compiled
-  // to) is smaller than what the roles ask for, and no bounded wait covers that: check the real allocation of
-  // this build once per variant and refuse to launch instead.
-  static int regs_ok[4] = {0, 0, 0, 0};   // 0 = not checked yet, 1 = fits, -1 = does not fit
-  if (regs_ok[variant] == 0) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return CP_ERR_CUDA;
-    regs_ok[variant] = (fa.numRegs * kThreads >= kRegPoolNeeded) ? 1 : -1;
-  }
-  if (regs_ok[variant] < 0) return CP_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return CP_ERR_CUDA;
   a.n_units = int(units);
+  // K and V of every head up to 160 MB (measured on both sides: see decode_unit; the L2 has 126 MB); a batch of sequences always (its neighbours in the order are the
+  // heads of one segment, so one sequence or two are in use at a time)
+  const int pp = (m.seg / kTile + 1) / 2;
+  a.long_first = (NS > 1 || kv_tokens * m.B * m.Hkv * m.d * m.es * 2 <= 160ll << 20) ? 1 : 0;
+  if (a.long_first && !dense) {
+    const int entries = order_units(a, pp);
+    if (entries > 0) a.n_units = m.B * m.Hq * entries;
+    else a.long_first = 0;                          // more segments than the table holds (never for a batch: see below)
+  }
   a.withhold_v = (p.flags & CP_FLAG_TEST_WITHHOLD_V) ? 1 : 0;
   // Moving every kEmulEvery-th pair of exponentials from the MUFU to the FMA pipes pays where units are long and the
   // kernel sits at the power cap (measured in 60-step loops: 1.6 % at 32 K/V tiles per unit) and costs where units are
   // short (3 % at 8 tiles per unit, the paper's operating point); a unit streams at most k*blk/128 tiles.
   a.emul = (dense || (long long)m.k * m.blk >= 12 * kTile) ? 1 : 0;
   a.o_vec32 = (reinterpret_cast<uintptr_t>(O) % 32 == 0 && p.o_stride[0] % 16 == 0 && p.o_stride[1] % 16 == 0 && p.o_stride[2] % 16 == 0) ? 1 : 0;
-  a.work_counter = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(st) + 128);   // inside the status block
-  if (cudaMemsetAsync(a.work_counter, 0, sizeof(unsigned int), s) != cudaSuccess) return CP_ERR_CUDA;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return CP_ERR_CUDA;
-  // persistent CTAs, one per SM (the kernel takes all of an SM's tensor memory and shared memory)
-  const unsigned grid = unsigned(units < sms ? units : sms);
-  kern<<<grid, kThreads, smem, s>>>(tmQ, tmKb, tmVb, tmKt, tmVt, a);
-  return check_launch();
+  if (m.d == 64) return f16 ? launch_variant<true, 64, NS>(maps, a, s) : launch_variant<false, 64, NS>(maps, a, s);
+  return f16 ? launch_variant<true, 128, NS>(maps, a, s) : launch_variant<false, 128, NS>(maps, a, s);
+}
+
+}  // namespace
+
+int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, const void* K, const void* V,
+                           const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st,
+                           bool dense, cudaStream_t s) {
+  const SeqSlot one{0, 0, 0, 0, m.n};
+  return launch_seqs<1>(p, m, &one, 1, Q, K, V, idx, cnt, O, lse, st, dense, s);
+}
+
+int launch_attention_sm100_varlen(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const void* Q, const void* K,
+                                  const void* V, const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st,
+                                  cudaStream_t s) {
+  const int pp = (m.seg / kTile + 1) / 2;
+  for (int i = 0; i < n_seqs;) {
+    // as many sequences as a launch has tensor maps and unit entries for; a lone one takes the single-problem launch
+    int c = 0;
+    long long entries = 0;
+    while (c < kMaxSeqs && i + c < n_seqs) {
+      entries += (long long)((slots[i + c].len + m.seg - 1) / m.seg) * pp;
+      if (entries > kMaxOrder) break;
+      ++c;
+    }
+    const int rc = c > 1 ? launch_seqs<kMaxSeqs>(p, m, slots + i, c, Q, K, V, idx, cnt, O, lse, st, false, s)
+                         : launch_seqs<1>(p, m, slots + i, 1, Q, K, V, idx, cnt, O, lse, st, false, s);
+    if (rc != CP_OK) return rc;
+    i += c > 1 ? c : 1;
+  }
+  return CP_OK;
 }
 
 }  // namespace cp

@@ -28,6 +28,9 @@ inline Dims make_dims(const cp_params& p) {
   return m;
 }
 
+// One sequence of a packed batch: where its S / idx / cnt arrays and its tokens start, and its length.
+struct SeqSlot { int64_t s, idx, cnt, tok; int len; };
+
 // Workspace layout: [status 256 B][Qmax][Qmin][Kmax][Kmin][stats][kabs]: summaries in the input dtype;
 // stats = the four log-sum-exps of every (head, segment) row, [B,Hq,n1,4] fp64; kabs = largest magnitude
 // in each key block's summaries, [B,Hkv,n2] fp32.
@@ -77,6 +80,9 @@ int launch_attention_simt(const cp_params& p, const Dims& m, const void* Q, cons
 int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, const void* K,
                            const void* V, const int32_t* idx, const int32_t* cnt, void* O,
                            float* lse, DeviceStatus* st, bool dense, cudaStream_t s);
+int launch_attention_sm100_varlen(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const void* Q, const void* K,
+                                  const void* V, const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st,
+                                  cudaStream_t s);
 bool sm100_path_applies(const cp_params& p, const Dims& m);
 int launch_project(const cp_params& p, const Dims& m, const void* X, const void* Wq, const void* Wk, const void* Wv,
                    const float* cosT, const float* sinT, int d_model, void* Q, void* K, void* V, char* ws, cudaStream_t st);

@@ -1,0 +1,40 @@
+"""More sequences than one attention launch takes, both head sizes: every sequence equals its single-sequence call bit for
+bit, and a neighbour's values that are not finite do not reach it."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2409_12490_b200 import binding as cp
+from paper_2409_12490_b200.inputs import make_uniform_qkv
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,dtype", [(128, torch.bfloat16), (64, torch.float16)])
+@pytest.mark.parametrize("lens", [[1], [1, 128, 129], [17 + 61 * i for i in range(19)], [1500, 33, 2049, 256] * 9,
+                                  [66000, 67000, 140000]])      # more segments than one launch's table of units
+def test_each_sequence_equals_its_own_call(d, dtype, lens):
+    Hq, Hkv, seg, blk, k = (4, 2, 256, 32, 12) if max(lens) < 5000 else (1, 1, 128, 128, 3)
+    total = sum(lens)
+    Q, K, V = make_uniform_qkv(1, Hq, Hkv, total, d, dtype={torch.bfloat16: "bf16", torch.float16: "f16"}[dtype], seed=len(lens))
+    pack = lambda t: t[0].permute(1, 0, 2).contiguous().cuda().permute(1, 0, 2)
+    Q, K, V = pack(Q), pack(K), pack(V)
+    cu = [0] + np.cumsum(lens).tolist()
+    if len(lens) > 1:
+        V[:, cu[1]:cu[2]] = float("inf")                       # the second sequence's values
+    prob = cp.Problem(1, Hq, Hkv, max(lens), d, seg, blk, k, dtype)
+    ws = cp.alloc_workspace(prob)
+    O, S, idx, cnt, _, lse = cp.prefill_varlen(prob, cu, Q, K, V, ws, want_lse=True)
+    assert cp.device_status(ws) == 0
+    for i, (lo, hi) in enumerate(zip(cu[:-1], cu[1:])):
+        one = cp.Problem(1, Hq, Hkv, hi - lo, d, seg, blk, k, dtype)
+        part = [t[None, :, lo:hi] for t in (Q, K, V)]
+        S1 = cp.estimate(one, part[0], part[1], ws)
+        idx1, cnt1 = cp.select(one, S1, ws)
+        O1, lse1 = cp.attention(one, *part, idx1, cnt1, ws, want_lse=True)
+        assert torch.equal(S[i], S1[0]) and torch.equal(idx[i], idx1[0]) and torch.equal(cnt[i], cnt1[0])
+        assert torch.equal(lse[Hq * lo:Hq * hi].view(Hq, hi - lo), lse1[0])
+        if i == 1:
+            assert not torch.isfinite(O[:, lo:hi].float()).any()
+        else:
+            assert torch.equal(O[:, lo:hi], O1[0]) and torch.isfinite(O[:, lo:hi].float()).all()
