@@ -9,6 +9,7 @@ from __future__ import annotations
 import ctypes
 import math
 import os
+import struct
 from dataclasses import dataclass
 
 import torch
@@ -101,17 +102,27 @@ def _check(rc: int, where: str):
         raise CritiPrefillError(rc, where)
 
 
+# cp_params as one flat record (10 int32, 12 int64 strides, 3 floats, 1 32-bit word): filling the ctypes fields and arrays one by
+# one takes longer than the call it is for (6.5 us against 2)
+_PARAMS = struct.Struct("=10i12q3fI")
+assert _PARAMS.size == ctypes.sizeof(CpParams)
+_DTYPES = {torch.bfloat16: CP_BF16, torch.float32: CP_F32, torch.float16: CP_F16}
+
+
 def _strides(t: torch.Tensor):
-    assert t.dim() == 4 and t.stride(3) == 1, "tensors are [batch, heads, tokens, head_dim] with head_dim contiguous"
-    return (ctypes.c_int64 * 3)(t.stride(0), t.stride(1), t.stride(2))
+    s = t.stride()
+    assert len(s) == 4 and s[3] == 1, "tensors are [batch, heads, tokens, head_dim] with head_dim contiguous"
+    return s[:3]
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())   # without the Stream object around it
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t):
+    return None if t is None else t.data_ptr()
 
 
 @dataclass
@@ -150,24 +161,17 @@ class Problem:
 
     def _contig(self, heads):
         n, d = self.seq_len, self.head_dim
-        return (ctypes.c_int64 * 3)(heads * n * d, n * d, d)
+        return heads * n * d, n * d, d
 
     def params(self, Q=None, K=None, V=None, O=None) -> CpParams:
-        p = CpParams()
-        p.batch, p.n_q_heads, p.n_kv_heads = self.batch, self.n_q_heads, self.n_kv_heads
-        p.seq_len, p.head_dim = self.seq_len, self.head_dim
-        p.segment_size, p.block_size, p.budget_blocks = self.segment_size, self.block_size, self.budget_blocks
-        p.dtype = {torch.bfloat16: CP_BF16, torch.float32: CP_F32, torch.float16: CP_F16}[self.dtype]
-        p.flags = self.flags
-        p.q_stride = _strides(Q) if Q is not None else self._contig(self.n_q_heads)
-        p.k_stride = _strides(K) if K is not None else self._contig(self.n_kv_heads)
-        p.v_stride = _strides(V) if V is not None else self._contig(self.n_kv_heads)
-        p.o_stride = _strides(O) if O is not None else self._contig(self.n_q_heads)
-        p.est_scale = self.est_scale
-        p.sm_scale = self.sm_scale if self.sm_scale is not None else 1.0 / math.sqrt(self.head_dim)
-        p.alpha = self.alpha
-        p.forced_blocks = self.n_sink | (self.n_local << 16)
-        return p
+        q, k = self._contig(self.n_q_heads), self._contig(self.n_kv_heads)
+        return CpParams.from_buffer_copy(_PARAMS.pack(
+            self.batch, self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim, self.segment_size, self.block_size,
+            self.budget_blocks, _DTYPES[self.dtype], self.flags,
+            *(_strides(Q) if Q is not None else q), *(_strides(K) if K is not None else k),
+            *(_strides(V) if V is not None else k), *(_strides(O) if O is not None else q),
+            self.est_scale, self.sm_scale if self.sm_scale is not None else 1.0 / math.sqrt(self.head_dim), self.alpha,
+            (self.n_sink | (self.n_local << 16)) & 0xffffffff))
 
 
 def workspace_bytes(prob: Problem) -> int:
@@ -351,7 +355,16 @@ def prefill_varlen(prob: Problem, cu_seqlens, Q, K, V, ws, S_prev=None, want_lse
 
 def prefill_layer(prob: Problem, Q, K, V, ws, S_prev=None):
     """One layer of the hot path: estimate -> select -> attention.  Returns (O, S, idx, cnt)."""
-    S = estimate(prob, Q, K, ws, S_prev=S_prev)
-    idx, cnt = select(prob, S, ws)
-    O = attention(prob, Q, K, V, idx, cnt, ws)
+    lib, stream, ws_ptr, ws_bytes = load_library(), _stream(), ws.data_ptr(), ws.numel()
+    S = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.n2), dtype=torch.float64, device=Q.device)
+    O = torch.empty_like(Q)
+    p = ctypes.byref(prob.params(Q=Q, K=K, V=V, O=O))
+    q_ptr, k_ptr, s_ptr = Q.data_ptr(), K.data_ptr(), S.data_ptr()
+    _check(lib.critiprefill_estimate(p, q_ptr, k_ptr, _ptr(S_prev), s_ptr, ws_ptr, ws_bytes, stream), "critiprefill_estimate")
+    idx = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.budget_blocks), dtype=torch.int32, device=S.device)
+    cnt = torch.empty((prob.batch, prob.n_q_heads, prob.n1), dtype=torch.int32, device=S.device)
+    idx_ptr, cnt_ptr = idx.data_ptr(), cnt.data_ptr()
+    _check(lib.critiprefill_select(p, s_ptr, idx_ptr, cnt_ptr, ws_ptr, ws_bytes, stream), "critiprefill_select")
+    _check(lib.critiprefill_attention(p, q_ptr, k_ptr, V.data_ptr(), idx_ptr, cnt_ptr, O.data_ptr(), None, ws_ptr, ws_bytes, stream),
+           "critiprefill_attention")
     return O, S, idx, cnt
