@@ -130,6 +130,7 @@ int critiprefill_decode_estimate(const cp_params* p, const void* q_last, const v
   pd.flags &= ~CP_FLAG_MASK_BEFORE_SOFTMAX;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   char* w = static_cast<char*>(ws);
+  if (decode_path_applies(m)) return launch_decode_score(pd, md, q_last, K, S_out, w, s);
   if ((rc = launch_summarize(pd, md, nullptr, K, w, s)) != CP_OK) return rc;
   const WsLayout wl = ws_layout(md);
   const size_t q_bytes = size_t(m.B) * m.Hq * m.d * m.es;      // Qmax = Qmin = q

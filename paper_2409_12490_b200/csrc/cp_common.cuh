@@ -87,6 +87,37 @@ bool sm100_path_applies(const cp_params& p, const Dims& m);
 int launch_project(const cp_params& p, const Dims& m, const void* X, const void* Wq, const void* Wk, const void* Wv,
                    const float* cosT, const float* sinT, int d_model, void* Q, void* K, void* V, char* ws, cudaStream_t st);
 
+int launch_decode_score(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* S_out, char* ws, cudaStream_t st);
+bool decode_path_applies(const Dims& m);
+
+// Programmatic dependent launch: a kernel of this library starts while its predecessor drains.  Every thread of such a kernel
+// calls pdl_wait before it touches global memory (the predecessor has then finished and its writes are visible, so nothing else
+// about stream order changes); pdl_trigger lets the successor start its own way to that point.  The pointers named in pdl_wait
+// pass through it, so that no read-only load through them (__ldg, const __restrict__) can be scheduled before the wait.
+template <typename P> __device__ __forceinline__ void asm_launder(P& ptr) { asm volatile("" : "+l"(ptr) :: "memory"); }
+template <typename... P>
+__device__ __forceinline__ void pdl_wait(P&... ptrs) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (asm_launder(ptrs), ...);
+}
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+int launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+  const cudaError_t last = cudaGetLastError();
+  return e == cudaSuccess && last == cudaSuccess ? CP_OK : CP_ERR_CUDA;
+}
+
 inline int check_launch() { return cudaGetLastError() == cudaSuccess ? CP_OK : CP_ERR_CUDA; }
 
 }  // namespace cp

@@ -1,0 +1,151 @@
+// Block criticality of the newest token (Algorithm 1 on a segment that holds one token: Qmax = Qmin = q), 16- or 32-bit keys.
+//
+// decode_logits_kernel reads the key cache once: a warp takes a key block, folds its rows into the per-channel max and min in
+// registers and multiplies them with the group's queries in fp64 right there, so the representatives never go to memory and
+// every SM takes part.  decode_score_kernel then normalises a head's two logit rows: ln S = max(l1 - lse1, l2 - lse2).  The general
+// kernels, which this replaces, wrote the representatives and scored each KV head's whole cache on one cluster of CTAs (130001
+// tokens, 8 KV heads, block 128: the pass 110 us, here 55; 41 us is the read of K at the copy rate, which bounds it).
+#include <math_constants.h>
+
+#include "score_common.cuh"
+#include "summarize.cuh"
+
+namespace cp {
+namespace {
+
+constexpr int kWarps = 8;
+constexpr int kThreads = kWarps * 32;
+
+template <typename T, int LPR>
+__global__ void __launch_bounds__(kThreads)
+decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, int64_t sb, int64_t sh, int64_t st, int Hkv, int g, int n,
+                     int blk, int n2, double est_scale, double* __restrict__ l_max, double* __restrict__ l_min) {
+  constexpr int CE = 16 / int(sizeof(T));          // channels per lane
+  constexpr int D = LPR * CE;
+  constexpr int SUBS = 32 / LPR;
+  extern __shared__ __align__(16) uint8_t smem[];
+  T* qs = reinterpret_cast<T*>(smem);              // [g][D]
+  pdl_trigger();
+  pdl_wait(q_last, K);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kvh = blockIdx.y, b = kvh / Hkv;       // b * Hkv + kv head
+  const int h0 = kvh * g;                          // b * Hq + first query head of the group
+  for (int e = threadIdx.x; e < g * LPR; e += kThreads)
+    reinterpret_cast<uint4*>(qs)[e] = __ldg(reinterpret_cast<const uint4*>(q_last + size_t(h0) * D) + e);
+  const int bb = blockIdx.x * kWarps + warp;
+  uint4 mx, mn;
+  if (bb < n2) {
+    const char* base = K + (int64_t(b) * sb + int64_t(kvh % Hkv) * sh + int64_t(bb) * blk * st) * int(sizeof(T));
+    scan_rows<T, LPR>(base, st * int(sizeof(T)), 0, min(blk, n - bb * blk), SUBS, lane, mx, mn);
+#pragma unroll
+    for (int m = LPR; m < 32; m <<= 1) { uint4 o = shfl_xor4(mx, m); vmax<T>(mx, o); o = shfl_xor4(mn, m); vmin<T>(mn, o); }
+  }
+  __syncthreads();
+  if (bb >= n2) return;
+  // (head u, max | min) products, dealt to the SUBS lane groups that hold a copy of the representatives each
+  const int sub = lane / LPR, col = lane % LPR;
+#pragma unroll 1
+  for (int t0 = 0; t0 < 2 * g; t0 += SUBS) {
+    const int t = t0 + sub;
+    const uint4 kv = (t & 1) ? mn : mx, qv = reinterpret_cast<const uint4*>(qs)[min(t >> 1, g - 1) * LPR + col];
+    const T *ke = reinterpret_cast<const T*>(&kv), *qe = reinterpret_cast<const T*>(&qv);
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int i = 0; i < CE; i += 2) {
+      s0 = fma(to_f64(qe[i]), to_f64(ke[i]), s0);
+      s1 = fma(to_f64(qe[i + 1]), to_f64(ke[i + 1]), s1);
+    }
+    s0 += s1;
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    if (col == 0 && t < 2 * g) ((t & 1) ? l_min : l_max)[size_t(h0 + (t >> 1)) * n2 + bb] = s0 * est_scale;
+  }
+}
+
+// One CTA per (batch, head): S[row] holds the Kmax logits on entry and ln S on return; l_min the Kmin logits.
+template <int NPT>
+__global__ void __launch_bounds__(kThreads)
+decode_score_kernel(double* __restrict__ S, const double* __restrict__ l_min, int n2) {
+  __shared__ double2 red[kWarps];
+  pdl_trigger();
+  pdl_wait(S, l_min);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* row = S + size_t(blockIdx.x) * n2;
+  const double* row2 = l_min + size_t(blockIdx.x) * n2;
+  double a[NPT], c[NPT];
+  double2 m = make_double2(-CUDART_INF, -CUDART_INF);
+#pragma unroll
+  for (int i = 0; i < NPT; ++i) {
+    const int x = tid + i * kThreads;
+    a[i] = x < n2 ? row[x] : -CUDART_INF;
+    c[i] = x < n2 ? row2[x] : -CUDART_INF;
+    m.x = fmax(m.x, a[i]); m.y = fmax(m.y, c[i]);
+  }
+  auto block_reduce = [&](double2 v, bool is_max) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, v.x, o), y = __shfl_xor_sync(0xffffffffu, v.y, o);
+      v.x = is_max ? fmax(v.x, x) : v.x + x; v.y = is_max ? fmax(v.y, y) : v.y + y;
+    }
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    v = red[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      v.x = is_max ? fmax(v.x, red[w].x) : v.x + red[w].x; v.y = is_max ? fmax(v.y, red[w].y) : v.y + red[w].y;
+    }
+    __syncthreads();
+    return v;
+  };
+  m = block_reduce(m, true);
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll 1
+  for (int i = 0; i < NPT; ++i) {                  // terms below e^-50 of the largest cannot change the rounded sum
+    if (tid + i * kThreads >= n2) break;
+    double av = a[0], cv = c[0];
+#pragma unroll
+    for (int x = 1; x < NPT; ++x) { av = x == i ? a[x] : av; cv = x == i ? c[x] : cv; }
+    if (!(av - m.x <= -50.0)) s.x += exp(av - m.x);
+    if (!(cv - m.y <= -50.0)) s.y += exp(cv - m.y);
+  }
+  s = block_reduce(s, false);
+  const double lse1 = m.x + log(s.x), lse2 = m.y + log(s.y);
+#pragma unroll
+  for (int i = 0; i < NPT; ++i) {
+    const int x = tid + i * kThreads;
+    if (x < n2) row[x] = fmax(a[i] - lse1, c[i] - lse2);
+  }
+}
+
+template <typename T, int LPR>
+int launch_logits(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* l_max, double* l_min, cudaStream_t st) {
+  const dim3 grid(unsigned((m.n2 + kWarps - 1) / kWarps), unsigned(m.B * m.Hkv));
+  return launch_pdl(decode_logits_kernel<T, LPR>, grid, kThreads, size_t(m.g) * m.d * m.es, st, static_cast<const T*>(q_last),
+                    static_cast<const char*>(K), p.k_stride[0], p.k_stride[1], p.k_stride[2], m.Hkv, m.g, m.n, m.blk, m.n2,
+                    double(p.est_scale), l_max, l_min);
+}
+
+}  // namespace
+
+// Blocks of up to 128 rows (a warp each), and query groups whose Kmin logits fit the workspace's key representatives
+// ([B,Hkv,n2,d] twice), whose place they take: 8 g <= 2 d es, at least 32 heads per KV head.
+bool decode_path_applies(const Dims& m) { return m.blk <= 128 && 8 * m.g <= 2 * m.d * m.es && m.B * (long long)m.Hkv <= 65535; }
+
+int launch_decode_score(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* S_out, char* ws, cudaStream_t st) {
+  double* l_min = reinterpret_cast<double*>(ws + ws_layout(m).kmax);
+  const int lpr = m.d * m.es / 16;
+  int rc = CP_ERR_UNSUPPORTED;
+  if (p.dtype == CP_BF16)
+    rc = lpr == 16 ? launch_logits<__nv_bfloat16, 16>(p, m, q_last, K, S_out, l_min, st) : launch_logits<__nv_bfloat16, 8>(p, m, q_last, K, S_out, l_min, st);
+  else if (p.dtype == CP_F16)
+    rc = lpr == 16 ? launch_logits<__half, 16>(p, m, q_last, K, S_out, l_min, st) : launch_logits<__half, 8>(p, m, q_last, K, S_out, l_min, st);
+  else
+    rc = lpr == 32 ? launch_logits<float, 32>(p, m, q_last, K, S_out, l_min, st) : launch_logits<float, 16>(p, m, q_last, K, S_out, l_min, st);
+  if (rc != CP_OK) return rc;
+  const dim3 grid(unsigned(m.B * m.Hq));
+  if (m.n2 <= 4 * kThreads) return launch_pdl(decode_score_kernel<4>, grid, kThreads, 0, st, S_out, l_min, m.n2);
+  if (m.n2 <= 16 * kThreads) return launch_pdl(decode_score_kernel<16>, grid, kThreads, 0, st, S_out, l_min, m.n2);
+  return launch_pdl(decode_score_kernel<32>, grid, kThreads, 0, st, S_out, l_min, m.n2);
+}
+
+}  // namespace cp

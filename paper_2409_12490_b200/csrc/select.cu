@@ -57,6 +57,8 @@ select_kernel(const double* __restrict__ S, int32_t* __restrict__ idx, int32_t* 
   __shared__ unsigned long long prefix_sh;
   __shared__ int remaining_sh, bin_count_sh;
   __shared__ int warp_tot[kWarps];
+  pdl_trigger();
+  pdl_wait(S);
 
   // CTA -> (batch * heads / pool + pooled head, segment); its first query head's unit is `unit`
   const int j = blockIdx.x % n1;
@@ -196,13 +198,12 @@ int launch_select(const cp_params& p, const Dims& m, const double* S, int32_t* i
   const long long units = (long long)m.B * (m.Hq / pool) * m.n1;
   if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   const int kpt = (m.n2 + kThreads - 1) / kThreads;
-  const unsigned grid = unsigned(units);
-  if (kpt <= 4) select_kernel<4><<<grid, kThreads, 0, st>>>(S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  else if (kpt <= 8) select_kernel<8><<<grid, kThreads, 0, st>>>(S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  else if (kpt <= 16) select_kernel<16><<<grid, kThreads, 0, st>>>(S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  else if (kpt <= 32) select_kernel<32><<<grid, kThreads, 0, st>>>(S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  else return CP_ERR_UNSUPPORTED;
-  return check_launch();
+  const dim3 grid(static_cast<unsigned>(units));
+  if (kpt <= 4) return launch_pdl(select_kernel<4>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 8) return launch_pdl(select_kernel<8>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 16) return launch_pdl(select_kernel<16>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 32) return launch_pdl(select_kernel<32>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  return CP_ERR_UNSUPPORTED;
 }
 
 }  // namespace cp

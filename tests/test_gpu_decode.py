@@ -1,0 +1,35 @@
+"""Block criticality of the newest token against the fp64 oracle: block sizes a warp takes and larger ones, ragged lengths, every
+type and head size, group sizes on both sides of the workspace rule, strided keys, and the longest rows of blocks."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2409_12490_b200 import binding as cp
+from paper_2409_12490_b200.inputs import make_uniform_qkv
+
+from helpers import f32
+
+pytestmark = pytest.mark.gpu
+
+TDT = {"bf16": torch.bfloat16, "f16": torch.float16, "f32": torch.float32}
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f16", 128), ("bf16", 64), ("f16", 64), ("f32", 64), ("f32", 128)])
+@pytest.mark.parametrize("B,Hkv,g,n,blk,k", [
+    (1, 1, 1, 1, 32, 4), (2, 2, 4, 257, 32, 5), (1, 2, 3, 1000, 16, 9), (1, 1, 40, 700, 64, 3), (3, 1, 8, 2049, 128, 20),
+    (1, 1, 2, 4096, 256, 6), (1, 1, 1, 4100, 4, 64), (1, 1, 2, 4096, 1, 64)])
+def test_scores_and_list_match_the_oracle(dtype, d, B, Hkv, g, n, blk, k):
+    Hq = Hkv * g
+    Q, K, V = make_uniform_qkv(B, Hq, Hkv, n, d, dtype=dtype, seed=n + g)
+    prob = cp.Problem(B, Hq, Hkv, n, d, blk, blk, k, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    q = Q[:, :, -1].contiguous()
+    Kd = K.permute(0, 2, 1, 3).contiguous().cuda().permute(0, 2, 1, 3)         # [batch, tokens, heads, d] storage
+    S = cp.decode_estimate(prob, q.cuda(), Kd, ws)
+    idx, cnt = cp.decode_select(prob, S, ws)
+    assert cp.device_status(ws) == 0
+    S_ref = oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))
+    assert np.abs(S.cpu().numpy() - S_ref).max() <= 1e-9
+    idx_ref, cnt_ref = oracle.decode_select(S.cpu().numpy(), k)
+    assert np.array_equal(idx.cpu().numpy(), idx_ref) and np.array_equal(cnt.cpu().numpy(), cnt_ref)
