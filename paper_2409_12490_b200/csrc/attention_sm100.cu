@@ -8,16 +8,17 @@
 //   warps 4-7  softmax for tile B
 //   warp  8    TMA producer: K/V tiles through a ring of 5 x 32 KB (head_dim 64: 8 x 16 KB); a gathered
 //              tile is assembled from 128/blk boxes addressed by the block list
-//   warp  9    MMA issuer (warps 10-11 idle; they complete the third warpgroup): S = Q K^T
-//              (operands in shared memory), O += P V (P read from tensor memory, where the
-//              softmax warps overwrite S with 16-bit probabilities)
+//   warp  9    MMA issuer: S = Q K^T (operands in shared memory), O += P V (P read from tensor
+//              memory, where the softmax warps overwrite S with 16-bit probabilities)
+//   warp  10   scheduler: draws the next unit, reads and checks its block list, publishes it
+//              (warp 11 is idle; it completes the third warpgroup)
 // Tensor memory (512 columns): S_A | S_B (128 fp32 columns each) | O_A | O_B (head_dim columns each).
 // The tile sequence of a unit is: gathered past tiles, contiguous unmasked tiles, then the
 // diagonal tiles; tile A stops one tile earlier than B.  The grid has one CTA per unit; those that
 // are resident take over the units of those that have not started yet, one after another
-// (clusterlaunchcontrol.try_cancel, producer warp), and publish them to the other warps, so faster SMs
+// (clusterlaunchcontrol.try_cancel, scheduler warp), and publish them to the other warps, so faster SMs
 // take more units without a counter in memory that a launch of its own would have to clear (and whose
-// round trip the producer had to wait out: 131072 tokens x 32 heads, segment 512, budget 1024: 2.03 -> 1.83 ms).  Every wait
+// round trip had to be waited out: 131072 tokens x 32 heads, segment 512, budget 1024: 2.03 -> 1.83 ms).  Every wait
 // is bounded: on expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
 // One launch serves one problem or a packed batch of up to kMaxSeqs sequences (each with tensor maps of
 // its own, so that reads past a sequence's end arrive as zeros and never as a neighbour's tokens).
@@ -28,7 +29,7 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kHalfBytes = kTile * 64 * 2;   // [128 rows x 64 cols] of 16-bit elements, 128-byte swizzled
-constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {producer, MMA, 2 idle}
+constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {producer, MMA, scheduler, idle}
 constexpr int kMaxSlots = 8;
 constexpr int kBarBytes = 512;
 // What head_dim decides.  Heads of 64 channels keep their probabilities to 32-bit accuracy: P is stored as the sum of two
@@ -91,6 +92,7 @@ struct Bars {
   unsigned long long sched_full[2];
   unsigned long long sched_empty[2];
   unsigned long long clc_full;
+  unsigned long long taken;            // the producer has begun the unit published last: the next one may be drawn
   __align__(16) uint32_t clc_resp[4];  // the hardware's answer to the last request for a further unit
   int sched_unit[2];
   Unit sched_u[2];                   // the published unit, decoded; its cnt carries kBadList / kEmptyUnit
@@ -131,24 +133,6 @@ template <int NS> struct Args {
 // tensor maps of each sequence; the launch's tensors have up to 4 dimensions, kQ .. kVt name their boxes
 enum { kQ = 0, kKb = 1, kVb = 2, kKt = 3, kVt = 4, kMaps = 5 };   // query tile, K / V block, K / V tile
 template <int NS> struct Maps { CUtensorMap m[NS][kMaps]; };
-
-// Optional event trace (compiled only with -DCP_TRACE, never in the product build): in CTA 0 the first softmax warp of
-// each query tile, the producer and the MMA warp each append (clock, tag) pairs for units 4..7 to a region of their own
-// in the workspace behind the status block (plain stores, a counter in a register: the traced warp never waits).
-#ifdef CP_TRACE
-__device__ __forceinline__ unsigned long long trace_clock() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%clock64;" : "=l"(t) :: "memory");
-  return t;
-}
-#define CP_EV_DECL unsigned ev_n = 0
-#define CP_EV(cond, q, tag) do { if ((cond) && blockIdx.x == 0 && (q) >= 4u && (q) < 8u && ev_n < 1024u) { \
-    reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(a.st) + 4096)[((tag) / 100 - 1 + ((tag) >= 110 && (tag) < 120 ? 3 : 0)) * 1024 + ev_n++] = \
-        (trace_clock() << 12) | (unsigned long long)(tag); } } while (0)
-#else
-#define CP_EV_DECL
-#define CP_EV(cond, q, tag) do { } while (0)
-#endif
 
 // bounded wait on one of this kernel's barriers (the CTA's abort flag lives in the barrier block)
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, Bars* bars, DeviceStatus* st, int site) {
@@ -269,10 +253,12 @@ __device__ __forceinline__ bool stop_requested(const Args<NS>& a, Bars* bars) {
 }
 
 // ---------------------------------------------------------------- unit scheduler
-// The producer warp gets the q-th unit of this CTA (its own block index first, then those of CTAs that the hardware
-// lets it cancel; the request for the next one is on its way while the current one is served), reads and checks
-// its block list, and publishes (unit, list length) through a two-entry ring; the MMA warp and
-// the eight softmax warps take it from there and touch no global memory at a unit's start.
+// The scheduler warp gets the q-th unit of this CTA (its own block index first, then those of CTAs that the hardware
+// lets it cancel), reads and checks its block list, and publishes (unit, list length) through a two-entry ring; the
+// other warps take it from there and touch no global memory at a unit's start.  This is a chain of three round trips
+// (3-4 K cycles): in the producer warp it held up the loads of the unit before (with it, and with one lane per box in the
+// producer: 131072 tokens, segment 512, budget 1024: 1.85 -> 1.80 ms; 1300 tokens: 36.6 -> 35.2 us; long units unchanged).
+// A unit is drawn when the producer begins the one before it, no earlier, so that no CTA sits on units at the end.
 // A list that breaks its contract is published with length kBadList and skipped by everyone.
 __device__ __forceinline__ void request_unit(Bars* bars) {
   mbar_expect_tx(&bars->clc_full, 16);
@@ -290,50 +276,56 @@ __device__ __forceinline__ int requested_unit(Bars* bars, int none) {
   return ok ? int(x) : none;
 }
 template <int NS>
-__device__ __forceinline__ bool publish_unit(const Args<NS>& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
-  const uint32_t slot = q & 1;
-  if (q >= 2 && !mbar_wait(&bars->sched_empty[slot], ((q >> 1) - 1) & 1, bars, a.st, 50)) return false;
-  int x = int(blockIdx.x);
-  if (q > 0) {
-    if (!mbar_wait(&bars->clc_full, (q - 1) & 1, bars, a.st, 52)) return false;
-    x = requested_unit(bars, a.n_units);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one is written
-  }
-  __syncwarp();
-  if (lane == 0 && x < a.n_units) request_unit(bars);
-  int cnt = 0;
-  if (x < a.n_units) {
-    *u_out = decode_unit(a, x, kLoadCnt);
-    cnt = u_out->cnt;
-    if (u_out->q_tok >= u_out->n) {
-      cnt = kEmptyUnit;                               // a short last segment has fewer units
-    } else {
-      const int cls = classify_unit(a, *u_out, lane);
-      if (cls < 0) {
-        if (lane == 0) report(a.st, CP_ERR_BOUNDS, 1, u_out->b, u_out->h, u_out->seg_j, u_out->cnt);
-        cnt = kBadList;
-      } else if (cls == 1) {
-        // any other valid list: all listed blocks are gathered, both query tiles consume every tile
-        u_out->generic = 1;
-        u_out->n_past = cnt;
-        u_out->n_past_tiles = (cnt * a.blk + kTile - 1) / kTile;
-        u_out->last_cols = cnt * a.blk - (u_out->n_past_tiles - 1) * kTile;
-        u_out->n_cont = 0;
-        u_out->nA = u_out->n_past_tiles;
-        u_out->nB = u_out->rowsB ? u_out->n_past_tiles : 0;
-        u_out->T = u_out->n_past_tiles;
-        if (u_out->T == 0) cnt = kZeroUnit;           // nothing listed: the rows are zeros
+__device__ __forceinline__ void scheduler_role(const Args<NS>& a, Bars* bars, int lane) {
+  for (uint32_t q = 0;; ++q) {
+    const uint32_t slot = q & 1;
+    if (q >= 2 && !mbar_wait(&bars->sched_empty[slot], ((q >> 1) - 1) & 1, bars, a.st, 50)) return;
+    int x = int(blockIdx.x);
+    if (q > 0) {
+      if (!mbar_wait(&bars->taken, (q - 1) & 1, bars, a.st, 53)) return;
+      __syncwarp();
+      if (lane == 0) request_unit(bars);
+      if (!mbar_wait(&bars->clc_full, (q - 1) & 1, bars, a.st, 52)) return;
+      x = requested_unit(bars, a.n_units);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one is written
+    }
+    Unit u;
+    int cnt = 0;
+    if (x < a.n_units) {
+      u = decode_unit(a, x, kLoadCnt);
+      cnt = u.cnt;
+      if (u.q_tok >= u.n) {
+        cnt = kEmptyUnit;                               // a short last segment has fewer units
+      } else {
+        const int cls = classify_unit(a, u, lane);
+        if (cls < 0) {
+          if (lane == 0) report(a.st, CP_ERR_BOUNDS, 1, u.b, u.h, u.seg_j, u.cnt);
+          cnt = kBadList;
+        } else if (cls == 1) {
+          // any other valid list: all listed blocks are gathered, both query tiles consume every tile
+          u.generic = 1;
+          u.n_past = cnt;
+          u.n_past_tiles = (cnt * a.blk + kTile - 1) / kTile;
+          u.last_cols = cnt * a.blk - (u.n_past_tiles - 1) * kTile;
+          u.n_cont = 0;
+          u.nA = u.n_past_tiles;
+          u.nB = u.rowsB ? u.n_past_tiles : 0;
+          u.T = u.n_past_tiles;
+          if (u.T == 0) cnt = kZeroUnit;           // nothing listed: the rows are zeros
+        }
       }
     }
+    u.cnt = cnt;
+    if (lane == 0) {
+      bars->sched_unit[slot] = x;
+      if (x < a.n_units) bars->sched_u[slot] = u;
+      mbar_arrive(&bars->sched_full[slot]);
+    }
+    if (x >= a.n_units) return;
+    // Only this warp reads the status word in global memory (a round trip the other roles would otherwise
+    // pay at every unit); it tells them through the CTA's abort flag, which their waits poll.
+    if (stop_requested(a, bars)) { bars->abort_flag = 1; return; }
   }
-  u_out->cnt = cnt;
-  if (lane == 0) {
-    bars->sched_unit[slot] = x;
-    if (x < a.n_units) bars->sched_u[slot] = *u_out;
-    mbar_arrive(&bars->sched_full[slot]);
-  }
-  *x_out = x;
-  return true;
 }
 template <int NS>
 __device__ __forceinline__ bool receive_unit(const Args<NS>& a, Bars* bars, uint32_t q, int lane, int* x_out, Unit* u_out) {
@@ -405,7 +397,6 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
   const uint32_t tO = tm + lane_off + 256 + which * D;
   const int row = warp_in_wg * 32 + lane;
   const float c = a.sm_scale * 1.4426950408889634f;   // logits -> log2 units
-  CP_EV_DECL;
   uint32_t n_tiles = 0;                               // S tiles consumed so far (all units)
   uint32_t n_units = 0;                               // units finished so far
 
@@ -430,9 +421,7 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
     float m_run = -CUDART_INF, l_run = 0.f;
 
     for (int jt = 0; jt < my_tiles; ++jt, ++n_tiles) {
-      CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 0);          // waiting for S
       if (!mbar_wait(&bars->s_full[which], n_tiles & 1, bars, a.st, 10 + which)) return;
-      CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 1);          // S ready
       tc_fence_after();
       uint32_t sv[128];
       tmem_ld128(tS, sv);
@@ -543,13 +532,11 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->p_full[which]);
-      CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 2);          // P handed over
     }
 
     // epilogue: O / l -> bf16 -> global.  The next unit's first PV cannot start before this
     // thread signals its next P, so O is not overwritten while it is being read.
     if (!mbar_wait(&bars->o_done[which], n_units & 1, bars, a.st, 20 + which)) return;
-    CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 3);            // O complete
     ++n_units;
     tc_fence_after();
     const int t = u.q_tok + which * kTile + row;
@@ -587,7 +574,6 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
     if constexpr (kSplitP) {
       if (!(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n) recompute_row<kF16>(&a, u.seq, u.b, u.h, u.list, u.cnt, t);
     }
-    CP_EV(warp_in_wg == 0 && lane == 0, q, 100 + which * 10 + 4);            // epilogue done
   }
 }
 
@@ -596,62 +582,57 @@ template <int D, int NS>
 __device__ __forceinline__ void producer_role(const Args<NS>& a, Bars* bars, uint32_t smem_base, const Maps<NS>& maps, int lane) {
   constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes, kHalves = Shape<D>::kHalves;
   const int bpt = kTile / a.blk;
-  CP_EV_DECL;
   uint32_t item = 0;      // K/V tiles issued so far (all units): item i lives in slot i % kSlots
   uint32_t n_units = 0;
-  // One unit of look-ahead: unit q+1 is drawn, checked and published before the loads of unit q
-  // are issued, so the other warps never wait for the counter or for the list to be read.
-  int x;
-  Unit u;
-  if (!publish_unit(a, bars, 0, lane, &x, &u)) return;
+  // lane -> box of a gathered tile: block `my_blk` of its 128/blk, half `my_hf` of head_dim
+  const int my_blk = lane / kHalves, my_hf = lane % kHalves;
   for (uint32_t q = 0;; ++q) {
-    if (x >= a.n_units) return;
-    // Only this warp reads the status word in global memory (a round trip the other roles would otherwise
-    // pay at every unit); it tells them through the CTA's abort flag, which their waits poll.
-    if (stop_requested(a, bars)) { bars->abort_flag = 1; return; }
-    const Unit u_cur = u;
-    CP_EV(lane == 0, q, 300);                                                // producer starts unit q
-    if (!publish_unit(a, bars, q + 1, lane, &x, &u)) return;
-    CP_EV(lane == 0, q, 301);                                                // unit q+1 published
-    if (u_cur.cnt == kBadList || u_cur.cnt == kEmptyUnit || u_cur.cnt == kZeroUnit) continue;
-    const CUtensorMap* tm = maps.m[NS > 1 ? u_cur.seq : 0];
+    int x;
+    Unit u;
+    if (!receive_unit(a, bars, q, lane, &x, &u) || x >= a.n_units || bars->abort_flag) return;
+    if (lane == 0) mbar_arrive(&bars->taken);
+    if (u.cnt == kBadList || u.cnt == kEmptyUnit || u.cnt == kZeroUnit) continue;
+    const CUtensorMap* tm = maps.m[NS > 1 ? u.seq : 0];
+    // token of this lane's block of gathered tile jt; boxes beyond the list read past the end of the tensor and arrive as zeros
+    auto token_of = [&](int jt) {
+      const int li = jt * bpt + my_blk;
+      return my_blk < bpt && jt < u.n_past_tiles && li < u.n_past ? u.list[li] * a.blk : u.n;
+    };
+    int tok = token_of(0);
     // Q tiles: the buffer is free once every QK^T of the previous unit has completed
     if (n_units > 0 && !mbar_wait(&bars->q_empty, (n_units - 1) & 1, bars, a.st, 31)) return;
-    CP_EV(lane == 0, q, 302);                                                // Q buffer free: Q loads go out
     if (lane == 0) {
-      const int nq = u_cur.nB ? 2 : 1;
+      const int nq = u.nB ? 2 : 1;
       mbar_expect_tx(&bars->q_full, nq * kTileBytes);
       for (int w = 0; w < nq; ++w)
         for (int hf = 0; hf < kHalves; ++hf)
           tma_load_4d(smem_base + Shape<D>::kSmemQ + w * kTileBytes + hf * kHalfBytes, tm + kQ, &bars->q_full, hf * 64,
-                      u_cur.q_tok + w * kTile, u_cur.h, u_cur.b);
+                      u.q_tok + w * kTile, u.h, u.b);
     }
     ++n_units;
-    for (int it = 0; it < 2 * u_cur.T; ++it, ++item) {   // 2*jt = K tile jt, 2*jt+1 = V tile jt
+    for (int it = 0; it < 2 * u.T; ++it, ++item) {   // 2*jt = K tile jt, 2*jt+1 = V tile jt
       const uint32_t slot = item % kSlots, use = item / kSlots;
+      const int jt = it >> 1;
+      const bool is_v = it & 1;
+      const int next_tok = is_v ? token_of(jt + 1) : 0;   // the next tile's list entries are on their way during the wait
       if (use > 0 && !mbar_wait(&bars->kv_empty[slot], (use - 1) & 1, bars, a.st, 30)) return;
-      CP_EV(lane == 0, q, 310 + (it < 40 ? it : 40));                        // slot free: K/V item `it` goes out
-      if (lane == 0 && !(a.withhold_v && (it & 1))) {
-        const int jt = it >> 1;
-        const bool is_v = it & 1;
+      if (!(a.withhold_v && is_v)) {
         const uint32_t dst = smem_base + Shape<D>::kSmemKV + slot * kTileBytes;
         unsigned long long* bar = &bars->kv_full[slot];
-        mbar_expect_tx(bar, kTileBytes);
-        if (jt < u_cur.n_past_tiles) {
-          for (int q = 0; q < bpt; ++q) {
-            const int li = jt * bpt + q;
-            // boxes beyond the list read past the end of the tensor and arrive as zeros
-            const int tok = li < u_cur.n_past ? u_cur.list[li] * a.blk : u_cur.n;
-            for (int hf = 0; hf < kHalves; ++hf)
-              tma_load_4d(dst + hf * kHalfBytes + q * a.blk * 128, tm + (is_v ? kVb : kKb), bar, hf * 64, tok, u_cur.kvh, u_cur.b);
-          }
-        } else {
-          const int ci = jt - u_cur.n_past_tiles;
-          const int tok = ci < u_cur.n_cont ? u_cur.c_tok + ci * kTile : u_cur.d_tok + (ci - u_cur.n_cont) * kTile;
-          for (int hf = 0; hf < kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm + (is_v ? kVt : kKt), bar, hf * 64, tok, u_cur.kvh, u_cur.b);
+        if (lane == 0) mbar_expect_tx(bar, kTileBytes);
+        __syncwarp();
+        // one lane per box: the list entries are read and the loads issued side by side, not one after another
+        if (jt < u.n_past_tiles) {
+          if (my_blk < bpt)
+            tma_load_4d(dst + my_hf * kHalfBytes + my_blk * a.blk * 128, tm + (is_v ? kVb : kKb), bar, my_hf * 64, tok, u.kvh, u.b);
+        } else if (lane < kHalves) {
+          const int ci = jt - u.n_past_tiles;
+          const int t0 = ci < u.n_cont ? u.c_tok + ci * kTile : u.d_tok + (ci - u.n_cont) * kTile;
+          tma_load_4d(dst + lane * kHalfBytes, tm + (is_v ? kVt : kKt), bar, lane * 64, t0, u.kvh, u.b);
         }
       }
       __syncwarp();
+      if (is_v) tok = next_tok;
     }
   }
 }
@@ -685,7 +666,6 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
   const uint32_t tm = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 256 + D};
   const uint32_t qA = smem_base + Shape<D>::kSmemQ, qB = qA + kTileBytes;
-  CP_EV_DECL;
   uint32_t item0 = 0;                 // first K/V item of the current unit
   uint32_t nA = 0, nB = 0;            // P tiles consumed so far per query tile (all units)
   uint32_t n_units = 0;
@@ -696,16 +676,12 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
   for (uint32_t q = 0;; ++q) {
     int x;
     Unit u;
-    CP_EV(lane == 0, q, 205);                                                // asks for the unit
     if (!receive_unit(a, bars, q, lane, &x, &u) || x >= a.n_units || bars->abort_flag) return;
     if (u.cnt == kBadList || u.cnt == kEmptyUnit || u.cnt == kZeroUnit) continue;
     const int T = u.T, TA = u.nA;
     const bool hasB = u.nB > 0;
-    CP_EV(lane == 0, q, 200);                                                // unit received
     if (!mbar_wait(&bars->q_full, n_units & 1, bars, a.st, 41)) return;
-    CP_EV(lane == 0, q, 201);                                                // Q ready
     if (!full_wait(item0)) return;
-    CP_EV(lane == 0, q, 202);                                                // K0 ready
     tc_fence_after();
     issue_qk<kF16, D>(tS[0], qA, slot_addr(item0)); umma_commit(&bars->s_full[0]);
     if (hasB) { issue_qk<kF16, D>(tS[1], qB, slot_addr(item0)); umma_commit(&bars->s_full[1]); }
@@ -719,7 +695,6 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
       const uint32_t v_smem = slot_addr(iv), kn_smem = slot_addr(ik);
       if (jt < TA) {
         if (!mbar_wait(&bars->p_full[0], nA & 1, bars, a.st, 42)) return;
-        CP_EV(lane == 0, q, 210);                                            // P_A ready
         ++nA;
         tc_fence_after();
         issue_pv<kF16, D>(tO[0], tS[0], v_smem, jt > 0);
@@ -727,9 +702,7 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
         else umma_commit(&bars->o_done[0]);
       }
       if (hasB) {
-        CP_EV(lane == 0, q, 211);                                            // group A issued
         if (!mbar_wait(&bars->p_full[1], nB & 1, bars, a.st, 43)) return;
-        CP_EV(lane == 0, q, 212);                                            // P_B ready
         ++nB;
         tc_fence_after();
         issue_pv<kF16, D>(tO[1], tS[1], v_smem, jt > 0);
@@ -742,7 +715,6 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
       } else if (hasB) {
         umma_commit(&bars->o_done[1]);
       }
-      CP_EV(lane == 0, q, 213);                                              // tile step issued
     }
     item0 += 2 * T;
     ++n_units;
@@ -766,7 +738,8 @@ attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_const
     for (int i = 0; i < Shape<D>::kSlots; ++i) { mbar_init(&bars->kv_full[i], 1); mbar_init(&bars->kv_empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->s_full[i], 1); mbar_init(&bars->p_full[i], 128); mbar_init(&bars->o_done[i], 1); }
     mbar_init(&bars->clc_full, 1);
-    for (int i = 0; i < 2; ++i) { mbar_init(&bars->sched_full[i], 1); mbar_init(&bars->sched_empty[i], 9); }
+    mbar_init(&bars->taken, 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(&bars->sched_full[i], 1); mbar_init(&bars->sched_empty[i], 10); }   // 8 softmax warps, producer, MMA
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -787,6 +760,7 @@ attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_const
     reg_dec<64>();
     if (warp == 8) producer_role<D, NS>(a, bars, smem_base, maps, lane);
     else if (warp == 9) mma_role<kF16, D, NS>(a, bars, smem_base, lane);
+    else if (warp == 10) scheduler_role<NS>(a, bars, lane);
   }
   if (bars->abort_flag) {
     // give copies and MMAs still in flight time to land before the CTA's resources go away
