@@ -234,9 +234,9 @@ int critiprefill_dense_attention(const cp_params* p, const void* Q, const void* 
  *   S_prev      in  device, nullable; S_out, idx, cnt  out device: the per-sequence arrays of critiprefill_estimate /
  *               critiprefill_select ([Hq,n1_i,n2_i] fp64, [Hq,n1_i,k] int32, [Hq,n1_i] int32 with n1_i, n2_i from
  *               len_i) stored one after another in sequence order; critiprefill_varlen_sizes gives the totals
- * The sequences go through the same kernels as the single-sequence calls (where the tensor-core attention kernel applies, all
- * of them in one launch), so each sequence's results are those of critiprefill_estimate + _select + _attention on its slice,
- * bit for bit.
+ * The sequences go through the same kernels as the single-sequence calls, many of them in one launch, so each sequence's
+ * results are those of critiprefill_estimate + _select + _attention on its slice, bit for bit.  Representatives live in `ws`
+ * while scores are formed: a workspace with room for more sequences (their workspace_bytes added up) saves launches.
  * Errors: CP_ERR_SHAPE for a bad cu_seqlens or batch != 1; otherwise as the single-sequence calls. */
 int critiprefill_prefill_varlen(const cp_params* p, const int32_t* cu_seqlens, int32_t n_seqs, const void* Q,
                                 const void* K, const void* V, const double* S_prev, double* S_out, int32_t* idx,

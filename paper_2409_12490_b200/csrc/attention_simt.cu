@@ -137,6 +137,9 @@ __global__ void __launch_bounds__(kThreads * NG)
 attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
   using S = SimtShape<T, D, RT, NG>;
   constexpr int kBM = S::kBM, kKS = S::kKS, kPS = S::kPS, kQS = D + 4;
+  const int32_t* idx = a.idx;
+  pdl_trigger();
+  pdl_wait(idx);
   extern __shared__ __align__(16) uint8_t smem[];
   float* qs = reinterpret_cast<float*>(smem);              // [kBM][kQS]
   const int grp = NG > 1 ? threadIdx.x / kThreads : 0;
@@ -169,7 +172,7 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
   int cnt = 0, n_keys = t_end;                                      // positions of the key sequence the CTA walks
   if (!a.dense) {
     const long long u = (long long)bh * n1 + j;
-    list = a.idx + u * a.k;
+    list = idx + u * a.k;
     cnt = a.cnt[u];
     if (warp == 0) {
       const bool ok = list_ok(list, cnt, j, a.r, n2, a.k, lane);
@@ -390,8 +393,7 @@ int launch_rt(const SimtArgs<T>& a0, const Dims& m, cudaStream_t s) {
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   auto kern = attention_simt_kernel<T, D, RT, NG>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kSmem)) != cudaSuccess) return CP_ERR_CUDA;
-  kern<<<unsigned(ctas), kThreads * NG, S::kSmem, s>>>(a);
-  return check_launch();
+  return launch_pdl(kern, dim3(unsigned(ctas)), kThreads * NG, S::kSmem, s, a);
 }
 
 template <typename T, int D>

@@ -749,6 +749,7 @@ attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_wait();
 
   // Register re-partition.  The pool is what the CTA was launched with (384 threads x 168):
   // 256 x 216 + 128 x 64 = 63488 fits; asking for more than the pool would block forever.
@@ -809,8 +810,7 @@ int launch_variant(const Maps<NS>& maps, const Args<NS>& a, cudaStream_t s) {
   if (regs_ok < 0) return CP_ERR_UNSUPPORTED;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<D>::kSmemTotal) != cudaSuccess)
     return CP_ERR_CUDA;
-  kern<<<unsigned(a.n_units), kThreads, Shape<D>::kSmemTotal, s>>>(maps, a);
-  return check_launch();
+  return launch_pdl(kern, dim3(unsigned(a.n_units)), kThreads, Shape<D>::kSmemTotal, s, maps, a);
 }
 
 // (segment, pair)s that have query rows, by the tiles they stream, longest first (counting sort; equal ones from the last

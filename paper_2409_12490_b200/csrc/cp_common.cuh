@@ -30,6 +30,15 @@ inline Dims make_dims(const cp_params& p) {
 
 // One sequence of a packed batch: where its S / idx / cnt arrays and its tokens start, and its length.
 struct SeqSlot { int64_t s, idx, cnt, tok; int len; };
+constexpr int kSeqsPerLaunch = 16;   // sequences whose descriptors travel in one launch's parameters
+
+inline Dims seq_dims(const Dims& m, int len) {
+  Dims x = m;
+  x.n = len;
+  x.n1 = (len + m.seg - 1) / m.seg;
+  x.n2 = (len + m.blk - 1) / m.blk;
+  return x;
+}
 
 // Workspace layout: [status 256 B][Qmax][Qmin][Kmax][Kmin][stats][kabs]: summaries in the input dtype;
 // stats = the four log-sum-exps of every (head, segment) row, [B,Hq,n1,4] fp64; kabs = largest magnitude
@@ -67,6 +76,14 @@ __device__ __forceinline__ void report(DeviceStatus* st, int code, int where, in
 // Kernel launchers (each returns a cp_status).
 int launch_summarize(const cp_params& p, const Dims& m, const void* Q, const void* K, char* ws,
                      cudaStream_t s);
+// the same for several sequences of a packed batch, each with a workspace of its own (ws[i])
+int launch_summarize_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, char* const* ws, int n_seqs, const void* Q,
+                          const void* K, cudaStream_t s);
+int launch_score_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, char* const* ws, int n_seqs, const double* S_prev,
+                      double* S_out, cudaStream_t s);      // sequences that score_is_split says no to
+int launch_select_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const double* S, int32_t* idx, int32_t* cnt,
+                       cudaStream_t s);
+bool score_is_split(const cp_params& p, const Dims& m);    // the scores take the two-kernel path
 int launch_score(const cp_params& p, const Dims& m, char* ws, const double* S_prev,
                  double* S_out, cudaStream_t s);
 int launch_lse(const cp_params& p, const Dims& m, char* ws, cudaStream_t s);   // stats region of ws <- row log-sum-exps

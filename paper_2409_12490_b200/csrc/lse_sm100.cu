@@ -84,8 +84,11 @@ __device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint32_t q_smem, uin
 // Kmin products of the same rows, warp 8 is the TMA producer, warp 9 the MMA issuer; all 12 warps share the exact pass.
 template <bool kF16>
 __global__ void __launch_bounds__(kThreads, 1)
-lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_constant__ CUtensorMap tmKmin, const LseArgs a) {
+lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_constant__ CUtensorMap tmKmin, const LseArgs args) {
   using T = typename Elem<kF16>::type;
+  LseArgs a = args;
+  pdl_trigger();
+  pdl_wait(a.Qmax, a.Qmin, a.Kmax, a.Kmin, a.kabs);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t smem_base = (raw + 1023u) & ~1023u;
@@ -514,8 +517,7 @@ int launch_lse(const cp_params& p, const Dims& m, char* ws, cudaStream_t st) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return CP_ERR_CUDA;
   const long long ctas = heads * (m.g / a.U) * a.n_qchunks;
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  kern<<<unsigned(ctas), kThreads, smem, st>>>(tmKmax, tmKmin, a);
-  return check_launch();
+  return launch_pdl(kern, dim3(unsigned(ctas)), kThreads, smem, st, tmKmax, tmKmin, a);
 }
 
 }  // namespace cp

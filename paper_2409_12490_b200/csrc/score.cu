@@ -20,26 +20,41 @@ constexpr int kWarps = kThreads / 32;
 // the log-sum-exp uses as a filter.  When the 4*U*n2 logits of a row group do not fit one CTA's shared
 // memory, CL CTAs of a thread-block cluster split the key blocks and merge their per-row (max, sum)
 // pairs through distributed shared memory.
-template <typename T, int D, int U>
+// One sequence of the launch (a single problem is one): its representatives, scores, sizes, and key blocks per CTA.
+template <typename T> struct ScoreSeq {
+  const T *Qmax, *Qmin, *Kmax, *Kmin;
+  const double* S_prev;
+  double* S_out;
+  int n1, n2, nb, cta_begin;
+};
+template <typename T, int NS> struct ScoreArgs { ScoreSeq<T> s[NS]; int n; };
+
+template <typename T, int D, int U, int NS>
 __global__ void __launch_bounds__(kThreads)
-score_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, const T* __restrict__ Kmax,
-             const T* __restrict__ Kmin, const double* __restrict__ S_prev, double* __restrict__ S_out,
-             int Hq, int g, int n1, int n2, int seg, int blk, double est_scale, double ln_alpha,
-             double ln_1m_alpha, int fuse, int mask_first, int CL, int nb, double* __restrict__ stats_out) {
+score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg, int blk, double est_scale, double ln_alpha,
+             double ln_1m_alpha, int fuse, int mask_first, int CL, double* stats_out) {
   extern __shared__ double smem[];
+  int si = 0;
+  while (NS > 1 && si + 1 < a.n && int(blockIdx.x) >= a.s[si + 1].cta_begin) ++si;
+  const ScoreSeq<T>& sq = a.s[NS > 1 ? si : 0];
+  const T *Qmax = sq.Qmax, *Qmin = sq.Qmin, *Kmax = sq.Kmax, *Kmin = sq.Kmin;
+  const double* S_prev = sq.S_prev;
+  double* S_out = sq.S_out;
+  const int n1 = sq.n1, n2 = sq.n2, nb = sq.nb;
+  const int cta = int(blockIdx.x) - sq.cta_begin;
   double* lg = smem;                                // [U][4][nb]
   float* lf = reinterpret_cast<float*>(smem + 4 * U * nb);   // the same logits rounded to fp32: a cheap filter for the log-sum-exp
   __shared__ double stat[4 * U];
   __shared__ double2 part[4 * U];                   // this CTA's (max, sum exp) per logit row
 
   // cluster rank -> owned key blocks [b_lo, b_lo + nloc)
-  const int rank = CL > 1 ? int(blockIdx.x % CL) : 0;
+  const int rank = CL > 1 ? cta % CL : 0;
   const int b_lo = rank * nb;
   const int nloc = max(0, min(n2, b_lo + nb) - b_lo);
 
   // CTA -> (b, kv head, head subgroup, segment)
   const int groups = g / U;
-  int x = blockIdx.x / CL;
+  int x = cta / CL;
   const int j = x % n1; x /= n1;
   const int sub = x % groups; x /= groups;
   const int kvh = x;                                 // b*Hkv + kv head
@@ -51,6 +66,11 @@ score_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, const T* __
 
   // blocks that start at or after the end of the segment are masked (line 13)
   const int visible = min(n2, ((j + 1) * seg + blk - 1) / blk);
+  __shared__ double sp_tab[kSpIntervals * kSpStride];
+  for (int e = threadIdx.x; e < kSpIntervals * kSpCoef; e += kThreads)
+    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
+  pdl_trigger();
+  pdl_wait(Qmax, Qmin, Kmax, Kmin, S_prev);
   const T* kmx_base = Kmax + size_t(kvh) * n2 * D;
   const T* kmn_base = Kmin + size_t(kvh) * n2 * D;
 
@@ -67,9 +87,6 @@ score_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, const T* __
   constexpr int SPC = CE / 4;               // MMA k-steps per load
   constexpr int QS = D + 2;                 // row stride of qs in doubles (odd number of 16-byte units: conflict-free)
   __shared__ __align__(16) double qs[8 * QS];   // B operand, row = column index n, laid out [k-step][tig][4 channels]
-  __shared__ double sp_tab[kSpIntervals * kSpStride];
-  for (int e = threadIdx.x; e < kSpIntervals * kSpCoef; e += kThreads)
-    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
   const int tig = lane & 3, grp = lane >> 2;
   if (fuse && (lane & 15) == 0) {
     // the previous layer's scores of this CTA's elements are read once, at the very end: start them towards L2 now
@@ -256,45 +273,84 @@ score_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, const T* __
   if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <typename T, int D, int U>
-int launch_u(const Dims& m, const char* ws, const WsLayout& w, const double* S_prev, double* S_out,
-             double est_scale, double alpha, int fuse, int mask_first, int CL, int nb, double* stats_out, cudaStream_t st) {
-  const size_t smem = (sizeof(double) + sizeof(float)) * (4 * size_t(U) * nb);   // fp64 logits + their fp32 copies
-  auto kern = score_kernel<T, D, U>;
+// key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until the logits of a row group fit ~200 KB per CTA; 0: they never do
+int cluster_of(const Dims& m, int U, int* nb) {
+  for (int CL = 1; CL <= 8; CL *= 2) {
+    *nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
+    if ((sizeof(double) + sizeof(float)) * 4 * size_t(U) * *nb <= 200 * 1024) return CL;
+  }
+  return 0;
+}
+// as many heads per CTA as divide the group (the fp64 MMA has 8 rows = 4 heads x 2 representatives)
+int heads_per_cta(const Dims& m) { return m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1); }
+
+struct ScoreProblem { Dims m; const char* ws; const double* S_prev; double* S_out; };
+
+// problems that need the same cluster size, in one launch
+template <typename T, int D, int U, int NS>
+int launch_u(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* stats_out, cudaStream_t st) {
+  ScoreArgs<T, NS> a;
+  a.n = n;
+  long long ctas = 0;
+  int nb_max = 0;
+  for (int i = 0; i < n; ++i) {
+    const Dims& m = pr[i].m;
+    const WsLayout w = ws_layout(m);
+    ScoreSeq<T>& s = a.s[i];
+    s.Qmax = reinterpret_cast<const T*>(pr[i].ws + w.qmax); s.Qmin = reinterpret_cast<const T*>(pr[i].ws + w.qmin);
+    s.Kmax = reinterpret_cast<const T*>(pr[i].ws + w.kmax); s.Kmin = reinterpret_cast<const T*>(pr[i].ws + w.kmin);
+    s.S_prev = pr[i].S_prev; s.S_out = pr[i].S_out; s.n1 = m.n1; s.n2 = m.n2;
+    cluster_of(m, U, &s.nb);
+    if (s.nb > nb_max) nb_max = s.nb;
+    if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+    s.cta_begin = int(ctas);
+    ctas += (long long)m.B * m.Hkv * (m.g / U) * m.n1 * CL;
+  }
+  if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+  const Dims& m = pr[0].m;
+  const size_t smem = (sizeof(double) + sizeof(float)) * (4 * size_t(U) * nb_max);   // fp64 logits + their fp32 copies
+  auto kern = score_kernel<T, D, U, NS>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return CP_ERR_CUDA;
-  const long long ctas = (long long)m.B * m.Hkv * (m.g / U) * m.n1 * CL;
-  if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(ctas));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = unsigned(CL); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = unsigned(CL); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = CL > 1 ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(
-      &cfg, kern, reinterpret_cast<const T*>(ws + w.qmax), reinterpret_cast<const T*>(ws + w.qmin),
-      reinterpret_cast<const T*>(ws + w.kmax), reinterpret_cast<const T*>(ws + w.kmin), S_prev, S_out,
-      m.Hq, m.g, m.n1, m.n2, m.seg, m.blk, est_scale, log(alpha), log1p(-alpha), fuse, mask_first, CL, nb, stats_out);
+  cfg.numAttrs = CL > 1 ? 2 : 1;
+  const double al = double(p.alpha);
+  const int fuse = (pr[0].S_prev != nullptr && p.alpha != 1.0f) ? 1 : 0, mask_first = (p.flags & CP_FLAG_MASK_BEFORE_SOFTMAX) ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, m.Hq, m.g, m.seg, m.blk, double(p.est_scale), log(al), log1p(-al), fuse,
+                                           mask_first, CL, stats_out);
   return e == cudaSuccess ? check_launch() : CP_ERR_CUDA;
 }
 
-template <typename T, int D>
-int launch_t(const Dims& m, const char* ws, const WsLayout& w, const double* S_prev, double* S_out,
-             double est_scale, double alpha, int fuse, int mask_first, double* stats_out, cudaStream_t st) {
-  // as many heads per CTA as divide the group (the fp64 MMA has 8 rows = 4 heads x 2 representatives);
-  // key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until the logits fit ~200 KB per CTA
-  const size_t budget = 200 * 1024;
-  const int U = m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1);
-  for (int CL = 1; CL <= 8; CL *= 2) {
-    const int nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
-    if ((sizeof(double) + sizeof(float)) * 4 * size_t(U) * nb > budget) continue;
-    if (U == 4) return launch_u<T, D, 4>(m, ws, w, S_prev, S_out, est_scale, alpha, fuse, mask_first, CL, nb, stats_out, st);
-    if (U == 2) return launch_u<T, D, 2>(m, ws, w, S_prev, S_out, est_scale, alpha, fuse, mask_first, CL, nb, stats_out, st);
-    return launch_u<T, D, 1>(m, ws, w, S_prev, S_out, est_scale, alpha, fuse, mask_first, CL, nb, stats_out, st);
+template <typename T, int D, int NS>
+int launch_t(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* stats_out, cudaStream_t st) {
+  const int U = heads_per_cta(pr[0].m);
+  if (U == 4) return launch_u<T, D, 4, NS>(p, pr, n, CL, stats_out, st);
+  if (U == 2) return launch_u<T, D, 2, NS>(p, pr, n, CL, stats_out, st);
+  return launch_u<T, D, 1, NS>(p, pr, n, CL, stats_out, st);
+}
+
+template <int NS>
+int launch_problems(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* stats_out, cudaStream_t st) {
+  const int d = pr[0].m.d;
+  if (p.dtype == CP_BF16) {
+    if (d == 128) return launch_t<__nv_bfloat16, 128, NS>(p, pr, n, CL, stats_out, st);
+    if (d == 64) return launch_t<__nv_bfloat16, 64, NS>(p, pr, n, CL, stats_out, st);
+  } else if (p.dtype == CP_F16) {
+    if (d == 128) return launch_t<__half, 128, NS>(p, pr, n, CL, stats_out, st);
+    if (d == 64) return launch_t<__half, 64, NS>(p, pr, n, CL, stats_out, st);
+  } else {
+    if (d == 128) return launch_t<float, 128, NS>(p, pr, n, CL, stats_out, st);
+    if (d == 64) return launch_t<float, 64, NS>(p, pr, n, CL, stats_out, st);
   }
   return CP_ERR_UNSUPPORTED;
 }
@@ -305,21 +361,32 @@ int launch_t(const Dims& m, const char* ws, const WsLayout& w, const double* S_p
 // of every (head, segment) row, [B,Hq,n1,4], and leaves S_out alone.
 int launch_score_generic(const cp_params& p, const Dims& m, const char* ws, const double* S_prev,
                          double* S_out, double* stats_out, cudaStream_t st) {
-  const WsLayout w = ws_layout(m);
-  const int fuse = (S_prev != nullptr && p.alpha != 1.0f) ? 1 : 0;
-  const int mask_first = (p.flags & CP_FLAG_MASK_BEFORE_SOFTMAX) ? 1 : 0;
-  const double es = double(p.est_scale), al = double(p.alpha);
-  if (p.dtype == CP_BF16) {
-    if (m.d == 128) return launch_t<__nv_bfloat16, 128>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
-    if (m.d == 64) return launch_t<__nv_bfloat16, 64>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
-  } else if (p.dtype == CP_F16) {
-    if (m.d == 128) return launch_t<__half, 128>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
-    if (m.d == 64) return launch_t<__half, 64>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
-  } else {
-    if (m.d == 128) return launch_t<float, 128>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
-    if (m.d == 64) return launch_t<float, 64>(m, ws, w, S_prev, S_out, es, al, fuse, mask_first, stats_out, st);
+  const ScoreProblem pr{m, ws, S_prev, S_out};
+  int nb;
+  const int CL = cluster_of(m, heads_per_cta(m), &nb);
+  return CL == 0 ? CP_ERR_UNSUPPORTED : launch_problems<1>(p, &pr, 1, CL, stats_out, st);
+}
+
+int launch_score_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, char* const* ws, int n_seqs, const double* S_prev,
+                      double* S_out, cudaStream_t st) {
+  int nb;
+  for (int CL = 1; CL <= 8; CL *= 2) {
+    ScoreProblem pr[kSeqsPerLaunch];
+    int n = 0;
+    for (int i = 0; i <= n_seqs; ++i) {
+      if (n == kSeqsPerLaunch || (i == n_seqs && n > 0)) {
+        const int rc = launch_problems<kSeqsPerLaunch>(p, pr, n, CL, nullptr, st);
+        if (rc != CP_OK) return rc;
+        n = 0;
+      }
+      if (i == n_seqs) break;
+      const Dims q = seq_dims(m, slots[i].len);
+      const int c = cluster_of(q, heads_per_cta(q), &nb);
+      if (c == 0) return CP_ERR_UNSUPPORTED;
+      if (c == CL) pr[n++] = {q, ws[i], S_prev ? S_prev + slots[i].s : nullptr, S_out + slots[i].s};
+    }
   }
-  return CP_ERR_UNSUPPORTED;
+  return CP_OK;
 }
 
 }  // namespace cp

@@ -59,6 +59,8 @@ score_visible_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, con
 
   for (int e = tid; e < kSpIntervals * kSpCoef; e += kThreads)
     sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
+  pdl_trigger();
+  pdl_wait(Qmax, Qmin, Kmax, Kmin, stats, S_prev);
   for (int e = tid; e < U * kG * 4; e += kThreads) {
     const int u = e / (kG * 4), s = (e / 4) % kG;
     st_sh[e] = s < n_seg ? stats[unit_of(u, s) * 4 + (e & 3)] : 0.0;
@@ -172,12 +174,12 @@ int launch_visible(const Dims& m, const char* ws, const WsLayout& w, const doubl
   const int n_chunks = (m.n1 + kG - 1) / kG;
   const long long ctas = (long long)m.B * m.Hkv * (m.g / U) * n_chunks;
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  score_visible_kernel<T, 128, U><<<unsigned(ctas), kThreads, 0, st>>>(
+  return launch_pdl(
+      score_visible_kernel<T, 128, U>, dim3(unsigned(ctas)), kThreads, 0, st,
       reinterpret_cast<const T*>(ws + w.qmax), reinterpret_cast<const T*>(ws + w.qmin),
       reinterpret_cast<const T*>(ws + w.kmax), reinterpret_cast<const T*>(ws + w.kmin),
       reinterpret_cast<const double*>(ws + w.stats), S_prev, S_out, m.Hq, m.g, m.n1, m.n2, m.seg, m.blk, est_scale,
       log(alpha), log1p(-alpha), fuse, n_chunks);
-  return check_launch();
 }
 
 template <typename T>
@@ -191,15 +193,18 @@ int launch_visible_t(const Dims& m, const char* ws, const WsLayout& w, const dou
 
 }  // namespace
 
+bool score_is_split(const cp_params& p, const Dims& m) {
+  const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2;
+  return (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 &&
+         (scores >= kFastMinScores || (p.flags & CP_FLAG_FORCE_SPLIT_SCORE));
+}
+
 // K2 dispatcher.  16-bit inputs with head_dim 128 take the two-kernel path (log-sum-exps, then exact logits of
 // the visible blocks); everything else the general kernel.
 int launch_score(const cp_params& p, const Dims& m, char* ws, const double* S_prev, double* S_out, cudaStream_t st) {
   // The two-kernel path pays for an extra launch and for the serial sweeps of the log-sum-exp kernel; it wins once the
   // score map is large (measured: 2x at 33 M scores, nothing below a few million), so small maps keep the general kernel.
-  const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2;
-  const bool fast = (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 &&
-                    (scores >= kFastMinScores || (p.flags & CP_FLAG_FORCE_SPLIT_SCORE));
-  if (!fast) return launch_score_generic(p, m, ws, S_prev, S_out, nullptr, st);
+  if (!score_is_split(p, m)) return launch_score_generic(p, m, ws, S_prev, S_out, nullptr, st);
   const WsLayout w = ws_layout(m);
   int rc = launch_lse(p, m, ws, st);
   if (rc != CP_OK) return rc;

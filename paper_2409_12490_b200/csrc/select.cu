@@ -48,21 +48,30 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int lane, int warp, i
 // before any scored block (the host has checked that they fit into the k - r free slots).
 // Resident CTAs per SM are set by registers: the kernel waits on barriers most of the time, so 16 keys per thread are held to 64
 // registers (4 CTAs instead of the 3 that 80 registers allow: 13 % faster at n2 = 4096; 48 registers spill and are slower).
-template <int KPT>
+// One sequence of the launch (a single problem is one).
+struct SelectSeq { const double* S; int32_t *idx, *cnt; int n1, n2, cta_begin; };
+template <int NS> struct SelectArgs { SelectSeq s[NS]; int n; };
+
+template <int KPT, int NS>
 __global__ void __launch_bounds__(kThreads, KPT <= 4 ? 5 : (KPT <= 16 ? 4 : 2))
-select_kernel(const double* __restrict__ S, int32_t* __restrict__ idx, int32_t* __restrict__ cnt,
-              int n1, int n2, int r, int k, int pool, int n_sink, int n_local, int past_fixed) {
+select_kernel(const __grid_constant__ SelectArgs<NS> a, int r, int k, int pool, int n_sink, int n_local, int past_fixed) {
   __shared__ unsigned int hist[256];
   __shared__ int warp_sum[kWarps];
   __shared__ unsigned long long prefix_sh;
   __shared__ int remaining_sh, bin_count_sh;
   __shared__ int warp_tot[kWarps];
+  int si = 0;
+  while (NS > 1 && si + 1 < a.n && int(blockIdx.x) >= a.s[si + 1].cta_begin) ++si;
+  const SelectSeq& sq = a.s[NS > 1 ? si : 0];
+  const double* S = sq.S;
+  int32_t *idx = sq.idx, *cnt = sq.cnt;
+  const int n1 = sq.n1, n2 = sq.n2, cta = int(blockIdx.x) - sq.cta_begin;
   pdl_trigger();
   pdl_wait(S);
 
   // CTA -> (batch * heads / pool + pooled head, segment); its first query head's unit is `unit`
-  const int j = blockIdx.x % n1;
-  const int unit = (blockIdx.x / n1) * pool * n1 + j;
+  const int j = cta % n1;
+  const int unit = (cta / n1) * pool * n1 + j;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double* row = S + size_t(unit) * n2;
   const int past = past_fixed >= 0 ? past_fixed : j * r;   // past_fixed: the caller names the first diagonal block (decoding: the last block)
@@ -189,21 +198,50 @@ select_kernel(const double* __restrict__ S, int32_t* __restrict__ idx, int32_t* 
   }
 }
 
+template <int NS>
+int launch_args(const cp_params& p, const Dims& m, const SelectArgs<NS>& a, long long units, int n2_max, int past_fixed, cudaStream_t st) {
+  const int pool = (p.flags & CP_FLAG_SHARED_GROUP_LISTS) ? m.g : 1;
+  const int n_sink = p.forced_blocks & 0xffff, n_local = (p.forced_blocks >> 16) & 0xffff;
+  if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+  const int kpt = (n2_max + kThreads - 1) / kThreads;
+  const dim3 grid(static_cast<unsigned>(units));
+  if (kpt <= 4) return launch_pdl(select_kernel<4, NS>, grid, kThreads, 0, st, a, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 8) return launch_pdl(select_kernel<8, NS>, grid, kThreads, 0, st, a, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 16) return launch_pdl(select_kernel<16, NS>, grid, kThreads, 0, st, a, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  if (kpt <= 32) return launch_pdl(select_kernel<32, NS>, grid, kThreads, 0, st, a, m.r, m.k, pool, n_sink, n_local, past_fixed);
+  return CP_ERR_UNSUPPORTED;
+}
+
 }  // namespace
 
 int launch_select(const cp_params& p, const Dims& m, const double* S, int32_t* idx, int32_t* cnt,
                   cudaStream_t st, int past_fixed) {
+  SelectArgs<1> a;
+  a.s[0] = {S, idx, cnt, m.n1, m.n2, 0};
+  a.n = 1;
   const int pool = (p.flags & CP_FLAG_SHARED_GROUP_LISTS) ? m.g : 1;
-  const int n_sink = p.forced_blocks & 0xffff, n_local = (p.forced_blocks >> 16) & 0xffff;
-  const long long units = (long long)m.B * (m.Hq / pool) * m.n1;
-  if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  const int kpt = (m.n2 + kThreads - 1) / kThreads;
-  const dim3 grid(static_cast<unsigned>(units));
-  if (kpt <= 4) return launch_pdl(select_kernel<4>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  if (kpt <= 8) return launch_pdl(select_kernel<8>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  if (kpt <= 16) return launch_pdl(select_kernel<16>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  if (kpt <= 32) return launch_pdl(select_kernel<32>, grid, kThreads, 0, st, S, idx, cnt, m.n1, m.n2, m.r, m.k, pool, n_sink, n_local, past_fixed);
-  return CP_ERR_UNSUPPORTED;
+  return launch_args<1>(p, m, a, (long long)m.B * (m.Hq / pool) * m.n1, m.n2, past_fixed, st);
+}
+
+int launch_select_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const double* S, int32_t* idx, int32_t* cnt,
+                       cudaStream_t st) {
+  const int pool = (p.flags & CP_FLAG_SHARED_GROUP_LISTS) ? m.g : 1;
+  for (int i = 0; i < n_seqs; i += kSeqsPerLaunch) {
+    SelectArgs<kSeqsPerLaunch> a;
+    a.n = 0;
+    long long units = 0;
+    int n2_max = 0;
+    for (int x = i; x < n_seqs && x < i + kSeqsPerLaunch; ++x) {
+      const Dims q = seq_dims(m, slots[x].len);
+      if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+      a.s[a.n++] = {S + slots[x].s, idx + slots[x].idx, cnt + slots[x].cnt, q.n1, q.n2, int(units)};
+      units += (long long)(m.Hq / pool) * q.n1;
+      if (q.n2 > n2_max) n2_max = q.n2;
+    }
+    const int rc = launch_args<kSeqsPerLaunch>(p, m, a, units, n2_max, -1, st);
+    if (rc != CP_OK) return rc;
+  }
+  return CP_OK;
 }
 
 }  // namespace cp

@@ -59,10 +59,17 @@ struct Side {            // one tensor (Q or K) and where its summaries go
   int groups_per_cta;    // kWarps (warp-owned groups) or 1 (CTA-owned group)
 };
 
-template <typename T, int LPR>
-__global__ void __launch_bounds__(kThreads) summarize_kernel(Side q, Side k, int d) {
+template <int NS> struct Sides { Side s[2 * NS]; int n; };   // Q and K of each sequence, by cta_begin
+
+template <typename T, int LPR, int NS>
+__global__ void __launch_bounds__(kThreads) summarize_kernel(const __grid_constant__ Sides<NS> t, int d) {
   __shared__ uint4 red[2][kWarps][LPR];
-  const Side& s = (blockIdx.x >= k.cta_begin) ? k : q;
+  int si = 0;
+  while (si + 1 < t.n && blockIdx.x >= t.s[si + 1].cta_begin) ++si;
+  const Side& s = t.s[si];
+  const char* base = s.base;
+  pdl_trigger();
+  pdl_wait(base);
   const long long cta = blockIdx.x - s.cta_begin;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int RPW = 32 / LPR;
@@ -75,7 +82,7 @@ __global__ void __launch_bounds__(kThreads) summarize_kernel(Side q, Side k, int
     const int gi = int(grp % s.groups_per_head);
     const long long bh = grp / s.groups_per_head;
     const int h = int(bh % s.H), b = int(bh / s.H);
-    const char* gbase = s.base + (int64_t(b) * s.sb + int64_t(h) * s.sh + int64_t(gi) * s.G * s.st) * es;
+    const char* gbase = base + (int64_t(b) * s.sb + int64_t(h) * s.sh + int64_t(gi) * s.G * s.st) * es;
     const int rows = min(s.G, s.n - gi * s.G);
     uint4 mx, mn;
     scan_rows<T, LPR>(gbase, st_bytes, warp * RPW, rows - warp * RPW, kWarps * RPW, lane, mx, mn);
@@ -105,7 +112,7 @@ __global__ void __launch_bounds__(kThreads) summarize_kernel(Side q, Side k, int
     const int gi = int(grp % s.groups_per_head);
     const long long bh = grp / s.groups_per_head;
     const int h = int(bh % s.H), b = int(bh / s.H);
-    const char* gbase = s.base + (int64_t(b) * s.sb + int64_t(h) * s.sh + int64_t(gi) * s.G * s.st) * es;
+    const char* gbase = base + (int64_t(b) * s.sb + int64_t(h) * s.sh + int64_t(gi) * s.G * s.st) * es;
     const int rows = min(s.G, s.n - gi * s.G);
     uint4 mx, mn;
     scan_rows<T, LPR>(gbase, st_bytes, 0, rows, RPW, lane, mx, mn);
@@ -123,47 +130,64 @@ __global__ void __launch_bounds__(kThreads) summarize_kernel(Side q, Side k, int
   }
 }
 
-template <typename T, int LPR>
-int launch_t(const Side& q, const Side& k, long long ctas, int d, cudaStream_t st) {
-  summarize_kernel<T, LPR><<<(unsigned)ctas, kThreads, 0, st>>>(q, k, d);
-  return check_launch();
+template <int NS>
+int launch_sides(const cp_params& p, const Dims& m, const Sides<NS>& t, long long ctas, cudaStream_t st) {
+  if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+  const dim3 grid(static_cast<unsigned>(ctas));
+  const int lpr = m.d * m.es / 16;
+  if (p.dtype == CP_BF16) {
+    if (lpr == 16) return launch_pdl(summarize_kernel<__nv_bfloat16, 16, NS>, grid, kThreads, 0, st, t, m.d);
+    if (lpr == 8) return launch_pdl(summarize_kernel<__nv_bfloat16, 8, NS>, grid, kThreads, 0, st, t, m.d);
+  } else if (p.dtype == CP_F16) {
+    if (lpr == 16) return launch_pdl(summarize_kernel<__half, 16, NS>, grid, kThreads, 0, st, t, m.d);
+    if (lpr == 8) return launch_pdl(summarize_kernel<__half, 8, NS>, grid, kThreads, 0, st, t, m.d);
+  } else {
+    if (lpr == 32) return launch_pdl(summarize_kernel<float, 32, NS>, grid, kThreads, 0, st, t, m.d);
+    if (lpr == 16) return launch_pdl(summarize_kernel<float, 16, NS>, grid, kThreads, 0, st, t, m.d);
+  }
+  return CP_ERR_UNSUPPORTED;
+}
+
+// appends the sides of one problem whose first token is `tok`; Q == nullptr: key side only (the caller supplies the query
+// representatives itself)
+template <int NS>
+void add_problem(Sides<NS>& t, long long& ctas, const cp_params& p, const Dims& m, int64_t tok, const void* Q, const void* K, char* ws) {
+  const WsLayout w = ws_layout(m);
+  auto add = [&](const void* base, const int64_t* s, int H, int G, char* omax, char* omin, float* oabs) {
+    Side& x = t.s[t.n++];
+    x.base = static_cast<const char*>(base) + tok * s[2] * m.es; x.sb = s[0]; x.sh = s[1]; x.st = s[2];
+    x.H = H; x.G = G; x.n = m.n; x.groups_per_head = (m.n + G - 1) / G; x.omax = omax; x.omin = omin; x.oabs = oabs;
+    x.n_groups = (long long)m.B * H * x.groups_per_head;
+    x.groups_per_cta = G > 128 ? 1 : kWarps;
+    x.cta_begin = ctas;
+    ctas += (x.n_groups + x.groups_per_cta - 1) / x.groups_per_cta;
+  };
+  if (Q != nullptr) add(Q, p.q_stride, m.Hq, m.seg, ws + w.qmax, ws + w.qmin, nullptr);
+  add(K, p.k_stride, m.Hkv, m.blk, ws + w.kmax, ws + w.kmin, reinterpret_cast<float*>(ws + w.kabs));
 }
 
 }  // namespace
 
 int launch_summarize(const cp_params& p, const Dims& m, const void* Q, const void* K, char* ws,
                      cudaStream_t st) {
-  const WsLayout w = ws_layout(m);
-  auto mk = [&](const void* base, const int64_t* s, int H, int G, char* omax, char* omin) {
-    Side x;
-    x.base = static_cast<const char*>(base); x.sb = s[0]; x.sh = s[1]; x.st = s[2];
-    x.H = H; x.G = G; x.n = m.n; x.groups_per_head = (m.n + G - 1) / G; x.omax = omax; x.omin = omin; x.oabs = nullptr;
-    x.n_groups = (long long)m.B * H * x.groups_per_head;
-    x.groups_per_cta = G > 128 ? 1 : kWarps;
-    x.cta_begin = 0;
-    return x;
-  };
-  Side q = mk(Q, p.q_stride, m.Hq, m.seg, ws + w.qmax, ws + w.qmin);
-  Side k = mk(K, p.k_stride, m.Hkv, m.blk, ws + w.kmax, ws + w.kmin);
-  if (Q == nullptr) q.n_groups = 0;          // key side only (the caller supplies the query representatives itself)
-  k.oabs = reinterpret_cast<float*>(ws + w.kabs);
-  const long long q_ctas = (q.n_groups + q.groups_per_cta - 1) / q.groups_per_cta;
-  const long long k_ctas = (k.n_groups + k.groups_per_cta - 1) / k.groups_per_cta;
-  k.cta_begin = q_ctas;
-  const long long ctas = q_ctas + k_ctas;
-  if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  const int lpr = m.d * m.es / 16;
-  if (p.dtype == CP_BF16) {
-    if (lpr == 16) return launch_t<__nv_bfloat16, 16>(q, k, ctas, m.d, st);
-    if (lpr == 8) return launch_t<__nv_bfloat16, 8>(q, k, ctas, m.d, st);
-  } else if (p.dtype == CP_F16) {
-    if (lpr == 16) return launch_t<__half, 16>(q, k, ctas, m.d, st);
-    if (lpr == 8) return launch_t<__half, 8>(q, k, ctas, m.d, st);
-  } else {
-    if (lpr == 32) return launch_t<float, 32>(q, k, ctas, m.d, st);
-    if (lpr == 16) return launch_t<float, 16>(q, k, ctas, m.d, st);
+  Sides<1> t;
+  t.n = 0;
+  long long ctas = 0;
+  add_problem(t, ctas, p, m, 0, Q, K, ws);
+  return launch_sides<1>(p, m, t, ctas, st);
+}
+
+int launch_summarize_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, char* const* ws, int n_seqs, const void* Q,
+                          const void* K, cudaStream_t st) {
+  for (int i = 0; i < n_seqs; i += kSeqsPerLaunch) {
+    Sides<kSeqsPerLaunch> t;
+    t.n = 0;
+    long long ctas = 0;
+    for (int x = i; x < n_seqs && x < i + kSeqsPerLaunch; ++x) add_problem(t, ctas, p, seq_dims(m, slots[x].len), slots[x].tok, Q, K, ws[x]);
+    const int rc = launch_sides<kSeqsPerLaunch>(p, m, t, ctas, st);
+    if (rc != CP_OK) return rc;
   }
-  return CP_ERR_UNSUPPORTED;
+  return CP_OK;
 }
 
 }  // namespace cp

@@ -1,5 +1,5 @@
-"""More sequences than one attention launch takes, both head sizes: every sequence equals its single-sequence call bit for
-bit, and a neighbour's values that are not finite do not reach it."""
+"""More sequences than one launch takes, workspaces that hold them in several groups, both head sizes, sequences on either score
+path: every sequence equals its single-sequence call bit for bit, and a neighbour's values that are not finite do not reach it."""
 import numpy as np
 import pytest
 import torch
@@ -38,3 +38,23 @@ def test_each_sequence_equals_its_own_call(d, dtype, lens):
             assert not torch.isfinite(O[:, lo:hi].float()).any()
         else:
             assert torch.equal(O[:, lo:hi], O1[0]) and torch.isfinite(O[:, lo:hi].float()).all()
+
+
+@pytest.mark.parametrize("flags,dtype,d", [(cp.FLAG_FORCE_SPLIT_SCORE, torch.bfloat16, 128), (0, torch.float32, 64),
+                                           (cp.FLAG_SHARED_GROUP_LISTS | cp.FLAG_MASK_BEFORE_SOFTMAX, torch.float16, 128)])
+@pytest.mark.parametrize("room", [1, 20])                      # workspaces of the longest sequence
+def test_fused_layers_equal_their_own_calls(flags, dtype, d, room):
+    lens, Hq, Hkv, seg, blk, k = [1500, 33, 2049, 256, 700] * 4, 4, 2, 256, 4, 80
+    name = {torch.bfloat16: "bf16", torch.float16: "f16", torch.float32: "f32"}[dtype]
+    total, cu = sum(lens), [0] + np.cumsum(lens).tolist()
+    layers = [[t[0].cuda() for t in make_uniform_qkv(1, Hq, Hkv, total, d, dtype=name, seed=s)] for s in (1, 2)]
+    prob = cp.Problem(1, Hq, Hkv, max(lens), d, seg, blk, k, dtype, flags=flags)
+    ws = torch.zeros(room * cp.workspace_bytes(prob), dtype=torch.uint8, device="cuda")
+    first = cp.prefill_varlen(prob, cu, *layers[0], ws)
+    O, S, idx, cnt, _ = cp.prefill_varlen(prob, cu, *layers[1], ws, S_prev=first[4])
+    assert cp.device_status(ws) == 0
+    for i, (lo, hi) in enumerate(zip(cu[:-1], cu[1:])):
+        one = cp.Problem(1, Hq, Hkv, hi - lo, d, seg, blk, k, dtype, flags=flags)
+        O1, S1, idx1, cnt1 = cp.prefill_layer(one, *[t[None, :, lo:hi] for t in layers[1]], ws, S_prev=first[1][i][None])
+        assert torch.equal(S[i], S1[0]) and torch.equal(idx[i], idx1[0]) and torch.equal(cnt[i], cnt1[0])
+        assert torch.equal(O[:, lo:hi], O1[0])
