@@ -4,12 +4,12 @@
 //
 // GEMM on the tcgen05 tensor cores: D[128 tokens x 128 channels] = X_tile[128 x d_model] * W_head[128 x d_model]^T per
 // head; an output tile is 128 tokens of two adjacent heads of one kind (one head where a kind has an odd head count),
-// so that both heads share the X operand of every MMA.  A work unit is (batch, head group, segment): its seg/128 token
-// tiles run back to back on one CTA, so the segment's running max / min stay on chip.  Warps 0-3: epilogue (one thread
+// so that both heads share the X operand of every MMA.  A query unit is (batch, head group, segment): its seg/128 token
+// tiles run back to back on one CTA, so the segment's running max / min stay on chip; key and value units are single tiles
+// (a key block never crosses a tile), which even out what the query units leave of the last round.  Warps 0-3: epilogue (one thread
 // per token row: tensor-memory load, rotation, rounding, stores; then one thread per channel for the column scans), warp 4:
 // TMA producer (X and W tiles of 64 d_model columns, 128-byte swizzle), warp 5: MMA issuer; the accumulator stages in
-// tensor memory let the epilogue of one tile run under the main loop of the next.  The value heads (Eq. 1, no rotation, no
-// representatives) follow the query / key units as a pass of their own.  Every wait is bounded.
+// tensor memory let the epilogue of one tile run under the main loop of the next.  Every wait is bounded.
 #include "sm100_ptx.cuh"
 
 namespace cp {
@@ -48,8 +48,10 @@ struct ProjArgs {
   float* kabs;
   DeviceStatus* st;
   int B, Hq, Hkv, Hv, n, seg, blk, n1, n2, d_model;   // Hv = Hkv when values are projected too, else 0
-  long long n_units;
+  long long n_q, n_kv;                        // query units; single tiles of the key and value heads
 };
+
+struct Work { int b, hh, j, tok0, nt; };      // batch, first head (query, then key, then value heads), segment, first token, tiles
 
 __device__ __forceinline__ float bf16_bits_to_f32(uint16_t v) { return __uint_as_float(uint32_t(v) << 16); }
 template <bool kF16> __device__ __forceinline__ float elem_to_f32(uint16_t v) {
@@ -86,42 +88,61 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   tc_fence_after();
   const uint32_t tm = bars->tmem_base;
 
-  const int Hqk = (a.Hq + a.Hkv) / kNH;    // head groups (kNH adjacent heads of one kind) in the order query, key, value
-  const long long n_qk_units = (long long)a.B * Hqk * a.n1;
-  const int tiles_per_seg = a.seg / kTileM;
   const int n_kb = a.d_model / kKB;
-  // unit -> (segment j, batch b, head hh); heads of one segment are adjacent so that its X rows stay in L2.  The value
-  // heads follow in a pass of their own after all query / key units: with all three weight matrices live at once
-  // the weights and the X tiles in flight no longer fit the L2 share of a die and every head slows down
-  auto decode = [&](long long u, int* b, int* hh, int* j) {
-    const bool vpass = u >= n_qk_units;
-    if (vpass) u -= n_qk_units;
-    const int H = vpass ? a.Hv / kNH : Hqk;
-    *hh = (int(u % H) + (vpass ? Hqk : 0)) * kNH; u /= H;      // first head of the group
-    *b = int(u % a.B); u /= a.B;
-    *j = int(u);
+  // The s-th unit of this CTA.  Query units are dealt round-robin, heads of one segment adjacent so that its X rows stay in
+  // L2; then come the single tiles of the key and value heads (heads of one tile adjacent), which the CTAs without a query unit in
+  // the last round begin one unit's length earlier.  At 16384 tokens, segment 512, 32 + 8 + 8 heads, units of a whole segment for
+  // every head left the last of 6 rounds a fifth full (768 units on 148 SMs): 648 us, here 576 us = 1430 TFLOP/s.  Keys and values
+  // share this pass because with all three weight matrices live at once the weights and the X tiles in flight no longer
+  // fit the L2 share of a die and every head slows down.
+  auto work = [&](long long s, Work* w) {
+    const long long G = gridDim.x, c = blockIdx.x;
+    const long long full = a.n_q / G, rem = a.n_q % G;
+    const long long mine = full + (c < rem ? 1 : 0);
+    const int t = a.seg / kTileM;
+    if (s < mine) {
+      long long u = c + s * G;
+      const int H = a.Hq / kNH;
+      w->hh = int(u % H) * kNH; u /= H;
+      w->b = int(u % a.B); u /= a.B;
+      w->j = int(u);
+      w->tok0 = w->j * a.seg;
+      w->nt = min(t, (a.n - w->tok0 + kTileM - 1) / kTileM);
+      return true;
+    }
+    const long long i = s - mine;
+    long long x;
+    if (rem == 0) x = i * G + c;
+    else if (c >= rem && i < t) x = i * (G - rem) + (c - rem);
+    else x = t * (G - rem) + (c >= rem ? i - t : i) * G + c;
+    if (x >= a.n_kv) return false;
+    const int H = (a.Hkv + a.Hv) / kNH;
+    w->hh = a.Hq + int(x % H) * kNH; x /= H;
+    w->b = int(x % a.B); x /= a.B;
+    w->tok0 = int(x) * kTileM;
+    w->j = 0;
+    w->nt = 1;
+    return true;
   };
-  auto n_tiles_of = [&](int j) { return min(tiles_per_seg, (a.n - j * a.seg + kTileM - 1) / kTileM); };
 
   if (warp == 4) {
     // ---------------- TMA producer
     uint32_t it = 0;
-    for (long long u = blockIdx.x; u < a.n_units; u += gridDim.x) {
-      int b, hh, j;
-      decode(u, &b, &hh, &j);
+    Work u;
+    for (long long s = 0; work(s, &u); ++s) {
+      const int b = u.b, hh = u.hh;
       const CUtensorMap* tw = hh < a.Hq ? &tmWq : (hh < a.Hq + a.Hkv ? &tmWk : &tmWv);
       const int wrow = (hh < a.Hq ? hh : (hh < a.Hq + a.Hkv ? hh - a.Hq : hh - a.Hq - a.Hkv)) * kD;
-      const int nt = n_tiles_of(j);
-      for (int t = 0; t < nt; ++t) {
-        const int tok0 = j * a.seg + t * kTileM;
+      for (int t = 0; t < u.nt; ++t) {
+        const int tok0 = u.tok0 + t * kTileM;
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
-          const uint32_t s = it % kRing, use = it / kRing;
-          if (use > 0 && !mbar_wait(&bars->empty[s], (use - 1) & 1, &bars->abort_flag, a.st, 70)) return;
+          const uint32_t st = it % kRing, use = it / kRing;
+          if (use > 0 && !mbar_wait(&bars->empty[st], (use - 1) & 1, &bars->abort_flag, a.st, 70)) return;
           if (lane == 0) {
-            const uint32_t dst = smem_base + s * kStageBytes;
-            mbar_expect_tx(&bars->full[s], kStageBytes);
-            tma_load_3d(dst, &tmX, &bars->full[s], kb * kKB, tok0, b);            // rows past n arrive as zeros
-            tma_load_3d(dst + kOpBytes, tw, &bars->full[s], kb * kKB, wrow, 0);   // 128 * kNH weight rows
+            const uint32_t dst = smem_base + st * kStageBytes;
+            mbar_expect_tx(&bars->full[st], kStageBytes);
+            tma_load_3d(dst, &tmX, &bars->full[st], kb * kKB, tok0, b);            // rows past n arrive as zeros
+            tma_load_3d(dst + kOpBytes, tw, &bars->full[st], kb * kKB, wrow, 0);   // 128 * kNH weight rows
           }
           __syncwarp();
         }
@@ -133,11 +154,9 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const uint64_t base = desc_base(16);
     // M = 128, N = 128 * kNH (bits 17-22 hold N / 8)
     constexpr uint32_t kIdesc = (Idesc<kF16>::qk & ~(0x3fu << 17)) | ((uint32_t(kD * kNH) >> 3) << 17);
-    for (long long u = blockIdx.x; u < a.n_units; u += gridDim.x) {
-      int b, hh, j;
-      decode(u, &b, &hh, &j);
-      const int nt = n_tiles_of(j);
-      for (int t = 0; t < nt; ++t, ++tile_no) {
+    Work u;
+    for (long long n = 0; work(n, &u); ++n) {
+      for (int t = 0; t < u.nt; ++t, ++tile_no) {
         const uint32_t as = tile_no % kAcc;
         if (tile_no >= kAcc && !mbar_wait(&bars->acc_empty[as], ((tile_no / kAcc) - 1) & 1, &bars->abort_flag, a.st, 71)) return;
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
@@ -158,18 +177,17 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const int row = tid;                         // 0..127
     const uint32_t t_row = tm + (uint32_t(warp * 32) << 16);
     uint32_t tile_no = 0;
-    for (long long u = blockIdx.x; u < a.n_units; u += gridDim.x) {
-      int b, hh, j;
-      decode(u, &b, &hh, &j);
+    Work u;
+    for (long long n = 0; work(n, &u); ++n) {
+      const int b = u.b, hh = u.hh, j = u.j;
       const bool is_q = hh < a.Hq, is_v = hh >= a.Hq + a.Hkv;
       const int h0 = is_q ? hh : (is_v ? hh - a.Hq - a.Hkv : hh - a.Hq);   // first head of the group within its kind
-      const int nt = n_tiles_of(j);
       float seg_max[kNH], seg_min[kNH];                            // channel `tid` over the segment (query heads)
 #pragma unroll
       for (int sub = 0; sub < kNH; ++sub) { seg_max[sub] = -CUDART_INF_F; seg_min[sub] = CUDART_INF_F; }
-      for (int t = 0; t < nt; ++t, ++tile_no) {
+      for (int t = 0; t < u.nt; ++t, ++tile_no) {
         const uint32_t as = tile_no % kAcc;
-        const int tok0 = j * a.seg + t * kTileM;
+        const int tok0 = u.tok0 + t * kTileM;
         const int tok = tok0 + row;
         if (!mbar_wait(&bars->acc_full[as], (tile_no / kAcc) & 1, &bars->abort_flag, a.st, 73)) return;
         tc_fence_after();
@@ -303,7 +321,8 @@ int launch_project(const cp_params& p, const Dims& m, const void* X, const void*
   a.B = m.B; a.Hq = m.Hq; a.Hkv = m.Hkv; a.n = m.n; a.seg = m.seg; a.blk = m.blk; a.n1 = m.n1; a.n2 = m.n2; a.d_model = d_model;
   // two heads per output tile where every kind has an even head count (see Geo)
   const int nh = (m.Hq % 2 == 0 && m.Hkv % 2 == 0) ? 2 : 1;
-  a.n_units = (long long)m.B * ((m.Hq + m.Hkv + a.Hv) / nh) * m.n1;
+  a.n_q = (long long)m.B * (m.Hq / nh) * m.n1;
+  a.n_kv = (long long)m.B * ((m.Hkv + a.Hv) / nh) * ((m.n + kTileM - 1) / kTileM);
   CUtensorMap tmX, tmWq, tmWk, tmWv;
   if (!make_map3(&tmX, X, d_model, m.n, m.B, f16) || !make_map3(&tmWq, Wq, d_model, (long long)m.Hq * kD, 1, f16, 128 * nh) ||
       !make_map3(&tmWk, Wk, d_model, (long long)m.Hkv * kD, 1, f16, 128 * nh))
@@ -317,7 +336,7 @@ int launch_project(const cp_params& p, const Dims& m, const void* X, const void*
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return CP_ERR_CUDA;
-  const unsigned grid = unsigned(a.n_units < sms ? a.n_units : sms);
+  const unsigned grid = unsigned(a.n_q + a.n_kv < sms ? a.n_q + a.n_kv : sms);
   kern<<<grid, kThreads, smem, st>>>(tmX, tmWq, tmWk, tmWv, a);
   return check_launch();
 }
