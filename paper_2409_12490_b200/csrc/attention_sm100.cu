@@ -342,10 +342,6 @@ __device__ __forceinline__ bool receive_unit(const Args<NS>& a, Bars* bars, uint
 // ---------------------------------------------------------------- softmax role
 constexpr int kMaskNone = 0, kMaskCausal = 1, kMaskCols = 2, kMaskGeneric = 3;
 
-__device__ __forceinline__ float elem_f32(uint16_t x, bool f16) {
-  return f16 ? __half2float(__ushort_as_half(x)) : __uint_as_float(uint32_t(x) << 16);
-}
-
 // One row of a 64-channel head in plain fp32, key by key, by one thread.  A tile's MMA multiplies the zero probability of a
 // key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row whose
 // output came out as NaN or infinite is therefore evaluated again over exactly the keys it sees.
@@ -358,31 +354,49 @@ __device__ __noinline__ void recompute_row(const Args<NS>* ap, int seq, int b, i
   const uint16_t* vb = a.V + b * a.vs[0] + (h / a.g) * a.vs[1] + sq.tok0 * a.vs[2];
   uint16_t* o = a.O + b * a.osb + h * a.osh + (sq.tok0 + t) * a.ost;
   const int n_ranges = a.dense ? 1 : cnt;
-  auto logit = [&](int key) {
-    float s = 0.f;
-    for (int c = 0; c < 64; ++c) s = fmaf(elem_f32(q[c], kF16), elem_f32(kb[int64_t(key) * a.ks[2] + c], kF16), s);
-    return s * a.sm_scale;
-  };
-  float m = -CUDART_INF_F;
-  for (int e = 0; e < n_ranges; ++e) {
-    const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
-    for (int key = u0; key < u1; ++key) m = fmaxf(m, logit(key));
-  }
-  float l = 0.f;
-  for (int c0 = 0; c0 < 64; c0 += 16) {
+  float m = 0.f, l = 0.f;
+#pragma unroll 1
+  for (int c0 = 0; c0 < 64; c0 += 16) {        // 16 channels at a time: few registers, or the caller's tile loop pays for them
     float acc[16];
+#pragma unroll
     for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-    l = 0.f;
+    m = -CUDART_INF_F; l = 0.f;
     for (int e = 0; e < n_ranges; ++e) {
       const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
       for (int key = u0; key < u1; ++key) {
-        const float p = expf(logit(key) - m);
-        l += p;
+        const uint4* q4 = reinterpret_cast<const uint4*>(q);
+        const uint4* k4 = reinterpret_cast<const uint4*>(kb + int64_t(key) * a.ks[2]);
+        const uint4* v4 = reinterpret_cast<const uint4*>(vb + int64_t(key) * a.vs[2] + c0);
+        float x = 0.f;
+#pragma unroll 2
+        for (int c = 0; c < 8; ++c) {
+          const uint4 qw = q4[c], kw = k4[c];
+          const uint32_t qe[4] = {qw.x, qw.y, qw.z, qw.w}, ke[4] = {kw.x, kw.y, kw.z, kw.w};
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = fmaf(p, elem_f32(vb[int64_t(key) * a.vs[2] + c0 + c], kF16), acc[c]);
+          for (int i = 0; i < 4; ++i) {
+            const float2 qf = unpack2<kF16>(qe[i]), kf = unpack2<kF16>(ke[i]);
+            x = fmaf(qf.y, kf.y, fmaf(qf.x, kf.x, x));
+          }
+        }
+        x *= a.sm_scale;
+        const float m_new = fmaxf(m, x), corr = m == -CUDART_INF_F ? 0.f : expf(m - m_new), p = expf(x - m_new);
+        l = l * corr + p;
+        m = m_new;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const uint4 vw = v4[c];
+          const uint32_t ve[4] = {vw.x, vw.y, vw.z, vw.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 vf = unpack2<kF16>(ve[i]);
+            acc[c * 8 + 2 * i] = fmaf(p, vf.x, acc[c * 8 + 2 * i] * corr);
+            acc[c * 8 + 2 * i + 1] = fmaf(p, vf.y, acc[c * 8 + 2 * i + 1] * corr);
+          }
+        }
       }
     }
     const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
     for (int c = 0; c < 16; ++c) o[c0 + c] = uint16_t(pack2<kF16>(acc[c] * inv, 0.f));
   }
   if (a.lse != nullptr) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m + logf(l);
