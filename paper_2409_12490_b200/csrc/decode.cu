@@ -120,7 +120,11 @@ decode_score_kernel(double* __restrict__ S, const double* __restrict__ l_min, in
 template <typename T, int LPR>
 int launch_logits(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* l_max, double* l_min, cudaStream_t st) {
   const dim3 grid(unsigned((m.n2 + kWarps - 1) / kWarps), unsigned(m.B * m.Hkv));
-  return launch_pdl(decode_logits_kernel<T, LPR>, grid, kThreads, size_t(m.g) * m.d * m.es, st, static_cast<const T*>(q_last),
+  const size_t smem = size_t(m.g) * m.d * m.es;    // the group's queries: up to 64 KB (fp32, 128 channels, 128 heads)
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(decode_logits_kernel<T, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+    return CP_ERR_CUDA;
+  return launch_pdl(decode_logits_kernel<T, LPR>, grid, kThreads, smem, st, static_cast<const T*>(q_last),
                     static_cast<const char*>(K), p.k_stride[0], p.k_stride[1], p.k_stride[2], m.Hkv, m.g, m.n, m.blk, m.n2,
                     double(p.est_scale), l_max, l_min);
 }

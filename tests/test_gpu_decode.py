@@ -33,3 +33,17 @@ def test_scores_and_list_match_the_oracle(dtype, d, B, Hkv, g, n, blk, k):
     assert np.abs(S.cpu().numpy() - S_ref).max() <= 1e-9
     idx_ref, cnt_ref = oracle.decode_select(S.cpu().numpy(), k)
     assert np.array_equal(idx.cpu().numpy(), idx_ref) and np.array_equal(cnt.cpu().numpy(), cnt_ref)
+
+
+@pytest.mark.parametrize("g", [96, 97, 128, 129])
+def test_large_query_groups_in_fp32(g):
+    """Up to 128 fp32 heads of 128 channels per KV head share the pass over the key cache (their queries fill up to 64 KB of shared
+    memory, 48 KB at 96 heads); one head more takes the general kernels."""
+    n, blk, k = 700, 64, 3
+    Q, K, V = make_uniform_qkv(1, g, 1, n, 128, dtype="f32", seed=g)
+    prob = cp.Problem(1, g, 1, n, 128, blk, blk, k, torch.float32)
+    ws = cp.alloc_workspace(prob)
+    q = Q[:, :, -1].contiguous()
+    S = cp.decode_estimate(prob, q.cuda(), K.cuda(), ws)
+    assert cp.device_status(ws) == 0
+    assert np.abs(S.cpu().numpy() - oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))).max() <= 1e-9
