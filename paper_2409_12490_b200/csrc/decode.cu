@@ -100,20 +100,23 @@ decode_score_kernel(double* __restrict__ S, const double* __restrict__ l_min, in
   m = block_reduce(m, true);
   double2 s = make_double2(0.0, 0.0);
 #pragma unroll 1
-  for (int i = 0; i < NPT; ++i) {                  // terms below e^-50 of the largest cannot change the rounded sum
+  for (int i = 0; i < NPT; ++i) {                  // terms below e^-50 of the largest cannot change the rounded sum; NaN stays out
     if (tid + i * kThreads >= n2) break;
     double av = a[0], cv = c[0];
 #pragma unroll
     for (int x = 1; x < NPT; ++x) { av = x == i ? a[x] : av; cv = x == i ? c[x] : cv; }
-    if (!(av - m.x <= -50.0)) s.x += exp(av - m.x);
-    if (!(cv - m.y <= -50.0)) s.y += exp(cv - m.y);
+    if (av - m.x > -50.0) s.x += exp(av - m.x);
+    if (cv - m.y > -50.0) s.y += exp(cv - m.y);
   }
   s = block_reduce(s, false);
-  const double lse1 = m.x + log(s.x), lse2 = m.y + log(s.y);
+  // Logits that are not finite end as in score_kernel, which larger blocks go through: a NaN logit is the NaN of its own block
+  // alone, and a row without a finite maximum has the sum 0 and ln 0 = -inf.
+  const double lse1 = s.x > 0.0 ? m.x + log(s.x) : -CUDART_INF, lse2 = s.y > 0.0 ? m.y + log(s.y) : -CUDART_INF;
 #pragma unroll
   for (int i = 0; i < NPT; ++i) {
     const int x = tid + i * kThreads;
-    if (x < n2) row[x] = fmax(a[i] - lse1, c[i] - lse2);
+    const double L1 = a[i] - lse1, L2 = c[i] - lse2;
+    if (x < n2) row[x] = L1 >= L2 ? L1 : L2;
   }
 }
 

@@ -47,3 +47,48 @@ def test_large_query_groups_in_fp32(g):
     S = cp.decode_estimate(prob, q.cuda(), K.cuda(), ws)
     assert cp.device_status(ws) == 0
     assert np.abs(S.cpu().numpy() - oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))).max() <= 1e-9
+
+
+def _bad_values(what, q, K, blk):
+    inf, nan = float("inf"), float("nan")
+    if what == "channel of a block NaN":
+        K[0, 0, 3 * blk:4 * blk, 7] = nan
+    elif what == "one key +inf":
+        K[0, 0, 3 * blk + blk // 2, 7] = inf
+    elif what == "one key -inf":
+        K[0, 0, 3 * blk + blk // 2, 7] = -inf
+    elif what == "NaN logits of one block":          # infinities of both signs in the representatives of two channels
+        K[0, 0, 3 * blk, 7] = K[0, 0, 3 * blk + 1, 9] = inf
+        K[0, 0, 3 * blk, 9] = K[0, 0, 3 * blk + 1, 7] = -inf
+        q[0, 0, 7], q[0, 0, 9] = 1.0, -1.0
+        q[0, 1, 7], q[0, 1, 9] = 1.0, 1.0
+    elif what == "q NaN":
+        q[0, 1, 3] = nan
+    elif what == "q inf":
+        q[0, 1, 3] = inf
+    elif what == "keys NaN":
+        K[...] = nan
+    return q, K
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 64), ("bf16", 64), ("f32", 128)])
+@pytest.mark.parametrize("blk,g", [(2, 2), (32, 4), (128, 2)])
+@pytest.mark.parametrize("what", ["channel of a block NaN", "one key +inf", "one key -inf", "NaN logits of one block", "q NaN", "q inf",
+                                  "keys NaN"])
+def test_values_that_are_not_finite_follow_the_general_kernel(dtype, d, blk, g, what):
+    """The last segment of a prefill may hold the newest token alone: its row of the general score kernel is then the decoding row,
+    and what NaN and infinite logits do to the other blocks has to be the same."""
+    n = 20 * blk + 1
+    Q, K, V = make_uniform_qkv(1, g, 1, n, d, dtype=dtype, seed=blk)
+    q = Q[:, :, -1].clone()
+    q, K = _bad_values(what, q, K.clone(), blk)
+    Q[:, :, -1] = q
+    prob = cp.Problem(1, g, 1, n, d, blk, blk, 4, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    row = cp.estimate(prob, Q.cuda(), K.cuda(), ws)[:, :, -1].cpu().numpy()
+    S = cp.decode_estimate(prob, q.contiguous().cuda(), K.cuda(), ws).cpu().numpy()
+    assert cp.device_status(ws) == 0
+    for kind in (np.isnan, np.isposinf, np.isneginf):
+        assert np.array_equal(kind(S), kind(row)), kind.__name__
+    fin = np.isfinite(row)
+    assert np.abs(S[fin] - row[fin]).max(initial=0.0) <= 1e-9
