@@ -10,6 +10,8 @@
 // 256, fp32: 230 us, here 17 us; error against fp64 at or below that kernel's (9.22e-7 against 9.24e-7 relative at 4001 tokens).
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "cp_common.cuh"
 
 namespace cp {
@@ -147,7 +149,7 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
   T* kt = reinterpret_cast<T*>(ps + kBM * kPS);             // [kBN][kKS]
   T* vt = kt + kBN * kKS;
   __shared__ int tok_all[NG][2][kBN];                         // token of each key of the tile; 0x7fffffff: no such key
-  __shared__ int list_state[2];                             // [0] the list is valid, [1] blocks that start at or before the last row
+  __shared__ int list_state[2];                             // [0] the list is valid, [1] listed keys up to the last row
   __shared__ int redo[kBM];
 
   const int tid = threadIdx.x % kThreads, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -181,14 +183,15 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
         for (int i = lane; i < cnt; i += 32) c += list[i] * a.blk < t_end;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-      if (lane == 0) { list_state[0] = ok; list_state[1] = c; }
+      // the list is ascending: later blocks are seen by no row, and of the last one only the keys up to the last row
+      if (lane == 0) { list_state[0] = ok; list_state[1] = c > 0 ? (c - 1) * a.blk + min(a.blk, t_end - list[c - 1] * a.blk) : 0; }
     }
     __syncthreads();
     if (!list_state[0]) {
       if (threadIdx.x == 0 && t0 == j * a.seg) report(a.st, CP_ERR_BOUNDS, 100, b, h, j, cnt);
       return;
     }
-    n_keys = list_state[1] * a.blk;                                  // the list is ascending: later blocks are seen by no row
+    n_keys = list_state[1];
   }
   for (int i = threadIdx.x; i < kBM; i += kThreads * NG) redo[i] = 0;
 
@@ -387,8 +390,8 @@ template <typename T, int D, int RT, int NG>
 int launch_rt(const SimtArgs<T>& a0, const Dims& m, cudaStream_t s) {
   using S = SimtShape<T, D, RT, NG>;
   SimtArgs<T> a = a0;
-  a.tiles_per_seg = (m.seg + S::kBM - 1) / S::kBM;
-  // the last segment may be short: its missing tiles return at once
+  // no segment has more rows than the sequence; the last one may be shorter than that: its missing tiles return at once
+  a.tiles_per_seg = (std::min(m.seg, m.n) + S::kBM - 1) / S::kBM;
   const long long ctas = (long long)m.B * m.Hq * m.n1 * a.tiles_per_seg;
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   auto kern = attention_simt_kernel<T, D, RT, NG>;

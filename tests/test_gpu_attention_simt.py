@@ -43,6 +43,23 @@ def test_sparse_and_dense_match_the_oracle(dtype, d, B, Hq, Hkv, n, seg, blk, k)
     assert_close(Od, oracle.dense_attention(Q, K, V, sm)[0], V, dtype)
 
 
+def test_segment_far_longer_than_the_sequence():
+    """2^29 tokens to the segment: tiles are counted over the rows there are, not over the segment's (2^33 tiles for 512 heads)."""
+    n, seg, H = 100, 1 << 29, 512
+    Q, K, V = make_uniform_qkv(1, H, 1, n, 64, dtype="f32", seed=2)
+    prob = cp.Problem(1, H, 1, n, 64, seg, seg, 1, torch.float32)
+    ws = cp.alloc_workspace(prob)
+    Qd, Kd, Vd = Q.cuda(), K.cuda(), V.cuda()
+    idx = torch.zeros((1, H, 1, 1), dtype=torch.int32, device="cuda")
+    cnt = torch.ones((1, H, 1), dtype=torch.int32, device="cuda")
+    O = cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws)
+    Od = cp.dense_attention(prob, Qd, Kd, Vd, ws)
+    assert cp.device_status(ws) == 0
+    O_ref, _ = oracle.dense_attention(Q, K, V, f32(0.125))
+    assert_close(O, O_ref, V, "f32")
+    assert_close(Od, O_ref, V, "f32")
+
+
 def test_value_that_is_not_finite_reaches_only_the_rows_that_see_it():
     n, seg, blk, k = 700, 256, 32, 12
     Q, K, V = make_uniform_qkv(1, 2, 1, n, 64, dtype="f32", seed=1)
