@@ -22,6 +22,8 @@
 // is bounded: on expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
 // One launch serves one problem or a packed batch of up to kMaxSeqs sequences (each with tensor maps of
 // its own, so that reads past a sequence's end arrive as zeros and never as a neighbour's tokens).
+#include <algorithm>
+
 #include "sm100_ptx.cuh"
 
 namespace cp {
@@ -116,6 +118,7 @@ template <int NS> struct Args {
   float* lse;
   DeviceStatus* st;
   int B, Hq, Hkv, g, seg, blk, k, r;
+  int pp;                       // units (pairs of query tiles) per segment, counted over the rows that a segment can have
   int64_t osb, osh, ost;
   const uint16_t *Q, *K, *V;    // only for rows that are recomputed one by one (recompute_row)
   int64_t qs[3], ks[3], vs[3];
@@ -180,7 +183,7 @@ __device__ __forceinline__ Unit decode_unit(const Args<NS>& a, int x, int cnt) {
     u.nB = (2 * pair + 1 < ntiles) ? 1 : 0;
   } else {
     const int q_tiles = a.seg / kTile;
-    const int pp = (q_tiles + 1) / 2;
+    const int pp = a.pp;
     int j, p;
     if (a.long_first) {
       const int heads = a.B * a.Hq, bh = x % heads;
@@ -827,10 +830,18 @@ int launch_variant(const Maps<NS>& maps, const Args<NS>& a, cudaStream_t s) {
   return launch_pdl(kern, dim3(unsigned(a.n_units)), kThreads, Shape<D>::kSmemTotal, s, maps, a);
 }
 
+// pairs of 128-row query tiles in a segment: a segment can be longer than every sequence, and empty units cost a hand-over each
+int pairs_per_segment(int seg, const SeqSlot* slots, int n_seqs) {
+  int rows = 0;
+  for (int i = 0; i < n_seqs; ++i) rows = std::max(rows, std::min(seg, slots[i].len));
+  return ((rows + kTile - 1) / kTile + 1) / 2;
+}
+
 // (segment, pair)s that have query rows, by the tiles they stream, longest first (counting sort; equal ones from the last
 // segment down).  Returns their number, 0 when there are more than the table holds.
 template <int NS>
-int order_units(Args<NS>& a, int pp) {
+int order_units(Args<NS>& a) {
+  const int pp = a.pp;
   if ((long long)a.n_segs * pp > kMaxOrder) return 0;
   constexpr int kCosts = 256;
   uint16_t cost[kMaxOrder];
@@ -860,6 +871,7 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
   Maps<NS> maps;
   Args<NS> a;
   a.n_segs = 0;
+  a.pp = pairs_per_segment(m.seg, slots, n_seqs);
   long long kv_tokens = 0;
   for (int i = 0; i < n_seqs; ++i) {
     const SeqSlot& q = slots[i];
@@ -888,15 +900,14 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
   a.sm_scale = p.sm_scale; a.dense = dense ? 1 : 0;
   // a unit is two 128-row query tiles (one when a segment, or the sequence, has an odd tile count)
   const long long units = dense ? (long long)m.B * m.Hq * (((m.n + kTile - 1) / kTile + 1) / 2)
-                                : (long long)m.B * m.Hq * a.n_segs * ((m.seg / kTile + 1) / 2);
+                                : (long long)m.B * m.Hq * a.n_segs * a.pp;
   if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   a.n_units = int(units);
   // K and V of every head up to 160 MB (measured on both sides: see decode_unit; the L2 has 126 MB); a batch of sequences always (its neighbours in the order are the
   // heads of one segment, so one sequence or two are in use at a time)
-  const int pp = (m.seg / kTile + 1) / 2;
   a.long_first = (NS > 1 || kv_tokens * m.B * m.Hkv * m.d * m.es * 2 <= 160ll << 20) ? 1 : 0;
   if (a.long_first && !dense) {
-    const int entries = order_units(a, pp);
+    const int entries = order_units(a);
     if (entries > 0) a.n_units = m.B * m.Hq * entries;
     else a.long_first = 0;                          // more segments than the table holds (never for a batch: see below)
   }
@@ -922,14 +933,13 @@ int launch_attention_sm100(const cp_params& p, const Dims& m, const void* Q, con
 int launch_attention_sm100_varlen(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_seqs, const void* Q, const void* K,
                                   const void* V, const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st,
                                   cudaStream_t s) {
-  const int pp = (m.seg / kTile + 1) / 2;
   for (int i = 0; i < n_seqs;) {
     // as many sequences as a launch has tensor maps and unit entries for; a lone one takes the single-problem launch
     int c = 0;
-    long long entries = 0;
+    long long segs = 0;
     while (c < kMaxSeqs && i + c < n_seqs) {
-      entries += (long long)((slots[i + c].len + m.seg - 1) / m.seg) * pp;
-      if (entries > kMaxOrder) break;
+      segs += (slots[i + c].len + m.seg - 1) / m.seg;
+      if (segs * pairs_per_segment(m.seg, slots + i, c + 1) > kMaxOrder) break;
       ++c;
     }
     const int rc = c > 1 ? launch_seqs<kMaxSeqs>(p, m, slots + i, c, Q, K, V, idx, cnt, O, lse, st, false, s)

@@ -49,6 +49,34 @@ def test_sparse_and_dense_match_the_oracle(dtype, B, Hq, Hkv, n, seg, blk, k):
     assert_close(Od, oracle.dense_attention(Q, K, V, SM)[0], V, dtype)
 
 
+def launched_grids(call):
+    """gridDim.x of every kernel that `call` enqueues, from a captured graph (nothing runs)."""
+    from cuda.bindings import runtime as rt
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        keep = call()
+    raw = rt.cudaGraph_t(g.raw_cuda_graph())
+    _, _, n = rt.cudaGraphGetNodes(raw, 0)
+    _, nodes, n = rt.cudaGraphGetNodes(raw, n)
+    grids = []
+    for node in nodes[:n]:
+        if rt.cudaGraphNodeGetType(node)[1] == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel:
+            grids.append(rt.cudaGraphKernelNodeGetParams(node)[1].gridDim.x)
+    del keep
+    return grids
+
+
+@pytest.mark.parametrize("B,n", [(1, 1), (2, 300), (1, 1301)])
+def test_segment_far_longer_than_the_sequence(B, n):
+    """Units are counted over the rows there are, not over the segment's 2^20."""
+    seg, blk = 1 << 20, 128
+    Q, K, V, prob, ws, Qd, Kd, Vd, idx, cnt = layer("f16", B, 4, 2, n, seg, blk, seg // blk)
+    O = cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws)
+    assert cp.device_status(ws) == 0
+    assert_close(O, oracle.dense_attention(Q, K, V, SM)[0], V, "f16")
+    assert launched_grids(lambda: cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws)) == [B * 4 * -(-n // 256)]
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f16"])
 def test_value_that_is_not_finite_reaches_only_the_rows_that_see_it(dtype):
     n, seg, blk, k = 700, 256, 32, 12
