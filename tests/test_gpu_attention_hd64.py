@@ -51,17 +51,18 @@ def test_sparse_and_dense_match_the_oracle(dtype, B, Hq, Hkv, n, seg, blk, k):
 
 def launched_grids(call):
     """gridDim.x of every kernel that `call` enqueues, from a captured graph (nothing runs)."""
-    from cuda.bindings import runtime as rt
+    from cuda.bindings import driver as cu
     g = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(g):
         keep = call()
-    raw = rt.cudaGraph_t(g.raw_cuda_graph())
-    _, _, n = rt.cudaGraphGetNodes(raw, 0)
-    _, nodes, n = rt.cudaGraphGetNodes(raw, n)
+    raw = cu.CUgraph(g.raw_cuda_graph())
+    n = cu.cuGraphGetNodes(raw, 0)[2]
     grids = []
-    for node in nodes[:n]:
-        if rt.cudaGraphNodeGetType(node)[1] == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel:
-            grids.append(rt.cudaGraphKernelNodeGetParams(node)[1].gridDim.x)
+    for node in cu.cuGraphGetNodes(raw, n)[1][:n]:
+        if cu.cuGraphNodeGetType(node)[1] == cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            rc, params = cu.cuGraphKernelNodeGetParams(node)
+            assert rc == cu.CUresult.CUDA_SUCCESS, rc
+            grids.append(params.gridDimX)
     del keep
     return grids
 
@@ -97,3 +98,26 @@ def test_value_that_is_not_finite_reaches_only_the_rows_that_see_it(dtype):
         assert np.isfinite(O[0][~sees]).all() and not np.isfinite(O[0][sees][:, 5]).any()
         O_ref = oracle.dense_attention(Q, K, Vf, SM)[0] if dense else oracle.sparse_attention(Q, K, Vf, li, cnt.cpu().numpy(), seg, blk, SM)[0]
         assert_close(torch.from_numpy(O[0][~sees]), O_ref[0][~sees], V, dtype)
+
+
+def test_value_that_is_not_finite_at_the_end_of_a_long_sequence():
+    """The last 300 rows of 1.3 M tokens see an infinite value and are evaluated one by one, over more keys than the kernel's waits
+    would sit out for a thread per row: the call ends without an error, every row before them is finite, and the rows are those of
+    the formula."""
+    n, bad = 1_300_000, 1_300_000 - 300
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    Q, K, V = (torch.randn((1, 1, n, 64), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(3))
+    V[0, 0, bad, 5] = float("inf")
+    prob = cp.Problem(1, 1, 1, n, 64, 1024, 128, 16, torch.bfloat16)
+    ws = cp.alloc_workspace(prob)
+    O, lse = cp.dense_attention(prob, Q, K, V, ws, want_lse=True)
+    assert cp.device_status(ws) == 0
+    assert torch.isfinite(O[0, 0, :bad]).all() and torch.isposinf(O[0, 0, bad:, 5]).all()
+    keep = torch.arange(64, device="cuda") != 5
+    assert torch.isfinite(O[0, 0, bad:][:, keep]).all()
+    for t in (bad - 1, bad, n - 1):
+        s = (K[0, 0, :t + 1].double() @ Q[0, 0, t].double()) * SM
+        ref = torch.softmax(s, 0) @ V[0, 0, :t + 1].double()
+        assert abs(float(torch.logsumexp(s, 0)) - float(lse[0, 0, t])) <= 1e-4
+        # outputs of about 1e-3: one rounding to bf16, and fp32 sums over 2^20 keys that add up to 1 (2^-17 of max|V| ~ 5)
+        assert (O[0, 0, t].double() - ref)[keep].abs().max() <= 2.0 ** -8 * ref[keep].abs().max() + 2.0 ** -17 * 5
