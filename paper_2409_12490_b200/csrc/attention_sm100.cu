@@ -100,6 +100,7 @@ struct Bars {
   Unit sched_u[2];                   // the published unit, decoded; its cnt carries kBadList / kEmptyUnit
   uint32_t tmem_base;
   volatile int abort_flag;
+  volatile uint32_t beat;            // advanced by warps that evaluate rows one by one (exact_row)
 };
 
 // One sequence: where its tokens, lists and rows of lse start in the arrays of the launch.
@@ -120,7 +121,7 @@ template <int NS> struct Args {
   int B, Hq, Hkv, g, seg, blk, k, r;
   int pp;                       // units (pairs of query tiles) per segment, counted over the rows that a segment can have
   int64_t osb, osh, ost;
-  const uint16_t *Q, *K, *V;    // only for rows that are recomputed one by one (recompute_row)
+  const uint16_t *Q, *K, *V;    // only for rows that are evaluated one by one (exact_row)
   int64_t qs[3], ks[3], vs[3];
   float sm_scale;
   int dense;
@@ -139,7 +140,7 @@ template <int NS> struct Maps { CUtensorMap m[NS][kMaps]; };
 
 // bounded wait on one of this kernel's barriers (the CTA's abort flag lives in the barrier block)
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, Bars* bars, DeviceStatus* st, int site) {
-  return mbar_wait(bar, parity, &bars->abort_flag, st, site);
+  return mbar_wait(bar, parity, &bars->abort_flag, st, site, &bars->beat);
 }
 
 // ---------------------------------------------------------------- unit geometry
@@ -345,33 +346,31 @@ __device__ __forceinline__ bool receive_unit(const Args<NS>& a, Bars* bars, uint
 // ---------------------------------------------------------------- softmax role
 constexpr int kMaskNone = 0, kMaskCausal = 1, kMaskCols = 2, kMaskGeneric = 3;
 
-// One row of a 64-channel head in plain fp32, key by key, by one thread.  A tile's MMA multiplies the zero probability of a
-// key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row whose
-// output came out as NaN or infinite is therefore evaluated again over exactly the keys it sees.
+// One row of a 64-channel head by one warp over exactly the keys it sees, in plain fp32.  A tile's MMA multiplies the zero
+// probability of a key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row
+// whose output came out as NaN or infinite is therefore evaluated again here.  A row of 131072 keys takes milliseconds and a unit
+// has up to 256 of them, so the CTA's other warps are told that this one is at work (`beat`), and their waits go on.
 template <bool kF16, int NS>
-__device__ __noinline__ void recompute_row(const Args<NS>* ap, int seq, int b, int h, const int32_t* list, int cnt, int t) {
+__device__ __noinline__ void exact_row(const Args<NS>* ap, Bars* bars, int seq, int b, int h, const int32_t* list, int cnt, int t, int lane) {
   const Args<NS>& a = *ap;
   const Seq& sq = a.seq[seq];
-  const uint16_t* q = a.Q + b * a.qs[0] + h * a.qs[1] + (sq.tok0 + t) * a.qs[2];
+  const uint4* q4 = reinterpret_cast<const uint4*>(a.Q + b * a.qs[0] + h * a.qs[1] + (sq.tok0 + t) * a.qs[2]);
   const uint16_t* kb = a.K + b * a.ks[0] + (h / a.g) * a.ks[1] + sq.tok0 * a.ks[2];
   const uint16_t* vb = a.V + b * a.vs[0] + (h / a.g) * a.vs[1] + sq.tok0 * a.vs[2];
-  uint16_t* o = a.O + b * a.osb + h * a.osh + (sq.tok0 + t) * a.ost;
   const int n_ranges = a.dense ? 1 : cnt;
-  float m = 0.f, l = 0.f;
-#pragma unroll 1
-  for (int c0 = 0; c0 < 64; c0 += 16) {        // 16 channels at a time: few registers, or the caller's tile loop pays for them
-    float acc[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-    m = -CUDART_INF_F; l = 0.f;
-    for (int e = 0; e < n_ranges; ++e) {
-      const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
-      for (int key = u0; key < u1; ++key) {
-        const uint4* q4 = reinterpret_cast<const uint4*>(q);
-        const uint4* k4 = reinterpret_cast<const uint4*>(kb + int64_t(key) * a.ks[2]);
-        const uint4* v4 = reinterpret_cast<const uint4*>(vb + int64_t(key) * a.vs[2] + c0);
+  float m_run = -CUDART_INF_F, l_run = 0.f;
+  float2 acc = make_float2(0.f, 0.f);                       // channels 2 * lane, 2 * lane + 1
+  uint32_t chunk = 0;
+  for (int e = 0; e < n_ranges; ++e) {
+    const int u0 = a.dense ? 0 : list[e] * a.blk, u1 = a.dense ? t + 1 : min(u0 + a.blk, t + 1);
+    for (int base = u0; base < u1; base += 32) {
+      if ((chunk++ & 63u) == 0 && lane == 0) bars->beat = bars->beat + 1;
+      const int u = base + lane;
+      float s = -CUDART_INF_F;
+      if (u < u1) {
+        const uint4* k4 = reinterpret_cast<const uint4*>(kb + int64_t(u) * a.ks[2]);
         float x = 0.f;
-#pragma unroll 2
+#pragma unroll
         for (int c = 0; c < 8; ++c) {
           const uint4 qw = q4[c], kw = k4[c];
           const uint32_t qe[4] = {qw.x, qw.y, qw.z, qw.w}, ke[4] = {kw.x, kw.y, kw.z, kw.w};
@@ -381,28 +380,33 @@ __device__ __noinline__ void recompute_row(const Args<NS>* ap, int seq, int b, i
             x = fmaf(qf.y, kf.y, fmaf(qf.x, kf.x, x));
           }
         }
-        x *= a.sm_scale;
-        const float m_new = fmaxf(m, x), corr = m == -CUDART_INF_F ? 0.f : expf(m - m_new), p = expf(x - m_new);
-        l = l * corr + p;
-        m = m_new;
+        s = x * a.sm_scale;
+      }
+      float mx = s;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint4 vw = v4[c];
-          const uint32_t ve[4] = {vw.x, vw.y, vw.z, vw.w};
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float m_new = fmaxf(m_run, mx);
+      const float corr = m_run == -CUDART_INF_F ? 0.f : expf(m_run - m_new);
+      const float p = u < u1 ? expf(s - m_new) : 0.f;
+      float ps = p;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 vf = unpack2<kF16>(ve[i]);
-            acc[c * 8 + 2 * i] = fmaf(p, vf.x, acc[c * 8 + 2 * i] * corr);
-            acc[c * 8 + 2 * i + 1] = fmaf(p, vf.y, acc[c * 8 + 2 * i + 1] * corr);
-          }
-        }
+      for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+      l_run = l_run * corr + ps;
+      m_run = m_new;
+      acc.x *= corr; acc.y *= corr;
+      const int here = min(32, u1 - base);
+#pragma unroll 8
+      for (int kk = 0; kk < here; ++kk) {
+        const float pk = __shfl_sync(0xffffffffu, p, kk);
+        const float2 vf = unpack2<kF16>(*reinterpret_cast<const uint32_t*>(vb + int64_t(base + kk) * a.vs[2] + 2 * lane));
+        acc.x = fmaf(pk, vf.x, acc.x); acc.y = fmaf(pk, vf.y, acc.y);
       }
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) o[c0 + c] = uint16_t(pack2<kF16>(acc[c] * inv, 0.f));
   }
-  if (a.lse != nullptr) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m + logf(l);
+  const float inv = l_run > 0.f ? 1.f / l_run : 0.f;        // a row without any visible key: zeros, lse = ln 0
+  uint16_t* o = a.O + b * a.osb + h * a.osh + (sq.tok0 + t) * a.ost;
+  *reinterpret_cast<uint32_t*>(o + 2 * lane) = pack2<kF16>(acc.x * inv, acc.y * inv);
+  if (a.lse != nullptr && lane == 0) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m_run + logf(l_run);
 }
 
 template <bool kF16, int D, int NS>
@@ -589,7 +593,12 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
       a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] =
           m_run * a.sm_scale + (kSplitP ? logf(l_run) - kPShift<kF16, D> * 0.693147180559945f : __logf(l_run));
     if constexpr (kSplitP) {
-      if (!(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n) recompute_row<kF16>(&a, u.seq, u.b, u.h, u.list, u.cnt, t);
+      // the warp's rows that came out as NaN or infinite, or saw no key, one after another
+      unsigned redo = __ballot_sync(0xffffffffu, !(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n);
+      for (; redo != 0; redo &= redo - 1) {
+        __syncwarp();                                // the row's own stores come first
+        exact_row<kF16>(&a, bars, u.seq, u.b, u.h, u.list, u.cnt, t - lane + (__ffs(redo) - 1), lane);
+      }
     }
   }
 }
@@ -758,6 +767,7 @@ attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_const
     mbar_init(&bars->taken, 1);
     for (int i = 0; i < 2; ++i) { mbar_init(&bars->sched_full[i], 1); mbar_init(&bars->sched_empty[i], 10); }   // 8 softmax warps, producer, MMA
     bars->abort_flag = 0;
+    bars->beat = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
