@@ -165,13 +165,17 @@ class Problem:
 
     def params(self, Q=None, K=None, V=None, O=None) -> CpParams:
         q, k = self._contig(self.n_q_heads), self._contig(self.n_kv_heads)
-        return CpParams.from_buffer_copy(_PARAMS.pack(
+        values = (
             self.batch, self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim, self.segment_size, self.block_size,
             self.budget_blocks, _DTYPES[self.dtype], self.flags,
             *(_strides(Q) if Q is not None else q), *(_strides(K) if K is not None else k),
             *(_strides(V) if V is not None else k), *(_strides(O) if O is not None else q),
             self.est_scale, self.sm_scale if self.sm_scale is not None else 1.0 / math.sqrt(self.head_dim), self.alpha,
-            (self.n_sink | (self.n_local << 16)) & 0xffffffff))
+            (self.n_sink | (self.n_local << 16)) & 0xffffffff)
+        try:
+            return CpParams.from_buffer_copy(_PARAMS.pack(*values))
+        except (struct.error, OverflowError):   # a number that its C type does not hold: converted as C does, for the library to judge
+            return CpParams(*values[:10], *(values[i:i + 3] for i in (10, 13, 16, 19)), *values[22:])
 
 
 def workspace_bytes(prob: Problem) -> int:

@@ -44,6 +44,15 @@ def test_host_validation_without_gpu():
     assert "workspace" in cp.status_string(4)
 
 
+def test_numbers_that_their_c_type_does_not_hold():
+    """They reach the library as C converts them: sizes it refuses with its own status, scales that are infinite."""
+    with pytest.raises(cp.CritiPrefillError):
+        cp.workspace_bytes(cp.Problem(1, 4, 2, 1 << 31, 64, 128, 32, 8))
+    p = cp.Problem(1, 4, 2, 1024, 64, 128, 32, 8, est_scale=1e39, sm_scale=-1e39, n_local=1 << 15).params()
+    assert (p.est_scale, p.sm_scale, p.forced_blocks) == (float("inf"), -float("inf"), -(1 << 31))
+    assert list(p.k_stride) == [2 * 1024 * 64, 1024 * 64, 64] and p.seq_len == 1024 and p.alpha == 0.25
+
+
 def test_varlen_sizes_and_cu_seqlens_validation_without_gpu():
     lib = cp.load_library()
     prob = cp.Problem(1, 4, 2, 1000, 64, 128, 32, 8)
