@@ -12,7 +12,8 @@
 //              memory, where the softmax warps overwrite S with 16-bit probabilities)
 //   warp  10   scheduler: draws the next unit, reads and checks its block list, publishes it
 //              (warp 11 is idle; it completes the third warpgroup)
-// Tensor memory (512 columns): S_A | S_B (128 fp32 columns each) | O_A | O_B (head_dim columns each).
+// Tensor memory (512 columns): S_A | S_B (128 fp32 columns each) | O_A | O_B (head_dim columns each) | head_dim 64 in bf16: the third
+// parts of P_A | P_B (64 columns each).
 // The tile sequence of a unit is: gathered past tiles, contiguous unmasked tiles, then the
 // diagonal tiles; tile A stops one tile earlier than B.  The grid has one CTA per unit; those that
 // are resident take over the units of those that have not started yet, one after another
@@ -34,14 +35,12 @@ constexpr int kHalfBytes = kTile * 64 * 2;   // [128 rows x 64 cols] of 16-bit e
 constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {producer, MMA, scheduler, idle}
 constexpr int kMaxSlots = 8;
 constexpr int kBarBytes = 512;
-// What head_dim decides.  Heads of 64 channels keep their probabilities to 32-bit accuracy: P is stored as the sum of two
-// 16-bit values (hi over the first 64 columns of S, lo over the other 64), and O += P V runs over both; O has 64 columns.
-// That costs 8 further N = 64 MMAs per tile, which hide under the softmax (the exponentials bound this shape: 128 per
-// row and tile against half the MMA work of 128 channels).  Measured on two sequences of 6001 tokens, 16 heads, segment 512,
-// block 64, budget 1024 (fp16): the whole layer 33.8 ms with the one-warp-per-row kernel of attention_simt.cu, 0.154 ms here;
-// error against fp64 the same to five digits (2.052e-4 relative at 4099 tokens in fp16, 1.645e-3 in bf16: the output's rounding).
+// What head_dim decides.  Heads of 64 channels keep 32-bit probabilities and sums (softmax_role64): P goes to the tensor cores as a
+// sum of 16-bit values of its own, two in fp16 (22 bits) and three in bf16 (24 bits), O += P V runs over each of them, and the
+// 64 columns of a tile's P V are added up in registers, because the tensor cores round every accumulation towards zero.
+// Tensor memory then holds, besides S, a tile's P V of each query tile and the third part of P (64 columns each).
 template <int D> struct Shape {
-  static constexpr bool kSplitP = D == 64;
+  static constexpr bool kSplitP = D == 64;                          // see above
   static constexpr int kHalves = D / 64;
   static constexpr int kTileBytes = kHalves * kHalfBytes;
   static constexpr int kSlots = D == 128 ? 5 : kMaxSlots;           // 5 x 32 KB + 64 KB of Q; 8 x 16 KB + 32 KB
@@ -50,9 +49,9 @@ template <int D> struct Shape {
   static constexpr int kSmemBar = kSmemKV + kSlots * kTileBytes;
   static constexpr int kSmemTotal = kSmemBar + kBarBytes + 1024;    // + barrier block + slack to align the tiles to 1024 bytes
 };
-// fp16 halves of P are scaled by 2^7: the reference maximum is at most 2^8 behind (lazy rescale), so P stays below 2^15,
-// and the low halves of small probabilities stay out of the subnormals
-template <bool kF16, int D> constexpr float kPShift = (kF16 && Shape<D>::kSplitP) ? 7.f : 0.f;
+// fp16 parts of P are scaled by 2^7: the reference maximum is at most 2^8 behind (lazy rescale), so P stays below 2^15,
+// and the low parts of small probabilities stay out of the subnormals
+template <bool kF16> constexpr float kPShift = kF16 ? 7.f : 0.f;
 constexpr float kRescaleThreshold = 8.0f;           // in log2 units
 #ifndef CP_EMUL_EVERY
 #define CP_EMUL_EVERY 8
@@ -409,9 +408,20 @@ __device__ __noinline__ void exact_row(const Args<NS>* ap, Bars* bars, int seq, 
   if (a.lse != nullptr && lane == 0) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m_run + logf(l_run);
 }
 
-template <bool kF16, int D, int NS>
+// an empty list: no key is visible to any row of the unit -- zeros, and lse = ln 0
+template <int D, int NS>
+__device__ __forceinline__ void write_zero_row(const Args<NS>& a, const Unit& u, int which, int t) {
+  if ((which == 0 || u.rowsB) && t < u.n) {
+    uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost);
+#pragma unroll
+    for (int i = 0; i < D * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (a.lse != nullptr) a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] = -CUDART_INF;
+  }
+}
+
+template <bool kF16, int NS>
 __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int which, int warp_in_wg, int lane) {
-  constexpr bool kSplitP = Shape<D>::kSplitP;
+  constexpr int D = 128;
   const uint32_t tm = bars->tmem_base;
   const uint32_t lane_off = uint32_t(warp_in_wg * 32) << 16;
   const uint32_t tS = tm + lane_off + which * 128;
@@ -427,14 +437,7 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
     if (!receive_unit(a, bars, q, lane, &x, &u) || x >= a.n_units || bars->abort_flag) return;
     if (u.cnt == kBadList || u.cnt == kEmptyUnit) continue;
     if (u.cnt == kZeroUnit) {
-      // an empty list: no key is visible to any row of the unit -- zeros, and lse = ln 0
-      const int t = u.q_tok + which * kTile + row;
-      if ((which == 0 || u.rowsB) && t < u.n) {
-        uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost);
-#pragma unroll
-        for (int i = 0; i < D * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (a.lse != nullptr) a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] = -CUDART_INF;
-      }
+      write_zero_row<D>(a, u, which, u.q_tok + which * kTile + row);
       continue;
     }
     const int my_tiles = which == 0 ? u.nA : u.nB;
@@ -508,26 +511,11 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
           tmem_st32(tO + q * 32, ov);
         }
       }
-      const float neg_mc = (m_run == -CUDART_INF) ? 0.f : kPShift<kF16, D> - m_run * c;   // a row that has not seen a key yet (generic lists only): exp2(-inf) = 0
+      const float neg_mc = (m_run == -CUDART_INF) ? 0.f : -m_run * c;   // a row that has not seen a key yet (generic lists only): exp2(-inf) = 0
       const float2 c2 = make_float2(c, c), nm2 = make_float2(neg_mc, neg_mc);
       float2 sum2 = make_float2(0.f, 0.f);
       uint32_t pk[64];
-      if constexpr (kSplitP) {
-        // P = hi + lo, each rounded to the operand type: 2^-22 (fp16) / 2^-17 (bf16) relative, far below the output's rounding
-        uint32_t lo[64];
-#pragma unroll
-        for (int i = 0; i < 128; i += 2) {
-          const float2 xx = __ffma2_rn(make_float2(s[i], s[i + 1]), c2, nm2);
-          float2 p;
-          p.x = ex2(xx.x); p.y = ex2(xx.y);
-          sum2 = __fadd2_rn(sum2, p);
-          const uint32_t hi = pack2<kF16>(p.x, p.y);
-          const float2 hf = unpack2<kF16>(hi);
-          pk[i >> 1] = hi;
-          lo[i >> 1] = pack2<kF16>(p.x - hf.x, p.y - hf.y);
-        }
-        tmem_st64(tS + 64, lo);
-      } else if (kind == kMaskNone && a.emul) {
+      if (kind == kMaskNone && a.emul) {
         // unmasked tile of a long unit: every kEmulEvery-th pair takes the polynomial path, the rest the MUFU
 #pragma unroll
         for (int i = 0; i < 128; i += 2) {
@@ -563,7 +551,6 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
     const int t = u.q_tok + which * kTile + row;
     uint16_t* orow = a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost;
     const float inv = l_run > 0.f ? 1.f / l_run : 0.f;   // a row without any visible key (generic lists only): zeros
-    float odd = 0.f;                                     // NaN as soon as one output of the row is NaN or infinite
 #pragma unroll
     for (int q = 0; q < D / 32; ++q) {
       uint32_t ov[32];
@@ -572,10 +559,6 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
       uint32_t w[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) w[i] = pack2<kF16>(__uint_as_float(ov[2 * i]) * inv, __uint_as_float(ov[2 * i + 1]) * inv);
-      if constexpr (kSplitP) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) odd = fmaf(__uint_as_float(ov[i]), 0.f, odd);
-      }
       if (t < u.n) {                                 // rows past the end of the sequence (ragged last tile) are dropped
         if (a.o_vec32) {
           // 32-byte stores: every store fills whole 32-byte sectors (a thread owns a row, so the lanes of a
@@ -590,15 +573,214 @@ __device__ __forceinline__ void softmax_role(const Args<NS>& a, Bars* bars, int 
       }
     }
     if (a.lse != nullptr && t < u.n)
-      a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] =
-          m_run * a.sm_scale + (kSplitP ? logf(l_run) - kPShift<kF16, D> * 0.693147180559945f : __logf(l_run));
-    if constexpr (kSplitP) {
-      // the warp's rows that came out as NaN or infinite, or saw no key, one after another
-      unsigned redo = __ballot_sync(0xffffffffu, !(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n);
-      for (; redo != 0; redo &= redo - 1) {
-        __syncwarp();                                // the row's own stores come first
-        exact_row<kF16>(&a, bars, u.seq, u.b, u.h, u.list, u.cnt, t - lane + (__ffs(redo) - 1), lane);
+      a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] = m_run * a.sm_scale + __logf(l_run);
+  }
+}
+
+// What the tensor cores lose.  QK^T over 64 channels is four accumulations, each rounded towards zero: half a unit in the last place,
+// 0.36 x 2^-23 of the running sum on average (the mean of 1/mantissa is 0.72).  The running sums of a large logit grow evenly, so it
+// comes out about (1/4 + 1/2 + 3/4 + 1) x 0.36 x 2^-23 = 0.9 x 2^-23 smaller than it is (measured: 1.0 in fp16, 0.7 in bf16, whose
+// 16-bit products leave some sums exact).  That cancels in O; lse, where the size of the logits itself counts, gets it back.  A
+// tile's P V loses 1 to 3.5 x 2^-23 in the same way (500 to 8000 keys, values of one sign or of both), of which O gets 2 x 2^-23 back.
+template <bool kF16> constexpr double kQkLoss = 1.0 + (kF16 ? 1.0 : 0.7) / 8388608.0;
+constexpr float kPvLoss = 1.0f + 2.0f / 8388608.0f;
+
+// Heads of 64 channels.  A tile costs a row 128 exponentials as with 128 channels, but half the MMA work and half the output
+// columns; that room goes into 32-bit accuracy:
+//   * P is stored as the sum of two (fp16) or three (bf16) 16-bit values, each the rounding of what the ones before leave;
+//   * each tile's P V starts from zero and is added here, in registers, to nearest (a chain of MMAs over 8192 keys loses up to
+//     512 roundings towards zero: 4e-6 of O, against 3e-7 with plain fp32 sums);
+//   * changes of the reference maximum, and lse, use the offsets that the exponentials were formed with.
+// S is read a half at a time, so that 64 columns of it, their parts of P and the output fit the registers.  Columns of a query
+// tile's S region once P is in it, per half (32 columns each): hi of keys 0..63 | lo | hi of keys 64..127 | lo.
+template <bool kF16, int NS>
+__device__ __forceinline__ void softmax_role64(const Args<NS>& a, Bars* bars, int which, int warp_in_wg, int lane) {
+  constexpr float kShift = kPShift<kF16>;
+  const uint32_t tm = bars->tmem_base + (uint32_t(warp_in_wg * 32) << 16);
+  const uint32_t tS = tm + which * 128, tO = tm + 256 + which * 64, tX = tm + 384 + which * 64;
+  const int row = warp_in_wg * 32 + lane;
+  const float c = a.sm_scale * 1.4426950408889634f;   // logits -> log2 units
+  uint32_t n_tiles = 0;                               // S tiles consumed so far (all units)
+  uint32_t n_units = 0;                               // units finished so far
+  float2 o[32];
+  auto add = [&](const uint32_t* ov) {                // O += P V of a tile
+#pragma unroll
+    for (int i = 0; i < 32; ++i) o[i] = __fadd2_rn(o[i], make_float2(__uint_as_float(ov[2 * i]), __uint_as_float(ov[2 * i + 1])));
+  };
+
+  for (uint32_t q = 0;; ++q) {
+    int x;
+    Unit u;
+    if (!receive_unit(a, bars, q, lane, &x, &u) || x >= a.n_units || bars->abort_flag) return;
+    if (u.cnt == kBadList || u.cnt == kEmptyUnit) continue;
+    const int t = u.q_tok + which * kTile + row;
+    if (u.cnt == kZeroUnit) {
+      write_zero_row<64>(a, u, which, t);
+      continue;
+    }
+    const int my_tiles = which == 0 ? u.nA : u.nB;
+    if (my_tiles == 0) continue;                        // this unit has no tile B
+    float m_run = -CUDART_INF, l_run = 0.f, offset = 0.f;   // p = 2^(s c + offset), offset = kShift - m_run c rounded
+#pragma unroll
+    for (int i = 0; i < 32; ++i) o[i] = make_float2(0.f, 0.f);
+
+    for (int jt = 0; jt < my_tiles; ++jt, ++n_tiles) {
+      // the QK^T of this tile was issued behind the P V of the one before: both are there
+      if (!mbar_wait(&bars->s_full[which], n_tiles & 1, bars, a.st, 10 + which)) return;
+      tc_fence_after();
+
+      // last visible offset in each 32 columns of the tile: causal in the own diagonal tile, the listed columns in the last gathered
+      // tile, and by token in the tiles of a generic list (128/blk listed blocks, -1 beyond the list)
+      bool masked = true;
+      int lim[4];
+      if (u.generic) {
+        const int bpt = kTile / a.blk;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const int li = jt * bpt + g * 32 / a.blk;
+          lim[g] = li < u.cnt ? t - __ldg(u.list + li) * a.blk - g * 32 % a.blk : -1;
+        }
+      } else {
+        const bool diagonal = jt == my_tiles - 1;
+        masked = diagonal || (jt == u.n_past_tiles - 1 && u.last_cols < kTile);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) lim[g] = (diagonal ? row : u.last_cols - 1) - g * 32;
       }
+      auto mask32 = [&](uint32_t* v, int g) {           // columns 32 g to 32 g + 31
+        if (masked) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = i > lim[g] ? 0xff800000u : v[i];
+        }
+      };
+      auto max64 = [&](const uint32_t* v) {
+        auto s = [&](int i) { return __uint_as_float(v[i]); };
+        float mx0 = s(0), mx1 = s(1), mx2 = s(2), mx3 = s(3);
+#pragma unroll
+        for (int i = 4; i < 60; i += 8) {
+          mx0 = max3(mx0, s(i), s(i + 1)); mx1 = max3(mx1, s(i + 2), s(i + 3));
+          mx2 = max3(mx2, s(i + 4), s(i + 5)); mx3 = max3(mx3, s(i + 6), s(i + 7));
+        }
+        return fmaxf(max3(mx0, s(60), s(61)), max3(max3(mx1, s(62), s(63)), mx2, mx3));
+      };
+      uint32_t sv[64];                                  // S: keys 0..63, then keys 64..127
+      float m_tile;
+      {
+        uint32_t ov[64], first[64];
+        tmem_ld64(tS, first);
+        if (jt > 0) {
+          tmem_ld64(tO, ov);
+          tmem_wait_ld();
+          add(ov);
+        } else {
+          tmem_wait_ld();
+        }
+        tmem_ld64(tS + 64, sv);
+        mask32(first, 0); mask32(first + 32, 1);
+        m_tile = max64(first);
+      }
+      tmem_wait_ld32(sv); tmem_wait_ld32(sv + 32);
+      mask32(sv, 2); mask32(sv + 32, 3);
+      m_tile = fmaxf(m_tile, max64(sv));
+      const float m_new = fmaxf(m_run, m_tile);
+      // lazy rescale: keep the old reference maximum while the new one exceeds it by < 2^8
+      float f = 1.f;
+      if (m_run == -CUDART_INF) {                       // no key seen yet (the first tile; later ones of generic lists only)
+        m_run = m_new;
+        if (m_new != -CUDART_INF) offset = fmaf(-m_new, c, kShift);
+      } else if ((m_new - m_run) * c > kRescaleThreshold) {
+        const float offset_new = fmaf(-m_new, c, kShift);
+        f = ex2(offset_new - offset);
+        m_run = m_new;
+        offset = offset_new;
+      }
+      if (__any_sync(0xffffffffu, f != 1.f)) {
+        l_run *= f;
+        const float2 f2 = make_float2(f, f);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) o[i] = __fmul2_rn(o[i], f2);
+      }
+      const float2 c2 = make_float2(c, c), off2 = make_float2(offset, offset);
+      float2 sum2[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sum2[i] = make_float2(0.f, 0.f);
+      auto probabilities = [&](const uint32_t* v, int g) {   // of keys 32 g to 32 g + 31, to tensor memory
+        uint32_t hi[16], lo[16], third[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float2 xx = __ffma2_rn(make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), c2, off2);
+          float2 p;
+          p.x = ex2(xx.x); p.y = ex2(xx.y);
+          sum2[i & 3] = __fadd2_rn(sum2[i & 3], p);
+          hi[i] = pack2<kF16>(p.x, p.y);
+          const float2 hf = unpack2<kF16>(hi[i]);
+          p.x -= hf.x; p.y -= hf.y;
+          lo[i] = pack2<kF16>(p.x, p.y);
+          if constexpr (!kF16) {
+            const float2 lf = unpack2<kF16>(lo[i]);
+            third[i] = pack2<kF16>(p.x - lf.x, p.y - lf.y);
+          }
+        }
+        tmem_st16(tS + (g >> 1) * 64 + (g & 1) * 16, hi);
+        tmem_st16(tS + (g >> 1) * 64 + 32 + (g & 1) * 16, lo);
+        if constexpr (!kF16) tmem_st16(tX + g * 16, third);
+      };
+      // the second half of S is at hand; the first comes back 32 columns at a time under the exponentials of the ones before
+      probabilities(sv, 2);
+      uint32_t sa[32], sb[32];
+      tmem_ld32(tS, sa);
+      probabilities(sv + 32, 3);
+      tmem_wait_ld32(sa);
+      mask32(sa, 0);
+      tmem_ld32(tS + 32, sb);
+      tmem_wait_ld32(sb);                               // before P of keys 0..31 goes over these columns
+      probabilities(sa, 0);
+      mask32(sb, 1);
+      probabilities(sb, 1);
+      sum2[0] = __fadd2_rn(__fadd2_rn(sum2[0], sum2[1]), __fadd2_rn(sum2[2], sum2[3]));
+      l_run += sum2[0].x + sum2[0].y;
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(&bars->p_full[which]);
+    }
+
+    // epilogue: the last tile's P V, O / l -> global.  The next unit's first PV cannot start before this thread signals its next P.
+    if (!mbar_wait(&bars->o_done[which], n_units & 1, bars, a.st, 20 + which)) return;
+    ++n_units;
+    tc_fence_after();
+    {
+      uint32_t ov[64];
+      tmem_ld64(tO, ov);
+      tmem_wait_ld();
+      add(ov);
+    }
+    uint16_t* orow = a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost;
+    const float inv = l_run > 0.f ? kPvLoss / l_run : 0.f;   // a row without any visible key (generic lists only): zeros
+    float odd = 0.f;                                     // NaN as soon as one output of the row is NaN or infinite
+#pragma unroll
+    for (int i = 0; i < 32; ++i) odd = fmaf(o[i].y, 0.f, fmaf(o[i].x, 0.f, odd));
+    if (t < u.n) {                                       // rows past the end of the sequence (ragged last tile) are dropped
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = pack2<kF16>(o[q4 * 8 + i].x * inv, o[q4 * 8 + i].y * inv);
+        if (a.o_vec32) {
+          st_global_v8(orow + q4 * 16, w);               // whole 32-byte sectors (see softmax_role)
+        } else {
+          uint4* dst = reinterpret_cast<uint4*>(orow + q4 * 16);
+          dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+          dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+      }
+      if (a.lse != nullptr)
+        a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] =
+            float(double(m_run) * (a.sm_scale * kQkLoss<kF16>) + (log(double(l_run)) - 0.693147180559945309417 * (double(m_run) * c + offset)));
+    }
+    // the warp's rows that came out as NaN or infinite, or saw no key, one after another
+    unsigned redo = __ballot_sync(0xffffffffu, !(odd == 0.f && l_run > 0.f && l_run < CUDART_INF_F) && t < u.n);
+    for (; redo != 0; redo &= redo - 1) {
+      __syncwarp();                                      // the row's own stores come first
+      exact_row<kF16>(&a, bars, u.seq, u.b, u.h, u.list, u.cnt, t - lane + (__ffs(redo) - 1), lane);
     }
   }
 }
@@ -674,15 +856,25 @@ __device__ __forceinline__ void issue_qk(uint32_t d_tmem, uint32_t q_smem, uint3
   }
 }
 template <bool kF16, int D>
-__device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint32_t v_smem, bool acc) {
+__device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint32_t x_tmem, uint32_t v_smem, bool acc) {
   const uint64_t base = desc_base(kHalfBytes);   // the two 64-column halves of head_dim are 16 KB apart
+  if constexpr (Shape<D>::kSplitP) {
+    // the parts of P, smallest first, into a sum that starts from zero (softmax_role64 adds the tiles up)
+    if constexpr (!kF16) {
 #pragma unroll
-  for (int kk = 0; kk < kTile / 16; ++kk)
-    umma_ts(d_tmem, p_tmem + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, (acc || kk > 0) ? 1u : 0u);
-  if constexpr (Shape<D>::kSplitP) {             // the low halves of P
+      for (int kk = 0; kk < kTile / 16; ++kk)
+        umma_ts(d_tmem, x_tmem + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, kk > 0);
+    }
+#pragma unroll
+    for (int part = 1; part >= 0; --part)
+#pragma unroll
+      for (int kk = 0; kk < kTile / 16; ++kk)
+        umma_ts(d_tmem, p_tmem + (kk >> 2) * 64 + part * 32 + (kk & 3) * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv,
+                (!kF16 || part == 0 || kk > 0) ? 1u : 0u);
+  } else {
 #pragma unroll
     for (int kk = 0; kk < kTile / 16; ++kk)
-      umma_ts(d_tmem, p_tmem + 64 + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, 1u);
+      umma_ts(d_tmem, p_tmem + kk * 8, desc_at(base, v_smem + kk * 16 * 128), Idesc<kF16, D>::pv, (acc || kk > 0) ? 1u : 0u);
   }
 }
 
@@ -690,7 +882,7 @@ template <bool kF16, int D, int NS>
 __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t smem_base, int lane) {
   constexpr int kSlots = Shape<D>::kSlots, kTileBytes = Shape<D>::kTileBytes;
   const uint32_t tm = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
-  const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 256 + D};
+  const uint32_t tS[2] = {tm, tm + 128}, tO[2] = {tm + 256, tm + 256 + D}, tX[2] = {tm + 384, tm + 448};   // tX: 64 channels only
   const uint32_t qA = smem_base + Shape<D>::kSmemQ, qB = qA + kTileBytes;
   uint32_t item0 = 0;                 // first K/V item of the current unit
   uint32_t nA = 0, nB = 0;            // P tiles consumed so far per query tile (all units)
@@ -723,7 +915,7 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
         if (!mbar_wait(&bars->p_full[0], nA & 1, bars, a.st, 42)) return;
         ++nA;
         tc_fence_after();
-        issue_pv<kF16, D>(tO[0], tS[0], v_smem, jt > 0);
+        issue_pv<kF16, D>(tO[0], tS[0], tX[0], v_smem, jt > 0);
         if (jt + 1 < TA) { issue_qk<kF16, D>(tS[0], qA, kn_smem); umma_commit(&bars->s_full[0]); }
         else umma_commit(&bars->o_done[0]);
       }
@@ -731,7 +923,7 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
         if (!mbar_wait(&bars->p_full[1], nB & 1, bars, a.st, 43)) return;
         ++nB;
         tc_fence_after();
-        issue_pv<kF16, D>(tO[1], tS[1], v_smem, jt > 0);
+        issue_pv<kF16, D>(tO[1], tS[1], tX[1], v_smem, jt > 0);
       }
       umma_commit(&bars->kv_empty[iv % kSlots]);             // every PV that reads this V tile has been issued
       if (has_next) {
@@ -783,7 +975,8 @@ attention_sm100_kernel(const __grid_constant__ Maps<NS> maps, const __grid_const
   static_assert(kRegPoolNeeded <= kThreads * 168, "setmaxnreg budget exceeds the launch allocation");
   if (warp < 8) {
     reg_inc<216>();
-    softmax_role<kF16, D, NS>(a, bars, warp >> 2, warp & 3, lane);
+    if constexpr (D == 64) softmax_role64<kF16, NS>(a, bars, warp >> 2, warp & 3, lane);
+    else softmax_role<kF16, NS>(a, bars, warp >> 2, warp & 3, lane);
   } else {
     reg_dec<64>();
     if (warp == 8) producer_role<D, NS>(a, bars, smem_base, maps, lane);

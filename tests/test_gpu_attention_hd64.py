@@ -1,12 +1,12 @@
-"""The tensor-core attention kernel on heads of 64 channels (probabilities held as the sum of two 16-bit values) against
+"""The tensor-core attention kernel on heads of 64 channels (probabilities held as sums of two or three 16-bit values) against
 the fp64 oracle: tile edges, ragged tails, odd tile counts, one-unit and long problems, and values that are not finite."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
-from paper_2409_12490_b200 import binding as cp
-from paper_2409_12490_b200.inputs import make_uniform_qkv
+from paper_2409_12490_b200 import CONFIGS, binding as cp
+from paper_2409_12490_b200.inputs import make_qkv, make_uniform_qkv
 
 from helpers import f32
 
@@ -26,7 +26,7 @@ def layer(dtype, B, Hq, Hkv, n, seg, blk, k, seed=3):
 
 
 def assert_close(O, O_ref, V, dtype):
-    """|O_gpu - O| <= u |O| + e max|V|: u is the unit roundoff of the one rounding of O; e covers the split of P (2^-17 for
+    """|O_gpu - O| <= u |O| + e max|V|: u is the unit roundoff of the one rounding of O; e covers the split of P (2^-24 for
     bf16, 2^-22 for fp16), exponentials and logits in fp32 (2^-20 each) and fp32 accumulation over up to 2^11 keys (2^-16 at
     most).  A single 16-bit rounding of P (2^-9 max|V| and 2^-12 max|V|) would not pass on averages of this length."""
     u, e = {"bf16": (2.0 ** -8, 2.0 ** -15), "f16": (2.0 ** -11, 2.0 ** -15)}[dtype]
@@ -47,6 +47,29 @@ def test_sparse_and_dense_match_the_oracle(dtype, B, Hq, Hkv, n, seg, blk, k):
     assert_close(O, O_ref, V, dtype)
     assert np.abs(lse.cpu().numpy() - lse_ref).max() <= 1e-4
     assert_close(Od, oracle.dense_attention(Q, K, V, SM)[0], V, dtype)
+
+
+@pytest.mark.parametrize("positive", [False, True])
+@pytest.mark.parametrize("dtype,share", [("bf16", 2.0 ** -11), ("f16", 2.0 ** -8)])
+def test_outputs_are_those_of_32_bit_arithmetic(dtype, share, positive):
+    """Before its rounding to 16 bits (spacing 2^-8 to 2^-7 of the output in bf16, 2^-11 to 2^-10 in fp16) O is good to 2^-19 of its
+    size: roundings in fp32 over 8000 keys, not a chain of accumulations towards zero (2^-16 when the values have one sign).  So
+    at most 2^-19 / 2^-8 or 2^-19 / 2^-11 of the outputs are rounded otherwise than the fp64 result."""
+    n = 8000
+    cfg = CONFIGS["C2"].with_(name="hd64", seq_len=n, n_q_heads=4, n_kv_heads=2, head_dim=64, segment_size=512, block_size=64,
+                              budget_tokens=1024, n_clusters=16, dtype=dtype)
+    Q, K, V = (t.cuda() for t in make_qkv(cfg))
+    V = V.abs() if positive else V
+    prob = cp.Problem.from_config(cfg)
+    ws = cp.alloc_workspace(prob)
+    O = cp.dense_attention(prob, Q, K, V, ws)
+    assert cp.device_status(ws) == 0
+    future = torch.ones((n, n), dtype=torch.bool, device="cuda").triu(1)
+    off = 0.0
+    for h in range(4):
+        s = ((Q[0, h].double() @ K[0, h // 2].double().T) * SM).masked_fill_(future, -float("inf"))
+        off += float((O[0, h] != (torch.softmax(s, 1) @ V[0, h // 2].double()).to(O.dtype)).double().mean()) / 4
+    assert off <= share, off
 
 
 def launched_grids(call):
