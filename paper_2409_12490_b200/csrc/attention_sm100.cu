@@ -998,7 +998,9 @@ bool make_map(CUtensorMap* map, const void* base, int B, int H, int n, int d, co
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return false;
   cuuint64_t dims[4] = {cuuint64_t(d), cuuint64_t(n), cuuint64_t(H), cuuint64_t(B)};
-  cuuint64_t strides[3] = {cuuint64_t(s[2]) * 2, cuuint64_t(s[1]) * 2, cuuint64_t(s[0]) * 2};
+  // nothing reads the stride of a dimension of extent 1, and the encoder takes no stride of 2^40 bytes
+  auto stride = [&](int extent, int64_t x) { return extent > 1 ? cuuint64_t(x) * 2 : cuuint64_t(d) * 2; };
+  cuuint64_t strides[3] = {stride(n, s[2]), stride(H, s[1]), stride(B, s[0])};
   cuuint32_t box[4] = {64, cuuint32_t(rows), 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,

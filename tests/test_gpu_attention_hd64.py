@@ -123,6 +123,41 @@ def test_value_that_is_not_finite_reaches_only_the_rows_that_see_it(dtype):
         assert_close(torch.from_numpy(O[0][~sees]), O_ref[0][~sees], V, dtype)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("storage", ["heads share their keys", "batches share their keys", "queries shared", "tokens first"])
+def test_strides(dtype, storage):
+    """Strides of 0 (expanded tensors), a token stride that is larger than the head stride, and the stride of a dimension of extent 1,
+    which nothing reads, at 2^40 bytes."""
+    B, H, n, seg, blk, k = 2, 3, 700, 256, 64, 6
+    Q, K, V = make_uniform_qkv(B, H, H, n, 64, dtype=dtype, seed=5)
+    if storage == "heads share their keys":
+        K, V = K[:, :1].expand(-1, H, -1, -1), V[:, :1].expand(-1, H, -1, -1)
+    elif storage == "batches share their keys":
+        K, V = K[:1].expand(B, -1, -1, -1), V[:1].expand(B, -1, -1, -1)
+    elif storage == "queries shared":
+        Q = Q[:, :1].expand(-1, H, -1, -1)
+    dense = [t.contiguous().cuda() for t in (Q, K, V)]
+    if storage == "tokens first":
+        Qd, Kd, Vd = (t.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for t in dense)
+        Qd, Kd, Vd = (t[:1].as_strided((1, H, n, 64), (1 << 39, 64, H * 64, 1)) for t in (Qd, Kd, Vd))
+        dense = [t[:1] for t in dense]
+    else:
+        Qd, Kd, Vd = (t.cuda() if t.is_contiguous() else _expand_like(t) for t in (Q, K, V))
+    prob = cp.Problem(Qd.shape[0], H, H, n, 64, seg, blk, k, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    idx, cnt = cp.select(prob, cp.estimate(prob, dense[0], dense[1], ws), ws)
+    O = torch.empty_like(dense[0])
+    for a, b in ((cp.attention(prob, Qd, Kd, Vd, idx, cnt, ws, O=O.clone()), cp.attention(prob, *dense, idx, cnt, ws)),
+                 (cp.dense_attention(prob, Qd, Kd, Vd, ws, O=O.clone()), cp.dense_attention(prob, *dense, ws))):
+        assert torch.equal(a, b)
+    assert cp.device_status(ws) == 0
+
+
+def _expand_like(t):
+    """The expanded CPU tensor's one copy on the device, expanded again."""
+    return t[tuple(slice(0, 1) if s == 0 else slice(None) for s in t.stride())].contiguous().cuda().expand(t.shape)
+
+
 def test_value_that_is_not_finite_at_the_end_of_a_long_sequence():
     """The last 300 rows of 1.3 M tokens see an infinite value and are evaluated one by one, over more keys than the kernel's waits
     would sit out for a thread per row: the call ends without an error, every row before them is finite, and the rows are those of
