@@ -58,3 +58,22 @@ def test_fused_layers_equal_their_own_calls(flags, dtype, d, room):
         O1, S1, idx1, cnt1 = cp.prefill_layer(one, *[t[None, :, lo:hi] for t in layers[1]], ws, S_prev=first[1][i][None])
         assert torch.equal(S[i], S1[0]) and torch.equal(idx[i], idx1[0]) and torch.equal(cnt[i], cnt1[0])
         assert torch.equal(O[:, lo:hi], O1[0])
+
+
+def test_batch_whose_scores_need_clusters_of_every_size():
+    """Four heads per CTA, blocks of 4 tokens: up to 1064 blocks fit one CTA's shared memory, 2128 two, 4256 four, 8192 eight.  Two sequences
+    of each size in one batch, alternating, so that every cluster launch holds several sequences with offsets of their own."""
+    lens, Hq, Hkv, d, seg, blk, k = [3000, 8000, 18000, 5000, 33, 9000, 4265, 20000, 4300, 17000], 4, 1, 64, 256, 4, 64
+    total, cu = sum(lens), [0] + np.cumsum(lens).tolist()
+    layers = [[t[0].cuda() for t in make_uniform_qkv(1, Hq, Hkv, total, d, dtype="f32", seed=s)] for s in (3, 4)]
+    prob = cp.Problem(1, Hq, Hkv, max(lens), d, seg, blk, k, torch.float32)
+    ws = torch.zeros(8 * cp.workspace_bytes(prob), dtype=torch.uint8, device="cuda")
+    first = cp.prefill_varlen(prob, cu, *layers[0], ws)
+    O, S, idx, cnt, _ = cp.prefill_varlen(prob, cu, *layers[1], ws, S_prev=first[4])
+    assert cp.device_status(ws) == 0
+    for i, (lo, hi) in enumerate(zip(cu[:-1], cu[1:])):
+        one = cp.Problem(1, Hq, Hkv, hi - lo, d, seg, blk, k, torch.float32)
+        S0 = cp.estimate(one, layers[0][0][None, :, lo:hi], layers[0][1][None, :, lo:hi], ws)
+        O1, S1, idx1, cnt1 = cp.prefill_layer(one, *[t[None, :, lo:hi] for t in layers[1]], ws, S_prev=S0)
+        assert torch.equal(first[1][i], S0[0]) and torch.equal(S[i], S1[0])
+        assert torch.equal(idx[i], idx1[0]) and torch.equal(cnt[i], cnt1[0]) and torch.equal(O[:, lo:hi], O1[0])
