@@ -14,7 +14,8 @@
  *   - Calls validate their arguments on the host, enqueue kernels on `cuda_stream`
  *     (a cudaStream_t passed as void*; NULL = the default stream) and return without
  *     synchronising.  Outputs are valid once the stream reaches that point.
- *     The calls (critiprefill_device_status excepted) only enqueue kernels (critiprefill_estimate_static also a small memset), so a stream
+ *     The calls (critiprefill_device_status excepted) only enqueue kernels (critiprefill_estimate_static also a small memset,
+ *     critiprefill_decode_estimate two copies inside the device for blocks of more than 128 rows and very large groups), so a stream
  *     that is being captured into a CUDA graph may carry them; the graph then refers to the buffers given at
  *     capture time (tensor maps are encoded on the host from those pointers).
  *   - Return value: a cp_status.  Conditions only the device can see (a block list that

@@ -208,7 +208,7 @@ int prefill_varlen(const cp_params* p, const int32_t* cu_seqlens, int32_t n_seqs
   Dims m;
   if ((rc = validate(p, &m)) != CP_OK) return rc;   // the longest sequence: strides, dtype, head geometry, budget
   if (!Q || !K || !V || !O || !S_out || !idx || !cnt) return CP_ERR_NULL;
-  if (p->flags & CP_FLAG_SUMMARIES_READY) return CP_ERR_UNSUPPORTED;   // the workspace holds one sequence's representatives at a time
+  if (p->flags & CP_FLAG_SUMMARIES_READY) return CP_ERR_UNSUPPORTED;   // they are formed here, group by group, wherever the workspace has room
   if ((rc = check_ws(m, ws, ws_bytes)) != CP_OK) return rc;
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || S_out == S_prev) return CP_ERR_SHAPE;
   if (S_prev != nullptr && !(p->alpha >= 0.0f && p->alpha <= 1.0f)) return CP_ERR_SHAPE;

@@ -417,7 +417,8 @@ int launch_t(const cp_params& p, const Dims& m, const void* Q, const void* K, co
   constexpr int kNG = D * sizeof(T) <= 256 ? 4 : 2;
   const long long ctas32 = (long long)m.B * m.Hq * ((m.n + 31) / 32);
   if (ctas32 < 4 * 148) return launch_rt<T, D, 4, kNG>(a, m, s);
-  if (D == 64 && m.seg >= 64) return launch_rt<T, D, 8, 1>(a, m, s);
+  if constexpr (D == 64)
+    if (m.seg >= 64) return launch_rt<T, D, 8, 1>(a, m, s);
   return launch_rt<T, D, 4, 1>(a, m, s);
 }
 

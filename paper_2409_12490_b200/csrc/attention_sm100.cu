@@ -59,7 +59,7 @@ constexpr float kRescaleThreshold = 8.0f;           // in log2 units
 constexpr int kEmulEvery = CP_EMUL_EVERY;           // 0: all exponentials on the MUFU; n: every n-th pair on the FMA pipes
 constexpr int kRegPoolNeeded = 256 * 216 + 128 * 64;   // registers the roles hold after setmaxnreg (softmax 216, producer/MMA 64)
 
-// One work unit, decoded (the producer warp decodes it once and publishes it to the other warps:
+// One work unit, decoded (the scheduler warp decodes it once and publishes it to the other warps:
 // the decoding is a chain of integer divisions that would otherwise sit at the start of every unit).
 struct Unit {
   int b, h, kvh;
@@ -148,9 +148,10 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
 // ordered KV-head-major (within a KV head from the sequence's end, longest first for the dense kernel): the CTAs that are
 // resident together then read the same tiles through L2.  When all K and V (nearly) fit L2 together that does not matter
 // and the order is longest units first over all heads and sequences (long_first; the host sorts the (segment, pair)s by
-// the tiles they stream), which leaves the short ones to even out the ends of the CTAs: 8192 tokens x 32 heads, segment 512,
-// budget 1024: 133 -> 118 us; 32768 tokens (134 MB), budget 2048: 857 -> 836 us; dense 24576 tokens (101 MB): 3.95 -> 3.80 ms;
-// but 131072 tokens (537 MB), segment 1024, budget 4096: 6.4 -> 6.8 ms.
+// the tiles they stream), which leaves the short ones to even out the ends of the CTAs.  Both orders, us, 32 query / 8 KV heads:
+// dense, KV-head-major / longest first: 34 MB of K and V 592 / 502, 101 MB 4479 / 4367, 168 MB 12125 / 12106, 201 MB 17344 / 17439,
+// 268 MB 30381 / 31149; segment 512, budget 1024: 67 MB 267 / 247, 134 MB 539 / 504, 268 MB 1069 / 1007, 537 MB 2113 / 2039; segment
+// 1024, budget 4096: 134 MB 1783 / 1749, 268 MB 3647 / 3586, 537 MB 7335 / 7285.  The line (160 MB) is the dense kernel's.
 // `cnt` is the unit's list length when the caller already has it, kLoadCnt to read it from global memory.
 constexpr int kLoadCnt = -2, kBadList = -1, kEmptyUnit = -3, kZeroUnit = -4;   // kEmptyUnit: no query row of the unit lies inside the sequence;
                                                                                 // kZeroUnit: an empty list -- the unit's rows are zeros
@@ -226,7 +227,7 @@ __device__ __forceinline__ Unit decode_unit(const Args<NS>& a, int x, int cnt) {
   return u;
 }
 
-// The list contract, checked by the producer warp before it publishes a unit: at most k entries, ascending, unique,
+// The list contract, checked by the scheduler warp before it publishes a unit: at most k entries, ascending, unique,
 // each a block the segment can see (0 <= b < (j+1)*r).  Returns 0 when the list has the form the selection emits
 // (past blocks, then exactly the diagonal blocks of the segment: the fast tile sequence applies), 1 for any other
 // valid list (generic tile sequence), -1 for a list that breaks the contract.
@@ -1108,8 +1109,9 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
                                 : (long long)m.B * m.Hq * a.n_segs * a.pp;
   if (units > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   a.n_units = int(units);
-  // K and V of every head up to 160 MB (measured on both sides: see decode_unit; the L2 has 126 MB); a batch of sequences always (its neighbours in the order are the
-  // heads of one segment, so one sequence or two are in use at a time)
+  // K and V of every head up to 160 MB (measured on both sides: see decode_unit; the L2 has 126 MB); a batch of sequences always: over
+  // lists the order pays at every size measured there, and one launch saves the end of another (two prompts of 131072 tokens,
+  // segment 1024, budget 4096, whole layers: 15.8 ms in one batch, 16.1 ms in two calls; of 65536 7.6 / 7.8 ms)
   a.long_first = (NS > 1 || kv_tokens * m.B * m.Hkv * m.d * m.es * 2 <= 160ll << 20) ? 1 : 0;
   if (a.long_first && !dense) {
     const int entries = order_units(a);

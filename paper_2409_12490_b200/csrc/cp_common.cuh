@@ -107,7 +107,8 @@ int launch_project(const cp_params& p, const Dims& m, const void* X, const void*
 int launch_decode_score(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* S_out, char* ws, cudaStream_t st);
 bool decode_path_applies(const Dims& m);
 
-// Programmatic dependent launch: a kernel of this library starts while its predecessor drains.  Every thread of such a kernel
+// Programmatic dependent launch: a kernel starts while its predecessor drains, if that one calls pdl_trigger (those of the estimate, the
+// selection, decoding and SIMT attention do; the projection and tensor-core attention don't, and have no successor before their end).  Every thread of such a kernel
 // calls pdl_wait before it touches global memory (the predecessor has then finished and its writes are visible, so nothing else
 // about stream order changes); pdl_trigger lets the successor start its own way to that point.  The pointers named in pdl_wait
 // pass through it, so that no read-only load through them (__ldg, const __restrict__) can be scheduled before the wait.

@@ -259,8 +259,8 @@ def test_single_token_segments_and_blocks_give_token_wise_critical_sets():
 
 
 def test_layer_replays_from_a_cuda_graph():
-    """estimate + select + attention captured once into a CUDA graph (the library only enqueues kernels and one
-    memset on the caller's stream, and encodes its tensor maps on the host) and replayed on new inputs written
+    """estimate + select + attention captured once into a CUDA graph (the library only enqueues kernels
+    on the caller's stream, and encodes its tensor maps on the host) and replayed on new inputs written
     into the same buffers: every replay must equal the eager result for those inputs."""
     cfg = BASE.with_(seq_len=1536)
     prob = problem(cfg)
