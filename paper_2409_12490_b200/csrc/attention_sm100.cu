@@ -700,7 +700,7 @@ __device__ __forceinline__ void softmax_role64(const Args<NS>& a, Bars* bars, in
 #pragma unroll
         for (int i = 0; i < 32; ++i) o[i] = __fmul2_rn(o[i], f2);
       }
-      const float2 c2 = make_float2(c, c), off2 = make_float2(offset, offset);
+      const float2 c2 = make_float2(c, c), off2 = make_float2(offset, offset), minus1 = make_float2(-1.f, -1.f);
       float2 sum2[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) sum2[i] = make_float2(0.f, 0.f);
@@ -713,12 +713,11 @@ __device__ __forceinline__ void softmax_role64(const Args<NS>& a, Bars* bars, in
           p.x = ex2(xx.x); p.y = ex2(xx.y);
           sum2[i & 3] = __fadd2_rn(sum2[i & 3], p);
           hi[i] = pack2<kF16>(p.x, p.y);
-          const float2 hf = unpack2<kF16>(hi[i]);
-          p.x -= hf.x; p.y -= hf.y;
+          p = __ffma2_rn(unpack2<kF16>(hi[i]), minus1, p);   // exact: what the part leaves
           lo[i] = pack2<kF16>(p.x, p.y);
           if constexpr (!kF16) {
-            const float2 lf = unpack2<kF16>(lo[i]);
-            third[i] = pack2<kF16>(p.x - lf.x, p.y - lf.y);
+            p = __ffma2_rn(unpack2<kF16>(lo[i]), minus1, p);
+            third[i] = pack2<kF16>(p.x, p.y);
           }
         }
         tmem_st16(tS + (g >> 1) * 64 + (g & 1) * 16, hi);
