@@ -19,8 +19,9 @@
 // are resident take over the units of those that have not started yet, one after another
 // (clusterlaunchcontrol.try_cancel, scheduler warp), and publish them to the other warps, so faster SMs
 // take more units without a counter in memory that a launch of its own would have to clear (and whose
-// round trip had to be waited out: 131072 tokens x 32 heads, segment 512, budget 1024: 2.03 -> 1.83 ms).  Every wait
-// is bounded: on expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
+// round trip had to be waited out).  With the scheduler warp and the order of units below, against a counter that the producer
+// warp read, 32 heads, segment 512, block 32, budget 1024, medians of nine: 1300 tokens 47.3 -> 32.4 us, 8192 145 -> 128, 131072
+// 2234 -> 2110 us; dense 4096 tokens 176 -> 141 us, 20001 unchanged (3.0 ms).  Every wait is bounded: on expiry the waiter raises a CTA-wide abort flag and CP_ERR_TIMEOUT, and all roles drain.
 // One launch serves one problem or a packed batch of up to kMaxSeqs sequences (each with tensor maps of
 // its own, so that reads past a sequence's end arrive as zeros and never as a neighbour's tokens).
 #include <algorithm>
@@ -260,8 +261,7 @@ __device__ __forceinline__ bool stop_requested(const Args<NS>& a, Bars* bars) {
 // The scheduler warp gets the q-th unit of this CTA (its own block index first, then those of CTAs that the hardware
 // lets it cancel), reads and checks its block list, and publishes (unit, list length) through a two-entry ring; the
 // other warps take it from there and touch no global memory at a unit's start.  This is a chain of three round trips
-// (3-4 K cycles): in the producer warp it held up the loads of the unit before (with it, and with one lane per box in the
-// producer: 131072 tokens, segment 512, budget 1024: 1.85 -> 1.80 ms; 1300 tokens: 36.6 -> 35.2 us; long units unchanged).
+// (3-4 K cycles): in the producer warp it held up the loads of the unit before (figures: head of this file).
 // A unit is drawn when the producer begins the one before it, no earlier, so that no CTA sits on units at the end.
 // A list that breaks its contract is published with length kBadList and skipped by everyone.
 __device__ __forceinline__ void request_unit(Bars* bars) {

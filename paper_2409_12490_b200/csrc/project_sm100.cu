@@ -92,7 +92,8 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   // The s-th unit of this CTA.  Query units are dealt round-robin, heads of one segment adjacent so that its X rows stay in
   // L2; then come the single tiles of the key and value heads (heads of one tile adjacent), which the CTAs without a query unit in
   // the last round begin one unit's length earlier.  At 16384 tokens, segment 512, 32 + 8 + 8 heads, units of a whole segment for
-  // every head left the last of 6 rounds a fifth full (768 units on 148 SMs): 648 us, here 576 us = 1430 TFLOP/s.  Keys and values
+  // every head left the last of 6 rounds a fifth full (768 units on 148 SMs): 759 us, here 726 us = 1136 TFLOP/s (medians of six
+  // loops at the power cap; 131072 tokens, segment 1024: 5.58 -> 5.45 ms).  Keys and values
   // share this pass because with all three weight matrices live at once the weights and the X tiles in flight no longer
   // fit the L2 share of a die and every head slows down.
   auto work = [&](long long s, Work* w) {
