@@ -5,7 +5,8 @@
 // GEMM on the tcgen05 tensor cores: D[128 tokens x 128 channels] = X_tile[128 x d_model] * W_head[128 x d_model]^T per
 // head; an output tile is 128 tokens of two adjacent heads of one kind (one head where a kind has an odd head count),
 // so that both heads share the X operand of every MMA.  A query unit is (batch, head group, segment): its seg/128 token
-// tiles run back to back on one CTA, so the segment's running max / min stay on chip; key and value units are single tiles
+// tiles run back to back on one CTA, so the segment's running max / min stay on chip; key and value units are single tiles (segments too where all units
+// have an SM of their own)
 // (a key block never crosses a tile), which even out what the query units leave of the last round.  Warps 0-3: epilogue (one thread
 // per token row: tensor-memory load, rotation, rounding, stores; then one thread per channel for the column scans), warp 4:
 // TMA producer (X and W tiles of 64 d_model columns, 128-byte swizzle), warp 5: MMA issuer; the accumulator stages in
@@ -48,7 +49,8 @@ struct ProjArgs {
   float* kabs;
   DeviceStatus* st;
   int B, Hq, Hkv, Hv, n, seg, blk, n1, n2, d_model;   // Hv = Hkv when values are projected too, else 0
-  long long n_q, n_kv;                        // query units; single tiles of the key and value heads
+  long long n_q, n_kv;                        // units of the query heads; of the key and value heads
+  int kv_t;                                   // tiles of a key or value unit
 };
 
 struct Work { int b, hh, j, tok0, nt; };      // batch, first head (query, then key, then value heads), segment, first token, tiles
@@ -120,9 +122,9 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const int H = (a.Hkv + a.Hv) / kNH;
     w->hh = a.Hq + int(x % H) * kNH; x /= H;
     w->b = int(x % a.B); x /= a.B;
-    w->tok0 = int(x) * kTileM;
+    w->tok0 = int(x) * a.kv_t * kTileM;
     w->j = 0;
-    w->nt = 1;
+    w->nt = min(a.kv_t, (a.n - w->tok0 + kTileM - 1) / kTileM);
     return true;
   };
 
@@ -323,7 +325,15 @@ int launch_project(const cp_params& p, const Dims& m, const void* X, const void*
   // two heads per output tile where every kind has an even head count (see Geo)
   const int nh = (m.Hq % 2 == 0 && m.Hkv % 2 == 0) ? 2 : 1;
   a.n_q = (long long)m.B * (m.Hq / nh) * m.n1;
-  a.n_kv = (long long)m.B * ((m.Hkv + a.Hv) / nh) * ((m.n + kTileM - 1) / kTileM);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return CP_ERR_CUDA;
+  // Key and value units are single tiles, unless whole segments of every head have an SM of their own: then the query units' time is
+  // the launch's, and more CTAs only take bandwidth from them (32 + 8 + 8 heads, segment 512: 1300 tokens 103.5 us with single
+  // tiles, 100.4 with segments; 300 tokens 71.7 either way).
+  const long long kv_heads = (long long)m.B * ((m.Hkv + a.Hv) / nh);
+  a.kv_t = a.n_q + kv_heads * m.n1 <= sms ? m.seg / kTileM : 1;
+  a.n_kv = a.kv_t > 1 ? kv_heads * m.n1 : kv_heads * ((m.n + kTileM - 1) / kTileM);
   CUtensorMap tmX, tmWq, tmWk, tmWv;
   if (!make_map3(&tmX, X, d_model, m.n, m.B, f16) || !make_map3(&tmWq, Wq, d_model, (long long)m.Hq * kD, 1, f16, 128 * nh) ||
       !make_map3(&tmWk, Wk, d_model, (long long)m.Hkv * kD, 1, f16, 128 * nh))
@@ -334,9 +344,6 @@ int launch_project(const cp_params& p, const Dims& m, const void* X, const void*
                       : (f16 ? project_sm100_kernel<true, 1> : project_sm100_kernel<false, 1>);
   const int smem = (nh == 2 ? Geo<2>::kSmemBar : Geo<1>::kSmemBar) + int(sizeof(ProjBars)) + 1024;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return CP_ERR_CUDA;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return CP_ERR_CUDA;
   const unsigned grid = unsigned(a.n_q + a.n_kv < sms ? a.n_q + a.n_kv : sms);
   kern<<<grid, kThreads, smem, st>>>(tmX, tmWq, tmWk, tmWv, a);
   return check_launch();

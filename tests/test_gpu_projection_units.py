@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("values", [True, False])
 @pytest.mark.parametrize("B,n,seg,blk,Hq,Hkv", [(1, 128, 128, 32, 2, 2), (1, 2000, 1024, 128, 4, 2), (2, 1300, 512, 64, 16, 4),
-                                                (1, 4500, 128, 32, 8, 8), (1, 1153, 256, 128, 3, 1)])
+                                                (1, 4500, 128, 32, 8, 8), (1, 1153, 256, 128, 3, 1),
+                                                (1, 3301, 256, 64, 32, 8), (1, 300, 512, 64, 32, 8)])
 def test_every_tile_is_projected_once(B, n, seg, blk, Hq, Hkv, values):
     torch.manual_seed(n)
     D, dm = 128, 256
