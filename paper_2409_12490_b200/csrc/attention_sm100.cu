@@ -594,6 +594,9 @@ constexpr float kPvLoss = 1.0f + 2.0f / 8388608.0f;
 //   * changes of the reference maximum, and lse, use the offsets that the exponentials were formed with.
 // S is read a half at a time, so that 64 columns of it, their parts of P and the output fit the registers.  Columns of a query
 // tile's S region once P is in it, per half (32 columns each): hi of keys 0..63 | lo | hi of keys 64..127 | lo.
+// Bound by the instructions of these threads (3700 cycles per pair of tiles in fp16, of which the exponentials need 2050).  Two
+// sequences of 6001 tokens, 16 heads, segment 512, block 64, budget 1024: fp16 112 us, bf16 130 us (90 and 88 us with two parts of P
+// in either type and one chain of accumulations, whose error was larger than that of plain fp32).
 template <bool kF16, int NS>
 __device__ __forceinline__ void softmax_role64(const Args<NS>& a, Bars* bars, int which, int warp_in_wg, int lane) {
   constexpr float kShift = kPShift<kF16>;

@@ -5,9 +5,9 @@
 // GEMM on the tcgen05 tensor cores: D[128 tokens x 128 channels] = X_tile[128 x d_model] * W_head[128 x d_model]^T per
 // head; an output tile is 128 tokens of two adjacent heads of one kind (one head where a kind has an odd head count),
 // so that both heads share the X operand of every MMA.  A query unit is (batch, head group, segment): its seg/128 token
-// tiles run back to back on one CTA, so the segment's running max / min stay on chip; key and value units are single tiles (segments too where all units
-// have an SM of their own)
-// (a key block never crosses a tile), which even out what the query units leave of the last round.  Warps 0-3: epilogue (one thread
+// tiles run back to back on one CTA, so the segment's running max / min stay on chip; key and value units are single tiles
+// (a key block never crosses a tile), which even out what the query units leave of the last round, or segments too where every
+// unit has an SM of its own.  Warps 0-3: epilogue (one thread
 // per token row: tensor-memory load, rotation, rounding, stores; then one thread per channel for the column scans), warp 4:
 // TMA producer (X and W tiles of 64 d_model columns, 128-byte swizzle), warp 5: MMA issuer; the accumulator stages in
 // tensor memory let the epilogue of one tile run under the main loop of the next.  Every wait is bounded.
