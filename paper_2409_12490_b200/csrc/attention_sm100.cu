@@ -26,13 +26,11 @@
 // its own, so that reads past a sequence's end arrive as zeros and never as a neighbour's tokens).
 #include <algorithm>
 
-#include "sm100_ptx.cuh"
+#include "attention_units.cuh"
 
 namespace cp {
 namespace {
 
-constexpr int kTile = 128;
-constexpr int kHalfBytes = kTile * 64 * 2;   // [128 rows x 64 cols] of 16-bit elements, 128-byte swizzled
 constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {producer, MMA, scheduler, idle}
 constexpr int kMaxSlots = 8;
 constexpr int kBarBytes = 512;
@@ -53,35 +51,7 @@ template <int D> struct Shape {
 // fp16 parts of P are scaled by 2^7: the reference maximum is at most 2^8 behind (lazy rescale), so P stays below 2^15,
 // and the low parts of small probabilities stay out of the subnormals
 template <bool kF16> constexpr float kPShift = kF16 ? 7.f : 0.f;
-constexpr float kRescaleThreshold = 8.0f;           // in log2 units
-#ifndef CP_EMUL_EVERY
-#define CP_EMUL_EVERY 8
-#endif
-constexpr int kEmulEvery = CP_EMUL_EVERY;           // 0: all exponentials on the MUFU; n: every n-th pair on the FMA pipes
 constexpr int kRegPoolNeeded = 256 * 216 + 128 * 64;   // registers the roles hold after setmaxnreg (softmax 216, producer/MMA 64)
-
-// One work unit, decoded (the scheduler warp decodes it once and publishes it to the other warps:
-// the decoding is a chain of integer divisions that would otherwise sit at the start of every unit).
-struct Unit {
-  int b, h, kvh;
-  int seq;          // sequence of a packed batch (0 for a single problem)
-  int n;            // its length
-  int q_tok;        // first query row of tile A
-  int n_past;       // listed blocks strictly before the segment
-  int n_past_tiles; // gathered tiles
-  int last_cols;    // valid key columns of the last gathered tile
-  int c_tok, n_cont;// contiguous unmasked tiles: first token, count
-  int d_tok;        // first token of diagonal tile d0 (d1 follows)
-  int T;            // K/V tiles the unit streams
-  int nA, nB;       // tiles query tile A / B consumes (nB = 0: the unit has no tile B)
-  const int32_t* list;
-  int seg_j;
-  int rj;           // diagonal blocks of the segment (r, fewer in a short last segment)
-  int cnt;
-  int generic;      // the list is not "past blocks, then exactly the diagonal blocks": every listed block is gathered and
-                    // every tile is masked element by element (a key counts iff its token is not after the query's)
-  int rowsB;        // the unit has a second 128-row query tile
-};
 
 struct Bars {
   unsigned long long q_full;
@@ -103,158 +73,9 @@ struct Bars {
   volatile uint32_t beat;            // advanced by warps that evaluate rows one by one (exact_row)
 };
 
-// One sequence: where its tokens, lists and rows of lse start in the arrays of the launch.
-struct Seq {
-  int n, n1, n2;
-  int seg0;                     // segments of the sequences before it
-  int64_t tok0, idx0, cnt0, lse0;
-};
-constexpr int kMaxSeqs = 16;
-constexpr int kMaxOrder = 1024;
-
-template <int NS> struct Args {
-  const int32_t* idx;
-  const int32_t* cnt;
-  uint16_t* O;                  // bf16 or fp16 elements
-  float* lse;
-  DeviceStatus* st;
-  int B, Hq, Hkv, g, seg, blk, k, r;
-  int pp;                       // units (pairs of query tiles) per segment, counted over the rows that a segment can have
-  int64_t osb, osh, ost;
-  const uint16_t *Q, *K, *V;    // only for rows that are evaluated one by one (exact_row)
-  int64_t qs[3], ks[3], vs[3];
-  float sm_scale;
-  int dense;
-  int n_units;
-  int n_seqs, n_segs;           // sequences, segments of all sequences
-  int long_first;               // order of the units: see decode_unit
-  Seq seq[NS];
-  uint16_t order[kMaxOrder];    // long_first, not dense: (segment * pairs per segment + pair), longest units first
-  int o_vec32;                  // O rows are 32-byte aligned: the epilogue may use 32-byte stores
-  int emul;                     // long units: part of the exponentials on the FMA pipes (see launch_attention_sm100)
-  int withhold_v;               // test hook: the producer never issues V tiles, so a bounded wait must expire
-};
-// tensor maps of each sequence; the launch's tensors have up to 4 dimensions, kQ .. kVt name their boxes
-enum { kQ = 0, kKb = 1, kVb = 2, kKt = 3, kVt = 4, kMaps = 5 };   // query tile, K / V block, K / V tile
-template <int NS> struct Maps { CUtensorMap m[NS][kMaps]; };
-
 // bounded wait on one of this kernel's barriers (the CTA's abort flag lives in the barrier block)
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, Bars* bars, DeviceStatus* st, int site) {
   return mbar_wait(bar, parity, &bars->abort_flag, st, site, &bars->beat);
-}
-
-// ---------------------------------------------------------------- unit geometry
-
-// Units of a segment or of a long sequence share K/V tiles with the other query heads of their KV head, so units are
-// ordered KV-head-major (within a KV head from the sequence's end, longest first for the dense kernel): the CTAs that are
-// resident together then read the same tiles through L2.  When all K and V (nearly) fit L2 together that does not matter
-// and the order is longest units first over all heads and sequences (long_first; the host sorts the (segment, pair)s by
-// the tiles they stream), which leaves the short ones to even out the ends of the CTAs.  Both orders, us, 32 query / 8 KV heads:
-// dense, KV-head-major / longest first: 34 MB of K and V 592 / 502, 101 MB 4479 / 4367, 168 MB 12125 / 12106, 201 MB 17344 / 17439,
-// 268 MB 30381 / 31149; segment 512, budget 1024: 67 MB 267 / 247, 134 MB 539 / 504, 268 MB 1069 / 1007, 537 MB 2113 / 2039; segment
-// 1024, budget 4096: 134 MB 1783 / 1749, 268 MB 3647 / 3586, 537 MB 7335 / 7285.  The line (160 MB) is the dense kernel's.
-// `cnt` is the unit's list length when the caller already has it, kLoadCnt to read it from global memory.
-constexpr int kLoadCnt = -2, kBadList = -1, kEmptyUnit = -3, kZeroUnit = -4;   // kEmptyUnit: no query row of the unit lies inside the sequence;
-                                                                                // kZeroUnit: an empty list -- the unit's rows are zeros
-template <int NS>
-__device__ __forceinline__ Unit decode_unit(const Args<NS>& a, int x, int cnt) {
-  Unit u;
-  u.list = nullptr;
-  u.cnt = 0;
-  u.seq = 0;
-  u.n = a.seq[0].n;
-  if (a.dense) {
-    const int ntiles = (u.n + kTile - 1) / kTile;
-    const int np = (ntiles + 1) / 2;
-    int pair;
-    if (a.long_first) {
-      const int heads = a.B * a.Hq, bh = x % heads;
-      pair = np - 1 - x / heads;
-      u.b = bh / a.Hq; u.h = bh % a.Hq; u.kvh = u.h / a.g;
-    } else {
-      const int per_kvh = a.g * np;
-      const int bkv = x / per_kvh;
-      const int rest = x - bkv * per_kvh;
-      pair = np - 1 - rest / a.g;
-      u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + rest % a.g;
-    }
-    u.q_tok = pair * 256;
-    u.n_past = 0; u.n_past_tiles = 0; u.last_cols = kTile;
-    u.c_tok = 0; u.n_cont = 2 * pair; u.d_tok = pair * 256;
-    u.seg_j = 0; u.rj = 0;
-    u.nB = (2 * pair + 1 < ntiles) ? 1 : 0;
-  } else {
-    const int q_tiles = a.seg / kTile;
-    const int pp = a.pp;
-    int j, p;
-    if (a.long_first) {
-      const int heads = a.B * a.Hq, bh = x % heads;
-      const int y = a.order[x / heads];
-      j = y / pp;
-      p = y % pp;
-      if constexpr (NS > 1) {
-        while (u.seq + 1 < a.n_seqs && j >= a.seq[u.seq + 1].seg0) ++u.seq;
-        j -= a.seq[u.seq].seg0;
-        u.n = a.seq[u.seq].n;
-      }
-      u.b = bh / a.Hq; u.h = bh % a.Hq; u.kvh = u.h / a.g;
-    } else {
-      const int gi_p = a.g * pp;
-      const int per_kvh = a.n_segs * gi_p;
-      const int bkv = x / per_kvh;
-      const int rest = x - bkv * per_kvh;
-      j = a.n_segs - 1 - rest / gi_p;
-      p = rest % pp;
-      u.b = bkv / a.Hkv; u.kvh = bkv % a.Hkv; u.h = u.kvh * a.g + (rest % gi_p) / pp;
-    }
-    const Seq& sq = a.seq[u.seq];
-    u.seg_j = j;
-    u.q_tok = j * a.seg + p * 256;
-    const long long unit = ((long long)u.b * a.Hq + u.h) * sq.n1 + j;
-    u.list = a.idx + sq.idx0 + unit * a.k;
-    u.cnt = cnt == kLoadCnt ? a.cnt[sq.cnt0 + unit] : cnt;
-    u.rj = min(sq.n2, (j + 1) * a.r) - j * a.r;
-    u.n_past = min(max(u.cnt - u.rj, 0), a.k);
-    u.n_past_tiles = (u.n_past * a.blk + kTile - 1) / kTile;
-    u.last_cols = u.n_past * a.blk - (u.n_past_tiles - 1) * kTile;
-    u.c_tok = j * a.seg; u.n_cont = 2 * p; u.d_tok = u.q_tok;
-    u.nB = (2 * p + 1 < q_tiles && u.q_tok + kTile < u.n) ? 1 : 0;   // tile B exists and starts inside the sequence
-  }
-  u.generic = 0;
-  u.rowsB = u.nB ? 1 : 0;
-  u.nA = u.n_past_tiles + u.n_cont + 1;       // up to and including its own diagonal tile
-  u.nB = u.nB ? u.nA + 1 : 0;                 // one more diagonal tile; 0 when the segment has an odd tile count
-  u.T = u.nB ? u.nB : u.nA;
-  return u;
-}
-
-// The list contract, checked by the scheduler warp before it publishes a unit: at most k entries, ascending, unique,
-// each a block the segment can see (0 <= b < (j+1)*r).  Returns 0 when the list has the form the selection emits
-// (past blocks, then exactly the diagonal blocks of the segment: the fast tile sequence applies), 1 for any other
-// valid list (generic tile sequence), -1 for a list that breaks the contract.
-template <int NS>
-__device__ __forceinline__ int classify_unit(const Args<NS>& a, const Unit& u, int lane) {
-  if (a.dense) return 0;
-  const int vis = min(a.seq[u.seq].n2, (u.seg_j + 1) * a.r);
-  bool gen_ok = (u.cnt >= 0) && (u.cnt <= a.k);
-  bool std_ok = gen_ok && (u.cnt >= u.rj);
-  if (gen_ok) {
-    for (int i = lane; i < u.cnt; i += 32) {
-      const int v = u.list[i];
-      const bool asc = v >= 0 && v < vis && (i == 0 || u.list[i - 1] < v);
-      gen_ok = gen_ok && asc;
-      if (i >= u.n_past) std_ok = std_ok && (v == u.seg_j * a.r + (i - u.n_past));
-      else std_ok = std_ok && asc && v < u.seg_j * a.r;
-    }
-  }
-  gen_ok = __all_sync(0xffffffffu, gen_ok);
-  std_ok = __all_sync(0xffffffffu, std_ok);
-  return !gen_ok ? -1 : (std_ok ? 0 : 1);
-}
-
-template <int NS>
-__device__ __forceinline__ bool stop_requested(const Args<NS>& a, Bars* bars) {
-  return bars->abort_flag || (a.st != nullptr && *reinterpret_cast<volatile int32_t*>(&a.st->code) == CP_ERR_TIMEOUT);
 }
 
 // ---------------------------------------------------------------- unit scheduler
@@ -345,7 +166,6 @@ __device__ __forceinline__ bool receive_unit(const Args<NS>& a, Bars* bars, uint
 
 // ---------------------------------------------------------------- softmax role
 constexpr int kMaskNone = 0, kMaskCausal = 1, kMaskCols = 2, kMaskGeneric = 3;
-
 // One row of a 64-channel head by one warp over exactly the keys it sees, in plain fp32.  A tile's MMA multiplies the zero
 // probability of a key that the row does not see with that key's value, which is NaN where the value is infinite or NaN; a row
 // whose output came out as NaN or infinite is therefore evaluated again here.  A row of 131072 keys takes milliseconds and a unit
@@ -407,17 +227,6 @@ __device__ __noinline__ void exact_row(const Args<NS>* ap, Bars* bars, int seq, 
   uint16_t* o = a.O + b * a.osb + h * a.osh + (sq.tok0 + t) * a.ost;
   *reinterpret_cast<uint32_t*>(o + 2 * lane) = pack2<kF16>(acc.x * inv, acc.y * inv);
   if (a.lse != nullptr && lane == 0) a.lse[sq.lse0 + ((long long)b * a.Hq + h) * sq.n + t] = m_run + logf(l_run);
-}
-
-// an empty list: no key is visible to any row of the unit -- zeros, and lse = ln 0
-template <int D, int NS>
-__device__ __forceinline__ void write_zero_row(const Args<NS>& a, const Unit& u, int which, int t) {
-  if ((which == 0 || u.rowsB) && t < u.n) {
-    uint4* dst = reinterpret_cast<uint4*>(a.O + u.b * a.osb + u.h * a.osh + (a.seq[u.seq].tok0 + t) * a.ost);
-#pragma unroll
-    for (int i = 0; i < D * 2 / 16; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (a.lse != nullptr) a.lse[a.seq[u.seq].lse0 + ((long long)u.b * a.Hq + u.h) * u.n + t] = -CUDART_INF;
-  }
 }
 
 template <bool kF16, int NS>
@@ -1045,6 +854,15 @@ int pairs_per_segment(int seg, const SeqSlot* slots, int n_seqs) {
   return ((rows + kTile - 1) / kTile + 1) / 2;
 }
 
+// units of a launch that have query rows
+long long count_units(const Dims& m, const SeqSlot* slots, int n_seqs, bool dense) {
+  auto pairs = [](int rows) { return (rows + 2 * kTile - 1) / (2 * kTile); };
+  long long per_head = 0;
+  for (int i = 0; i < n_seqs; ++i)
+    per_head += dense ? pairs(slots[i].len) : (long long)(slots[i].len / m.seg) * pairs(m.seg) + pairs(slots[i].len % m.seg);
+  return per_head * m.B * m.Hq;
+}
+
 // (segment, pair)s that have query rows, by the tiles they stream, longest first (counting sort; equal ones from the last
 // segment down).  Returns their number, 0 when there are more than the table holds.
 template <int NS>
@@ -1077,7 +895,22 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
                 const int32_t* idx, const int32_t* cnt, void* O, float* lse, DeviceStatus* st, bool dense, cudaStream_t s) {
   const bool f16 = p.dtype == CP_F16;
   Maps<NS> maps;
+  OMaps<NS> o_maps;
   Args<NS> a;
+  // Moving every kEmulEvery-th pair of exponentials from the MUFU to the FMA pipes pays where units are long and the
+  // kernel sits at the power cap (measured in 60-step loops: 1.6 % at 32 K/V tiles per unit) and costs where units are
+  // short (3 % at 8 tiles per unit, the paper's operating point); a unit streams at most k*blk/128 tiles.
+  a.emul = (dense || (long long)m.k * m.blk >= 12 * kTile) ? 1 : 0;
+  // The kernel of CTA pairs (attention_pair_sm100.cu): heads of 128 channels whose units have two query tiles (segments of an odd
+  // number of tiles would leave half of every pair idle), in launches of few units.  A unit takes half as long there, which counts while
+  // the SMs see up to three units each, or up to 14 short ones (their beginnings and ends overlap there); with more of them this kernel
+  // needs fewer cycles or, at the power cap, less energy per tile.  The results are the same bits.  Graph replays, this kernel / pairs, us,
+  // by units of a launch: segment 1024, budget 4096: 24 (8 / 2 heads, 600 tokens) 15.1 / 12.9, 64 35.5 / 23.2, 128 (32 / 8 heads, 1000
+  // tokens) 23.4 / 20.6, 192 86.0 / 70.7, 256 51.9 / 42.1, 288 112 / 105, 384 81.6 / 77.4, 408 162 / 158, 576 152 / 156, 1152 408 / 421; dense:
+  // 64 35.0 / 22.4, 192 108 / 79, 288 188 / 151, 408 299 / 298, 576 155 / 155, 1152 623 / 644.  Short units (budget 1024): 192 32.3 / 29.1,
+  // 1024 115 / 111, 1632 187 / 177; whole layer in long loops, a batch of 3296 units: 474 / 484.
+  const bool pair = m.d == 128 && (dense || m.seg % (2 * kTile) == 0) &&
+                    count_units(m, slots, n_seqs, dense) <= (a.emul ? 3 * 148 : 14 * 148);
   a.n_segs = 0;
   a.pp = pairs_per_segment(m.seg, slots, n_seqs);
   long long kv_tokens = 0;
@@ -1086,10 +919,11 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
     auto at = [&](const void* base, const int64_t* stride) { return static_cast<const char*>(base) + q.tok * stride[2] * m.es; };
     CUtensorMap* t = maps.m[i];
     if (!make_map(t + kQ, at(Q, p.q_stride), m.B, m.Hq, q.len, m.d, p.q_stride, kTile, f16) ||
-        !make_map(t + kKb, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, m.blk, f16) ||
+        !make_map(t + kKb, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, pair ? std::min(m.blk, 64) : m.blk, f16) ||
         !make_map(t + kVb, at(V, p.v_stride), m.B, m.Hkv, q.len, m.d, p.v_stride, m.blk, f16) ||
-        !make_map(t + kKt, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, kTile, f16) ||
-        !make_map(t + kVt, at(V, p.v_stride), m.B, m.Hkv, q.len, m.d, p.v_stride, kTile, f16))
+        !make_map(t + kKt, at(K, p.k_stride), m.B, m.Hkv, q.len, m.d, p.k_stride, pair ? 64 : kTile, f16) ||
+        !make_map(t + kVt, at(V, p.v_stride), m.B, m.Hkv, q.len, m.d, p.v_stride, kTile, f16) ||
+        (pair && !make_map(&o_maps.m[i], at(O, p.o_stride), m.B, m.Hq, q.len, m.d, p.o_stride, 32, f16)))
       return CP_ERR_CUDA;
     Seq& x = a.seq[i];
     x.n = q.len; x.n1 = (q.len + m.seg - 1) / m.seg; x.n2 = (q.len + m.blk - 1) / m.blk;
@@ -1121,11 +955,8 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
     else a.long_first = 0;                          // more segments than the table holds (never for a batch: see below)
   }
   a.withhold_v = (p.flags & CP_FLAG_TEST_WITHHOLD_V) ? 1 : 0;
-  // Moving every kEmulEvery-th pair of exponentials from the MUFU to the FMA pipes pays where units are long and the
-  // kernel sits at the power cap (measured in 60-step loops: 1.6 % at 32 K/V tiles per unit) and costs where units are
-  // short (3 % at 8 tiles per unit, the paper's operating point); a unit streams at most k*blk/128 tiles.
-  a.emul = (dense || (long long)m.k * m.blk >= 12 * kTile) ? 1 : 0;
   a.o_vec32 = (reinterpret_cast<uintptr_t>(O) % 32 == 0 && p.o_stride[0] % 16 == 0 && p.o_stride[1] % 16 == 0 && p.o_stride[2] % 16 == 0) ? 1 : 0;
+  if (pair) return launch_attention_pair<NS>(maps, o_maps, a, f16, s);
   if (m.d == 64) return f16 ? launch_variant<true, 64, NS>(maps, a, s) : launch_variant<false, 64, NS>(maps, a, s);
   return f16 ? launch_variant<true, 128, NS>(maps, a, s) : launch_variant<false, 128, NS>(maps, a, s);
 }
