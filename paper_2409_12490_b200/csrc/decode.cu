@@ -15,11 +15,18 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
+constexpr int kMaxFusedGroup = 32;
+constexpr int kMaxFusedHeads = (kStatusBytes - int(sizeof(DeviceStatus))) / int(sizeof(unsigned));   // counters behind the status word
+
+// Rows that the logits kernel normalises itself, one launch less: those of a KV head are one CTA's work then, so it has to be little: a
+// row per warp, eight values per lane.  Both calls of a token, us, normalised by a kernel of its own / by the last CTA, 32 / 8 heads: 256
+// blocks 24.5 / 19.8 (both bound by the host), 1016 blocks 55.6 / 71.1; with a head per KV head and some 1000 blocks 26.2 / 30.8.
+bool fused_rows(const Dims& m) { return m.g <= kMaxFusedGroup && m.B * m.Hkv <= kMaxFusedHeads && m.n2 <= kThreads && 2 * m.g * m.n2 <= 2048; }
 
 template <typename T, int LPR>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 5)
 decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, int64_t sb, int64_t sh, int64_t st, int Hkv, int g, int n,
-                     int blk, int n2, double est_scale, double* __restrict__ l_max, double* __restrict__ l_min) {
+                     int blk, int n2, double est_scale, double* l_max, double* l_min, unsigned* done) {
   constexpr int CE = 16 / int(sizeof(T));          // channels per lane
   constexpr int D = LPR * CE;
   constexpr int SUBS = 32 / LPR;
@@ -41,11 +48,10 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
     for (int m = LPR; m < 32; m <<= 1) { uint4 o = shfl_xor4(mx, m); vmax<T>(mx, o); o = shfl_xor4(mn, m); vmin<T>(mn, o); }
   }
   __syncthreads();
-  if (bb >= n2) return;
   // (head u, max | min) products, dealt to the SUBS lane groups that hold a copy of the representatives each
   const int sub = lane / LPR, col = lane % LPR;
 #pragma unroll 1
-  for (int t0 = 0; t0 < 2 * g; t0 += SUBS) {
+  for (int t0 = 0; t0 < (bb < n2 ? 2 * g : 0); t0 += SUBS) {
     const int t = t0 + sub;
     const uint4 kv = (t & 1) ? mn : mx, qv = reinterpret_cast<const uint4*>(qs)[min(t >> 1, g - 1) * LPR + col];
     const T *ke = reinterpret_cast<const T*>(&kv), *qe = reinterpret_cast<const T*>(&qv);
@@ -59,6 +65,46 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
 #pragma unroll
     for (int o = LPR / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
     if (col == 0 && t < 2 * g) ((t & 1) ? l_min : l_max)[size_t(h0 + (t >> 1)) * n2 + bb] = s0 * est_scale;
+  }
+  if (done == nullptr) return;
+
+  // The last CTA of a KV head normalises the rows of its group (small ones: fused_rows): a warp per row, from L2, where the other CTAs
+  // left them.
+  __shared__ bool last;
+  __shared__ double lse[2 * kMaxFusedGroup];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(done + kvh, 1u) == gridDim.x - 1;
+    if (last) done[kvh] = 0;                       // for the next call
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int r = warp; r < 2 * g; r += kWarps) {
+    const double* l = ((r & 1) ? l_min : l_max) + size_t(h0 + (r >> 1)) * n2;
+    double m = -CUDART_INF, s = 0.0;
+#pragma unroll 8
+    for (int x = lane; x < n2; x += 32) m = fmax(m, __ldcg(l + x));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+#pragma unroll 8
+    for (int x = lane; x < n2; x += 32) {          // terms below e^-50 of the largest cannot change the rounded sum; NaN stays out
+      const double v = __ldcg(l + x) - m;
+      if (v > -50.0) s += exp(v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) lse[r] = s > 0.0 ? m + log(s) : -CUDART_INF;
+  }
+  __syncthreads();
+  for (int u = 0; u < g; ++u) {
+    const double e1 = lse[2 * u], e2 = lse[2 * u + 1];
+    const size_t row = size_t(h0 + u) * n2;
+    for (int x = threadIdx.x; x < n2; x += kThreads) {
+      const double L1 = __ldcg(l_max + row + x) - e1, L2 = __ldcg(l_min + row + x) - e2;
+      l_max[row + x] = L1 >= L2 ? L1 : L2;
+    }
   }
 }
 
@@ -121,15 +167,16 @@ decode_score_kernel(double* __restrict__ S, const double* __restrict__ l_min, in
 }
 
 template <typename T, int LPR>
-int launch_logits(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* l_max, double* l_min, cudaStream_t st) {
+int launch_logits(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* l_max, double* l_min, unsigned* done,
+                  cudaStream_t st) {
   const dim3 grid(unsigned((m.n2 + kWarps - 1) / kWarps), unsigned(m.B * m.Hkv));
   const size_t smem = size_t(m.g) * m.d * m.es;    // the group's queries: up to 64 KB (fp32, 128 channels, 128 heads)
-  if (smem > 48 * 1024 &&
+  if (smem > 47 * 1024 &&                          // 48 KB with the kernel's own
       cudaFuncSetAttribute(decode_logits_kernel<T, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return CP_ERR_CUDA;
   return launch_pdl(decode_logits_kernel<T, LPR>, grid, kThreads, smem, st, static_cast<const T*>(q_last),
                     static_cast<const char*>(K), p.k_stride[0], p.k_stride[1], p.k_stride[2], m.Hkv, m.g, m.n, m.blk, m.n2,
-                    double(p.est_scale), l_max, l_min);
+                    double(p.est_scale), l_max, l_min, done);
 }
 
 }  // namespace
@@ -140,15 +187,16 @@ bool decode_path_applies(const Dims& m) { return m.blk <= 128 && 8 * m.g <= 2 * 
 
 int launch_decode_score(const cp_params& p, const Dims& m, const void* q_last, const void* K, double* S_out, char* ws, cudaStream_t st) {
   double* l_min = reinterpret_cast<double*>(ws + ws_layout(m).kmax);
+  unsigned* done = fused_rows(m) ? reinterpret_cast<unsigned*>(ws + sizeof(DeviceStatus)) : nullptr;
   const int lpr = m.d * m.es / 16;
   int rc = CP_ERR_UNSUPPORTED;
   if (p.dtype == CP_BF16)
-    rc = lpr == 16 ? launch_logits<__nv_bfloat16, 16>(p, m, q_last, K, S_out, l_min, st) : launch_logits<__nv_bfloat16, 8>(p, m, q_last, K, S_out, l_min, st);
+    rc = lpr == 16 ? launch_logits<__nv_bfloat16, 16>(p, m, q_last, K, S_out, l_min, done, st) : launch_logits<__nv_bfloat16, 8>(p, m, q_last, K, S_out, l_min, done, st);
   else if (p.dtype == CP_F16)
-    rc = lpr == 16 ? launch_logits<__half, 16>(p, m, q_last, K, S_out, l_min, st) : launch_logits<__half, 8>(p, m, q_last, K, S_out, l_min, st);
+    rc = lpr == 16 ? launch_logits<__half, 16>(p, m, q_last, K, S_out, l_min, done, st) : launch_logits<__half, 8>(p, m, q_last, K, S_out, l_min, done, st);
   else
-    rc = lpr == 32 ? launch_logits<float, 32>(p, m, q_last, K, S_out, l_min, st) : launch_logits<float, 16>(p, m, q_last, K, S_out, l_min, st);
-  if (rc != CP_OK) return rc;
+    rc = lpr == 32 ? launch_logits<float, 32>(p, m, q_last, K, S_out, l_min, done, st) : launch_logits<float, 16>(p, m, q_last, K, S_out, l_min, done, st);
+  if (rc != CP_OK || done != nullptr) return rc;
   const dim3 grid(unsigned(m.B * m.Hq));
   if (m.n2 <= 4 * kThreads) return launch_pdl(decode_score_kernel<4>, grid, kThreads, 0, st, S_out, l_min, m.n2);
   if (m.n2 <= 16 * kThreads) return launch_pdl(decode_score_kernel<16>, grid, kThreads, 0, st, S_out, l_min, m.n2);

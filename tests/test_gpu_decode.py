@@ -89,3 +89,22 @@ def test_values_that_are_not_finite_follow_the_general_kernel(dtype, d, blk, g, 
         assert np.array_equal(kind(S), kind(row)), kind.__name__
     fin = np.isfinite(row)
     assert np.abs(S[fin] - row[fin]).max(initial=0.0) <= 1e-9
+
+
+@pytest.mark.parametrize("B,Hkv,g,n,blk", [
+    (1, 2, 4, 256 * 16, 16), (1, 2, 4, 256 * 16 + 1, 16),    # 2 g n2 = 2048 and one block more
+    (1, 56, 1, 300, 32), (3, 19, 1, 300, 32),                 # 56 KV heads have a counter behind the status word each; 57 do not
+    (1, 1, 32, 1024, 32), (1, 1, 33, 500, 32)])
+def test_rows_normalised_behind_their_logits_or_by_a_kernel_of_their_own(B, Hkv, g, n, blk):
+    """Two calls on one workspace (the counters start from zero again), another problem between them."""
+    Q, K, V = make_uniform_qkv(B, Hkv * g, Hkv, n, 64, dtype="bf16", seed=n + g)
+    prob = cp.Problem(B, Hkv * g, Hkv, n, 64, blk, blk, 2, torch.bfloat16)
+    ws = cp.alloc_workspace(prob)
+    q, Kd = Q[:, :, -1].contiguous(), K.cuda()
+    S_ref = oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))
+    small = cp.Problem(1, g, 1, 100, 64, blk, blk, 2, torch.bfloat16)
+    for _ in range(2):
+        S = cp.decode_estimate(prob, q.cuda(), Kd, ws)
+        cp.decode_estimate(small, q[:1, :g].contiguous().cuda(), Kd[:1, :1, :100].contiguous(), ws)
+        assert cp.device_status(ws) == 0
+        assert np.abs(S.cpu().numpy() - S_ref).max() <= 1e-9
