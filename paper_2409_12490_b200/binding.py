@@ -193,7 +193,7 @@ def alloc_workspace(prob: Problem, device="cuda") -> torch.Tensor:
 def estimate(prob: Problem, Q, K, ws, S_prev=None, S_out=None) -> torch.Tensor:
     """critiprefill_estimate: ln S [B,Hq,n1,n2] fp64 (Algorithm 1)."""
     if S_out is None:
-        S_out = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.n2), dtype=torch.float64, device=Q.device)
+        S_out = torch.empty(prob.batch, prob.n_q_heads, prob.n1, prob.n2, dtype=torch.float64, device=Q.device)
     p = prob.params(Q=Q, K=K)
     _check(load_library().critiprefill_estimate(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(S_prev), _ptr(S_out),
                                                 _ptr(ws), ws.numel(), _stream()), "critiprefill_estimate")
@@ -204,7 +204,7 @@ def estimate_static(prob: Problem, Q, K, S_prev=None, S_out=None) -> torch.Tenso
     """critiprefill_estimate_static: critiprefill_estimate without a caller workspace, for callers
     that cannot allocate device memory (the scratch is a fixed array inside the library)."""
     if S_out is None:
-        S_out = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.n2), dtype=torch.float64, device=Q.device)
+        S_out = torch.empty(prob.batch, prob.n_q_heads, prob.n1, prob.n2, dtype=torch.float64, device=Q.device)
     p = prob.params(Q=Q, K=K)
     _check(load_library().critiprefill_estimate_static(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(S_prev), _ptr(S_out),
                                                        _stream()), "critiprefill_estimate_static")
@@ -218,9 +218,9 @@ def static_scratch_bytes() -> int:
 def select(prob: Problem, S, ws, idx=None, cnt=None):
     """critiprefill_select: (idx [B,Hq,n1,k] int32, cnt [B,Hq,n1] int32) (Algorithm 2, line 8)."""
     if idx is None:
-        idx = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.budget_blocks), dtype=torch.int32, device=S.device)
+        idx = torch.empty(prob.batch, prob.n_q_heads, prob.n1, prob.budget_blocks, dtype=torch.int32, device=S.device)
     if cnt is None:
-        cnt = torch.empty((prob.batch, prob.n_q_heads, prob.n1), dtype=torch.int32, device=S.device)
+        cnt = torch.empty(prob.batch, prob.n_q_heads, prob.n1, dtype=torch.int32, device=S.device)
     p = prob.params()
     _check(load_library().critiprefill_select(ctypes.byref(p), _ptr(S), _ptr(idx), _ptr(cnt), _ptr(ws), ws.numel(),
                                               _stream()), "critiprefill_select")
@@ -233,9 +233,9 @@ def project_qk(prob: Problem, X, Wq, Wk, ws, rope_cos=None, rope_sin=None, Q_out
     B, n, d_model = X.shape
     assert X.is_contiguous() and Wq.is_contiguous() and Wk.is_contiguous()
     if Q_out is None:
-        Q_out = torch.empty((B, prob.n_q_heads, n, prob.head_dim), dtype=X.dtype, device=X.device)
+        Q_out = torch.empty(B, prob.n_q_heads, n, prob.head_dim, dtype=X.dtype, device=X.device)
     if K_out is None:
-        K_out = torch.empty((B, prob.n_kv_heads, n, prob.head_dim), dtype=X.dtype, device=X.device)
+        K_out = torch.empty(B, prob.n_kv_heads, n, prob.head_dim, dtype=X.dtype, device=X.device)
     p = prob.params(Q=Q_out, K=K_out)
     _check(load_library().critiprefill_project_qk(ctypes.byref(p), _ptr(X), _ptr(Wq), _ptr(Wk), _ptr(rope_cos), _ptr(rope_sin),
                                                   int(d_model), _ptr(Q_out), _ptr(K_out), _ptr(ws), ws.numel(), _stream()),
@@ -247,7 +247,7 @@ def project_qkv(prob: Problem, X, Wq, Wk, Wv, ws, rope_cos=None, rope_sin=None, 
     """critiprefill_project_qkv: project_qk plus V = W_V X (no rotation) in the same launch.  Returns (Q, K, V)."""
     B, n, d_model = X.shape
     assert X.is_contiguous() and Wq.is_contiguous() and Wk.is_contiguous() and Wv.is_contiguous()
-    mk = lambda h: torch.empty((B, h, n, prob.head_dim), dtype=X.dtype, device=X.device)
+    mk = lambda h: torch.empty(B, h, n, prob.head_dim, dtype=X.dtype, device=X.device)
     Q_out = mk(prob.n_q_heads) if Q_out is None else Q_out
     K_out = mk(prob.n_kv_heads) if K_out is None else K_out
     V_out = mk(prob.n_kv_heads) if V_out is None else V_out
@@ -263,7 +263,7 @@ def decode_estimate(prob: Problem, q_last, K, ws, S_out=None) -> torch.Tensor:
     """critiprefill_decode_estimate: ln S [B,Hq,n2] fp64 of the last query token (Section 2.1)."""
     assert q_last.is_contiguous() and q_last.shape == (prob.batch, prob.n_q_heads, prob.head_dim)
     if S_out is None:
-        S_out = torch.empty((prob.batch, prob.n_q_heads, prob.n2), dtype=torch.float64, device=K.device)
+        S_out = torch.empty(prob.batch, prob.n_q_heads, prob.n2, dtype=torch.float64, device=K.device)
     p = prob.params(K=K)
     _check(load_library().critiprefill_decode_estimate(ctypes.byref(p), _ptr(q_last), _ptr(K), _ptr(S_out), _ptr(ws),
                                                        ws.numel(), _stream()), "critiprefill_decode_estimate")
@@ -272,8 +272,8 @@ def decode_estimate(prob: Problem, q_last, K, ws, S_out=None) -> torch.Tensor:
 
 def decode_select(prob: Problem, S, ws):
     """critiprefill_decode_select: (idx [B,Hq,k] int32, cnt [B,Hq] int32) for the last query token."""
-    idx = torch.empty((prob.batch, prob.n_q_heads, prob.budget_blocks), dtype=torch.int32, device=S.device)
-    cnt = torch.empty((prob.batch, prob.n_q_heads), dtype=torch.int32, device=S.device)
+    idx = torch.empty(prob.batch, prob.n_q_heads, prob.budget_blocks, dtype=torch.int32, device=S.device)
+    cnt = torch.empty(prob.batch, prob.n_q_heads, dtype=torch.int32, device=S.device)
     p = prob.params()
     _check(load_library().critiprefill_decode_select(ctypes.byref(p), _ptr(S), _ptr(idx), _ptr(cnt), _ptr(ws), ws.numel(),
                                                      _stream()), "critiprefill_decode_select")
@@ -285,7 +285,7 @@ def attention(prob: Problem, Q, K, V, idx, cnt, ws, O=None, lse=None, want_lse=F
     if O is None:
         O = torch.empty_like(Q)
     if lse is None and want_lse:
-        lse = torch.empty((prob.batch, prob.n_q_heads, prob.seq_len), dtype=torch.float32, device=Q.device)
+        lse = torch.empty(prob.batch, prob.n_q_heads, prob.seq_len, dtype=torch.float32, device=Q.device)
     p = prob.params(Q=Q, K=K, V=V, O=O)
     _check(load_library().critiprefill_attention(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(idx), _ptr(cnt),
                                                  _ptr(O), _ptr(lse), _ptr(ws), ws.numel(), _stream()),
@@ -298,7 +298,7 @@ def dense_attention(prob: Problem, Q, K, V, ws, O=None, lse=None, want_lse=False
     if O is None:
         O = torch.empty_like(Q)
     if lse is None and want_lse:
-        lse = torch.empty((prob.batch, prob.n_q_heads, prob.seq_len), dtype=torch.float32, device=Q.device)
+        lse = torch.empty(prob.batch, prob.n_q_heads, prob.seq_len, dtype=torch.float32, device=Q.device)
     p = prob.params(Q=Q, K=K, V=V, O=O)
     _check(load_library().critiprefill_dense_attention(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(lse),
                                                        _ptr(ws), ws.numel(), _stream()), "critiprefill_dense_attention")
@@ -340,7 +340,7 @@ def prefill_varlen(prob: Problem, cu_seqlens, Q, K, V, ws, S_prev=None, want_lse
     S_flat = torch.empty(sizes[0].value, dtype=torch.float64, device=Q.device)
     idx_flat = torch.empty(sizes[1].value, dtype=torch.int32, device=Q.device)
     cnt_flat = torch.empty(sizes[2].value, dtype=torch.int32, device=Q.device)
-    lse = torch.empty((prob.n_q_heads * Q.shape[1],), dtype=torch.float32, device=Q.device) if want_lse else None
+    lse = torch.empty(prob.n_q_heads * Q.shape[1], dtype=torch.float32, device=Q.device) if want_lse else None
     _check(lib.critiprefill_prefill_varlen(ctypes.byref(p), cu, n_seqs, _ptr(Q), _ptr(K), _ptr(V), _ptr(S_prev), _ptr(S_flat),
                                            _ptr(idx_flat), _ptr(cnt_flat), _ptr(O), _ptr(lse), _ptr(ws), ws.numel(), _stream()),
            "critiprefill_prefill_varlen")
@@ -360,13 +360,13 @@ def prefill_varlen(prob: Problem, cu_seqlens, Q, K, V, ws, S_prev=None, want_lse
 def prefill_layer(prob: Problem, Q, K, V, ws, S_prev=None):
     """One layer of the hot path: estimate -> select -> attention.  Returns (O, S, idx, cnt)."""
     lib, stream, ws_ptr, ws_bytes = load_library(), _stream(), ws.data_ptr(), ws.numel()
-    S = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.n2), dtype=torch.float64, device=Q.device)
+    S = torch.empty(prob.batch, prob.n_q_heads, prob.n1, prob.n2, dtype=torch.float64, device=Q.device)
     O = torch.empty_like(Q)
     p = ctypes.byref(prob.params(Q=Q, K=K, V=V, O=O))
     q_ptr, k_ptr, s_ptr = Q.data_ptr(), K.data_ptr(), S.data_ptr()
     _check(lib.critiprefill_estimate(p, q_ptr, k_ptr, _ptr(S_prev), s_ptr, ws_ptr, ws_bytes, stream), "critiprefill_estimate")
-    idx = torch.empty((prob.batch, prob.n_q_heads, prob.n1, prob.budget_blocks), dtype=torch.int32, device=S.device)
-    cnt = torch.empty((prob.batch, prob.n_q_heads, prob.n1), dtype=torch.int32, device=S.device)
+    idx = torch.empty(prob.batch, prob.n_q_heads, prob.n1, prob.budget_blocks, dtype=torch.int32, device=S.device)
+    cnt = torch.empty(prob.batch, prob.n_q_heads, prob.n1, dtype=torch.int32, device=S.device)
     idx_ptr, cnt_ptr = idx.data_ptr(), cnt.data_ptr()
     _check(lib.critiprefill_select(p, s_ptr, idx_ptr, cnt_ptr, ws_ptr, ws_bytes, stream), "critiprefill_select")
     _check(lib.critiprefill_attention(p, q_ptr, k_ptr, V.data_ptr(), idx_ptr, cnt_ptr, O.data_ptr(), None, ws_ptr, ws_bytes, stream),
