@@ -15,13 +15,14 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kMaxFusedGroup = 32;
+constexpr int kMaxFusedGroup = 32, kMaxFusedLogits = 2048;
 constexpr int kMaxFusedHeads = (kStatusBytes - int(sizeof(DeviceStatus))) / int(sizeof(unsigned));   // counters behind the status word
 
 // Rows that the logits kernel normalises itself, one launch less: those of a KV head are one CTA's work then, so it has to be little: a
-// row per warp, eight values per lane.  Both calls of a token, us, normalised by a kernel of its own / by the last CTA, 32 / 8 heads: 256
-// blocks 24.5 / 19.8 (both bound by the host), 1016 blocks 55.6 / 71.1; with a head per KV head and some 1000 blocks 26.2 / 30.8.
-bool fused_rows(const Dims& m) { return m.g <= kMaxFusedGroup && m.B * m.Hkv <= kMaxFusedHeads && m.n2 <= kThreads && 2 * m.g * m.n2 <= 2048; }
+// row per warp, eight values per lane.  Both calls of a token, us, 32 / 8 heads, 256 blocks, normalised by a kernel of its own / by the last
+// CTA: 24.1 / 19.4 where the host launches them (that bounds both; about half of it is the launch), 12.5 / 14.7 in a graph.  1016 blocks 55.6 /
+// 71.1, a head per KV head and some 1000 blocks 26.2 / 30.8 (rows read from L2 by the warps, one after another).
+bool fused_rows(const Dims& m) { return m.g <= kMaxFusedGroup && m.B * m.Hkv <= kMaxFusedHeads && m.n2 <= kThreads && 2 * m.g * m.n2 <= kMaxFusedLogits; }
 
 template <typename T, int LPR>
 __global__ void __launch_bounds__(kThreads, 5)
@@ -68,10 +69,11 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
   }
   if (done == nullptr) return;
 
-  // The last CTA of a KV head normalises the rows of its group (small ones: fused_rows): a warp per row, from L2, where the other CTAs
-  // left them.
+  // The last CTA of a KV head normalises the rows of its group (small ones: fused_rows): all of them come from L2, where the other CTAs
+  // left them, in one go, a warp takes a row at a time from shared memory, and all are written in one go.
   __shared__ bool last;
   __shared__ double lse[2 * kMaxFusedGroup];
+  __shared__ double rows[kMaxFusedLogits];         // [Kmax | Kmin][head][block]
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -81,16 +83,22 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
   __syncthreads();
   if (!last) return;
   __threadfence();
+  const int gn = g * n2;
+  double *out = l_max + size_t(h0) * n2, *other = l_min + size_t(h0) * n2;
+#pragma unroll
+  for (int i = 0; i < kMaxFusedLogits / 2 / kThreads; ++i) {
+    const int x = i * kThreads + threadIdx.x;
+    if (x < gn) { rows[x] = __ldcg(out + x); rows[gn + x] = __ldcg(other + x); }
+  }
+  __syncthreads();
   for (int r = warp; r < 2 * g; r += kWarps) {
-    const double* l = ((r & 1) ? l_min : l_max) + size_t(h0 + (r >> 1)) * n2;
+    const double* l = rows + r * n2;
     double m = -CUDART_INF, s = 0.0;
-#pragma unroll 8
-    for (int x = lane; x < n2; x += 32) m = fmax(m, __ldcg(l + x));
+    for (int x = lane; x < n2; x += 32) m = fmax(m, l[x]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-#pragma unroll 8
     for (int x = lane; x < n2; x += 32) {          // terms below e^-50 of the largest cannot change the rounded sum; NaN stays out
-      const double v = __ldcg(l + x) - m;
+      const double v = l[x] - m;
       if (v > -50.0) s += exp(v);
     }
 #pragma unroll
@@ -98,13 +106,10 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
     if (lane == 0) lse[r] = s > 0.0 ? m + log(s) : -CUDART_INF;
   }
   __syncthreads();
-  for (int u = 0; u < g; ++u) {
-    const double e1 = lse[2 * u], e2 = lse[2 * u + 1];
-    const size_t row = size_t(h0 + u) * n2;
-    for (int x = threadIdx.x; x < n2; x += kThreads) {
-      const double L1 = __ldcg(l_max + row + x) - e1, L2 = __ldcg(l_min + row + x) - e2;
-      l_max[row + x] = L1 >= L2 ? L1 : L2;
-    }
+  for (int x = threadIdx.x; x < gn; x += kThreads) {
+    const int u = x / n2;
+    const double L1 = rows[x] - lse[u], L2 = rows[gn + x] - lse[g + u];
+    out[x] = L1 >= L2 ? L1 : L2;
   }
 }
 
@@ -171,7 +176,7 @@ int launch_logits(const cp_params& p, const Dims& m, const void* q_last, const v
                   cudaStream_t st) {
   const dim3 grid(unsigned((m.n2 + kWarps - 1) / kWarps), unsigned(m.B * m.Hkv));
   const size_t smem = size_t(m.g) * m.d * m.es;    // the group's queries: up to 64 KB (fp32, 128 channels, 128 heads)
-  if (smem > 47 * 1024 &&                          // 48 KB with the kernel's own
+  if (smem > 30 * 1024 &&                          // 48 KB with the kernel's own
       cudaFuncSetAttribute(decode_logits_kernel<T, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return CP_ERR_CUDA;
   return launch_pdl(decode_logits_kernel<T, LPR>, grid, kThreads, smem, st, static_cast<const T*>(q_last),
