@@ -74,15 +74,15 @@ decode_logits_kernel(const T* __restrict__ q_last, const char* __restrict__ K, i
   __shared__ bool last;
   __shared__ double lse[2 * kMaxFusedGroup];
   __shared__ double rows[kMaxFusedLogits];         // [Kmax | Kmin][head][block]
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();                               // the CTA's logits, which the barrier has ordered before this, are visible
     last = atomicAdd(done + kvh, 1u) == gridDim.x - 1;
     if (last) done[kvh] = 0;                       // for the next call
+    __threadfence();
   }
   __syncthreads();
   if (!last) return;
-  __threadfence();
   const int gn = g * n2;
   double *out = l_max + size_t(h0) * n2, *other = l_min + size_t(h0) * n2;
 #pragma unroll
