@@ -74,7 +74,13 @@ __device__ __forceinline__ uint32_t first_cta(const void* p) {      // the addre
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ bool mbar_ready(unsigned long long* bar, uint32_t parity) {      // never suspends
+// Never suspends.  Like every test of a parity it is true before the phase that it asks about has begun, while the one before is open, so the
+// caller has to know that that one is over.  v_full, ahead of a tile: the tile three before has gone through P V.  k_full, three tiles ahead of
+// the next one: only if QK^T of that next tile has been issued, which it has not been (gq == gp + 1) where a unit ended and its successor was
+// published too late; the wait then comes before the QK^T itself.  The other waits: each barrier's phases are waited for one after
+// another by the same warp; s_full of every second tile by either softmax warpgroup, which has the tile before from the other one (row_get)
+// by then; v_empty before a rescale: commits of one thread, in order, and s_full of a later one has been seen.
+__device__ __forceinline__ bool mbar_ready(unsigned long long* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
@@ -637,7 +643,7 @@ __device__ __forceinline__ void mma_role(const Args<NS>& a, Bars* bars, uint32_t
     umma2_commit(&bars->v_empty[slot]);
     // under the MMAs just issued: what the next turn would wait for
     v_ok = mbar_ready(&bars->v_full[slot1], par1);
-    k_ok = mbar_ready(&bars->k_full[slot1], par1 ^ 1);
+    k_ok = gq != gp + 1 && mbar_ready(&bars->k_full[slot1], par1 ^ 1);
     if (CP_LIKELY(next)) {
       umma2_qk8(tP, dq, dk, Idesc2<kF16>::qk);
       umma2_commit(&bars->s_full[slot]);
