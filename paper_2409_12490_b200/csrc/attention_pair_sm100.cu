@@ -53,7 +53,7 @@ struct Bars {
   unsigned long long clc_full;
   unsigned long long taken;              // both producers have begun the unit published last: the next one may be drawn
   __align__(16) uint32_t clc_resp[4];    // the hardware's answer to the last request for a further unit
-  uint2 ref[2][kTile];                   // a row's reference maximum after a tile of either warpgroup, and that tile's number + 1
+  unsigned long long ref[2][kTile];      // a row's reference maximum after a tile of either warpgroup, and (upper half) that tile's number + 1
   int sched_unit[kSched];
   Unit sched_u[kSched];
   uint32_t mma_unit[4];                  // units between the MMA warp's QK^T and its P V: tiles | 2^31 if only the second CTA's rows see the last
@@ -97,18 +97,19 @@ __device__ __forceinline__ bool wait(unsigned long long* bar, uint32_t parity, B
   if (CP_LIKELY(mbar_test(bar, parity))) return true;
   return wait_slow(bar, parity, bars, st, site);
 }
-// A row's reference maximum after tile `tag` - 1, from the thread of the other warpgroup that has the same row.  Value and tag
-// are one 8-byte word: a barrier would cost each side a hundred cycles and more per tile.  Every tile takes the value of the one before,
-// also where it has no use for it (a unit's first), so neither side writes over a value that the other has not seen.
-__device__ __forceinline__ void row_put(uint2* p, float m, uint32_t tag) {
-  asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(smem_u32(p)), "r"(__float_as_uint(m)), "r"(tag) : "memory");
+// A row's reference maximum after tile `tag` - 1, from the thread of the other warpgroup that has the same row.  Value and tag are one
+// 8-byte word, written and read as one scalar (the parts of a vector access may be seen one without the other): a barrier would cost each side
+// a hundred cycles and more per tile.  Every tile takes the value of the one before, also where it has no use for it (a unit's first),
+// so neither side writes over a value that the other has not seen.
+__device__ __forceinline__ void row_put(unsigned long long* p, float m, uint32_t tag) {
+  asm volatile("{\n.reg .b64 v;\nmov.b64 v, {%1, %2};\nst.volatile.shared.b64 [%0], v;\n}" ::"r"(smem_u32(p)), "r"(__float_as_uint(m)), "r"(tag) : "memory");
 }
-__device__ __forceinline__ uint2 row_load(const uint2* p) {
+__device__ __forceinline__ uint2 row_load(const unsigned long long* p) {
   uint2 v;
-  asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(smem_u32(p)) : "memory");
+  asm volatile("{\n.reg .b64 v;\nld.volatile.shared.b64 v, [%2];\nmov.b64 {%0, %1}, v;\n}" : "=r"(v.x), "=r"(v.y) : "r"(smem_u32(p)) : "memory");
   return v;
 }
-__device__ __noinline__ bool row_wait(const uint2* p, uint32_t tag, float* m, Bars* bars, DeviceStatus* st, int site) {
+__device__ __noinline__ bool row_wait(const unsigned long long* p, uint32_t tag, float* m, Bars* bars, DeviceStatus* st, int site) {
   unsigned long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
     const uint2 v = row_load(p);
@@ -127,7 +128,7 @@ __device__ __noinline__ bool row_wait(const uint2* p, uint32_t tag, float* m, Ba
   }
 }
 // `early`: what an earlier row_load found there, most often the value already
-__device__ __forceinline__ bool row_get(const uint2* p, uint2 early, uint32_t tag, float* m, Bars* bars, DeviceStatus* st, int site) {
+__device__ __forceinline__ bool row_get(const unsigned long long* p, uint2 early, uint32_t tag, float* m, Bars* bars, DeviceStatus* st, int site) {
   *m = __uint_as_float(early.x);
   if (CP_LIKELY(__all_sync(0xffffffffu, early.y == tag))) return true;
   float v;
@@ -697,7 +698,7 @@ attention_pair_kernel(const __grid_constant__ Maps<NS> maps, const __grid_consta
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp < 8) bars->ref[warp >> 2][threadIdx.x & 127] = make_uint2(0u, 0u);
+  if (warp < 8) bars->ref[warp >> 2][threadIdx.x & 127] = 0ull;
   if (warp == 12 && lane < kMaps && NS == 1) prefetch_tmap(&maps.m[0][lane]);
   if (warp == 14) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&bars->tmem_base)) : "memory");

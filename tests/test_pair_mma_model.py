@@ -22,3 +22,11 @@ def test_no_product_is_issued_before_its_operands(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-O1", "-w", f'-DROLE_FILE="{role}"', "-o", str(exe), str(TESTS / "pair_mma_model.cpp")], check=True)
     out = subprocess.run([str(exe), "3000"], capture_output=True, text=True, timeout=300)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
+
+
+def test_a_row_and_its_tag_are_exchanged_as_one_scalar():
+    """PTX guarantees that a scalar access is seen whole; a vector access is one access per part."""
+    text = SOURCE.read_text()
+    for name, access in (("void row_put(", "st.volatile.shared.b64 "), ("uint2 row_load(", "ld.volatile.shared.b64 ")):
+        body = _between(text, name, "\n}\n")
+        assert body.count(access) == 1 and ".v2" not in body and body.count("asm volatile") == 1
