@@ -78,3 +78,85 @@ def test_keys_that_only_the_second_tile_sees_stay_out_of_the_first():
         clean, odd = f(V), f(W)
         assert torch.equal(clean[:, :, :384], odd[:, :, :384]) and not torch.isfinite(odd[:, :, 400:]).any()
     assert cp.device_status(ws) == 0
+
+
+def mixed_lists(Hq, n, seg, blk, k, seed, broken):
+    """Lists of length 0, 1 and k in every order, any visible blocks among them; broken: some that break their contract."""
+    rng = np.random.default_rng(seed)
+    n1, n2, r = -(-n // seg), -(-n // blk), seg // blk
+    idx = np.full((1, Hq, n1, k), -1, dtype=np.int32)
+    cnt = np.zeros((1, Hq, n1), dtype=np.int32)
+    for h in range(Hq):
+        for j in range(n1):
+            own = list(range(j * r, min(n2, (j + 1) * r)))
+            mode = rng.choice(["empty", "empty", "one", "standard", "standard", "any", "broken"])
+            if mode == "empty":
+                sel = []
+            elif mode == "one":
+                sel = [int(rng.integers(own[-1] + 1))]
+            elif mode == "any":
+                sel = sorted(rng.choice(own[-1] + 1, size=min(k, own[-1] + 1), replace=False).tolist())
+            else:
+                sel = sorted(rng.choice(j * r, size=min(k - r, j * r), replace=False).tolist() if j else []) + own
+                if mode == "broken" and broken:
+                    sel[-1] = n2 + 1000
+            cnt[0, h, j] = len(sel)
+            idx[0, h, j, :len(sel)] = sel
+    return torch.from_numpy(idx), torch.from_numpy(cnt)
+
+
+@pytest.mark.parametrize("broken", [False, True])
+@pytest.mark.parametrize("dtype,blk,k,items", [("bf16", 32, 32, 7), ("f16", 128, 8, 7), ("bf16", 64, 32, 2)])
+def test_mixed_lists_over_many_units(dtype, blk, k, items, broken):
+    """Each pair of CTAs draws five units or so, with empty and one-block lists before and behind full ones.  One item alone (320 units: pairs)
+    and in a batch (640 long units, 2240 short ones: one CTA each); rows of a broken list are left as they were by both."""
+    Hq, Hkv, n, seg = 16, 4, 5000, 256
+    Q, K, V = (t.cuda() for t in make_uniform_qkv(items, Hq, Hkv, n, 128, dtype=dtype, seed=k))
+    lists = [mixed_lists(Hq, n, seg, blk, k, 10 * i + k, broken) for i in range(items)]
+    idx, cnt = (torch.cat([x[i] for x in lists]).cuda() for i in (0, 1))
+
+    def run(b):
+        q, kk, v = Q[b].contiguous(), K[b].contiguous(), V[b].contiguous()
+        prob = cp.Problem(q.shape[0], Hq, Hkv, n, 128, seg, blk, k, TDT[dtype])
+        ws = cp.alloc_workspace(prob)
+        O, lse = torch.full_like(q, 7.0), torch.full(q.shape[:3], 7.0, device="cuda")
+        cp.attention(prob, q, kk, v, idx[b].contiguous(), cnt[b].contiguous(), ws, O=O, lse=lse)
+        assert cp.device_status(ws) == (7 if broken else 0)
+        return O, lse
+    O, lse = run(slice(0, items))
+    for i in range(items):
+        Oi, lse_i = run(slice(i, i + 1))
+        assert torch.equal(O[i], Oi[0]) and torch.equal(lse[i], lse_i[0])
+    assert (O == 0).all(-1).any() and bool((lse == 7).any()) == broken
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("seg,blk,k", [(384, 32, 20), (384, 128, 7), (128, 64, 9)])
+def test_mixed_lists_on_the_single_cta_kernel(dtype, seg, blk, k):
+    """Segments of an odd number of 128-row tiles never take pairs of CTAs."""
+    Hq, Hkv, n = 4, 2, 2500
+    Q, K, V = make_uniform_qkv(1, Hq, Hkv, n, 128, dtype=dtype, seed=seg + k)
+    idx, cnt = mixed_lists(Hq, n, seg, blk, k, k, False)
+    prob = cp.Problem(1, Hq, Hkv, n, 128, seg, blk, k, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    O, lse = cp.attention(prob, Q.cuda(), K.cuda(), V.cuda(), idx.cuda(), cnt.cuda(), ws, want_lse=True)
+    assert cp.device_status(ws) == 0
+    O_ref, lse_ref = oracle.sparse_attention(Q, K, V, idx.numpy(), cnt.numpy(), seg, blk, SM)
+    assert_close(O, O_ref, V, dtype)
+    none = np.isneginf(lse_ref)
+    assert none.any() and np.array_equal(np.isneginf(lse.cpu().numpy()), none)
+    assert np.abs(lse.cpu().numpy()[~none] - lse_ref[~none]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("seg", [256, 384])
+def test_a_wait_that_runs_out_is_reported(seg):
+    """V tiles never requested (test hook): pairs of CTAs (segment 256) and the single-CTA kernel give up after their limit, and the next call works."""
+    Q, K, V = (t.cuda() for t in make_uniform_qkv(1, 2, 1, 700, 128, seed=seg))
+    out = []
+    for flags, status in ((0, 0), (cp.FLAG_TEST_WITHHOLD_V, 6), (0, 0)):
+        prob = cp.Problem(1, 2, 1, 700, 128, seg, 64, 8, torch.bfloat16, flags=flags)
+        ws = cp.alloc_workspace(prob)
+        idx, cnt = cp.select(prob, cp.estimate(prob, Q, K, ws), ws)
+        out.append(cp.attention(prob, Q, K, V, idx, cnt, ws))
+        assert cp.device_status(ws) == status
+    assert torch.equal(out[0], out[2])
