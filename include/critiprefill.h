@@ -93,10 +93,9 @@ typedef struct {
 
 /* Bytes of scratch (`ws`) the calls below need for these parameters; the same buffer serves
  * all of them.  `ws` must be 256-byte aligned.  Its first 256 bytes are the device status
- * block, which the caller zeroes once (cudaMemset) before the first call; critiprefill_decode_estimate
- * also keeps counters there and sets them back at every launch.  Calls that
- * may execute concurrently (different streams without ordering) need separate workspaces;
- * calls ordered on one stream can share one.  Host pointers. */
+ * block, which the caller zeroes once (cudaMemset) before the first call.  Calls that may execute
+ * concurrently (different streams without ordering) need separate workspaces; calls ordered on one
+ * stream can share one.  Host pointers. */
 int critiprefill_workspace_bytes(const cp_params* p, size_t* bytes_out);
 
 /* Algorithm 1 (estimation of query criticality in one layer).

@@ -120,20 +120,26 @@ __device__ __forceinline__ void pdl_wait(P&... ptrs) {
 }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
-int launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+int launch_pdl_cluster(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, unsigned cluster_x, cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster_x > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
   const cudaError_t last = cudaGetLastError();
   return e == cudaSuccess && last == cudaSuccess ? CP_OK : CP_ERR_CUDA;
+}
+template <typename... P, typename... A>
+int launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+  return launch_pdl_cluster(kern, grid, block, smem, 1, st, args...);
 }
 
 inline int check_launch() { return cudaGetLastError() == cudaSuccess ? CP_OK : CP_ERR_CUDA; }

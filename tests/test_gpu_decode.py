@@ -108,3 +108,29 @@ def test_rows_normalised_behind_their_logits_or_by_a_kernel_of_their_own(B, Hkv,
         cp.decode_estimate(small, q[:1, :g].contiguous().cuda(), Kd[:1, :1, :100].contiguous(), ws)
         assert cp.device_status(ws) == 0
         assert np.abs(S.cpu().numpy() - S_ref).max() <= 1e-9
+
+
+@pytest.mark.parametrize("Hkv,g,n,blk", [(8, 4, 256 * 8, 8), (2, 4, 300, 32), (1, 1, 5, 32)])
+def test_decoding_needs_nothing_of_what_the_workspace_holds(Hkv, g, n, blk):
+    Q, K, V = make_uniform_qkv(1, Hkv * g, Hkv, n, 128, dtype="bf16", seed=n)
+    prob = cp.Problem(1, Hkv * g, Hkv, n, 128, blk, blk, 2, torch.bfloat16)
+    q, Kd = Q[:, :, -1].contiguous().cuda(), K.cuda()
+    ws = cp.alloc_workspace(prob)
+    S = cp.decode_estimate(prob, q, Kd, ws)
+    assert torch.equal(S, cp.decode_estimate(prob, q, Kd, torch.full_like(ws, 1)))
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f16", 64), ("f32", 128), ("f32", 64)])
+@pytest.mark.parametrize("B,Hkv,g,n2,blk", [
+    (1, 1, 1, 8, 4), (1, 2, 3, 9, 4), (2, 1, 4, 64, 4), (1, 2, 5, 65, 4), (1, 1, 8, 255, 4), (2, 3, 7, 256, 4),    # 1 to 16 CTAs of 8 to 16 warps
+    (1, 1, 9, 256, 4), (1, 2, 4, 257, 4), (2, 65, 1, 130, 4),                                                     # a head, a block, a batch too many
+    (1, 13, 2, 250, 32), (2, 75, 1, 40, 32)])                                                                     # two blocks per warp where these are long
+def test_short_rows_over_clusters_of_every_size(dtype, d, B, Hkv, g, n2, blk):
+    """The last block has one row."""
+    n = (n2 - 1) * blk + 1
+    Q, K, V = make_uniform_qkv(B, Hkv * g, Hkv, n, d, dtype=dtype, seed=n2 + g)
+    prob = cp.Problem(B, Hkv * g, Hkv, n, d, blk, blk, 2, TDT[dtype])
+    ws = cp.alloc_workspace(prob)
+    q = Q[:, :, -1].contiguous()
+    S = cp.decode_estimate(prob, q.cuda(), K.cuda(), ws)
+    assert np.abs(S.cpu().numpy() - oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))).max() <= 1e-9
