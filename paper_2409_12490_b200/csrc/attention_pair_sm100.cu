@@ -18,7 +18,7 @@
 // tile against 1040 of MMAs; in long loops the power cap, where the other kernel takes less energy over long units.  Both kernels
 // in graph replays, us (attention_sm100.cu / this one): 32 query / 8 KV heads, segment 512, block 32, budget 1024: 1300 tokens
 // 32.3 / 29.1, 2000 38.0 / 33.8, 13000 187 / 177; 8 / 2 heads, segment 256, budget 2048: 1000 tokens 21.9 / 15.3, 2000 35.5 / 23.0;
-// dense, 8 / 2 heads: 2000 tokens 35.0 / 22.4, 6000 108 / 79.  The line between them: launch_seqs in attention_sm100.cu.
+// dense, 8 / 2 heads: 2000 tokens 35.0 / 22.4, 6000 108 / 79.  The line between them: pairs_are_faster in attention_sm100.cu.
 #include "attention_units.cuh"
 
 namespace cp {

@@ -863,6 +863,42 @@ long long count_units(const Dims& m, const SeqSlot* slots, int n_seqs, bool dens
   return per_head * m.B * m.Hq;
 }
 
+// Whether pairs of CTAs take a launch in less time than single ones.  Units are handed out one ahead, so the SMs go through them in
+// rounds, as it were, longest units first, and each round lasts as long as its longest unit: rounds of 148 units on single CTAs, of 74 on
+// pairs, which take 0.5 of a single CTA's time per tile of a short unit, 0.62 of a long one (0.60 without a list), and 0.75 tiles more per launch.
+// Over 336 launches (37 to 3000 units of 2 to 1200 tiles; 1 / 1, 8 / 2 and 32 / 8 heads; loops of 0.1 s) the faster kernel but for 0.5 % on average;
+// the worst seen, single / pairs: 8 / 2 heads, 7104 tokens, budget 8192, 113 / 123 us on pairs; 16 / 4, 4000, 8192, 90 / 81 on single ones.  Single CTAs / pairs, us: segment 512, budget 1024: 37 units 22.5 / 15.8, 111 23.3 /
+// 23.0, 222 36.8 / 31.5, 296 39.5 / 41.5; segment 1024, budget 4096: 74 64.3 / 44.2, 110 64.6 / 73.6, 185 112 / 105, 260 128 / 144, 444 206 / 231;
+// dense, 8 / 2 heads: 80 units 39.1 / 30.3, 192 105 / 92, 296 201 / 204, 448 395 / 445.
+// With more than three units per SM the ends of the rounds no longer count.  Long units then cost pairs 5 to 15 % more (power); short ones cost
+// the same in long loops and 4 to 20 % less between other kernels, as their beginnings and ends overlap: whole layer of 8192 tokens (1024
+// units) 163.7 / 161.5 us; units of two tiles 12 % more (segment = budget = 256, 2072 units 107 / 122), of four 0.5 % less, so the line lies at 3.5
+// on average.  Beyond 14 per SM not even the former (whole layers, a batch of 3296 units 474 / 484).
+bool pairs_are_faster(const Dims& m, const SeqSlot* slots, int n_seqs, bool dense, bool long_units) {
+  constexpr int kMany = 3 * 148;
+  const long long units = count_units(m, slots, n_seqs, dense);
+  if (units > kMany) return !long_units && units <= 14 * 148 && 2 * ((m.k - m.r) * (long long)m.blk + m.seg / 2 + kTile) >= 7 * kTile;
+  int tiles[kMany], classes = 0;                    // of each unit of a head
+  for (int i = 0; i < n_seqs; ++i) {
+    const int seg = dense ? slots[i].len : m.seg;
+    for (int j = 0; j * seg < slots[i].len; ++j) {
+      const int rows = std::min(seg, slots[i].len - j * seg);
+      const long long past = dense ? 0 : std::min((long long)j * m.r, (long long)m.k - m.r) * m.blk;
+      for (int x = 0; x < rows; x += 2 * kTile)
+        tiles[classes++] = int((past + kTile - 1) / kTile) + x / kTile + (x + kTile < rows ? 2 : 1);
+    }
+  }
+  std::sort(tiles, tiles + classes, [](int a, int b) { return a > b; });
+  const long long heads = (long long)m.B * m.Hq;
+  auto rounds = [&](int places) {
+    long long sum = 0;
+    for (long long x = 0; x < units; x += places) sum += tiles[x / heads];
+    return sum;
+  };
+  const long long single = rounds(148), pair = rounds(74);
+  return long_units ? (dense ? 60 : 62) * pair + 75 < 100 * single : 50 * pair + 75 < 100 * single;
+}
+
 // (segment, pair)s that have query rows, by the tiles they stream, longest first (counting sort; equal ones from the last
 // segment down).  Returns their number, 0 when there are more than the table holds.
 template <int NS>
@@ -901,16 +937,9 @@ int launch_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, int n_s
   // kernel sits at the power cap (measured in 60-step loops: 1.6 % at 32 K/V tiles per unit) and costs where units are
   // short (3 % at 8 tiles per unit, the paper's operating point); a unit streams at most k*blk/128 tiles.
   a.emul = (dense || (long long)m.k * m.blk >= 12 * kTile) ? 1 : 0;
-  // The kernel of CTA pairs (attention_pair_sm100.cu): heads of 128 channels whose units have two query tiles (segments of an odd
-  // number of tiles would leave half of every pair idle), in launches of few units.  A unit takes half as long there, which counts while
-  // the SMs see up to three units each, or up to 14 short ones (their beginnings and ends overlap there); with more of them this kernel
-  // needs fewer cycles or, at the power cap, less energy per tile.  The results are the same bits.  Graph replays, this kernel / pairs, us,
-  // by units of a launch: segment 1024, budget 4096: 24 (8 / 2 heads, 600 tokens) 15.1 / 12.9, 64 35.5 / 23.2, 128 (32 / 8 heads, 1000
-  // tokens) 23.4 / 20.6, 192 86.0 / 70.7, 256 51.9 / 42.1, 288 112 / 105, 384 81.6 / 77.4, 408 162 / 158, 576 152 / 156, 1152 408 / 421; dense:
-  // 64 35.0 / 22.4, 192 108 / 79, 288 188 / 151, 408 299 / 298, 576 155 / 155, 1152 623 / 644.  Short units (budget 1024): 192 32.3 / 29.1,
-  // 1024 115 / 111, 1632 187 / 177; whole layer in long loops, a batch of 3296 units: 474 / 484.
-  const bool pair = m.d == 128 && (dense || m.seg % (2 * kTile) == 0) &&
-                    count_units(m, slots, n_seqs, dense) <= (a.emul ? 3 * 148 : 14 * 148);
+  // The kernel of CTA pairs (attention_pair_sm100.cu) takes heads of 128 channels whose units have two query tiles (segments of an odd number
+  // of tiles would leave half of every pair idle), where it is the faster one.  The results are the same bits.
+  const bool pair = m.d == 128 && (dense || m.seg % (2 * kTile) == 0) && pairs_are_faster(m, slots, n_seqs, dense, a.emul != 0);
   a.n_segs = 0;
   a.pp = pairs_per_segment(m.seg, slots, n_seqs);
   long long kv_tokens = 0;

@@ -106,11 +106,11 @@ def mixed_lists(Hq, n, seg, blk, k, seed, broken):
 
 
 @pytest.mark.parametrize("broken", [False, True])
-@pytest.mark.parametrize("dtype,blk,k,items", [("bf16", 32, 32, 7), ("f16", 128, 8, 7), ("bf16", 64, 32, 2)])
-def test_mixed_lists_over_many_units(dtype, blk, k, items, broken):
-    """Each pair of CTAs draws five units or so, with empty and one-block lists before and behind full ones.  One item alone (320 units: pairs)
-    and in a batch (640 long units, 2240 short ones: one CTA each); rows of a broken list are left as they were by both."""
-    Hq, Hkv, n, seg = 16, 4, 5000, 256
+@pytest.mark.parametrize("dtype,blk,k,items,Hq,Hkv,n", [("bf16", 32, 32, 7, 16, 4, 5000), ("f16", 128, 8, 7, 16, 4, 5000), ("bf16", 64, 32, 3, 2, 1, 27000)])
+def test_mixed_lists_over_many_units(dtype, blk, k, items, Hq, Hkv, n, broken):
+    """Each pair of CTAs draws three units or more, with empty and one-block lists before and behind full ones.  One item alone (320 short
+    or 212 long units: pairs) and in a batch (2240 short units, 636 long ones: one CTA each); rows of a broken list are left as they were by both."""
+    seg = 256
     Q, K, V = (t.cuda() for t in make_uniform_qkv(items, Hq, Hkv, n, 128, dtype=dtype, seed=k))
     lists = [mixed_lists(Hq, n, seg, blk, k, 10 * i + k, broken) for i in range(items)]
     idx, cnt = (torch.cat([x[i] for x in lists]).cuda() for i in (0, 1))
