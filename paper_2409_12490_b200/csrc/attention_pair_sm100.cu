@@ -12,8 +12,9 @@
 //   warp  14        MMA issuer of the pair (first CTA only)
 //   warp  15        scheduler
 // Tensor memory (512 columns): S_0 | S_1 | S_2 | O, 128 fp32 columns each; P goes over the first half of its S.
-// QK^T runs three tiles ahead of P V, across the ends of units.  The reference maximum and the row sum of a row go from tile to tile,
-// from one warpgroup to the other; O is rescaled (only when the maximum grew by more than 2^8) by the threads that form the tile's P.
+// QK^T runs three tiles ahead of P V, across the ends of units.  The reference maximum of a row goes from tile to tile, from one warpgroup
+// to the other; what each tile adds to the row's sum goes to the epilogue warps, which add up in the tiles' order.  O is rescaled (only when
+// the maximum grew by more than 2^8) by the threads that form the tile's P.
 // What bounds a unit: a tile's P -> P V -> QK^T three tiles on -> softmax (1800 + 2900 cycles) over three S buffers, 1600 to 1850 cycles per
 // tile against 1040 of MMAs; in long loops the power cap, where the other kernel takes less energy over long units.  Both kernels
 // in graph replays, us (attention_sm100.cu / this one): 32 query / 8 KV heads, segment 512, block 32, budget 1024: 1300 tokens
@@ -686,7 +687,6 @@ attention_pair_kernel(const __grid_constant__ Maps<NS> maps, const __grid_consta
     mbar_init(&bars->o_full, 1);
     mbar_init(&bars->o_empty, 8);
     for (int i = 0; i < kSched; ++i) {
-      
       mbar_init(&bars->sched_full[i], 1);
       mbar_init(&bars->sched_empty[i], kReaders - (rank == 0 ? 0 : 1));   // the MMA warp is the first CTA's
     }

@@ -866,10 +866,12 @@ long long count_units(const Dims& m, const SeqSlot* slots, int n_seqs, bool dens
 // Whether pairs of CTAs take a launch in less time than single ones.  Units are handed out one ahead, so the SMs go through them in
 // rounds, as it were, longest units first, and each round lasts as long as its longest unit: rounds of 148 units on single CTAs, of 74 on
 // pairs, which take 0.5 of a single CTA's time per tile of a short unit, 0.62 of a long one (0.60 without a list), and 0.75 tiles more per launch.
-// Over 336 launches (37 to 3000 units of 2 to 1200 tiles; 1 / 1, 8 / 2 and 32 / 8 heads; loops of 0.1 s) the faster kernel but for 0.5 % on average;
-// the worst seen, single / pairs: 8 / 2 heads, 7104 tokens, budget 8192, 113 / 123 us on pairs; 16 / 4, 4000, 8192, 90 / 81 on single ones.  Single CTAs / pairs, us: segment 512, budget 1024: 37 units 22.5 / 15.8, 111 23.3 /
-// 23.0, 222 36.8 / 31.5, 296 39.5 / 41.5; segment 1024, budget 4096: 74 64.3 / 44.2, 110 64.6 / 73.6, 185 112 / 105, 260 128 / 144, 444 206 / 231;
-// dense, 8 / 2 heads: 80 units 39.1 / 30.3, 192 105 / 92, 296 201 / 204, 448 395 / 445.
+// Over 336 launches (37 to 3000 units of 2 to 1200 tiles; 1 / 1, 8 / 2 and 32 / 8 heads; loops of 0.1 s) the choice costs 0.4 % on average against
+// the faster kernel; the worst seen, single CTAs / pairs, us: 8 / 2 heads, 7104 tokens, budget 8192, 113 / 123, on pairs; 16 / 4 heads, 4000 tokens,
+// budget 8192, 90 / 81, on single ones.
+// Single CTAs / pairs, us: segment 512, budget 1024: 37 units 22.5 / 15.8, 111 23.3 / 23.0, 222 36.8 / 31.5, 296 39.5 / 41.5; segment 1024, budget
+// 4096: 74 64.3 / 44.2, 110 64.6 / 73.6, 185 112 / 105, 260 128 / 144, 444 206 / 231; dense, 8 / 2 heads: 80 units 39.1 / 30.3, 192 105 / 92, 296 201 /
+// 204, 448 395 / 445.
 // With more than three units per SM the ends of the rounds no longer count.  Long units then cost pairs 5 to 15 % more (power); short ones cost
 // the same in long loops and 4 to 20 % less between other kernels, as their beginnings and ends overlap: whole layer of 8192 tokens (1024
 // units) 163.7 / 161.5 us; units of two tiles 12 % more (segment = budget = 256, 2072 units 107 / 122), of four 0.5 % less, so the line lies at 3.5

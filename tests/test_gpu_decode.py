@@ -134,3 +134,19 @@ def test_short_rows_over_clusters_of_every_size(dtype, d, B, Hkv, g, n2, blk):
     q = Q[:, :, -1].contiguous()
     S = cp.decode_estimate(prob, q.cuda(), K.cuda(), ws)
     assert np.abs(S.cpu().numpy() - oracle.decode_estimate(q, K, blk, est_scale=f32(1.0))).max() <= 1e-9
+
+
+@pytest.mark.parametrize("n", [300, 8000, 8200])
+def test_decoding_replays_from_a_cuda_graph(n):
+    """One launch of clusters of 2 or 16 CTAs, and two kernels, captured and replayed over other keys."""
+    prob = cp.Problem(1, 8, 2, n, 128, 32, 32, 8, torch.bfloat16)
+    (Q, K, _), (Q1, K1, _) = (make_uniform_qkv(1, 8, 2, n, 128, dtype="bf16", seed=x) for x in (1, 2))
+    q, Kd, ws = Q[:, :, -1].contiguous().cuda(), K.cuda(), cp.alloc_workspace(prob)
+    cp.decode_estimate(prob, q, Kd, ws)
+    S = torch.empty(1, 8, prob.n2, dtype=torch.float64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cp.decode_estimate(prob, q, Kd, ws, S_out=S)
+    q.copy_(Q1[:, :, -1]); Kd.copy_(K1)
+    graph.replay()
+    assert torch.equal(S, cp.decode_estimate(prob, q, Kd, ws))
