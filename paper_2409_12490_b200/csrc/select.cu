@@ -1,9 +1,9 @@
 // K3: critical block selection (Algorithm 2, line 8).  One CTA per (batch, query head,
 // segment j).  The r diagonal blocks are always taken; the other m = k - r slots go to the
-// strictly-past blocks with the largest score, ties to the larger block index.  Exact:
-// an MSB-first radix select (8 bits per pass, at most 8 passes, usually 3-4) on order-preserving 64-bit
-// keys held in registers finds the m-th largest score, equal keys are resolved towards larger indices by
-// counting, and an ordered block-wide compaction (two scans) writes the list ascending.
+// strictly-past blocks with the largest score, ties to the larger block index.  Exact: order-preserving
+// 64-bit keys are held in registers; a histogram over one 8-bit digit after the other leaves the blocks
+// that may hold the m-th largest score, until they are few enough to be ranked against each other (usually
+// after the first digit), and an ordered compaction by warp ballots writes the list ascending.
 #include "cp_common.cuh"
 
 namespace cp {
@@ -18,36 +18,33 @@ __device__ __forceinline__ unsigned long long ordered_key(double x) {
   return (u & 0x8000000000000000ull) ? ~u : (u | 0x8000000000000000ull);
 }
 
-// Block-wide exclusive scan of one int per thread (256 threads); *total receives the sum.  Two barriers.
-__device__ __forceinline__ int block_exclusive_scan(int v, int lane, int warp, int* warp_tot, int* total) {
-  int incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  if (lane == 31) warp_tot[warp] = incl;
-  __syncthreads();
-  int before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const int t = warp_tot[w];
-    before += w < warp ? t : 0;
-    all += t;
-  }
-  __syncthreads();                      // warp_tot may be reused by the next scan
-  *total = all;
-  return before + incl - v;
+constexpr int kRank = 32;        // as many candidates are ranked against each other instead of by a further digit
+constexpr int kLastLevel = 9;
+
+// The digit of a level of the search; larger keys (equal keys: larger indices) never have the smaller digit.
+//   0     sign, exponent and four bits of the mantissa, clamped to scores from -2^12 to -2^-4: ln S lies there, so that this
+//         digit alone spreads a row over 256 bins (its plain top byte is the same for nearly all of them)
+//   1-8   the bytes of the key
+//   9     the block index (all keys left are equal)
+__device__ __forceinline__ int digit_of(int level, unsigned long long key, int b) {
+  const uint32_t hi = uint32_t(key >> 32);
+  if (level == 0) return min(max(int(hi >> 16) - 0x3F50, 0), 255);
+  if (level == kLastLevel) return b >> 5;
+  return ((level <= 4 ? hi : uint32_t(key)) >> ((32 - 8 * level) & 31)) & 0xff;
 }
 
-// KPT = keys per thread; thread t owns the KPT consecutive blocks [t*KPT, (t+1)*KPT), so the ordered
-// compaction at the end is two block-wide scans instead of a barrier-separated step per key slot.
+// KPT = keys per thread at most.  The past blocks are dealt to the warps in consecutive parts of equal size, whatever the segment,
+// and inside a part lane by lane, so that reads and the written list are coalesced and the list is in order.  The kernel is bound by
+// latency: barriers, shared-memory atomics, one read of a row of scores.  When a thread owned KPT consecutive blocks each load of a
+// warp touched 32 lines, and the first two of three to four byte digits hit one or two bins.  Before / now, us, calls back to back in a
+// graph, 32 heads, segment 512, block 32: 1300 tokens 4.3 / 2.5, 4096 4.9 / 4.2, 8192 5.6 / 5.1, 16384 8.8 / 7.2, 131072 142 / 120;
+// segment 1024, block 128, 131072 tokens 26.9 / 23.0.  Candidates ranked, 32 / 64 / 128: 8192 tokens 5.1 / 5.3 / 6.8; several lanes
+// per candidate 8.4.
 // `pool` > 1: one CTA per (batch, KV head, segment); the key of a block is the largest of the pool's `pool`
 // consecutive query heads' scores, and the one list is written for each of them.  n_sink / n_local: the first
 // n_sink blocks and the n_local blocks right before the segment get the largest possible key, so they are taken
 // before any scored block (the host has checked that they fit into the k - r free slots).
-// Resident CTAs per SM are set by registers: the kernel waits on barriers most of the time, so 16 keys per thread are held to 64
-// registers (4 CTAs instead of the 3 that 80 registers allow: 13 % faster at n2 = 4096; 48 registers spill and are slower).
+// Resident CTAs per SM are set by registers; 16 keys per thread are held to 64 registers (4 CTAs).
 // One sequence of the launch (a single problem is one).
 struct SelectSeq { const double* S; int32_t *idx, *cnt; int n1, n2, cta_begin; };
 template <int NS> struct SelectArgs { SelectSeq s[NS]; int n; };
@@ -57,9 +54,9 @@ __global__ void __launch_bounds__(kThreads, KPT <= 4 ? 5 : (KPT <= 16 ? 4 : 2))
 select_kernel(const __grid_constant__ SelectArgs<NS> a, int r, int k, int pool, int n_sink, int n_local, int past_fixed) {
   __shared__ unsigned int hist[256];
   __shared__ int warp_sum[kWarps];
-  __shared__ unsigned long long prefix_sh;
-  __shared__ int remaining_sh, bin_count_sh;
-  __shared__ int warp_tot[kWarps];
+  __shared__ int bin_sh, remaining_sh, count_sh, n_cand;
+  __shared__ unsigned long long cand_key[kRank], thr_sh;
+  __shared__ int cand_blk[kRank], thr_blk_sh;
   int si = 0;
   while (NS > 1 && si + 1 < a.n && int(blockIdx.x) >= a.s[si + 1].cta_begin) ++si;
   const SelectSeq& sq = a.s[NS > 1 ? si : 0];
@@ -99,42 +96,42 @@ select_kernel(const __grid_constant__ SelectArgs<NS> a, int r, int k, int pool, 
     return;
   }
 
-  const int b0 = tid * KPT;                  // first block owned by this thread
+  const int part = (past + kThreads - 1) / kThreads * 32;   // blocks per warp, a multiple of 32, at most 32 * KPT
+  const int b0 = warp * part + lane, b_end = min(past, (warp + 1) * part);
   unsigned long long key[KPT];
+  unsigned alive = 0;                        // bit s: block b0 + 32 s may be the one that holds the m-th largest key
 #pragma unroll
   for (int s = 0; s < KPT; ++s) {
-    const int bb = b0 + s;
-    unsigned long long kk = 0ull;
-    if (bb < past) {
-      if (bb < n_sink || bb >= past - n_local) {
-        kk = ~0ull;                          // forced block
-      } else {
-        kk = ordered_key(__ldg(row + bb));
-        for (int u = 1; u < pool; ++u) kk = max(kk, ordered_key(__ldg(row + size_t(u) * n1 * n2 + bb)));
-      }
-    }
-    key[s] = kk;
+    key[s] = 0ull;
+    if (b0 + 32 * s < b_end) alive |= 1u << s;
   }
-  hist[tid] = 0;
-  __syncthreads();
-
-  // ---- radix select: key of the m-th largest past score --------------------------------
-  // MSB-first, 8 bits per pass.  A pass ends the search early when the bin that holds the m-th largest key
-  // holds exactly as many keys as are still to be taken: then every key of that bin (and above) is selected
-  // and no tie has to be resolved.  With distinct scores this happens after 3-4 of the 8 passes.
-  unsigned long long prefix = 0;   // bits decided so far (high bits)
-  int remaining = m;               // how many still to take among keys matching the prefix
-  bool all_of_bin = false;
-  for (int pass = 0; pass < 8; ++pass) {
-    const int shift = 56 - 8 * pass;
-    const unsigned long long himask = pass == 0 ? 0ull : (~0ull << (shift + 8));
+#pragma unroll 1
+  for (int u = 0; u < pool; ++u, row += size_t(n1) * n2) {
 #pragma unroll
     for (int s = 0; s < KPT; ++s)
-      if (b0 + s < past && (key[s] & himask) == prefix) atomicAdd(&hist[(key[s] >> shift) & 0xff], 1u);
+      if (alive >> s & 1u) key[s] = max(key[s], ordered_key(__ldg(row + b0 + 32 * s)));
+  }
+  if ((n_sink | n_local) != 0) {             // forced blocks
+#pragma unroll
+    for (int s = 0; s < KPT; ++s)
+      if (b0 + 32 * s < n_sink || b0 + 32 * s >= past - n_local) key[s] = ~0ull;
+  }
+  hist[tid] = 0;
+  if (tid == 0) n_cand = 0;
+  __syncthreads();
+
+  // ---- the block that holds the m-th largest past score (equal scores: the larger index is the larger) ----
+  int remaining = m;                         // its rank among those alive
+  int count = past;                          // how many are alive
+  unsigned above_mask = 0;                   // bit s: the block is certainly taken
+  for (int level = 0; count > kRank && level <= kLastLevel;) {
+#pragma unroll
+    for (int s = 0; s < KPT; ++s)
+      if (alive >> s & 1u) atomicAdd(&hist[digit_of(level, key[s], b0 + 32 * s)], 1u);
     __syncthreads();
     // suffix sums over the 256 bins: thread t owns bin t; above(t) = keys with a larger digit
     const int mine = int(hist[tid]);
-    hist[tid] = 0;                 // only its owner reads a bin, so it can be cleared for the next pass right away
+    hist[tid] = 0;                 // only its owner reads a bin, so it can be cleared for the next level right away
     int incl = mine;               // inclusive suffix sum within the warp (towards higher lanes)
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -146,52 +143,64 @@ select_kernel(const __grid_constant__ SelectArgs<NS> a, int r, int k, int pool, 
     int above = incl - mine;
     for (int w = warp + 1; w < kWarps; ++w) above += warp_sum[w];
     if (above < remaining && remaining <= above + mine) {   // exactly one bin satisfies this
-      prefix_sh = prefix | ((unsigned long long)tid << shift);
+      bin_sh = tid;
       remaining_sh = remaining - above;
-      bin_count_sh = mine;
+      count_sh = mine;
     }
     __syncthreads();
-    prefix = prefix_sh;
+    const int bin = bin_sh;
     remaining = remaining_sh;
-    if (bin_count_sh == remaining) { all_of_bin = true; break; }   // uniform: read from shared memory by all
-  }
-  // all_of_bin: take every key >= prefix (its undecided low bits are zero).  Otherwise prefix is the m-th
-  // largest key itself: take the keys above it and, of the keys equal to it, the `remaining` largest indices.
-  const unsigned long long thr = prefix;
-  int n_gt = 0, n_eq = 0;
+    count = count_sh;
 #pragma unroll
-  for (int s = 0; s < KPT; ++s) {
-    const bool in = b0 + s < past;
-    n_gt += in && (all_of_bin ? key[s] >= thr : key[s] > thr);
-    n_eq += in && !all_of_bin && key[s] == thr;
+    for (int s = 0; s < KPT; ++s) {
+      if (!(alive >> s & 1u)) continue;
+      const int dg = digit_of(level, key[s], b0 + 32 * s);
+      if (dg > bin) above_mask |= 1u << s;
+      if (dg != bin) alive &= ~(1u << s);
+    }
+    level = level == 0 && bin > 0 && bin < 255 ? 3 : level + 1;   // not clamped: the keys left agree in their top two bytes
   }
-  int eq_before = 0, eq_skip = 0;
-  if (!all_of_bin) {                         // uniform branch
-    int total_eq;
-    eq_before = block_exclusive_scan(n_eq, lane, warp, warp_tot, &total_eq);
-    eq_skip = total_eq - remaining;          // equal keys with the smallest indices are dropped
-  }
-  int n_take = n_gt;
-  if (!all_of_bin) {
+  // at most kRank blocks are left (the index digit leaves 32): each counts those before it
 #pragma unroll
-    for (int s = 0, e = eq_before; s < KPT; ++s)
-      if (b0 + s < past && key[s] == thr) { n_take += e >= eq_skip; ++e; }
+  for (int s = 0; s < KPT; ++s)
+    if (alive >> s & 1u) {
+      const int at = atomicAdd(&n_cand, 1);
+      cand_key[at] = key[s];
+      cand_blk[at] = b0 + 32 * s;
+    }
+  __syncthreads();
+  if (tid < count) {
+    const unsigned long long kk = cand_key[tid];
+    const int bb = cand_blk[tid];
+    int before = 0;
+    for (int i = 0; i < count; ++i) before += (cand_key[i] > kk) | ((cand_key[i] == kk) & (cand_blk[i] > bb));
+    if (before == remaining - 1) { thr_sh = kk; thr_blk_sh = bb; }
   }
+  __syncthreads();
+  const unsigned long long thr = thr_sh;
+  const int thr_blk = thr_blk_sh;
+  unsigned take = above_mask;
+#pragma unroll
+  for (int s = 0; s < KPT; ++s)
+    if ((alive >> s & 1u) && (key[s] > thr || (key[s] == thr && b0 + 32 * s >= thr_blk))) take |= 1u << s;
 
-  // ---- ordered compaction: blocks are owned in index order, so positions are an exclusive scan ----
-  int total_take;
-  const int pos0 = block_exclusive_scan(n_take, lane, warp, warp_tot, &total_take);
+  // ---- ordered compaction ----
+  int n_warp = 0;
+#pragma unroll
+  for (int s = 0; s < KPT; ++s) n_warp += __popc(__ballot_sync(0xffffffffu, take >> s & 1u));
+  if (lane == 0) warp_sum[warp] = n_warp;
+  __syncthreads();
+  int first = 0;
+  for (int w = 0; w < warp; ++w) first += warp_sum[w];
   for (int u = 0; u < pool; ++u) {           // the same list for every head of the pool
     int32_t* out = idx + (size_t(unit) + size_t(u) * n1) * k;
-    int pos = pos0;
+    int pos = first;
 #pragma unroll
-    for (int s = 0, e = eq_before; s < KPT; ++s) {
-      if (b0 + s >= past) break;
-      bool take;
-      if (all_of_bin) take = key[s] >= thr;
-      else if (key[s] == thr) { take = e >= eq_skip; ++e; }
-      else take = key[s] > thr;
-      if (take) { if (pos < m) out[pos] = b0 + s; ++pos; }
+    for (int s = 0; s < KPT; ++s) {
+      const unsigned taken = __ballot_sync(0xffffffffu, take >> s & 1u);
+      const int at = pos + __popc(taken & ((1u << lane) - 1u));
+      if ((take >> s & 1u) && at < m) out[at] = b0 + 32 * s;
+      pos += __popc(taken);
     }
     for (int i = tid; i < rj; i += kThreads) out[m + i] = past + i;   // diagonal blocks
     if (tid == 0) cnt[unit + u * n1] = k;
