@@ -1,200 +1,661 @@
 // K2 for 16-bit inputs with head_dim 128 (Algorithm 1, lines 9-14), split in two kernels:
-//   lse (see lse_sm100.cu / the general kernel)  the four log-sum-exps of every (head, segment) row, which need every
-//        key block of the row but only to the accuracy with which a term can still change the sum, and
-//   score_visible_kernel (this file)  the exact fp64 logits of the blocks a segment can see, combined
-//        straight out of the MMA accumulators:  ln S = max( ln((S1+S3)/2), ln((S2+S4)/2) ), fusion with S'.
-// Blocks that start at or after the end of the segment are masked by line 13 whatever their logits, so the
-// exact fp64 products -- the cost of this step -- are spent on the visible half of the map only.
-#include "score_common.cuh"
+//   lse (lse_sm100.cu)   the four log-sum-exps of every (head, segment) row, which need every key block of the row but only to
+//        the accuracy with which a term can still change the sum, and
+//   score_visible_kernel (this file)   the exact logits of the blocks a segment can see, combined straight out of tensor memory:
+//        ln S = max( ln((S1+S3)/2), ln((S2+S4)/2) ), fusion with S'.
+// Blocks that start at or after the end of the segment are masked by line 13 whatever their logits, so exact products are
+// spent on the visible half of the map only.
+//
+// Exact products without the fp64 pipe.  A representative is an integer multiple of a power of two: with 2^E above the largest
+// magnitude of its row, X = v 2^(30-E) is an integer of 31 bits unless v is smaller than the row's largest by some 2^22, and X is the
+// sum of four signed bytes, d0 + d1 2^8 + d2 2^16 + d3 2^24.  A logit is then the sum of 16 products of byte rows, which
+// tcgen05.mma.kind::i8 forms without any rounding; those of equal weight (i + j) share one of 7 accumulators of 32 bits (at most
+// 2^23).  Put together in 64-bit integers and rounded once to fp64 they give the dot product correctly rounded, which a chain of 128
+// fp64 additions does not.  Rows and blocks that do not fit (tiny values beside large ones, infinities, NaN) are marked, and their
+// logits are summed in fp64 by the threads that own them.
+//
+// One CTA per SM, 128 logit rows (the Qmax / Qmin representatives of 64 / U segments x U heads of a KV group) against tiles
+// of 32 key blocks (64 rows: Kmax, Kmin).  The tiles of all (row group, visible block) pairs are dealt to the CTAs in equal
+// consecutive parts.  Roles (768 threads):
+//   warps 0-15  epilogue: a thread per logit row and quarter of a tile; 7 accumulators -> logits, then the four logits of a score
+//               meet in one of the two lanes that hold them (Qmax and Qmin rows alternate) and are combined in fp64; at the
+//               start of a row group, the bytes of its query rows
+//   warps 16-19 bytes of the next tile's key rows into shared memory
+//   warp 20     MMA issuer: 64 MMAs of 128 x 64 x 32 per tile, under the fp64 part of the epilogue
+//   warps 21-23 the masked part of the map: -inf
+// Bound by MMAs and fp64 operations, which do not run at the same time: a tile's combination takes 1900 cycles alone (50 fp64 operations
+// per score) and 6100 with the next tile's MMAs under way, which take 3400 to 4600 (6 KB of operands each from shared memory).  A tile
+// takes 10 to 13 thousand cycles, with 8 epilogue warps 14 thousand (latency).  Half tiles with accumulators of their own, so that half of the
+// warps combine while the others convert: slower (N = 32: 5 KB per MMA of half the work; 131072 tokens 665 -> 780 us).
+// Both kernels of the scores, this one with fp64 MMAs (m16n8k16, 8 to 12 warps each on its own tiles) -> now, us, in graphs, 32 / 8 heads:
+// 131072 tokens, segment 512, block 32, fused 982 -> 665; segment 1024, block 128 184 -> 153; 65536 tokens, segment 512, block 64 166 -> 161.
+#include "sm100_ptx.cuh"
 
 namespace cp {
 namespace {
 
-constexpr int kThreads = 256;   // 8 warps x <= 85 registers: three CTAs per SM, so a CTA's set-up and tile epilogues run under the others' MMAs
-constexpr int kWarps = kThreads / 32;
-#ifndef CP_SCORE_FAST_MIN
-#define CP_SCORE_FAST_MIN 3000000
-#endif
-constexpr long long kFastMinScores = CP_SCORE_FAST_MIN;   // (batch x heads x segments x blocks) from which the two-kernel path is used
-constexpr int kG = 4;                       // segments per CTA: one MMA column group = 4 segments x {Qmax, Qmin} of one head
+constexpr long long kFastMinScores = 1500000;   // see score_is_split
+constexpr int kEpilogueWarps = 16, kThreads = (kEpilogueWarps + 8) * 32, kMmaWarp = kEpilogueWarps + 4;
+constexpr int kD = 128;
+constexpr int kRows = 128;                     // logit rows (MMA M) per CTA
+constexpr int kTileBlocks = 32;                // key blocks per tile
+constexpr int kTileN = 2 * kTileBlocks;        // their Kmax rows, then their Kmin rows (MMA N)
+constexpr int kDigits = 4, kAccs = 7;
+constexpr int kQPlane = kRows * kD, kKPlane = kTileN * kD;      // bytes of one byte plane
+constexpr int kStages = 2;                     // tiles of key rows
+constexpr int kInfo = 4;                       // what goes with a tile (scales, marks) outlives its bytes: read until its epilogue ends
+constexpr int kSmemK = kDigits * kQPlane;
+constexpr int kSmemFixed = kSmemK + kStages * kDigits * kKPlane;
 
-// One CTA: G = 4 consecutive segments x U query heads of one KV group.  The fp64 MMA m16n8k16 runs with 16 key
-// blocks on the M side (streamed from the summaries, widened to fp64 once and used for all 4*U segment-head
-// pairs) and, on the N side, the 8 columns (segment s, representative) = (s0 max, s0 min, s1 max, ...) of one
-// head.  Lane (grp = lane/4, tig = lane%4) then owns, for head u, segment tig and the two blocks grp, grp+8,
-// all four logits l1..l4 in its accumulators (Kmax product: cx, Kmin product: cn; even element: Qmax, odd:
-// Qmin) and finishes the element without shared memory.
-template <typename T, int D, int U>
-__global__ void __launch_bounds__(kThreads, 3)
-score_visible_kernel(const T* __restrict__ Qmax, const T* __restrict__ Qmin, const T* __restrict__ Kmax,
-                     const T* __restrict__ Kmin, const double* __restrict__ stats, const double* __restrict__ S_prev,
-                     double* __restrict__ S_out, int Hq, int g, int n1, int n2, int seg, int blk, double est_scale,
-                     double ln_alpha, double ln_1m_alpha, int fuse, int n_chunks) {
-  constexpr int KS = D / 4;                 // channels per lane slice (lane tig owns channels [tig*KS, (tig+1)*KS))
-  constexpr int CE = 16 / sizeof(T);        // elements per 16-byte load
-  constexpr int NCH = KS / CE;              // loads per slice
-  constexpr int SPC = CE / 4;               // MMA k-steps per load
-  constexpr int QS = D + 2;                 // row stride of qs in doubles (odd number of 16-byte units: conflict-free)
-  __shared__ __align__(16) double qs[U * 8 * QS];   // B operand: row = (head u, column c = 2*s + rep), [k-step][tig][4 channels]
-  __shared__ double st_sh[U * kG * 4];              // log-sum-exps of the (head, segment) rows of this CTA
-  __shared__ double sp_tab[kSpIntervals * kSpStride];
+constexpr int kNodes = 40 * 32 + 1;
+static __device__ const double2 kSoftplusNodes[kNodes] = {
+#include "softplus_nodes.inc"
+};
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tig = lane & 3, grp = lane >> 2;
-  // CTA -> (chunk of 4 segments, b, kv head, head subgroup); the chunks with the most visible blocks go first
-  const int groups = g / U;
-  int x = blockIdx.x;
-  const int per_chunk = gridDim.x / n_chunks;
-  const int chunk = n_chunks - 1 - x / per_chunk; x %= per_chunk;
-  const int sub = x % groups; x /= groups;
-  const int kvh = x;                                 // b*Hkv + kv head
-  const int Hkv = Hq / g;
-  const int b = kvh / Hkv;
-  const int h0 = (kvh % Hkv) * g + sub * U;          // first query head of this CTA
-  const int j0 = chunk * kG;
-  auto unit_of = [&](int u, int s) { return (size_t(b) * Hq + h0 + u) * n1 + j0 + s; };
-  auto visible_of = [&](int j) { return min(n2, ((j + 1) * seg + blk - 1) / blk); };   // first masked block of segment j
-  const int n_seg = min(kG, n1 - j0);                // segments of this chunk that exist
-  const int vis_hi = visible_of(j0 + n_seg - 1);
+struct Info {
+  double scale[kTileBlocks];                   // 2^(E-30) of a block's bytes; 1 if it is marked
+  uint32_t bad[4];                             // marked blocks, 8 per converting warp
+};
+struct __align__(16) RowInfo {
+  double scale[kRows];                         // likewise for the logit rows
+  double lse[kRows][2];                        // their log-sum-exps (Kmax, Kmin)
+  uint8_t bad[kRows / 8], special[kRows / 8];  // marked rows, 8 per converting warp; whether some of the 8 have log-sum-exps that are not finite
+};
+struct Bars {
+  double2 nodes[kNodes];                       // ln(1 + e^-x) and its derivative at the multiples of 1/32
+  Info info[kInfo];
+  RowInfo rows[2];                             // by parity of the CTA's row groups
+  unsigned long long q_full, k_full[kStages], k_empty[kStages], info_full[kInfo], acc_full, acc_empty;
+  uint32_t tmem_base;
+  volatile int abort_flag;
+};
+constexpr int kEpilogueRegs = 96, kOtherRegs = 48, kRegPoolNeeded = kEpilogueWarps * 32 * kEpilogueRegs + 256 * kOtherRegs;
+constexpr int kSmemTotal = kSmemFixed + int(sizeof(Bars)) + 1024;
 
-  for (int e = tid; e < kSpIntervals * kSpCoef; e += kThreads)
-    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
-  pdl_trigger();
-  pdl_wait(Qmax, Qmin, Kmax, Kmin, stats, S_prev);
-  for (int e = tid; e < U * kG * 4; e += kThreads) {
-    const int u = e / (kG * 4), s = (e / 4) % kG;
-    st_sh[e] = s < n_seg ? stats[unit_of(u, s) * 4 + (e & 3)] : 0.0;
+struct ScoreExactArgs {
+  const void *Qmax, *Qmin, *Kmax, *Kmin;       // representatives in the workspace
+  const float* kabs;                           // [B*Hkv, n2]
+  const double* stats;                         // [B,Hq,n1,4]
+  const double* S_prev;
+  double* S_out;
+  DeviceStatus* st;
+  int Hq, g, U, n1, n2, seg, blk, segs, n_qchunks, n_combos, fuse, vec;
+  int tiles_per_combo, n_tiles;
+  double est_scale, ln_alpha, ln_1m_alpha;
+};
+
+template <bool kF16> struct Elem { using type = __nv_bfloat16; };
+template <> struct Elem<true> { using type = __half; };
+
+// d s32, a and b s8, K-major; M = 128, N = 64
+constexpr uint32_t kIdesc = (2u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kTileN >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
+__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p, e;\n.reg .b32 lid;\nelect.sync lid|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
+      "@e tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, int* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+// The integer a0 + a1 2^8 + ... + a6 2^48, rounded once.  |a_s| <= 2^22.6 (the top digits are at most 64), so the sums of two fit 32
+// bits; the low four and the high three become fp64 exactly, through the mantissa of 1.5 x 2^52.
+__device__ __forceinline__ double digits_to_f64(int a0, int a1, int a2, int a3, int a4, int a5, int a6) {
+  constexpr long long kMagic = 0x4338000000000000ll;
+  constexpr double kMagicF = 6755399441055744.0;
+  const double lo = __longlong_as_double(mad_wide(a2 + (a3 << 8), 1 << 16, mad_wide(a0 + (a1 << 8), 1, kMagic))) - kMagicF;
+  const double hi = __longlong_as_double(mad_wide(a6, 1 << 16, mad_wide(a4 + (a5 << 8), 1, kMagic))) - kMagicF;
+  return fma(hi, 4294967296.0, lo);
+}
+
+// E with 2^(E-1) <= m < 2^E; kMarked: m is infinite, NaN or so large or small that the scales leave fp32
+constexpr int kMarked = 1 << 20;
+__device__ __forceinline__ int exponent_of(float m) {
+  const int e = int(__float_as_uint(m) >> 23) - 126;
+  return m == 0.f ? 30 : (e < -60 || e > 60) ? kMarked : e;
+}
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// 8 elements -> 8 bytes of each digit; true if the row is marked or an element is not a multiple of 2^(E-30)
+template <bool kF16>
+__device__ __forceinline__ bool to_digits(const uint4& v, int e, uint2 (&out)[kDigits]) {
+  const float mul = e == kMarked ? 0.f : __uint_as_float(uint32_t(127 + 30 - e) << 23);
+  // smallest magnitude whose last bit (2^-7 or 2^-10 of its leading one) is still at least 1; an fp16 is a multiple of 2^-24
+  const float least = kF16 ? (e <= 6 ? 0.f : 1024.f) : 128.f;
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint32_t dg[8];
+  bool bad = e == kMarked;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = unpack2<kF16>(w[i]);
+    const float x = f.x * mul, y = f.y * mul;
+    bad |= !(fabsf(x) >= least || x == 0.f) || !(fabsf(y) >= least || y == 0.f);
+    // signed bytes: adding 0x80 to each but the top one carries, the exclusive or takes it off again
+    dg[2 * i] = (uint32_t(__float2int_rz(x)) + 0x00808080u) ^ 0x00808080u;
+    dg[2 * i + 1] = (uint32_t(__float2int_rz(y)) + 0x00808080u) ^ 0x00808080u;
   }
-  for (int e = tid; e < U * 8 * D; e += kThreads) {
-    const int row = e / D, ch = e % D;               // row = u*8 + s*2 + rep
-    const int u = row >> 3, s = (row >> 1) & 3, rep = row & 1;
-    const int tq = ch / KS, within = ch % KS;        // owner lane-in-quad, position in its slice
-    const double v = s < n_seg ? to_f64(((rep == 0 ? Qmax : Qmin) + unit_of(u, s) * D)[ch]) : 0.0;
-    qs[row * QS + ((within >> 2) * 4 + tq) * 4 + (within & 3)] = v;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {                // 4 x 4 bytes transposed: digit p of four elements
+    const uint32_t* d = dg + 4 * h;
+    const uint32_t ab_lo = __byte_perm(d[0], d[1], 0x5140), cd_lo = __byte_perm(d[2], d[3], 0x5140);
+    const uint32_t ab_hi = __byte_perm(d[0], d[1], 0x7362), cd_hi = __byte_perm(d[2], d[3], 0x7362);
+    const uint32_t p0 = __byte_perm(ab_lo, cd_lo, 0x5410), p1 = __byte_perm(ab_lo, cd_lo, 0x7632);
+    const uint32_t p2 = __byte_perm(ab_hi, cd_hi, 0x5410), p3 = __byte_perm(ab_hi, cd_hi, 0x7632);
+    if (h == 0) { out[0].x = p0; out[1].x = p1; out[2].x = p2; out[3].x = p3; }
+    else { out[0].y = p0; out[1].y = p1; out[2].y = p2; out[3].y = p3; }
   }
-  // blocks at or after the end of a segment: -inf (line 13)
-  for (int r = warp; r < U * n_seg; r += kWarps) {
-    const int u = r / n_seg, s = r % n_seg;
-    double* row = S_out + unit_of(u, s) * n2;
-    for (int bb = visible_of(j0 + s) + lane; bb < n2; bb += 32) row[bb] = -CUDART_INF;
+  return bad;
+}
+template <bool kF16>
+__device__ __forceinline__ float absmax8(const uint4& v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  float m = 0.f;
+  bool nan = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = unpack2<kF16>(w[i]);
+    m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+    nan |= f.x != f.x || f.y != f.y;
   }
-  __syncthreads();
+  return nan ? CUDART_INF_F : m;
+}
+// 8-byte piece `c` (channels 8 c to 8 c + 7) of row `row` in a 128-byte-swizzled plane of 128-byte rows
+__device__ __forceinline__ uint32_t digit_at(int row, int c) { return row * kD + (((c >> 1) ^ (row & 7)) << 4) + (c & 1) * 8; }
 
-  const T* kmx_base = Kmax + size_t(kvh) * n2 * D;
-  const T* kmn_base = Kmin + size_t(kvh) * n2 * D;
-  const int my_vis = tig < n_seg ? visible_of(j0 + tig) : 0;     // this lane's segment
+// Part of a logit of a marked row or block, in fp64: `pieces` of 8 channels.  In line and rolled up: a call would cost the code around
+// it registers.
+template <bool kF16>
+__device__ __forceinline__ double slow_logit(const uint4* q, const uint4* k, int pieces) {
+  double x = 0.0, y = 0.0;
+#pragma unroll 1
+  for (int c = 0; c < pieces; ++c) {
+    const uint4 a = q[c], b = k[c];
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 af = unpack2<kF16>(aw[e]), bf = unpack2<kF16>(bw[e]);
+      x = fma(double(af.x), double(bf.x), x);
+      y = fma(double(af.y), double(bf.y), y);
+    }
+  }
+  return x + y;
+}
+
+// ln(1 + e^-x), x >= 0, for N independent values: Taylor series around the nearest node, whose coefficients are polynomials in the
+// derivative there (gen_softplus_nodes.py; absolute error 1.2e-16).  Written step by step for all N, so that the chains of 19 operations
+// run side by side.  The twelve coefficients of a piecewise polynomial, read from shared memory by index, kept that memory busy for
+// some 75 cycles per warp and evaluation.
+template <int N>
+__device__ __forceinline__ void softplus_nodes(const double2* nodes, double (&x)[N]) {
+  constexpr double kRound = 211106232532992.0;             // 1.5 x 2^47: sums keep multiples of 1/32
+  double s[N], w[N], h[N];
+  int at[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    // beyond 40 (infinity and NaN included) as at 40, where f = 4e-18 is below the rounding of what it is added to
+    if (uint32_t(__double2hiint(x[i])) >= 0x40440000u) x[i] = 40.0;
+    const double y = x[i] + kRound;
+    at[i] = __double2loint(y);
+    s[i] = nodes[at[i]].y;
+    x[i] -= y - kRound;
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) w[i] = fma(-s[i], s[i], s[i]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) h[i] = fma(fma(w[i], 120.0 / 720, -30.0 / 720), w[i], 1.0 / 720);
+#pragma unroll
+  for (int i = 0; i < N; ++i) h[i] = fma(h[i], x[i], fma(-2.0, s[i], 1.0) * fma(w[i], 12.0 / 120, -1.0 / 120));
+#pragma unroll
+  for (int i = 0; i < N; ++i) h[i] = fma(h[i], x[i], fma(w[i], -6.0 / 24, 1.0 / 24)) * x[i];
+#pragma unroll
+  for (int i = 0; i < N; ++i) h[i] = fma(fma(fma(-2.0, s[i], 1.0), -1.0 / 6, h[i]), x[i], 0.5);
+#pragma unroll
+  for (int i = 0; i < N; ++i) x[i] = fma(x[i], fma(w[i] * x[i], h[i], -s[i]), nodes[at[i]].x);
+}
+// the same by fmax and fmin, which leave a NaN out: for rows and blocks with infinities or NaN
+__device__ __forceinline__ double logaddexp_any(const double2* nodes, double a, double b) {
+  const double hi = fmax(a, b), lo = fmin(a, b);
+  double x[1] = {hi - lo};
+  if (!(x[0] >= 0.0)) return hi;
+  softplus_nodes(nodes, x);
+  return hi + x[0];
+}
+__device__ __noinline__ double combine_any(const double2* nodes, double L1, double L2, double L3, double L4) {
   const double ln2 = 0.693147180559945309417232121458;
-  const int n_tiles = (vis_hi + 15) / 16;
-  for (int t = warp; t < n_tiles; t += kWarps) {
-    const int blk0 = min(t * 16 + grp, n2 - 1), blk1 = min(t * 16 + grp + 8, n2 - 1);   // clamped in a ragged last tile
-    const uint4* src[4] = {reinterpret_cast<const uint4*>(kmx_base + size_t(blk0) * D + tig * KS),
-                           reinterpret_cast<const uint4*>(kmx_base + size_t(blk1) * D + tig * KS),
-                           reinterpret_cast<const uint4*>(kmn_base + size_t(blk0) * D + tig * KS),
-                           reinterpret_cast<const uint4*>(kmn_base + size_t(blk1) * D + tig * KS)};
-    double cx[U][4], cn[U][4];
+  const double h13 = fmax(L1, L3), h24 = fmax(L2, L4);
+  const bool first = h13 >= h24;
+  double y = logaddexp_any(nodes, first ? L1 : L2, first ? L3 : L4);
+  if (fabs(h13 - h24) < ln2) y = fmax(y, logaddexp_any(nodes, first ? L2 : L1, first ? L4 : L3));
+  return y;
+}
+
+__device__ __forceinline__ void ld4(const double* p, bool vec, int n, double* v) {
+  if (vec && n == 4) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+  } else {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int i = 0; i < 4; ++i) v[i] = i < n ? p[i] : 0.0;
+  }
+}
+__device__ __forceinline__ void st4(double* p, bool vec, int n, const double* v) {
+  if (vec && n == 4) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
+  } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { cx[u][i] = 0.0; cn[u][i] = 0.0; }
-    uint4 cur[4], nxt[4];
+    for (int i = 0; i < 4; ++i)
+      if (i < n) p[i] = v[i];
+  }
+}
+
+// The row groups and tiles of one CTA: consecutive tiles [lo, hi) of the list (combo, chunk of segments, tile of visible blocks).
+struct Walk {
+  int at, hi;
+  int combo, chunk, tile, n;                   // the current piece: tiles [tile, tile + n) of row group (combo, chunk)
+};
+__device__ __forceinline__ int visible_of(const ScoreExactArgs& a, int j) { return min(a.n2, ((j + 1) * a.seg + a.blk - 1) / a.blk); }
+__device__ __forceinline__ int chunk_tiles(const ScoreExactArgs& a, int chunk) {
+  return (visible_of(a, min(a.n1, (chunk + 1) * a.segs) - 1) + kTileBlocks - 1) / kTileBlocks;
+}
+__device__ __forceinline__ bool next_piece(const ScoreExactArgs& a, Walk& w) {
+  if (w.at >= w.hi) return false;
+  w.combo = w.at / a.tiles_per_combo;
+  int rest = w.at % a.tiles_per_combo;
+  int nt;
+  for (w.chunk = 0; rest >= (nt = chunk_tiles(a, w.chunk)); ++w.chunk) rest -= nt;
+  w.tile = rest;
+  w.n = min(nt - rest, w.hi - w.at);
+  w.at += w.n;
+  return true;
+}
+// row m of a row group: column m / 8 = (4 segments, head); within it (segment, representative)
+struct RowGroup { int kvh, b, h0, j0; };
+__device__ __forceinline__ RowGroup row_group(const ScoreExactArgs& a, const Walk& w) {
+  const int groups = a.g / a.U, Hkv = a.Hq / a.g;
+  RowGroup r;
+  r.kvh = w.combo / groups;
+  r.b = r.kvh / Hkv;
+  r.h0 = (r.kvh % Hkv) * a.g + (w.combo % groups) * a.U;
+  r.j0 = w.chunk * a.segs;
+  return r;
+}
+__device__ __forceinline__ int row_seg(const ScoreExactArgs& a, const RowGroup& r, int m) {
+  return min(a.n1, r.j0 + ((m >> 3) / a.U) * 4 + ((m >> 1) & 3));
+}
+__device__ __forceinline__ size_t row_unit(const ScoreExactArgs& a, const RowGroup& r, int m) {
+  return (size_t(r.b) * a.Hq + r.h0 + (m >> 3) % a.U) * a.n1 + row_seg(a, r, m);
+}
+
+// ---------------------------------------------------------------- warps 16-19
+template <bool kF16>
+__device__ __forceinline__ void convert_role(const ScoreExactArgs& a, Bars* bars, uint8_t* sm, Walk w, int warp, int lane) {
+  const int c = lane & 15, half = lane >> 4;   // a warp takes 8 blocks: Kmax rows by the lower half warp, Kmin rows by the upper; 8 channels per lane
+  uint32_t t = 0;                              // tiles so far
+  while (next_piece(a, w)) {
+    const RowGroup r = row_group(a, w);
+    const uint4* src = static_cast<const uint4*>(half ? a.Kmin : a.Kmax) + size_t(r.kvh) * a.n2 * (kD / 8) + c;
+    const float* abs_src = a.kabs + size_t(r.kvh) * a.n2;
+    for (int x = 0; x < w.n; ++x, ++t) {
+      const uint32_t stage = t % kStages;
+      uint8_t* dst = sm + kSmemK + stage * kDigits * kKPlane;
+      Info& info = bars->info[t % kInfo];
+      const int blk0 = (w.tile + x) * kTileBlocks + warp * 8;
+      uint32_t bad_blocks = 0;
+#pragma unroll 1
+      for (int i0 = 0; i0 < 8; i0 += 2) {
+        uint4 v[2];
+        float ka[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) cur[i] = __ldg(src[i]);
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-      if (ch + 1 < NCH) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) nxt[i] = __ldg(src[i] + ch + 1);
-      }
-#pragma unroll
-      for (int sp = 0; sp < SPC; ++sp) {
-        const int step = ch * SPC + sp;
-        double ax[8], an[8];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          ax[2 * c] = to_f64(reinterpret_cast<const T*>(&cur[0])[sp * 4 + c]);
-          ax[2 * c + 1] = to_f64(reinterpret_cast<const T*>(&cur[1])[sp * 4 + c]);
-          an[2 * c] = to_f64(reinterpret_cast<const T*>(&cur[2])[sp * 4 + c]);
-          an[2 * c + 1] = to_f64(reinterpret_cast<const T*>(&cur[3])[sp * 4 + c]);
+        for (int i = 0; i < 2; ++i) {
+          const bool in = blk0 + i0 + i < a.n2;
+          v[i] = in ? src[size_t(blk0 + i0 + i) * (kD / 8)] : make_uint4(0u, 0u, 0u, 0u);
+          ka[i] = in ? abs_src[blk0 + i0 + i] : 0.f;
         }
+        if (i0 == 0 && t >= kStages && !mbar_wait(&bars->k_empty[stage], (t / kStages - 1) & 1, &bars->abort_flag, a.st, 71)) return;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const double* qrow = &qs[(u * 8 + grp) * QS + (step * 4 + tig) * 4];
-          const double2 b01 = *reinterpret_cast<const double2*>(qrow);
-          const double2 b23 = *reinterpret_cast<const double2*>(qrow + 2);
-          asm volatile(
-              "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, {%4,%5,%6,%7,%8,%9,%10,%11}, "
-              "{%12,%13,%14,%15}, {%0,%1,%2,%3};"
-              : "+d"(cx[u][0]), "+d"(cx[u][1]), "+d"(cx[u][2]), "+d"(cx[u][3])
-              : "d"(ax[0]), "d"(ax[1]), "d"(ax[2]), "d"(ax[3]), "d"(ax[4]), "d"(ax[5]), "d"(ax[6]), "d"(ax[7]),
-                "d"(b01.x), "d"(b01.y), "d"(b23.x), "d"(b23.y));
-          asm volatile(
-              "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, {%4,%5,%6,%7,%8,%9,%10,%11}, "
-              "{%12,%13,%14,%15}, {%0,%1,%2,%3};"
-              : "+d"(cn[u][0]), "+d"(cn[u][1]), "+d"(cn[u][2]), "+d"(cn[u][3])
-              : "d"(an[0]), "d"(an[1]), "d"(an[2]), "d"(an[3]), "d"(an[4]), "d"(an[5]), "d"(an[6]), "d"(an[7]),
-                "d"(b01.x), "d"(b01.y), "d"(b23.x), "d"(b23.y));
+        for (int i = 0; i < 2; ++i) {
+          const int e = exponent_of(ka[i]);
+          uint2 dg[kDigits];
+          const bool bad = __ballot_sync(0xffffffffu, to_digits<kF16>(v[i], e, dg)) != 0;
+          const int at = warp * 8 + i0 + i;
+#pragma unroll
+          for (int p = 0; p < kDigits; ++p) *reinterpret_cast<uint2*>(dst + p * kKPlane + digit_at(half * kTileBlocks + at, c)) = dg[p];
+          bad_blocks |= (bad ? 1u : 0u) << (i0 + i);
+          if (lane == 0) info.scale[at] = bad ? 1.0 : pow2(e - 30);
         }
       }
-      if (ch + 1 < NCH) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
-      }
-    }
-    // C[i]: block grp + 8*(i/2), column 2*tig + (i%2) = (segment tig, representative i%2).
-    // Qmax columns: cx = l1, cn = l2; Qmin columns: cx = l3, cn = l4.
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const double* stp = &st_sh[(u * kG + tig) * 4];
-      const double st1 = stp[0], st2 = stp[1], st3 = stp[2], st4 = stp[3];
-      const size_t out_row = unit_of(u, tig) * n2;
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const int bb = t * 16 + grp + half * 8;
-        if (bb < my_vis) {
-          const double L1 = cx[u][2 * half] * est_scale - st1, L2 = cn[u][2 * half] * est_scale - st2;
-          const double L3 = cx[u][2 * half + 1] * est_scale - st3, L4 = cn[u][2 * half + 1] * est_scale - st4;
-          // max( ln (S1+S3)/2, ln (S2+S4)/2 ).  ln(e^a + e^b) lies in [max(a,b), max(a,b) + ln 2], so the pair with the
-          // larger maximum wins outright unless the two maxima are within ln 2 of each other: one evaluation, rarely two.
-          const double h13 = fmax(L1, L3), h24 = fmax(L2, L4);
-          const bool first = h13 >= h24;
-          double v = logaddexp(first ? L1 : L2, first ? L3 : L4, sp_tab);
-          if (fabs(h13 - h24) < ln2) v = fmax(v, logaddexp(first ? L2 : L1, first ? L4 : L3, sp_tab));
-          v -= ln2;
-          if (fuse) v = logaddexp(ln_alpha + v, ln_1m_alpha + S_prev[out_row + bb], sp_tab);
-          S_out[out_row + bb] = v;
-        }
-      }
+      if (lane == 0) info.bad[warp] = bad_blocks;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the planes through the async proxy
+      mbar_arrive(&bars->info_full[t % kInfo]);
+      mbar_arrive(&bars->k_full[stage]);
     }
   }
 }
 
-template <typename T, int U>
-int launch_visible(const Dims& m, const char* ws, const WsLayout& w, const double* S_prev, double* S_out,
-                   double est_scale, double alpha, int fuse, cudaStream_t st) {
-  const int n_chunks = (m.n1 + kG - 1) / kG;
-  const long long ctas = (long long)m.B * m.Hkv * (m.g / U) * n_chunks;
-  if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
-  return launch_pdl(
-      score_visible_kernel<T, 128, U>, dim3(unsigned(ctas)), kThreads, 0, st,
-      reinterpret_cast<const T*>(ws + w.qmax), reinterpret_cast<const T*>(ws + w.qmin),
-      reinterpret_cast<const T*>(ws + w.kmax), reinterpret_cast<const T*>(ws + w.kmin),
-      reinterpret_cast<const double*>(ws + w.stats), S_prev, S_out, m.Hq, m.g, m.n1, m.n2, m.seg, m.blk, est_scale,
-      log(alpha), log1p(-alpha), fuse, n_chunks);
+// ---------------------------------------------------------------- warp 20
+__device__ __forceinline__ void mma_role(const ScoreExactArgs& a, Bars* bars, uint32_t smem, Walk w) {
+  const uint32_t tm = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  const uint64_t base = desc_base(16);
+  uint32_t t = 0;
+  for (uint32_t piece = 0; next_piece(a, w); ++piece) {
+    if (!mbar_wait(&bars->q_full, piece & 1, &bars->abort_flag, a.st, 70)) return;
+    for (int x = 0; x < w.n; ++x, ++t) {
+      const uint32_t stage = t % kStages;
+      if (!mbar_wait(&bars->k_full[stage], (t / kStages) & 1, &bars->abort_flag, a.st, 72)) return;
+      if (t > 0 && !mbar_wait(&bars->acc_empty, (t - 1) & 1, &bars->abort_flag, a.st, 73)) return;
+      tc_fence_after();
+      const uint32_t k_smem = smem + kSmemK + stage * kDigits * kKPlane;
+#pragma unroll
+      for (int s = 0; s < kAccs; ++s)
+#pragma unroll
+        for (int i = s > 3 ? s - 3 : 0; i <= (s < 3 ? s : 3); ++i)
+#pragma unroll
+          for (int kk = 0; kk < kD / 32; ++kk)
+            umma_i8(tm + s * kTileN, desc_at(base, smem + i * kQPlane + kk * 32), desc_at(base, k_smem + (s - i) * kKPlane + kk * 32),
+                    i > (s > 3 ? s - 3 : 0) || kk > 0);
+      umma_commit(&bars->acc_full);
+      umma_commit(&bars->k_empty[stage]);
+    }
+  }
 }
 
-template <typename T>
-int launch_visible_t(const Dims& m, const char* ws, const WsLayout& w, const double* S_prev, double* S_out,
-                     double est_scale, double alpha, int fuse, cudaStream_t st) {
-  // One head per CTA: 80 registers, three CTAs of 8 warps per SM.  More heads per CTA amortise the widening of the A operand
-  // over more MMAs but leave fewer CTAs to overlap (measured at n2 = 4096: U = 4 with one CTA of 12 warps 0.69 ms, U = 2 with two
-  // CTAs 0.65 ms, U = 1 with three 0.62 ms; four CTAs at 64 registers spill and gain nothing).
-  return launch_visible<T, 1>(m, ws, w, S_prev, S_out, est_scale, alpha, fuse, st);
+// ---------------------------------------------------------------- warps 0-15
+template <bool kF16>
+__device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bars, uint8_t* sm, Walk w, int warp, int lane) {
+  const int m = (warp & 3) * 32 + lane, hc = warp >> 2;     // logit row; quarter of the tile's blocks
+  const uint32_t tm = bars->tmem_base + (uint32_t((warp & 3) * 32) << 16) + hc * 8;
+  const bool odd = lane & 1;                                // Qmin rows; the lane takes the upper 4 of its 8 blocks
+  const double ln2 = 0.693147180559945309417232121458;
+  uint32_t t = 0;
+  for (uint32_t piece = 0; next_piece(a, w); ++piece) {
+    const RowGroup r = row_group(a, w);
+    RowInfo& ri = bars->rows[piece & 1];
+    {
+      // The bytes of the row group's query rows, 8 rows per warp, two at a time.  The MMAs on the row group before have all been
+      // completed: this warp has seen the last of them.
+      const int c = lane & 15, m0 = (warp & 3) * 32 + hc * 8 + (lane >> 4);
+      uint4 q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int mq = m0 + 2 * i;
+        q[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (row_seg(a, r, mq) < a.n1) q[i] = static_cast<const uint4*>((mq & 1) ? a.Qmin : a.Qmax)[row_unit(a, r, mq) * (kD / 8) + c];
+      }
+      uint32_t bad_rows = 0;
+      bool not_finite = false;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int mq = m0 + 2 * i;
+        float mx = absmax8<kF16>(q[i]);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const int e = exponent_of(mx);
+        uint2 dg[kDigits];
+        const unsigned bad = __ballot_sync(0xffffffffu, to_digits<kF16>(q[i], e, dg));
+#pragma unroll
+        for (int p = 0; p < kDigits; ++p) *reinterpret_cast<uint2*>(sm + p * kQPlane + digit_at(mq, c)) = dg[p];
+        const uint32_t both = ((bad & 0xffffu) != 0 ? 1u : 0u) | ((bad >> 16) != 0 ? 2u : 0u);
+        bad_rows |= both << (2 * i);
+        if (c < 2) {
+          const double l = row_seg(a, r, mq) < a.n1 ? a.stats[row_unit(a, r, mq) * 4 + 2 * (mq & 1) + c] : 0.0;
+          ri.lse[mq][c] = l;
+          not_finite |= !(fabs(l) < CUDART_INF);
+        }
+        if (c == 0) ri.scale[mq] = (both >> (lane >> 4) & 1u) ? 1.0 : pow2(e - 30);
+      }
+      not_finite = __any_sync(0xffffffffu, not_finite);
+      if (lane == 0) { ri.bad[(warp & 3) * 4 + hc] = uint8_t(bad_rows); ri.special[(warp & 3) * 4 + hc] = not_finite; }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the planes through the async proxy
+      mbar_arrive(&bars->q_full);
+    }
+    const int j = row_seg(a, r, m);
+    const bool valid = j < a.n1;
+    const size_t unit = row_unit(a, r, m);
+    const int vis = valid ? visible_of(a, j) : 0;
+    const int warp_vis = __reduce_max_sync(0xffffffffu, vis);
+    if (!mbar_wait(&bars->q_full, piece & 1, &bars->abort_flag, a.st, 76)) return;
+    const uint32_t bad_rows = *reinterpret_cast<const uint32_t*>(&ri.bad[(warp & 3) * 4]);        // of the warp's rows
+    const bool special = *reinterpret_cast<const uint32_t*>(&ri.special[(warp & 3) * 4]) != 0;
+    for (int x = 0; x < w.n; ++x, ++t) {
+      const int b_tile = (w.tile + x) * kTileBlocks + hc * 8, b0 = b_tile + (odd ? 4 : 0);
+      const int n_in = valid ? min(4, a.n2 - b0) : 0;       // blocks of this lane that exist
+      const size_t out = unit * a.n2 + b0;
+      double sp[4];
+      const bool any = b_tile < warp_vis;                   // some row of the warp sees some of its 8 blocks
+      if (a.fuse && any) ld4(a.S_prev + out, a.vec, n_in, sp);
+      if (!mbar_wait(&bars->info_full[t % kInfo], (t / kInfo) & 1, &bars->abort_flag, a.st, 74)) return;
+      if (!mbar_wait(&bars->acc_full, t & 1, &bars->abort_flag, a.st, 75)) return;
+      tc_fence_after();
+      if (!any) {
+        tc_fence_before();
+        mbar_arrive(&bars->acc_empty);
+        const double v[4] = {-CUDART_INF, -CUDART_INF, -CUDART_INF, -CUDART_INF};
+        st4(a.S_out + out, a.vec, n_in, v);
+        continue;
+      }
+      const Info& info = bars->info[t % kInfo];
+      double vx[8], vn[8];                                  // integer dot products with the Kmax / Kmin rows of the 8 blocks
+#pragma unroll
+      for (int part = 0; part < 4; ++part) {
+        const uint32_t col = tm + (part >> 1) * kTileBlocks + (part & 1) * 4;
+        int acc[kAccs][4];
+#pragma unroll
+        for (int s = 0; s < kAccs; ++s) tmem_ld4(col + s * kTileN, acc[s]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const double d = digits_to_f64(acc[0][i], acc[1][i], acc[2][i], acc[3][i], acc[4][i], acc[5][i], acc[6][i]);
+          if (part < 2) vx[(part & 1) * 4 + i] = d; else vn[(part & 1) * 4 + i] = d;
+        }
+      }
+      tc_fence_before();
+      mbar_arrive(&bars->acc_empty);
+      const uint32_t bad_blocks = info.bad[hc];
+      if (bad_blocks | bad_rows) {
+        // marked blocks: every lane the two logits of its row; marked rows: the lanes share the row's 16 logits, half of the channels each
+        const uint4 *kx = static_cast<const uint4*>(a.Kmax) + (size_t(r.kvh) * a.n2 + b_tile) * (kD / 8);
+        const uint4 *kn = static_cast<const uint4*>(a.Kmin) + (size_t(r.kvh) * a.n2 + b_tile) * (kD / 8);
+        const int last = min(8, a.n2 - b_tile) - 1;         // blocks past the end: any logit will do
+#pragma unroll 1
+        for (uint32_t left = bad_blocks; left; left &= left - 1) {
+          const int ib = __ffs(left) - 1, at = min(ib, last) * (kD / 8);
+          const uint4* q = static_cast<const uint4*>((m & 1) ? a.Qmin : a.Qmax) + (valid ? unit : 0) * (kD / 8);
+          const double un = 1.0 / (ri.scale[m] * info.scale[hc * 8 + ib]);     // a power of two: taken off again below
+#pragma unroll 1
+          for (int kr = 0; kr < 2; ++kr) {
+            const double l = slow_logit<kF16>(q, (kr ? kn : kx) + at, kD / 8) * un;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (i == ib && kr == 0) vx[i] = l;
+              if (i == ib && kr == 1) vn[i] = l;
+            }
+          }
+        }
+#pragma unroll 1
+        for (uint32_t left = bad_rows; left; left &= left - 1) {
+          const int owner = __ffs(left) - 1, ib = lane & 7, mo = (warp & 3) * 32 + owner, c0 = (lane >> 4) * (kD / 16);
+          const uint4* q = static_cast<const uint4*>((mo & 1) ? a.Qmin : a.Qmax) + row_unit(a, r, mo) * (kD / 8) + c0;
+          double l = slow_logit<kF16>(q, ((lane & 8) == 0 ? kx : kn) + min(ib, last) * (kD / 8) + c0, kD / 16);
+          l = (l + __shfl_xor_sync(0xffffffffu, l, 16)) / info.scale[hc * 8 + ib];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const double lx = __shfl_sync(0xffffffffu, l, i), ln = __shfl_sync(0xffffffffu, l, 8 + i);
+            if (lane == owner) { vx[i] = lx; vn[i] = ln; }
+          }
+        }
+      }
+      // The Qmax lane gives its upper blocks for the Qmin lane's lower ones: each then has all four logits of 4 blocks, less
+      // their log-sum-exps.  Which of a pair is l1 (l2) and which l3 (l4) makes no difference.
+      const double f_own = ri.scale[m] * a.est_scale, f_other = ri.scale[m ^ 1] * a.est_scale;
+      const double2 lse_own = *reinterpret_cast<const double2*>(ri.lse[m]), lse_other = *reinterpret_cast<const double2*>(ri.lse[m ^ 1]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const double ox = __shfl_xor_sync(0xffffffffu, odd ? vx[i] : vx[4 + i], 1), on = __shfl_xor_sync(0xffffffffu, odd ? vn[i] : vn[4 + i], 1);
+        const double mx = odd ? vx[4 + i] : vx[i], mn = odd ? vn[4 + i] : vn[i];
+        const double bs = info.scale[hc * 8 + (odd ? 4 : 0) + i];
+        const double fm = f_own * bs, fo = f_other * bs;
+        vx[i] = fma(mx, fm, -lse_own.x); vn[i] = fma(mn, fm, -lse_own.y);
+        vx[4 + i] = fma(ox, fo, -lse_other.x); vn[4 + i] = fma(on, fo, -lse_other.y);
+      }
+      // max( ln (S1+S3)/2, ln (S2+S4)/2 ), fusion with S'
+      double v[4];
+      if (special | bad_blocks | bad_rows) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = combine_any(bars->nodes, vx[i], vn[i], vx[4 + i], vn[4 + i]) - ln2;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+          double hi[4], d[4];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const double L1 = vx[q + i], L2 = vn[q + i], L3 = vx[4 + q + i], L4 = vn[4 + q + i];
+            d[i] = L1 - L3; d[2 + i] = L2 - L4;
+            hi[i] = __double2hiint(d[i]) >= 0 ? L1 : L3; hi[2 + i] = __double2hiint(d[2 + i]) >= 0 ? L2 : L4;
+            d[i] = fabs(d[i]); d[2 + i] = fabs(d[2 + i]);
+          }
+          softplus_nodes(bars->nodes, d);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const double y13 = hi[i] + d[i], y24 = hi[2 + i] + d[2 + i];
+            v[q + i] = (y13 >= y24 ? y13 : y24) - ln2;
+          }
+        }
+      }
+      if (a.fuse) {
+        double d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const double y = a.ln_alpha + v[i], z = a.ln_1m_alpha + sp[i];
+          v[i] = fmax(y, z);
+          d[i] = v[i] - fmin(y, z);
+        }
+        softplus_nodes(bars->nodes, d);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] += d[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = b0 + i < vis ? v[i] : -CUDART_INF;     // blocks at or after the end of the segment (line 13)
+      st4(a.S_out + out, a.vec, n_in, v);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- warps 21-23: blocks after the tiles of a row group
+__device__ __forceinline__ void mask_role(const ScoreExactArgs& a, int warp, int lane) {
+  const size_t rows = size_t(a.n_combos) * a.U * a.n1;      // = batch x heads x segments
+  for (size_t u = size_t(blockIdx.x) * 3 + warp; u < rows; u += size_t(gridDim.x) * 3) {
+    const int lo = chunk_tiles(a, int(u % a.n1) / a.segs) * kTileBlocks;
+    double* row = a.S_out + u * a.n2;
+    if (a.vec) {
+      for (int b = lo + lane * 4; b < a.n2; b += 128)
+        asm volatile("st.global.v4.f64 [%0], {%1, %1, %1, %1};" ::"l"(row + b), "d"(-CUDART_INF) : "memory");
+    } else {
+      for (int b = lo + lane; b < a.n2; b += 32) row[b] = -CUDART_INF;
+    }
+  }
+}
+
+template <bool kF16>
+__global__ void __launch_bounds__(kThreads, 1) score_visible_kernel(const __grid_constant__ ScoreExactArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t smem_base = (raw + 1023u) & ~1023u;
+  uint8_t* sm = smem_raw + (smem_base - raw);
+  Bars* bars = reinterpret_cast<Bars*>(sm + kSmemFixed);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int i = 0; i < kStages; ++i) { mbar_init(&bars->k_full[i], 128); mbar_init(&bars->k_empty[i], 1); }
+    for (int i = 0; i < kInfo; ++i) mbar_init(&bars->info_full[i], 128);
+    mbar_init(&bars->q_full, kEpilogueWarps * 32);
+    mbar_init(&bars->acc_full, 1);
+    mbar_init(&bars->acc_empty, kEpilogueWarps * 32);
+    bars->abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kMmaWarp) { tmem_alloc(&bars->tmem_base, 512); tmem_relinquish(); }
+  for (int e = tid; e < kNodes; e += kThreads) bars->nodes[e] = kSoftplusNodes[e];
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_trigger();
+  pdl_wait();                                  // the loads behind it are plain ones, which stay behind it
+
+  Walk w;
+  w.at = int((long long)a.n_tiles * blockIdx.x / gridDim.x);
+  w.hi = int((long long)a.n_tiles * (blockIdx.x + 1) / gridDim.x);
+  static_assert(kRegPoolNeeded <= kThreads * 80, "setmaxnreg budget exceeds the launch allocation");
+  if (warp < kEpilogueWarps) {
+    reg_inc<kEpilogueRegs>();
+    epilogue_role<kF16>(a, bars, sm, w, warp, lane);
+  } else {
+    reg_dec<kOtherRegs>();
+    if (warp < kMmaWarp) convert_role<kF16>(a, bars, sm, w, warp - kEpilogueWarps, lane);
+    else if (warp == kMmaWarp) mma_role(a, bars, smem_base, w);
+    else mask_role(a, warp - kMmaWarp - 1, lane);
+  }
+  if (bars->abort_flag) {
+    for (int i = 0; i < 200; ++i) __nanosleep(1000);        // let MMAs in flight land before the CTA's resources go
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) tmem_dealloc(bars->tmem_base, 512);
+}
+
+template <bool kF16>
+int launch_visible(const Dims& m, char* ws, const double* S_prev, double* S_out, double est_scale, double alpha, int fuse, cudaStream_t st) {
+  const WsLayout w = ws_layout(m);
+  ScoreExactArgs a;
+  a.Qmax = ws + w.qmax; a.Qmin = ws + w.qmin; a.Kmax = ws + w.kmax; a.Kmin = ws + w.kmin;
+  a.kabs = reinterpret_cast<const float*>(ws + w.kabs);
+  a.stats = reinterpret_cast<const double*>(ws + w.stats);
+  a.S_prev = S_prev; a.S_out = S_out;
+  a.st = reinterpret_cast<DeviceStatus*>(ws);
+  a.Hq = m.Hq; a.g = m.g; a.U = m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1);
+  a.n1 = m.n1; a.n2 = m.n2; a.seg = m.seg; a.blk = m.blk;
+  a.segs = 64 / a.U;
+  a.n_qchunks = (m.n1 + a.segs - 1) / a.segs;
+  a.n_combos = m.B * m.Hkv * (m.g / a.U);
+  a.fuse = fuse;
+  // whole 32-byte sectors where every row of the map starts on one
+  a.vec = m.n2 % 4 == 0 && (reinterpret_cast<uintptr_t>(S_out) & 31u) == 0 && (!fuse || (reinterpret_cast<uintptr_t>(S_prev) & 31u) == 0);
+  long long per_combo = 0;
+  for (int c = 0; c < a.n_qchunks; ++c) {
+    const int j = (c + 1) * a.segs < m.n1 ? (c + 1) * a.segs - 1 : m.n1 - 1;
+    const long long end = ((long long)(j + 1) * m.seg + m.blk - 1) / m.blk;
+    per_combo += ((end < m.n2 ? end : m.n2) + kTileBlocks - 1) / kTileBlocks;
+  }
+  if (per_combo * a.n_combos > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
+  a.tiles_per_combo = int(per_combo);
+  a.n_tiles = int(per_combo * a.n_combos);
+  a.est_scale = est_scale; a.ln_alpha = log(alpha); a.ln_1m_alpha = log1p(-alpha);
+  auto kern = score_visible_kernel<kF16>;
+  // setmaxnreg.inc blocks forever when the registers that the kernel was compiled to are fewer than what the roles ask for: refuse
+  // to launch such a build instead
+  static int regs_ok = 0;
+  if (regs_ok == 0) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return CP_ERR_CUDA;
+    regs_ok = fa.numRegs * kThreads >= kRegPoolNeeded ? 1 : -1;
+  }
+  if (regs_ok < 0) return CP_ERR_UNSUPPORTED;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal) != cudaSuccess) return CP_ERR_CUDA;
+  const unsigned grid = unsigned(a.n_tiles < 148 ? a.n_tiles : 148);   // one CTA per SM
+  return launch_pdl(kern, dim3(grid), kThreads, kSmemTotal, st, a);
 }
 
 }  // namespace
 
+// From which size on the two-kernel path is used.  What counts is the general kernel's work: its MMAs have 8 columns, the Qmax and
+// Qmin rows of up to 4 heads of a group, of which groups of 2 heads fill half and single heads a quarter.
+// General kernel / two kernels, us, 32 / 8 heads: segment 512, block 32, 16384 tokens (0.5 M scores) 36 / 68; block 64, 32768 tokens
+// (1.05 M, fused) 77 / 78; segment 1024, block 128, 65536 tokens (1.05 M) 70 / 74; block 32, 32768 tokens (2.1 M) 122 / 105; 8 / 8 heads, segment
+// 128, block 32, 16384 tokens (0.5 M, counted as 2.1 M) 103 / 75.
 bool score_is_split(const cp_params& p, const Dims& m) {
-  const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2;
+  const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2 * (m.g % 4 == 0 ? 1 : (m.g % 2 == 0 ? 2 : 4));
   return (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 &&
          (scores >= kFastMinScores || (p.flags & CP_FLAG_FORCE_SPLIT_SCORE));
 }
@@ -203,15 +664,14 @@ bool score_is_split(const cp_params& p, const Dims& m) {
 // the visible blocks); everything else the general kernel.
 int launch_score(const cp_params& p, const Dims& m, char* ws, const double* S_prev, double* S_out, cudaStream_t st) {
   // The two-kernel path pays for an extra launch and for the serial sweeps of the log-sum-exp kernel; it wins once the
-  // score map is large (measured: 2x at 33 M scores, nothing below a few million), so small maps keep the general kernel.
+  // score map is large, so small maps keep the general kernel.
   if (!score_is_split(p, m)) return launch_score_generic(p, m, ws, S_prev, S_out, nullptr, st);
-  const WsLayout w = ws_layout(m);
-  int rc = launch_lse(p, m, ws, st);
+  const int rc = launch_lse(p, m, ws, st);
   if (rc != CP_OK) return rc;
   const int fuse = (S_prev != nullptr && p.alpha != 1.0f) ? 1 : 0;
   const double es = double(p.est_scale), al = double(p.alpha);
-  if (p.dtype == CP_BF16) return launch_visible_t<__nv_bfloat16>(m, ws, w, S_prev, S_out, es, al, fuse, st);
-  return launch_visible_t<__half>(m, ws, w, S_prev, S_out, es, al, fuse, st);
+  return p.dtype == CP_F16 ? launch_visible<true>(m, ws, S_prev, S_out, es, al, fuse, st)
+                           : launch_visible<false>(m, ws, S_prev, S_out, es, al, fuse, st);
 }
 
 }  // namespace cp
