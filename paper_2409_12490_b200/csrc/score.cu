@@ -13,8 +13,12 @@
 namespace cp {
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
+// Threads per CTA.  A CTA's phases (products on the fp64 tensor cores, log-sum-exps, combination) use different units one after
+// another; with 256 threads two CTAs share an SM and work in different phases (the registers of 512 allow one).  With no more CTAs than
+// SMs a CTA has its SM to itself anyway and is faster with 512.
+// One CTA of 512 threads / two of 256 per SM, us, in graphs, 32 / 8 heads, segment 512: 16384 tokens, block 32 (256 CTAs) 35.9 / 33.6, block 64 23.4 /
+// 19.4; 32768 tokens, block 64, fused (512 CTAs) 77.0 / 70.0.
+constexpr int kThreadsFew = 512, kThreadsMany = 256;
 
 // Shared memory: logits lg[U][4][nb] (fp64) for the nb key blocks this CTA owns, plus an fp32 copy that
 // the log-sum-exp uses as a filter.  When the 4*U*n2 logits of a row group do not fit one CTA's shared
@@ -29,10 +33,11 @@ template <typename T> struct ScoreSeq {
 };
 template <typename T, int NS> struct ScoreArgs { ScoreSeq<T> s[NS]; int n; };
 
-template <typename T, int D, int U, int NS>
-__global__ void __launch_bounds__(kThreads)
+template <typename T, int D, int U, int NS, int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreadsFew / kThreads)
 score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg, int blk, double est_scale, double ln_alpha,
              double ln_1m_alpha, int fuse, int mask_first, int CL, double* stats_out) {
+  constexpr int kWarps = kThreads / 32;
   extern __shared__ double smem[];
   int si = 0;
   while (NS > 1 && si + 1 < a.n && int(blockIdx.x) >= a.s[si + 1].cta_begin) ++si;
@@ -66,9 +71,6 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
 
   // blocks that start at or after the end of the segment are masked (line 13)
   const int visible = min(n2, ((j + 1) * seg + blk - 1) / blk);
-  __shared__ double sp_tab[kSpIntervals * kSpStride];
-  for (int e = threadIdx.x; e < kSpIntervals * kSpCoef; e += kThreads)
-    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
   pdl_trigger();
   pdl_wait(Qmax, Qmin, Kmax, Kmin, S_prev);
   const T* kmx_base = Kmax + size_t(kvh) * n2 * D;
@@ -86,7 +88,9 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
   constexpr int NCH = KS / CE;              // loads per slice
   constexpr int SPC = CE / 4;               // MMA k-steps per load
   constexpr int QS = D + 2;                 // row stride of qs in doubles (odd number of 16-byte units: conflict-free)
-  __shared__ __align__(16) double qs[8 * QS];   // B operand, row = column index n, laid out [k-step][tig][4 channels]
+  static_assert(8 * QS <= kSpIntervals * kSpStride, "the B operand fits where the table goes");
+  __shared__ __align__(16) double sp_tab[kSpIntervals * kSpStride];   // read by the combination; until the products are done its place holds
+  double* qs = sp_tab;                      // the B operand, row = column index n, laid out [k-step][tig][4 channels]
   const int tig = lane & 3, grp = lane >> 2;
   if (fuse && (lane & 15) == 0) {
     // the previous layer's scores of this CTA's elements are read once, at the very end: start them towards L2 now
@@ -178,6 +182,8 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
     }
   }
   __syncthreads();
+  for (int e = threadIdx.x; e < kSpIntervals * kSpCoef; e += kThreads)
+    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
 
   // log-sum-exp of each of the 4U logit rows (softmax over blocks, lines 9-10): a warp owns a row, so only
   // shuffles are needed.  Terms more than e^-50 below the row maximum cannot change the rounded sum and
@@ -273,12 +279,15 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
   if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until the logits of a row group fit ~200 KB per CTA; 0: they never do
+// Key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until two CTAs fit an SM (104 KB of logits each), or, where 8 do not get
+// there, until one does (200 KB); 0: they never do.
+constexpr size_t kSmemShared = 104 * 1024, kSmemAlone = 200 * 1024;
 int cluster_of(const Dims& m, int U, int* nb) {
-  for (int CL = 1; CL <= 8; CL *= 2) {
-    *nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
-    if ((sizeof(double) + sizeof(float)) * 4 * size_t(U) * *nb <= 200 * 1024) return CL;
-  }
+  for (size_t limit : {kSmemShared, kSmemAlone})
+    for (int CL = 1; CL <= 8; CL *= 2) {
+      *nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
+      if ((sizeof(double) + sizeof(float)) * 4 * size_t(U) * *nb <= limit) return CL;
+    }
   return 0;
 }
 // as many heads per CTA as divide the group (the fp64 MMA has 8 rows = 4 heads x 2 representatives)
@@ -309,26 +318,14 @@ int launch_u(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* 
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   const Dims& m = pr[0].m;
   const size_t smem = (sizeof(double) + sizeof(float)) * (4 * size_t(U) * nb_max);   // fp64 logits + their fp32 copies
-  auto kern = score_kernel<T, D, U, NS>;
+  const bool many = ctas > 148 && smem <= kSmemShared;
+  auto kern = many ? score_kernel<T, D, U, NS, kThreadsMany> : score_kernel<T, D, U, NS, kThreadsFew>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return CP_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(ctas));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = unsigned(CL); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = CL > 1 ? 2 : 1;
   const double al = double(p.alpha);
   const int fuse = (pr[0].S_prev != nullptr && p.alpha != 1.0f) ? 1 : 0, mask_first = (p.flags & CP_FLAG_MASK_BEFORE_SOFTMAX) ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, m.Hq, m.g, m.seg, m.blk, double(p.est_scale), log(al), log1p(-al), fuse,
-                                           mask_first, CL, stats_out);
-  return e == cudaSuccess ? check_launch() : CP_ERR_CUDA;
+  return launch_pdl_cluster(kern, dim3(unsigned(ctas)), many ? kThreadsMany : kThreadsFew, smem, unsigned(CL), st, a, m.Hq, m.g, m.seg, m.blk,
+                            double(p.est_scale), log(al), log1p(-al), fuse, mask_first, CL, stats_out);
 }
 
 template <typename T, int D, int NS>
