@@ -98,7 +98,7 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
   uint16_t* queues = reinterpret_cast<uint16_t*>(masks + kLists * n_words);   // [kWarps][kQueue]
   float* mref = reinterpret_cast<float*>(queues + kWarps * kQueue);     // [kRows][2]
   float* ql1 = mref + kRows * 2;                                        // [kRows]
-  double* exact_sum = reinterpret_cast<double*>(ql1 + kRows);           // [kRows][2]
+  double* exact_sum = reinterpret_cast<double*>(ql1 + kRows);           // [rows in use][2][parts]: at most kRows * 2
   LseBars* bars = reinterpret_cast<LseBars*>(exact_sum + kRows * 2);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -259,15 +259,28 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
           }
           Mx = fmaxf(m0, m1);
         } else {
+          // own: bit i = element i is flagged.  In a full piece the sign of flagT - x is shifted in, four chains side by side; a
+          // compare, a select and an or per element, with the piece's end looked at for each, took 2.5 times as long.
           uint32_t own = 0;
+          const bool full = n_in >= 32;
+          if (full) {
+            uint32_t part[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-          for (int i = 0; i < 32; ++i) own |= ((i < n_in) && (__uint_as_float(v[i]) * es > flagT)) ? (1u << i) : 0u;
+            for (int i = 7; i >= 0; --i)
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                part[q] = __funnelshift_l(__float_as_uint(fmaf(-__uint_as_float(v[8 * q + i]), es, flagT)), part[q], 1);
+            own = part[0] | part[1] << 8 | part[2] << 16 | part[3] << 24;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) own |= ((i < n_in) && (__uint_as_float(v[i]) * es > flagT)) ? (1u << i) : 0u;
+          }
           if (!my_valid) own = 0;
           uint32_t gm = own;                                  // OR over the 8 rows of the column group
           gm |= __shfl_xor_sync(0xffffffffu, gm, 1);
           gm |= __shfl_xor_sync(0xffffffffu, gm, 2);
           gm |= __shfl_xor_sync(0xffffffffu, gm, 4);
-          const uint32_t add = ~gm & (n_in >= 32 ? 0xffffffffu : (n_in <= 0 ? 0u : ((1u << n_in) - 1u)));
+          const uint32_t add = ~gm & (full ? 0xffffffffu : (n_in <= 0 ? 0u : ((1u << n_in) - 1u)));
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
           for (int i = 0; i < 32; i += 2) {
@@ -306,19 +319,27 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
 #endif
 
   // ---------------- exact pass over the flagged blocks: list l = (column group, Kmax | Kmin)
+  // A list is summed by one warp in a fixed order.  With at most 64 (32) rows in the CTA there are 16 (8) lists for 12 warps: each is then cut
+  // into 2 (4) parts of its blocks with sums of their own, added up in order at the end.  With all 32 lists cutting them costs more in B-operand
+  // set-up than it balances (127 K / 144 K cycles).  Both score kernels, us, whole lists / parts: 8 / 8 heads, segment 128, block 32, 16384 tokens
+  // 76.9 / 66.8; 32 / 8 heads, segment 512, block 32, 32768 tokens 104.8 / 99.6; segment 1024, block 128, 131072 tokens 152.5 / 147.5.
+  const int n_lists = 2 * min(kLists / 2, a.U * ((a.segs_per_cta + 3) / 4));
+  const int parts = n_lists > 16 ? 1 : (n_lists > 8 ? 2 : 4);
   if (!aborted) {
     const int grp = lane >> 2, tig = lane & 3;
     uint16_t* queue = queues + warp * kQueue;
     double* qs = reinterpret_cast<double*>(sm + kSmemKV) + warp * 8 * kQS;   // this warp's B operand, in the idle K ring
     const double es_d = double(a.es);
+    const int part_words = (n_tiles * 4 + parts - 1) / parts;
     for (;;) {
       // lists differ a lot in length (a few rows near their maximum flag most of the blocks), so they are taken first
-      // come, first served (a fixed round-robin left the slowest warp 25 % behind; halving the lists for a finer grain
-      // costs more in B-operand set-up than it balances)
+      // come, first served (a fixed round-robin left the slowest warp 25 % behind)
       int l = 0;
       if (lane == 0) l = atomicAdd(&bars->next_list, 1);
       l = __shfl_sync(0xffffffffu, l, 0);
-      if (l >= kLists) break;
+      if (l >= n_lists * parts) break;
+      const int part = l % parts;
+      l /= parts;
       const int cg = l >> 1, kr = l & 1;
       if (row_seg(cg * 8) >= a.n1) continue;              // the group's first segment does not exist: nothing flagged
       // B operand: the 8 rows of the group widened to fp64, [row][k-step][lane-in-quad][4 channels]
@@ -389,8 +410,8 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
 
       int qn = 0;
       const uint32_t* lm = masks + l * n_words;
-      const int words = n_tiles * 4;
-      for (int w0i = 0; w0i < words; w0i += 32) {
+      const int words = min(n_tiles * 4, (part + 1) * part_words);
+      for (int w0i = part * part_words; w0i < words; w0i += 32) {
         const int wi = w0i + lane;
         const uint32_t word = wi < words ? lm[wi] : 0u;
         const int c = __popc(word);
@@ -446,7 +467,7 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
         acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
         acc1 += __shfl_xor_sync(0xffffffffu, acc1, o);
       }
-      if (grp == 0) { exact_sum[mc * 2 + kr] = acc0; exact_sum[(mc + 1) * 2 + kr] = acc1; }
+      if (grp == 0) { exact_sum[(mc * 2 + kr) * parts + part] = acc0; exact_sum[((mc + 1) * 2 + kr) * parts + part] = acc1; }
     }
   }
   __syncthreads();
@@ -458,7 +479,8 @@ lse_sm100_kernel(const __grid_constant__ CUtensorMap tmKmax, const __grid_consta
 #endif
   if (!aborted && my_valid) {
     // row my_row = (segment, representative rep = my_row % 2): Qmax rows give l1 (Kmax) and l2 (Kmin), Qmin rows l3 and l4
-    const double tot = double(asum) + exact_sum[my_row * 2 + my_kr];
+    double tot = double(asum);
+    for (int i = 0; i < parts; ++i) tot += exact_sum[(my_row * 2 + my_kr) * parts + i];
     a.stats[row_unit(my_row) * 4 + (my_row & 1) * 2 + my_kr] = double(Mx) + log(tot);
   }
   if (aborted) {
