@@ -71,6 +71,11 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
 
   // blocks that start at or after the end of the segment are masked (line 13)
   const int visible = min(n2, ((j + 1) * seg + blk - 1) / blk);
+  // the table of ln(1 + e^-x), read while the predecessor ends; it goes to shared memory when the products are done (see sp_tab)
+  constexpr int kTabPer = (kSpIntervals * kSpCoef + kThreads - 1) / kThreads;
+  double tab[kTabPer];
+#pragma unroll
+  for (int i = 0; i < kTabPer; ++i) tab[i] = kSoftplusTable[min(int(threadIdx.x) + i * kThreads, kSpIntervals * kSpCoef - 1)];
   pdl_trigger();
   pdl_wait(Qmax, Qmin, Kmax, Kmin, S_prev);
   const T* kmx_base = Kmax + size_t(kvh) * n2 * D;
@@ -182,8 +187,11 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kSpIntervals * kSpCoef; e += kThreads)
-    sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = kSoftplusTable[e];
+#pragma unroll
+  for (int i = 0; i < kTabPer; ++i) {
+    const int e = threadIdx.x + i * kThreads;
+    if (e < kSpIntervals * kSpCoef) sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = tab[i];
+  }
 
   // log-sum-exp of each of the 4U logit rows (softmax over blocks, lines 9-10): a warp owns a row, so only
   // shuffles are needed.  Terms more than e^-50 below the row maximum cannot change the rounded sum and
