@@ -163,19 +163,32 @@ class Problem:
         n, d = self.seq_len, self.head_dim
         return heads * n * d, n * d, d
 
+    # A few records are kept, by the strides they were made for: building one took 2.5 us of Python in each call, a quarter of what a
+    # decoding call's two launches cost the host.  Setting any field drops them.
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        self.__dict__["_records"] = {}
+
     def params(self, Q=None, K=None, V=None, O=None) -> CpParams:
+        strides = (Q if Q is None else _strides(Q), K if K is None else _strides(K), V if V is None else _strides(V), O if O is None else _strides(O))
+        records = self.__dict__.get("_records", {})
+        record = records.get(strides)
+        if record is not None:
+            return CpParams.from_buffer_copy(record)
         q, k = self._contig(self.n_q_heads), self._contig(self.n_kv_heads)
         values = (
             self.batch, self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim, self.segment_size, self.block_size,
             self.budget_blocks, _DTYPES[self.dtype], self.flags,
-            *(_strides(Q) if Q is not None else q), *(_strides(K) if K is not None else k),
-            *(_strides(V) if V is not None else k), *(_strides(O) if O is not None else q),
+            *(strides[0] or q), *(strides[1] or k), *(strides[2] or k), *(strides[3] or q),
             self.est_scale, self.sm_scale if self.sm_scale is not None else 1.0 / math.sqrt(self.head_dim), self.alpha,
             (self.n_sink | (self.n_local << 16)) & 0xffffffff)
         try:
-            return CpParams.from_buffer_copy(_PARAMS.pack(*values))
+            record = _PARAMS.pack(*values)
         except (struct.error, OverflowError):   # a number that its C type does not hold: converted as C does, for the library to judge
             return CpParams(*values[:10], *(values[i:i + 3] for i in (10, 13, 16, 19)), *values[22:])
+        if len(records) < 8:
+            records[strides] = record
+        return CpParams.from_buffer_copy(record)
 
 
 def workspace_bytes(prob: Problem) -> int:
