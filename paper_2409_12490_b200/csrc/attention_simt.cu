@@ -45,19 +45,6 @@ __device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// The list contract: at most k entries, ascending, unique, each a block that segment j can see.
-__device__ __forceinline__ bool list_ok(const int32_t* list, int c, int j, int r_full, int n2, int k, int lane) {
-  const int vis = min(n2, (j + 1) * r_full);
-  bool ok = (c >= 0) && (c <= k);
-  if (ok) {
-    for (int i = lane; i < c; i += 32) {
-      const int v = list[i];
-      ok = ok && (v >= 0) && (v < vis) && (i == 0 || list[i - 1] < v);
-    }
-  }
-  return __all_sync(0xffffffffu, ok);
-}
-
 template <typename T>
 struct SimtArgs {
   const T *Q, *K, *V;
@@ -170,31 +157,28 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
   if (t0 >= t_end) return;
   const int n1 = (a.n + a.seg - 1) / a.seg, n2 = (a.n + a.blk - 1) / a.blk;
 
+  // Everything the first tile needs is asked for at once: the list and its length, the tokens of the tile's keys, the rows of Q.  One after
+  // the other -- length, list, rows, tokens -- it was three to four round trips: whole layer, 1024 tokens x 4 heads x 64 channels, fp32, caches
+  // cold, 30.9 us, now 29.6 (a third of the attention's 16.5 us is such latency).
   const int32_t* list = nullptr;
   int cnt = 0, n_keys = t_end;                                      // positions of the key sequence the CTA walks
   if (!a.dense) {
     const long long u = (long long)bh * n1 + j;
     list = idx + u * a.k;
     cnt = a.cnt[u];
-    if (warp == 0) {
-      const bool ok = list_ok(list, cnt, j, a.r, n2, a.k, lane);
-      int c = 0;
-      if (ok)
-        for (int i = lane; i < cnt; i += 32) c += list[i] * a.blk < t_end;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-      // the list is ascending: later blocks are seen by no row, and of the last one only the keys up to the last row
-      if (lane == 0) { list_state[0] = ok; list_state[1] = c > 0 ? (c - 1) * a.blk + min(a.blk, t_end - list[c - 1] * a.blk) : 0; }
-    }
-    __syncthreads();
-    if (!list_state[0]) {
-      if (threadIdx.x == 0 && t0 == j * a.seg) report(a.st, CP_ERR_BOUNDS, 100, b, h, j, cnt);
-      return;
-    }
-    n_keys = list_state[1];
   }
-  for (int i = threadIdx.x; i < kBM; i += kThreads * NG) redo[i] = 0;
-
+  // token of a position, 0x7fffffff: none.  An entry that is no block of the sequence is not followed, whatever the list turns out to be.
+  auto token_at = [&](int pos) {
+    if (a.dense) return pos < t_end ? pos : 0x7fffffff;
+    const int e = pos / a.blk;
+    const int entry = e < a.k ? __ldg(list + e) : -1;
+    if (e >= cnt || uint32_t(entry) >= uint32_t(n2)) return 0x7fffffff;
+    const int tok = entry * a.blk + pos % a.blk;
+    return tok < t_end ? tok : 0x7fffffff;
+  };
+  auto make_tokens = [&](int tile_i) {                               // threads 0..63
+    if (tid < kBN) tok_sh[(tile_i / NG) & 1][tid] = token_at(tile_i * kBN + tid);
+  };
   // Q rows, widened to fp32
   const T* qg = a.Q + b * a.qs[0] + h * a.qs[1];
   for (int e = threadIdx.x; e < kBM * (D / 4); e += kThreads * NG) {
@@ -203,21 +187,38 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
     if (t0 + row < t_end) v = ld4(qg + int64_t(t0 + row) * a.qs[2] + c4 * 4);
     *reinterpret_cast<float4*>(qs + row * kQS + c4 * 4) = v;
   }
+  make_tokens(grp);
+  for (int i = threadIdx.x; i < kBM; i += kThreads * NG) redo[i] = 0;
+  if (!a.dense) {
+    if (warp == 0) {
+      bool ok = cnt >= 0 && cnt <= a.k;
+      const int vis = min(n2, (j + 1) * a.r);
+      int end = 0;                                                  // positions up to the last key that a row can see
+      for (int i = lane; i < a.k; i += 32) {
+        const int v = list[i], before = i > 0 ? list[i - 1] : -1;
+        if (i < cnt) {
+          ok = ok && v >= 0 && v < vis && before < v;
+          if (v * a.blk < t_end) end = max(end, i * a.blk + min(a.blk, t_end - v * a.blk));
+        }
+      }
+      ok = __all_sync(0xffffffffu, ok);
+      // the list is ascending: later blocks are seen by no row, and of the last one only the keys up to the last row
+      end = __reduce_max_sync(0xffffffffu, end);
+      if (lane == 0) { list_state[0] = ok; list_state[1] = end; }
+    }
+    __syncthreads();
+    if (!list_state[0]) {
+      if (threadIdx.x == 0 && t0 == j * a.seg) report(a.st, CP_ERR_BOUNDS, 100, b, h, j, cnt);
+      return;
+    }
+    n_keys = list_state[1];
+  } else {
+    __syncthreads();
+  }
 
   const T* kg = a.K + b * a.ks[0] + (h / a.g) * a.ks[1];
   const T* vg = a.V + b * a.vs[0] + (h / a.g) * a.vs[1];
   const int n_tiles = (n_keys + kBN - 1) / kBN;
-  auto make_tokens = [&](int tile_i) {                               // threads 0..63
-    if (tid < kBN) {
-      const int pos = tile_i * kBN + tid;
-      int tok = 0x7fffffff;
-      if (pos < n_keys) {
-        tok = a.dense ? pos : __ldg(list + pos / a.blk) * a.blk + pos % a.blk;
-        if (tok >= t_end) tok = 0x7fffffff;
-      }
-      tok_sh[(tile_i / NG) & 1][tid] = tok;
-    }
-  };
   constexpr int VPR = D * int(sizeof(T)) / 16;                        // 16-byte vectors per row
   auto load_tile = [&](const T* base, int64_t stride, T* dst, int tile_i) {
     for (int e = tid; e < kBN * VPR; e += kThreads) {
@@ -236,8 +237,6 @@ attention_simt_kernel(const __grid_constant__ SimtArgs<T> a) {
 #pragma unroll
     for (int c = 0; c < D / 16; ++c) o[i][c] = 0.f;
   }
-  if (grp < n_tiles) make_tokens(grp);
-  __syncthreads();
   if (grp < n_tiles) load_tile(kg, a.ks[2], kt, grp);
   for (int it = grp; it < n_tiles; it += NG) {
     load_tile(vg, a.vs[2], vt, it);                                   // lands under Q K^T
