@@ -71,11 +71,22 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
 
   // blocks that start at or after the end of the segment are masked (line 13)
   const int visible = min(n2, ((j + 1) * seg + blk - 1) / blk);
-  // the table of ln(1 + e^-x), read while the predecessor ends; it goes to shared memory when the products are done (see sp_tab)
+  // The table of ln(1 + e^-x) goes to shared memory while the predecessor ends.  Where two CTAs share an SM there is no room for it beside the B
+  // operand: it is read here, and goes to the operand's place when the products are done.
+  constexpr bool kShared = kThreads == kThreadsMany;
   constexpr int kTabPer = (kSpIntervals * kSpCoef + kThreads - 1) / kThreads;
+  __shared__ __align__(16) double sp_tab[kSpIntervals * kSpStride];
   double tab[kTabPer];
+  auto put_table = [&] {
+#pragma unroll
+    for (int i = 0; i < kTabPer; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      if (e < kSpIntervals * kSpCoef) sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = tab[i];
+    }
+  };
 #pragma unroll
   for (int i = 0; i < kTabPer; ++i) tab[i] = kSoftplusTable[min(int(threadIdx.x) + i * kThreads, kSpIntervals * kSpCoef - 1)];
+  if constexpr (!kShared) put_table();
   pdl_trigger();
   pdl_wait(Qmax, Qmin, Kmax, Kmin, S_prev);
   const T* kmx_base = Kmax + size_t(kvh) * n2 * D;
@@ -94,8 +105,8 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
   constexpr int SPC = CE / 4;               // MMA k-steps per load
   constexpr int QS = D + 2;                 // row stride of qs in doubles (odd number of 16-byte units: conflict-free)
   static_assert(8 * QS <= kSpIntervals * kSpStride, "the B operand fits where the table goes");
-  __shared__ __align__(16) double sp_tab[kSpIntervals * kSpStride];   // read by the combination; until the products are done its place holds
-  double* qs = sp_tab;                      // the B operand, row = column index n, laid out [k-step][tig][4 channels]
+  __shared__ __align__(16) double qs_own[kShared ? 1 : 8 * QS];
+  double* qs = kShared ? sp_tab : qs_own;   // B operand, row = column index n, laid out [k-step][tig][4 channels]
   const int tig = lane & 3, grp = lane >> 2;
   if (fuse && (lane & 15) == 0) {
     // the previous layer's scores of this CTA's elements are read once, at the very end: start them towards L2 now
@@ -187,11 +198,7 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < kTabPer; ++i) {
-    const int e = threadIdx.x + i * kThreads;
-    if (e < kSpIntervals * kSpCoef) sp_tab[(e / kSpCoef) * kSpStride + e % kSpCoef] = tab[i];
-  }
+  if constexpr (kShared) put_table();
 
   // log-sum-exp of each of the 4U logit rows (softmax over blocks, lines 9-10): a warp owns a row, so only
   // shuffles are needed.  Terms more than e^-50 below the row maximum cannot change the rounded sum and
