@@ -28,7 +28,8 @@
 // takes 10 to 13 thousand cycles, with 8 epilogue warps 14 thousand (latency).  Half tiles with accumulators of their own, so that half of the
 // warps combine while the others convert: slower (N = 32: 5 KB per MMA of half the work; 131072 tokens 665 -> 780 us).
 // Both kernels of the scores, this one with fp64 MMAs (m16n8k16, 8 to 12 warps each on its own tiles) -> now, us, in graphs, 32 / 8 heads:
-// 131072 tokens, segment 512, block 32, fused 982 -> 665; segment 1024, block 128 184 -> 153; 65536 tokens, segment 512, block 64 166 -> 161.
+// 131072 tokens, segment 512, block 32, fused 982 -> 665 (641 with lse_sm100.cu as it is now); segment 1024, block 128 184 -> 153 (147.5);
+// 65536 tokens, segment 512, block 64 166 -> 161 (156).
 #include "sm100_ptx.cuh"
 
 namespace cp {
@@ -651,9 +652,9 @@ int launch_visible(const Dims& m, char* ws, const double* S_prev, double* S_out,
 
 // From which size on the two-kernel path is used.  What counts is the general kernel's work: its MMAs have 8 columns, the Qmax and
 // Qmin rows of up to 4 heads of a group, of which groups of 2 heads fill half and single heads a quarter.
-// General kernel / two kernels, us, 32 / 8 heads: segment 512, block 32, 16384 tokens (0.5 M scores) 36 / 68; block 64, 32768 tokens
-// (1.05 M, fused) 77 / 78; segment 1024, block 128, 65536 tokens (1.05 M) 70 / 74; block 32, 32768 tokens (2.1 M) 122 / 105; 8 / 8 heads, segment
-// 128, block 32, 16384 tokens (0.5 M, counted as 2.1 M) 103 / 75.
+// General kernel / two kernels, us, 32 / 8 heads: segment 512, block 32, 16384 tokens (0.5 M scores) 34 / 65; block 64, 32768 tokens
+// (1.05 M, fused) 70 / 75; segment 1024, block 128, 65536 tokens (1.05 M) 63 / 72; the general kernel with one CTA per SM: block 32, 32768 tokens
+// (2.1 M) 122 / 100; 8 / 8 heads, segment 128, block 32, 16384 tokens (0.5 M, counted as 2.1 M) 103 / 67.
 bool score_is_split(const cp_params& p, const Dims& m) {
   const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2 * (m.g % 4 == 0 ? 1 : (m.g % 2 == 0 ? 2 : 4));
   return (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 &&
