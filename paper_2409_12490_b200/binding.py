@@ -159,36 +159,39 @@ class Problem:
     def n2(self):
         return -(-self.seq_len // self.block_size)
 
-    def _contig(self, heads):
-        n, d = self.seq_len, self.head_dim
-        return heads * n * d, n * d, d
-
-    # A few records are kept, by the strides they were made for: building one took 2.5 us of Python in each call, a quarter of what a
-    # decoding call's two launches cost the host.  Setting any field drops them.
-    def __setattr__(self, name, value):
-        object.__setattr__(self, name, value)
-        self.__dict__["_records"] = {}
-
+    # Written out flat: a decoding call's two launches cost the host some 17 us, of which building its two records was 3.4 us with a tuple
+    # and a helper call per tensor and is 2.5 us now.  Nothing is kept for the next call: records kept per object took 1.4 us where
+    # nothing had changed, but 5.1 us where the length had and 9.3 us on a new object (a cache that grows by a token per step).
     def params(self, Q=None, K=None, V=None, O=None) -> CpParams:
-        strides = (Q if Q is None else _strides(Q), K if K is None else _strides(K), V if V is None else _strides(V), O if O is None else _strides(O))
-        records = self.__dict__.get("_records", {})
-        record = records.get(strides)
-        if record is not None:
-            return CpParams.from_buffer_copy(record)
-        q, k = self._contig(self.n_q_heads), self._contig(self.n_kv_heads)
-        values = (
-            self.batch, self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim, self.segment_size, self.block_size,
-            self.budget_blocks, _DTYPES[self.dtype], self.flags,
-            *(strides[0] or q), *(strides[1] or k), *(strides[2] or k), *(strides[3] or q),
-            self.est_scale, self.sm_scale if self.sm_scale is not None else 1.0 / math.sqrt(self.head_dim), self.alpha,
-            (self.n_sink | (self.n_local << 16)) & 0xffffffff)
+        q_heads, kv_heads, n, d = self.n_q_heads, self.n_kv_heads, self.seq_len, self.head_dim
+        head = n * d
+        q_all, kv_all = q_heads * head, kv_heads * head
+        if Q is None:
+            q0, q1, q2 = q_all, head, d
+        else:
+            q0, q1, q2 = _strides(Q)
+        if K is None:
+            k0, k1, k2 = kv_all, head, d
+        else:
+            k0, k1, k2 = _strides(K)
+        if V is None:
+            v0, v1, v2 = kv_all, head, d
+        else:
+            v0, v1, v2 = _strides(V)
+        if O is None:
+            o0, o1, o2 = q_all, head, d
+        else:
+            o0, o1, o2 = _strides(O)
+        sm_scale = 1.0 / math.sqrt(d) if self.sm_scale is None else self.sm_scale
+        forced = (self.n_sink | (self.n_local << 16)) & 0xffffffff
         try:
-            record = _PARAMS.pack(*values)
+            return CpParams.from_buffer_copy(_PARAMS.pack(
+                self.batch, q_heads, kv_heads, n, d, self.segment_size, self.block_size, self.budget_blocks, _DTYPES[self.dtype], self.flags,
+                q0, q1, q2, k0, k1, k2, v0, v1, v2, o0, o1, o2, self.est_scale, sm_scale, self.alpha, forced))
         except (struct.error, OverflowError):   # a number that its C type does not hold: converted as C does, for the library to judge
-            return CpParams(*values[:10], *(values[i:i + 3] for i in (10, 13, 16, 19)), *values[22:])
-        if len(records) < 8:
-            records[strides] = record
-        return CpParams.from_buffer_copy(record)
+            return CpParams(
+                self.batch, q_heads, kv_heads, n, d, self.segment_size, self.block_size, self.budget_blocks, _DTYPES[self.dtype], self.flags,
+                (q0, q1, q2), (k0, k1, k2), (v0, v1, v2), (o0, o1, o2), self.est_scale, sm_scale, self.alpha, forced)
 
 
 def workspace_bytes(prob: Problem) -> int:

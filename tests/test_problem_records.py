@@ -1,4 +1,4 @@
-"""The records that Problem.params keeps: the same bytes as a fresh Problem gives, whatever was set, copied or passed before."""
+"""The records that Problem.params makes: the same bytes as a fresh Problem gives, whatever was set, copied or passed before."""
 import copy
 import dataclasses
 import pickle
@@ -34,3 +34,14 @@ def test_strides_and_records_are_the_callers_own():
         rec.k_stride[1] = 7                                # a copy: the next call does not see it
         assert tuple(p.params(K=K).k_stride) == K.stride()[:3]
     assert bytes(p.params()) == plain
+
+
+def test_nothing_but_the_fields():
+    p = cp.Problem(*ARGS)
+    p.params()
+    assert set(vars(p)) == {f.name for f in dataclasses.fields(p)}
+    assert cp.Problem(**vars(p)) == p
+    vars(p).update(seq_len=290, alpha=0.5)                 # fields set behind the object's back
+    assert bytes(p.params()) == bytes(cp.Problem(1, 8, 2, 290, 64, 64, 16, 8, alpha=0.5).params())
+    # making an object and setting a field run no code of the class: a decoding step does both per token
+    assert cp.Problem.__setattr__ is object.__setattr__
