@@ -12,7 +12,11 @@
 // tcgen05.mma.kind::i8 forms without any rounding; those of equal weight (i + j) share one of 7 accumulators of 32 bits (at most
 // 2^23).  Put together in 64-bit integers and rounded once to fp64 they give the dot product correctly rounded, which a chain of 128
 // fp64 additions does not.  Rows and blocks that do not fit (tiny values beside large ones, infinities, NaN) are marked, and their
-// logits are summed in fp64 by the threads that own them.
+// scores follow once more, from fp64 MMAs, at the end of their row group (redo_marked).
+// What marks cost depends on the data.  Both kernels of the scores, us, 131072 tokens, 32 / 8 heads, segment 512, block 32, fused, fp16 with a
+// channel of 80: 1 % of the blocks marked 608, 5 % 642, a third 929, all 1347 (840 with the products of all blocks on the fp64 pipe, whatever the
+// values).  Normal bf16 inputs of that size have one marked row of 16384: 653 against 622 without.  With the marked logits summed by
+// the threads that own them 1237, 1521, 3379, 7293 and 777.
 //
 // One CTA per SM, 128 logit rows (the Qmax / Qmin representatives of 64 / U segments x U heads of a KV group) against tiles
 // of 32 key blocks (64 rows: Kmax, Kmin).  The tiles of all (row group, visible block) pairs are dealt to the CTAs in equal
@@ -47,6 +51,8 @@ constexpr int kStages = 2;                     // tiles of key rows
 constexpr int kInfo = 4;                       // what goes with a tile (scales, marks) outlives its bytes: read until its epilogue ends
 constexpr int kSmemK = kDigits * kQPlane;
 constexpr int kSmemFixed = kSmemK + kStages * kDigits * kKPlane;
+constexpr int kMarks = 512;                    // tiles whose marks are kept: a row group has at most kMaxBlocksN2 / kTileBlocks = 256, the converter is at most 2 ahead
+static_assert(kMaxBlocksN2 / kTileBlocks + kStages <= kMarks, "marks of a row group");
 
 constexpr int kNodes = 40 * 32 + 1;
 static __device__ const double2 kSoftplusNodes[kNodes] = {
@@ -54,8 +60,7 @@ static __device__ const double2 kSoftplusNodes[kNodes] = {
 };
 
 struct Info {
-  double scale[kTileBlocks];                   // 2^(E-30) of a block's bytes; 1 if it is marked
-  uint32_t bad[4];                             // marked blocks, 8 per converting warp
+  double scale[kTileBlocks];                   // 2^(E-30) of a block's bytes
 };
 struct __align__(16) RowInfo {
   double scale[kRows];                         // likewise for the logit rows
@@ -66,12 +71,16 @@ struct Bars {
   double2 nodes[kNodes];                       // ln(1 + e^-x) and its derivative at the multiples of 1/32
   Info info[kInfo];
   RowInfo rows[2];                             // by parity of the CTA's row groups
-  unsigned long long q_full, k_full[kStages], k_empty[kStages], info_full[kInfo], acc_full, acc_empty;
+  uint32_t marks[kMarks];                      // marked blocks of a tile, by the CTA's tiles
+  uint16_t redo_blocks[kMaxBlocksN2];          // of a row group that has marks: its marked blocks, from its first on
+  uint8_t redo_pairs[kRows / 2];               // and its marked (Qmax, Qmin) pairs of rows
+  unsigned long long q_full, k_full[kStages], k_empty[kStages], info_full[kInfo], acc_full, acc_empty, redo;
   uint32_t tmem_base;
   volatile int abort_flag;
 };
 constexpr int kEpilogueRegs = 96, kOtherRegs = 48, kRegPoolNeeded = kEpilogueWarps * 32 * kEpilogueRegs + 256 * kOtherRegs;
 constexpr int kSmemTotal = kSmemFixed + int(sizeof(Bars)) + 1024;
+static_assert(kSmemTotal <= 227 * 1024, "shared memory of an SM");
 
 struct ScoreExactArgs {
   const void *Qmax, *Qmin, *Kmax, *Kmin;       // representatives in the workspace
@@ -84,9 +93,6 @@ struct ScoreExactArgs {
   int tiles_per_combo, n_tiles;
   double est_scale, ln_alpha, ln_1m_alpha;
 };
-
-template <bool kF16> struct Elem { using type = __nv_bfloat16; };
-template <> struct Elem<true> { using type = __half; };
 
 // d s32, a and b s8, K-major; M = 128, N = 64
 constexpr uint32_t kIdesc = (2u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kTileN >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
@@ -126,8 +132,6 @@ __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + 
 template <bool kF16>
 __device__ __forceinline__ bool to_digits(const uint4& v, int e, uint2 (&out)[kDigits]) {
   const float mul = e == kMarked ? 0.f : __uint_as_float(uint32_t(127 + 30 - e) << 23);
-  // smallest magnitude whose last bit (2^-7 or 2^-10 of its leading one) is still at least 1; an fp16 is a multiple of 2^-24
-  const float least = kF16 ? (e <= 6 ? 0.f : 1024.f) : 128.f;
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
   uint32_t dg[8];
   bool bad = e == kMarked;
@@ -135,10 +139,11 @@ __device__ __forceinline__ bool to_digits(const uint4& v, int e, uint2 (&out)[kD
   for (int i = 0; i < 4; ++i) {
     const float2 f = unpack2<kF16>(w[i]);
     const float x = f.x * mul, y = f.y * mul;
-    bad |= !(fabsf(x) >= least || x == 0.f) || !(fabsf(y) >= least || y == 0.f);
+    const int ix = __float2int_rz(x), iy = __float2int_rz(y);
+    bad |= float(ix) != x || float(iy) != y;
     // signed bytes: adding 0x80 to each but the top one carries, the exclusive or takes it off again
-    dg[2 * i] = (uint32_t(__float2int_rz(x)) + 0x00808080u) ^ 0x00808080u;
-    dg[2 * i + 1] = (uint32_t(__float2int_rz(y)) + 0x00808080u) ^ 0x00808080u;
+    dg[2 * i] = (uint32_t(ix) + 0x00808080u) ^ 0x00808080u;
+    dg[2 * i + 1] = (uint32_t(iy) + 0x00808080u) ^ 0x00808080u;
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {                // 4 x 4 bytes transposed: digit p of four elements
@@ -168,23 +173,28 @@ __device__ __forceinline__ float absmax8(const uint4& v) {
 // 8-byte piece `c` (channels 8 c to 8 c + 7) of row `row` in a 128-byte-swizzled plane of 128-byte rows
 __device__ __forceinline__ uint32_t digit_at(int row, int c) { return row * kD + (((c >> 1) ^ (row & 7)) << 4) + (c & 1) * 8; }
 
-// Part of a logit of a marked row or block, in fp64: `pieces` of 8 channels.  In line and rolled up: a call would cost the code around
-// it registers.
+// fp64 products of 16 rows with 8 (A and B rows of 128 channels; lane (grp, tig) = (lane / 4, lane % 4) gives A rows grp and grp + 8 and B row grp).
+// c: (A row grp, B rows 2 tig, 2 tig + 1), then the same of A row grp + 8.  The order of the channels inside a product is free: a lane takes
+// 8 consecutive ones for two MMAs.
 template <bool kF16>
-__device__ __forceinline__ double slow_logit(const uint4* q, const uint4* k, int pieces) {
-  double x = 0.0, y = 0.0;
-#pragma unroll 1
-  for (int c = 0; c < pieces; ++c) {
-    const uint4 a = q[c], b = k[c];
-    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+__device__ __forceinline__ void exact_16x8(const uint4* a0, const uint4* a1, const uint4* b, int tig, double (&c)[4]) {
+  uint4 v0[4], v1[4], vb[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 af = unpack2<kF16>(aw[e]), bf = unpack2<kF16>(bw[e]);
-      x = fma(double(af.x), double(bf.x), x);
-      y = fma(double(af.y), double(bf.y), y);
-    }
+  for (int i = 0; i < 4; ++i) { v0[i] = a0[i * 4 + tig]; v1[i] = a1[i * 4 + tig]; vb[i] = b[i * 4 + tig]; }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) c[i] = 0.0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 &x = v0[i >> 1], &y = v1[i >> 1], &z = vb[i >> 1];
+    const float2 x0 = unpack2<kF16>(i & 1 ? x.z : x.x), x1 = unpack2<kF16>(i & 1 ? x.w : x.y);
+    const float2 y0 = unpack2<kF16>(i & 1 ? y.z : y.x), y1 = unpack2<kF16>(i & 1 ? y.w : y.y);
+    const float2 z0 = unpack2<kF16>(i & 1 ? z.z : z.x), z1 = unpack2<kF16>(i & 1 ? z.w : z.y);
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, {%4,%5,%6,%7,%8,%9,%10,%11}, {%12,%13,%14,%15}, {%0,%1,%2,%3};"
+        : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+        : "d"(double(x0.x)), "d"(double(y0.x)), "d"(double(x0.y)), "d"(double(y0.y)), "d"(double(x1.x)), "d"(double(y1.x)), "d"(double(x1.y)),
+          "d"(double(y1.y)), "d"(double(z0.x)), "d"(double(z0.y)), "d"(double(z1.x)), "d"(double(z1.y)));
   }
-  return x + y;
 }
 
 // ln(1 + e^-x), x >= 0, for N independent values: Taylor series around the nearest node, whose coefficients are polynomials in the
@@ -235,6 +245,35 @@ __device__ __noinline__ double combine_any(const double2* nodes, double L1, doub
   return y;
 }
 
+// max( ln (S1+S3), ln (S2+S4) ) of N scores with finite logits
+template <int N>
+__device__ __forceinline__ void combine_n(const double2* nodes, const double (&L1)[N], const double (&L2)[N], const double (&L3)[N], const double (&L4)[N],
+                                          double (&out)[N]) {
+  double hi[2 * N], d[2 * N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    d[i] = L1[i] - L3[i]; d[N + i] = L2[i] - L4[i];
+    hi[i] = __double2hiint(d[i]) >= 0 ? L1[i] : L3[i]; hi[N + i] = __double2hiint(d[N + i]) >= 0 ? L2[i] : L4[i];
+    d[i] = fabs(d[i]); d[N + i] = fabs(d[N + i]);
+  }
+  softplus_nodes(nodes, d);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const double y13 = hi[i] + d[i], y24 = hi[N + i] + d[N + i];
+    out[i] = y13 >= y24 ? y13 : y24;
+  }
+}
+// ln(e^y + e^z) for N scores; fmax and fmin leave a NaN out
+template <int N>
+__device__ __forceinline__ void fuse_n(const double2* nodes, double (&v)[N], const double (&y)[N], const double (&z)[N]) {
+  double d[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) { v[i] = fmax(y[i], z[i]); d[i] = v[i] - fmin(y[i], z[i]); }
+  softplus_nodes(nodes, d);
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] += d[i];
+}
+
 __device__ __forceinline__ void ld4(const double* p, bool vec, int n, double* v) {
   if (vec && n == 4) {
     asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
@@ -275,13 +314,13 @@ __device__ __forceinline__ bool next_piece(const ScoreExactArgs& a, Walk& w) {
 }
 // row m of a row group: column m / 8 = (4 segments, head); within it (segment, representative)
 struct RowGroup { int kvh, b, h0, j0; };
-__device__ __forceinline__ RowGroup row_group(const ScoreExactArgs& a, const Walk& w) {
+__device__ __forceinline__ RowGroup row_group(const ScoreExactArgs& a, int combo, int chunk) {
   const int groups = a.g / a.U, Hkv = a.Hq / a.g;
   RowGroup r;
-  r.kvh = w.combo / groups;
+  r.kvh = combo / groups;
   r.b = r.kvh / Hkv;
-  r.h0 = (r.kvh % Hkv) * a.g + (w.combo % groups) * a.U;
-  r.j0 = w.chunk * a.segs;
+  r.h0 = (r.kvh % Hkv) * a.g + (combo % groups) * a.U;
+  r.j0 = chunk * a.segs;
   return r;
 }
 __device__ __forceinline__ int row_seg(const ScoreExactArgs& a, const RowGroup& r, int m) {
@@ -297,7 +336,7 @@ __device__ __forceinline__ void convert_role(const ScoreExactArgs& a, Bars* bars
   const int c = lane & 15, half = lane >> 4;   // a warp takes 8 blocks: Kmax rows by the lower half warp, Kmin rows by the upper; 8 channels per lane
   uint32_t t = 0;                              // tiles so far
   while (next_piece(a, w)) {
-    const RowGroup r = row_group(a, w);
+    const RowGroup r = row_group(a, w.combo, w.chunk);
     const uint4* src = static_cast<const uint4*>(half ? a.Kmin : a.Kmax) + size_t(r.kvh) * a.n2 * (kD / 8) + c;
     const float* abs_src = a.kabs + size_t(r.kvh) * a.n2;
     for (int x = 0; x < w.n; ++x, ++t) {
@@ -321,20 +360,26 @@ __device__ __forceinline__ void convert_role(const ScoreExactArgs& a, Bars* bars
         for (int i = 0; i < 2; ++i) {
           const int e = exponent_of(ka[i]);
           uint2 dg[kDigits];
-          const bool bad = __ballot_sync(0xffffffffu, to_digits<kF16>(v[i], e, dg)) != 0;
+          const bool bad = __any_sync(0xffffffffu, to_digits<kF16>(v[i], e, dg));
           const int at = warp * 8 + i0 + i;
 #pragma unroll
           for (int p = 0; p < kDigits; ++p) *reinterpret_cast<uint2*>(dst + p * kKPlane + digit_at(half * kTileBlocks + at, c)) = dg[p];
           bad_blocks |= (bad ? 1u : 0u) << (i0 + i);
-          if (lane == 0) info.scale[at] = bad ? 1.0 : pow2(e - 30);
+          if (lane == 0) info.scale[at] = e == kMarked ? 1.0 : pow2(e - 30);
         }
       }
-      if (lane == 0) info.bad[warp] = bad_blocks;
+      if (lane == 0) reinterpret_cast<uint8_t*>(&bars->marks[t % kMarks])[warp] = uint8_t(bad_blocks);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the planes through the async proxy
       mbar_arrive(&bars->info_full[t % kInfo]);
       mbar_arrive(&bars->k_full[stage]);
     }
   }
+}
+
+// all logit rows are marked: like a tile of marked blocks alone, such tiles are left to redo_marked
+__device__ __forceinline__ bool all_marked(const RowInfo& ri) {
+  const uint4 v = *reinterpret_cast<const uint4*>(ri.bad);
+  return (v.x & v.y & v.z & v.w) == ~0u;
 }
 
 // ---------------------------------------------------------------- warp 20
@@ -344,20 +389,23 @@ __device__ __forceinline__ void mma_role(const ScoreExactArgs& a, Bars* bars, ui
   uint32_t t = 0;
   for (uint32_t piece = 0; next_piece(a, w); ++piece) {
     if (!mbar_wait(&bars->q_full, piece & 1, &bars->abort_flag, a.st, 70)) return;
+    const bool all_rows = all_marked(bars->rows[piece & 1]);
     for (int x = 0; x < w.n; ++x, ++t) {
       const uint32_t stage = t % kStages;
       if (!mbar_wait(&bars->k_full[stage], (t / kStages) & 1, &bars->abort_flag, a.st, 72)) return;
       if (t > 0 && !mbar_wait(&bars->acc_empty, (t - 1) & 1, &bars->abort_flag, a.st, 73)) return;
       tc_fence_after();
       const uint32_t k_smem = smem + kSmemK + stage * kDigits * kKPlane;
+      if (!all_rows && bars->marks[t % kMarks] != ~0u) {
 #pragma unroll
-      for (int s = 0; s < kAccs; ++s)
+        for (int s = 0; s < kAccs; ++s)
 #pragma unroll
-        for (int i = s > 3 ? s - 3 : 0; i <= (s < 3 ? s : 3); ++i)
+          for (int i = s > 3 ? s - 3 : 0; i <= (s < 3 ? s : 3); ++i)
 #pragma unroll
-          for (int kk = 0; kk < kD / 32; ++kk)
-            umma_i8(tm + s * kTileN, desc_at(base, smem + i * kQPlane + kk * 32), desc_at(base, k_smem + (s - i) * kKPlane + kk * 32),
-                    i > (s > 3 ? s - 3 : 0) || kk > 0);
+            for (int kk = 0; kk < kD / 32; ++kk)
+              umma_i8(tm + s * kTileN, desc_at(base, smem + i * kQPlane + kk * 32), desc_at(base, k_smem + (s - i) * kKPlane + kk * 32),
+                      i > (s > 3 ? s - 3 : 0) || kk > 0);
+      }
       umma_commit(&bars->acc_full);
       umma_commit(&bars->k_empty[stage]);
     }
@@ -365,15 +413,95 @@ __device__ __forceinline__ void mma_role(const ScoreExactArgs& a, Bars* bars, ui
 }
 
 // ---------------------------------------------------------------- warps 0-15
+// The scores of a row group's marked blocks and of its marked rows once more, from fp64 products; t: the CTA's tiles up to the end of the group.  An MMA tile
+// is 8 blocks (Kmax, Kmin) with 4 pairs of rows (Qmax, Qmin) of a (head, segment): each lane then holds the four logits of a score.  Marked
+// blocks are gathered over the whole group, so that few of them cost little: 8 with 64 pairs take 4100 cycles of the fp64 pipes.  Returns how
+// often the epilogue warps have met here by then.
+constexpr uint32_t kGaveUp = ~0u;
+template <bool kF16>
+__device__ __forceinline__ uint32_t redo_marked(const ScoreExactArgs& a, Bars* bars, int combo, int chunk, int tile, int n_tiles, uint32_t piece, uint32_t t,
+                                             uint32_t redone) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane >> 2, tig = lane & 3;
+  const RowInfo& ri = bars->rows[piece & 1];
+  const uint32_t t0 = t - n_tiles;
+  int n_blocks = 0;                            // marked blocks; bits of the lanes' words first
+  for (int i = lane; i < n_tiles; i += 32) n_blocks += __popc(bars->marks[(t0 + i) % kMarks]);
+  n_blocks = __reduce_add_sync(0xffffffffu, n_blocks);
+  const uint32_t* row_words = reinterpret_cast<const uint32_t*>(ri.bad);
+  auto pair_marked = [&](int p) { return (row_words[p >> 4] >> (2 * (p & 15)) & 3u) != 0; };
+  const uint32_t pairs_lo = __ballot_sync(0xffffffffu, pair_marked(lane)), pairs_hi = __ballot_sync(0xffffffffu, pair_marked(32 + lane));
+  int n_pairs = __popc(pairs_lo) + __popc(pairs_hi);
+  if (n_blocks + n_pairs == 0) return redone;
+  const int first = tile * kTileBlocks, in_group = min(n_tiles * kTileBlocks, a.n2 - first);
+  // all pairs with the marked blocks, then the marked pairs with all blocks; or, where that is no more, all with all
+  const int all_units = (kRows / 8) * ((in_group + 7) / 8);
+  int block_units = (kRows / 8) * ((n_blocks + 7) / 8);
+  const bool whole = block_units + (n_pairs + 3) / 4 * ((in_group + 7) / 8) >= all_units;
+  if (whole) { block_units = 0; n_pairs = kRows / 2; }
+  if (warp == 0) {                             // the lists; nobody reads those of the group before any more: all have passed the wait for q_full
+    int at = 0;
+    for (int i0 = 0; i0 < n_tiles && !whole; i0 += 32) {
+      uint32_t word = i0 + lane < n_tiles ? bars->marks[(t0 + i0 + lane) % kMarks] : 0u;
+      int incl = __popc(word);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+      }
+      int pos = at + incl - __popc(word);
+      for (; word; word &= word - 1) bars->redo_blocks[pos++] = uint16_t((i0 + lane) * kTileBlocks + __ffs(word) - 1);
+      at += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    const uint32_t below = (1u << lane) - 1u;
+    if (whole || (pairs_lo >> lane & 1u)) bars->redo_pairs[whole ? lane : __popc(pairs_lo & below)] = uint8_t(lane);
+    if (whole || (pairs_hi >> lane & 1u)) bars->redo_pairs[whole ? 32 + lane : __popc(pairs_lo) + __popc(pairs_hi & below)] = uint8_t(32 + lane);
+  }
+  // what is stored below overwrites what other threads have stored for these scores
+  mbar_arrive(&bars->redo);
+  if (!mbar_wait(&bars->redo, redone++ & 1, &bars->abort_flag, a.st, 77)) return kGaveUp;
+
+  const RowGroup r = row_group(a, combo, chunk);
+  const int pair_units = (n_pairs + 3) / 4, units = block_units + pair_units * ((in_group + 7) / 8);
+#pragma unroll 1
+  for (int u = warp; u < units; u += kEpilogueWarps) {
+    const bool by_block = u < block_units;
+    const int n_groups = by_block ? kRows / 8 : pair_units, v = by_block ? u : u - block_units;
+    const int pg = v % n_groups * 4, bg = v / n_groups * 8 + grp;           // the unit's first pair; the lane's block
+    auto pair_at = [&](int i) { return by_block ? i : int(bars->redo_pairs[min(i, n_pairs - 1)]); };
+    const int block = first + (by_block ? int(bars->redo_blocks[min(bg, n_blocks - 1)]) : min(bg, in_group - 1));
+    const int mq = 2 * pair_at(pg + (grp >> 1)) + (grp & 1), ms = 2 * pair_at(pg + tig);    // the lane's B row; Qmax row of its score
+    const int j = row_seg(a, r, ms);
+    const bool here = j < a.n1 && (by_block ? bg < n_blocks : bg < in_group && pg + tig < n_pairs), seen = here && block < visible_of(a, j);
+    const size_t key = (size_t(r.kvh) * a.n2 + block) * (kD / 8), at = (here ? row_unit(a, r, ms) : 0) * a.n2 + block;
+    const double sp = a.fuse && seen ? a.S_prev[at] : 0.0;
+    double c[4];
+    exact_16x8<kF16>(static_cast<const uint4*>(a.Kmax) + key, static_cast<const uint4*>(a.Kmin) + key,
+                     static_cast<const uint4*>((mq & 1) ? a.Qmin : a.Qmax) + (row_seg(a, r, mq) < a.n1 ? row_unit(a, r, mq) : 0) * (kD / 8), tig, c);
+    const double L1[1] = {fma(c[0], a.est_scale, -ri.lse[ms][0])}, L2[1] = {fma(c[2], a.est_scale, -ri.lse[ms][1])};
+    const double L3[1] = {fma(c[1], a.est_scale, -ri.lse[ms + 1][0])}, L4[1] = {fma(c[3], a.est_scale, -ri.lse[ms + 1][1])};
+    const bool finite = fabs(L1[0]) < CUDART_INF && fabs(L2[0]) < CUDART_INF && fabs(L3[0]) < CUDART_INF && fabs(L4[0]) < CUDART_INF;
+    double s[1];
+    if (__all_sync(0xffffffffu, finite)) combine_n(bars->nodes, L1, L2, L3, L4, s);
+    else s[0] = combine_any(bars->nodes, L1[0], L2[0], L3[0], L4[0]);
+    s[0] -= 0.693147180559945309417232121458;
+    if (a.fuse) {
+      const double y[1] = {a.ln_alpha + s[0]}, z[1] = {a.ln_1m_alpha + sp};
+      fuse_n(bars->nodes, s, y, z);
+    }
+    if (here) a.S_out[at] = seen ? s[0] : -CUDART_INF;
+  }
+  return redone;
+}
+
 template <bool kF16>
 __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bars, uint8_t* sm, Walk w, int warp, int lane) {
   const int m = (warp & 3) * 32 + lane, hc = warp >> 2;     // logit row; quarter of the tile's blocks
   const uint32_t tm = bars->tmem_base + (uint32_t((warp & 3) * 32) << 16) + hc * 8;
   const bool odd = lane & 1;                                // Qmin rows; the lane takes the upper 4 of its 8 blocks
   const double ln2 = 0.693147180559945309417232121458;
-  uint32_t t = 0;
+  uint32_t t = 0, redone = 0;
   for (uint32_t piece = 0; next_piece(a, w); ++piece) {
-    const RowGroup r = row_group(a, w);
+    const RowGroup r = row_group(a, w.combo, w.chunk);
     RowInfo& ri = bars->rows[piece & 1];
     {
       // The bytes of the row group's query rows, 8 rows per warp, two at a time.  The MMAs on the row group before have all been
@@ -406,7 +534,7 @@ __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bar
           ri.lse[mq][c] = l;
           not_finite |= !(fabs(l) < CUDART_INF);
         }
-        if (c == 0) ri.scale[mq] = (both >> (lane >> 4) & 1u) ? 1.0 : pow2(e - 30);
+        if (c == 0) ri.scale[mq] = e == kMarked ? 1.0 : pow2(e - 30);
       }
       not_finite = __any_sync(0xffffffffu, not_finite);
       if (lane == 0) { ri.bad[(warp & 3) * 4 + hc] = uint8_t(bad_rows); ri.special[(warp & 3) * 4 + hc] = not_finite; }
@@ -419,7 +547,7 @@ __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bar
     const int vis = valid ? visible_of(a, j) : 0;
     const int warp_vis = __reduce_max_sync(0xffffffffu, vis);
     if (!mbar_wait(&bars->q_full, piece & 1, &bars->abort_flag, a.st, 76)) return;
-    const uint32_t bad_rows = *reinterpret_cast<const uint32_t*>(&ri.bad[(warp & 3) * 4]);        // of the warp's rows
+    const bool all_rows = all_marked(ri);
     const bool special = *reinterpret_cast<const uint32_t*>(&ri.special[(warp & 3) * 4]) != 0;
     for (int x = 0; x < w.n; ++x, ++t) {
       const int b_tile = (w.tile + x) * kTileBlocks + hc * 8, b0 = b_tile + (odd ? 4 : 0);
@@ -431,6 +559,11 @@ __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bar
       if (!mbar_wait(&bars->info_full[t % kInfo], (t / kInfo) & 1, &bars->abort_flag, a.st, 74)) return;
       if (!mbar_wait(&bars->acc_full, t & 1, &bars->abort_flag, a.st, 75)) return;
       tc_fence_after();
+      if (all_rows || bars->marks[t % kMarks] == ~0u) {     // every score of the tile follows from redo_marked
+        tc_fence_before();
+        mbar_arrive(&bars->acc_empty);
+        continue;
+      }
       if (!any) {
         tc_fence_before();
         mbar_arrive(&bars->acc_empty);
@@ -455,40 +588,6 @@ __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bar
       }
       tc_fence_before();
       mbar_arrive(&bars->acc_empty);
-      const uint32_t bad_blocks = info.bad[hc];
-      if (bad_blocks | bad_rows) {
-        // marked blocks: every lane the two logits of its row; marked rows: the lanes share the row's 16 logits, half of the channels each
-        const uint4 *kx = static_cast<const uint4*>(a.Kmax) + (size_t(r.kvh) * a.n2 + b_tile) * (kD / 8);
-        const uint4 *kn = static_cast<const uint4*>(a.Kmin) + (size_t(r.kvh) * a.n2 + b_tile) * (kD / 8);
-        const int last = min(8, a.n2 - b_tile) - 1;         // blocks past the end: any logit will do
-#pragma unroll 1
-        for (uint32_t left = bad_blocks; left; left &= left - 1) {
-          const int ib = __ffs(left) - 1, at = min(ib, last) * (kD / 8);
-          const uint4* q = static_cast<const uint4*>((m & 1) ? a.Qmin : a.Qmax) + (valid ? unit : 0) * (kD / 8);
-          const double un = 1.0 / (ri.scale[m] * info.scale[hc * 8 + ib]);     // a power of two: taken off again below
-#pragma unroll 1
-          for (int kr = 0; kr < 2; ++kr) {
-            const double l = slow_logit<kF16>(q, (kr ? kn : kx) + at, kD / 8) * un;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              if (i == ib && kr == 0) vx[i] = l;
-              if (i == ib && kr == 1) vn[i] = l;
-            }
-          }
-        }
-#pragma unroll 1
-        for (uint32_t left = bad_rows; left; left &= left - 1) {
-          const int owner = __ffs(left) - 1, ib = lane & 7, mo = (warp & 3) * 32 + owner, c0 = (lane >> 4) * (kD / 16);
-          const uint4* q = static_cast<const uint4*>((mo & 1) ? a.Qmin : a.Qmax) + row_unit(a, r, mo) * (kD / 8) + c0;
-          double l = slow_logit<kF16>(q, ((lane & 8) == 0 ? kx : kn) + min(ib, last) * (kD / 8) + c0, kD / 16);
-          l = (l + __shfl_xor_sync(0xffffffffu, l, 16)) / info.scale[hc * 8 + ib];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const double lx = __shfl_sync(0xffffffffu, l, i), ln = __shfl_sync(0xffffffffu, l, 8 + i);
-            if (lane == owner) { vx[i] = lx; vn[i] = ln; }
-          }
-        }
-      }
       // The Qmax lane gives its upper blocks for the Qmin lane's lower ones: each then has all four logits of 4 blocks, less
       // their log-sum-exps.  Which of a pair is l1 (l2) and which l3 (l4) makes no difference.
       const double f_own = ri.scale[m] * a.est_scale, f_other = ri.scale[m ^ 1] * a.est_scale;
@@ -504,44 +603,30 @@ __device__ __forceinline__ void epilogue_role(const ScoreExactArgs& a, Bars* bar
       }
       // max( ln (S1+S3)/2, ln (S2+S4)/2 ), fusion with S'
       double v[4];
-      if (special | bad_blocks | bad_rows) {
+      if (special) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) v[i] = combine_any(bars->nodes, vx[i], vn[i], vx[4 + i], vn[4 + i]) - ln2;
       } else {
 #pragma unroll
         for (int q = 0; q < 4; q += 2) {
-          double hi[4], d[4];
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const double L1 = vx[q + i], L2 = vn[q + i], L3 = vx[4 + q + i], L4 = vn[4 + q + i];
-            d[i] = L1 - L3; d[2 + i] = L2 - L4;
-            hi[i] = __double2hiint(d[i]) >= 0 ? L1 : L3; hi[2 + i] = __double2hiint(d[2 + i]) >= 0 ? L2 : L4;
-            d[i] = fabs(d[i]); d[2 + i] = fabs(d[2 + i]);
-          }
-          softplus_nodes(bars->nodes, d);
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const double y13 = hi[i] + d[i], y24 = hi[2 + i] + d[2 + i];
-            v[q + i] = (y13 >= y24 ? y13 : y24) - ln2;
-          }
+          const double L1[2] = {vx[q], vx[q + 1]}, L2[2] = {vn[q], vn[q + 1]}, L3[2] = {vx[4 + q], vx[5 + q]}, L4[2] = {vn[4 + q], vn[5 + q]};
+          double y[2];
+          combine_n(bars->nodes, L1, L2, L3, L4, y);
+          v[q] = y[0] - ln2; v[q + 1] = y[1] - ln2;
         }
       }
       if (a.fuse) {
-        double d[4];
+        double y[4], z[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const double y = a.ln_alpha + v[i], z = a.ln_1m_alpha + sp[i];
-          v[i] = fmax(y, z);
-          d[i] = v[i] - fmin(y, z);
-        }
-        softplus_nodes(bars->nodes, d);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] += d[i];
+        for (int i = 0; i < 4; ++i) { y[i] = a.ln_alpha + v[i]; z[i] = a.ln_1m_alpha + sp[i]; }
+        fuse_n(bars->nodes, v, y, z);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[i] = b0 + i < vis ? v[i] : -CUDART_INF;     // blocks at or after the end of the segment (line 13)
       st4(a.S_out + out, a.vec, n_in, v);
     }
+    redone = redo_marked<kF16>(a, bars, w.combo, w.chunk, w.tile, w.n, piece, t, redone);
+    if (redone == kGaveUp) return;
   }
 }
 
@@ -574,6 +659,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_visible_kernel(const __grid
     mbar_init(&bars->q_full, kEpilogueWarps * 32);
     mbar_init(&bars->acc_full, 1);
     mbar_init(&bars->acc_empty, kEpilogueWarps * 32);
+    mbar_init(&bars->redo, kEpilogueWarps * 32);
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
