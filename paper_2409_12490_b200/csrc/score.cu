@@ -294,17 +294,30 @@ score_kernel(const __grid_constant__ ScoreArgs<T, NS> a, int Hq, int g, int seg,
   if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until two CTAs fit an SM (104 KB of logits each), or, where 8 do not get
-// there, until one does (200 KB); 0: they never do.
-constexpr size_t kSmemShared = 104 * 1024, kSmemAlone = 200 * 1024;
+// Key blocks are split over a cluster of 1, 2, 4 or 8 CTAs until one fits an SM (200 KB of logits each), and twice as often where two then fit
+// an SM (104 KB) and that is the faster split; 0: 8 are not enough.  With 4 heads it is the faster one only while all CTAs run at once:
+// 552 < n2 <= 1064, one CTA with 512 threads / two of half the blocks, us, in graphs, bf16: 5 segments x 8 KV heads, n2 600 25.6 / 16.4; 15 x 8,
+// n2 938 33.2 / 37.0; 34 x 8, n2 576 46.0 / 52.1; 145 x 8, n2 580 10 to 12 % slower split.  With 1 or 2 heads, whose MMAs are a quarter or half empty
+// columns, the split is never slower: 30 x 8, 2 heads, n2 1132 65.9 / 65.8 (64 channels 52.1 / 48.1); 25 x 12, one head, n2 2268 119.4 / 95.2.
+constexpr size_t kSmemShared = 104 * 1024, kSmemWideRows = 88 * 1024 + 512, kSmemAlone = 200 * 1024;
 int cluster_of(const Dims& m, int U, int* nb) {
-  for (size_t limit : {kSmemShared, kSmemAlone})
-    for (int CL = 1; CL <= 8; CL *= 2) {
-      *nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
-      if ((sizeof(double) + sizeof(float)) * 4 * size_t(U) * *nb <= limit) return CL;
-    }
-  return 0;
+  auto split = [&](int CL) {
+    *nb = (((m.n2 + CL - 1) / CL) + 7) & ~7;
+    return (sizeof(double) + sizeof(float)) * 4 * size_t(U) * *nb;
+  };
+  int CL = 1;
+  while (split(CL) > kSmemAlone)
+    if ((CL *= 2) > 8) return 0;
+  const bool twice = CL < 8 && split(CL) > kSmemShared && split(2 * CL) <= kSmemShared &&
+                     (U < 4 || (long long)m.B * m.Hkv * (m.g / U) * m.n1 * 2 * CL <= 148);
+  if (twice) CL *= 2;
+  split(CL);
+  return CL;
 }
+// CTAs of 256 threads, two per SM, where there are more of them than SMs (see kThreadsMany).  Rows of 512 bytes (fp32, 128 channels) need
+// the L1 that two CTAs of more than 88.5 KB (196 KB of the SM with their static part) leave no room for: n2 464 / 480, 34 / 32 segments x 8 KV
+// heads, one CTA 55.1 / 55.4 us, two 54.2 / 71.2.
+bool two_per_sm(const Dims& m, long long ctas, size_t smem) { return ctas > 148 && smem <= (m.d * m.es == 512 ? kSmemWideRows : kSmemShared); }
 // as many heads per CTA as divide the group (the fp64 MMA has 8 rows = 4 heads x 2 representatives)
 int heads_per_cta(const Dims& m) { return m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1); }
 
@@ -333,7 +346,7 @@ int launch_u(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* 
   if (ctas > 0x7fffffffLL) return CP_ERR_UNSUPPORTED;
   const Dims& m = pr[0].m;
   const size_t smem = (sizeof(double) + sizeof(float)) * (4 * size_t(U) * nb_max);   // fp64 logits + their fp32 copies
-  const bool many = ctas > 148 && smem <= kSmemShared;
+  const bool many = two_per_sm(m, ctas, smem);
   auto kern = many ? score_kernel<T, D, U, NS, kThreadsMany> : score_kernel<T, D, U, NS, kThreadsFew>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return CP_ERR_CUDA;

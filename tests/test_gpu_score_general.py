@@ -1,5 +1,6 @@
-"""The general score kernel where its launches change shape: key blocks at the limits of a cluster's shared memory (552 per CTA for four
-heads when two CTAs share an SM, 1064 when one has it to itself), CTAs as many as SMs and one more."""
+"""The general score kernel where its launches change shape: key blocks at the limits of a cluster's shared memory (four heads: 1064 per CTA, 552
+where twice the CTAs still run at once; fewer heads: 552 x 4 / heads), CTAs as many as SMs and one more, fp32 rows at the
+limit of two CTAs per SM (472 blocks)."""
 import numpy as np
 import pytest
 import torch
@@ -16,7 +17,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,d,g,n2,segments", [
     ("bf16", 128, 4, 552, 138), ("f16", 128, 4, 552, 184), ("bf16", 128, 4, 553, 93), ("f32", 128, 4, 553, 111),
     ("f16", 64, 4, 148, 148), ("bf16", 128, 4, 149, 149), ("f32", 64, 2, 1105, 79), ("bf16", 64, 1, 2209, 60),
-    ("bf16", 128, 4, 1105, 12), ("f16", 64, 4, 2209, 6), ("bf16", 64, 4, 4417, 3), ("f16", 64, 4, 8191, 2),
+    ("bf16", 128, 4, 553, 74), ("f32", 64, 4, 553, 79), ("bf16", 64, 4, 1064, 152), ("f16", 128, 4, 1065, 153), ("f32", 128, 4, 472, 158),
+    ("f32", 128, 4, 473, 158), ("f32", 128, 1, 1889, 158), ("bf16", 128, 4, 1105, 12), ("f16", 64, 4, 2209, 6), ("bf16", 64, 4, 4417, 3), ("f16", 64, 4, 8191, 2),
 ])
 def test_shapes_of_the_launch(dtype, d, g, n2, segments):
     r = -(-n2 // segments)

@@ -61,9 +61,10 @@ def test_fused_layers_equal_their_own_calls(flags, dtype, d, room):
 
 
 def test_batch_whose_scores_need_clusters_of_every_size():
-    """Four heads per CTA, blocks of 4 tokens: up to 1064 blocks fit one CTA's shared memory, 2128 two, 4256 four, 8192 eight.  Two sequences
-    of each size in one batch, alternating, so that every cluster launch holds several sequences with offsets of their own."""
-    lens, Hq, Hkv, d, seg, blk, k = [3000, 8000, 18000, 5000, 33, 9000, 4265, 20000, 4300, 17000], 4, 1, 64, 256, 4, 64
+    """Four heads per CTA, blocks of 4 tokens: up to 1064 blocks fit one CTA's shared memory, 2128 two, 4256 four, 8192 eight; half of that are
+    split twice as often where that makes no more than 148 CTAs.  Two sequences or more of each size (1: 33, 1500; 2: 3000, 4265, 4300; 4: 8000,
+    5000, 9000, 17000; 8: 18000, 20000) in one batch, so that every cluster launch holds several sequences with offsets of their own."""
+    lens, Hq, Hkv, d, seg, blk, k = [3000, 8000, 18000, 5000, 33, 9000, 4265, 20000, 4300, 1500, 17000], 4, 1, 64, 256, 4, 64
     total, cu = sum(lens), [0] + np.cumsum(lens).tolist()
     layers = [[t[0].cuda() for t in make_uniform_qkv(1, Hq, Hkv, total, d, dtype="f32", seed=s)] for s in (3, 4)]
     prob = cp.Problem(1, Hq, Hkv, max(lens), d, seg, blk, k, torch.float32)
