@@ -58,6 +58,17 @@ inline WsLayout ws_layout(const Dims& m) {
   return w;
 }
 
+// Query heads of a KV group that share a CTA of a score kernel.
+inline int score_heads(const Dims& m) { return m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1); }
+// Segments per CTA of the log-sum-exp kernel.  A CTA has 128 logit rows = 64 / U segments; on mid-sized problems fewer segments per CTA (rows left
+// unused) put more SMs to work on the sweeps and the exact pass, which run per CTA one after the other.
+inline int lse_segments(const Dims& m) {
+  int segs = 64 / score_heads(m);
+  const long long groups = (long long)m.B * m.Hkv * (m.g / score_heads(m));
+  while (segs > 4 && groups * ((m.n1 + segs - 1) / segs) < 100) segs /= 2;
+  return segs;
+}
+
 // Device status block.
 struct DeviceStatus {
   int32_t code;     // cp_status, first error wins

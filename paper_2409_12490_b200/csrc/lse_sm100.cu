@@ -516,13 +516,9 @@ int launch_lse(const cp_params& p, const Dims& m, char* ws, cudaStream_t st) {
   a.kabs = reinterpret_cast<const float*>(ws + w.kabs);
   a.stats = stats;
   a.st = reinterpret_cast<DeviceStatus*>(ws);
-  a.Hq = m.Hq; a.g = m.g; a.U = m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1);
+  a.Hq = m.Hq; a.g = m.g; a.U = score_heads(m);
   a.n1 = m.n1; a.n2 = m.n2; a.seg = m.seg; a.blk = m.blk;
-  // a CTA has 128 logit rows = 64 / U segments; on mid-sized problems fewer segments per CTA (rows left unused) put more
-  // SMs to work on the sweeps and the exact pass, which run per CTA one after the other
-  a.segs_per_cta = 64 / a.U;
-  const long long per_chunk = (long long)m.B * m.Hkv * (m.g / a.U);
-  while (a.segs_per_cta > 4 && per_chunk * ((m.n1 + a.segs_per_cta - 1) / a.segs_per_cta) < 100) a.segs_per_cta /= 2;
+  a.segs_per_cta = lse_segments(m);
   a.n_qchunks = (m.n1 + a.segs_per_cta - 1) / a.segs_per_cta;
   a.mask_first = (p.flags & CP_FLAG_MASK_BEFORE_SOFTMAX) ? 1 : 0;
   a.box_rows = m.n2 < kTileN ? m.n2 : kTileN;

@@ -318,9 +318,6 @@ int cluster_of(const Dims& m, int U, int* nb) {
 // the L1 that two CTAs of more than 88.5 KB (196 KB of the SM with their static part) leave no room for: n2 464 / 480, 34 / 32 segments x 8 KV
 // heads, one CTA 55.1 / 55.4 us, two 54.2 / 71.2.
 bool two_per_sm(const Dims& m, long long ctas, size_t smem) { return ctas > 148 && smem <= (m.d * m.es == 512 ? kSmemWideRows : kSmemShared); }
-// as many heads per CTA as divide the group (the fp64 MMA has 8 rows = 4 heads x 2 representatives)
-int heads_per_cta(const Dims& m) { return m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1); }
-
 struct ScoreProblem { Dims m; const char* ws; const double* S_prev; double* S_out; };
 
 // problems that need the same cluster size, in one launch
@@ -358,7 +355,7 @@ int launch_u(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* 
 
 template <typename T, int D, int NS>
 int launch_t(const cp_params& p, const ScoreProblem* pr, int n, int CL, double* stats_out, cudaStream_t st) {
-  const int U = heads_per_cta(pr[0].m);
+  const int U = score_heads(pr[0].m);
   if (U == 4) return launch_u<T, D, 4, NS>(p, pr, n, CL, stats_out, st);
   if (U == 2) return launch_u<T, D, 2, NS>(p, pr, n, CL, stats_out, st);
   return launch_u<T, D, 1, NS>(p, pr, n, CL, stats_out, st);
@@ -388,7 +385,7 @@ int launch_score_generic(const cp_params& p, const Dims& m, const char* ws, cons
                          double* S_out, double* stats_out, cudaStream_t st) {
   const ScoreProblem pr{m, ws, S_prev, S_out};
   int nb;
-  const int CL = cluster_of(m, heads_per_cta(m), &nb);
+  const int CL = cluster_of(m, score_heads(m), &nb);
   return CL == 0 ? CP_ERR_UNSUPPORTED : launch_problems<1>(p, &pr, 1, CL, stats_out, st);
 }
 
@@ -406,7 +403,7 @@ int launch_score_seqs(const cp_params& p, const Dims& m, const SeqSlot* slots, c
       }
       if (i == n_seqs) break;
       const Dims q = seq_dims(m, slots[i].len);
-      const int c = cluster_of(q, heads_per_cta(q), &nb);
+      const int c = cluster_of(q, score_heads(q), &nb);
       if (c == 0) return CP_ERR_UNSUPPORTED;
       if (c == CL) pr[n++] = {q, ws[i], S_prev ? S_prev + slots[i].s : nullptr, S_out + slots[i].s};
     }

@@ -39,7 +39,6 @@
 namespace cp {
 namespace {
 
-constexpr long long kFastMinScores = 1500000;   // see score_is_split
 constexpr int kEpilogueWarps = 16, kThreads = (kEpilogueWarps + 8) * 32, kMmaWarp = kEpilogueWarps + 4;
 constexpr int kD = 128;
 constexpr int kRows = 128;                     // logit rows (MMA M) per CTA
@@ -701,7 +700,7 @@ int launch_visible(const Dims& m, char* ws, const double* S_prev, double* S_out,
   a.stats = reinterpret_cast<const double*>(ws + w.stats);
   a.S_prev = S_prev; a.S_out = S_out;
   a.st = reinterpret_cast<DeviceStatus*>(ws);
-  a.Hq = m.Hq; a.g = m.g; a.U = m.g % 4 == 0 ? 4 : (m.g % 2 == 0 ? 2 : 1);
+  a.Hq = m.Hq; a.g = m.g; a.U = score_heads(m);
   a.n1 = m.n1; a.n2 = m.n2; a.seg = m.seg; a.blk = m.blk;
   a.segs = 64 / a.U;
   a.n_qchunks = (m.n1 + a.segs - 1) / a.segs;
@@ -736,15 +735,25 @@ int launch_visible(const Dims& m, char* ws, const double* S_prev, double* S_out,
 
 }  // namespace
 
-// From which size on the two-kernel path is used.  What counts is the general kernel's work: its MMAs have 8 columns, the Qmax and
-// Qmin rows of up to 4 heads of a group, of which groups of 2 heads fill half and single heads a quarter.
-// General kernel / two kernels, us, 32 / 8 heads: segment 512, block 32, 16384 tokens (0.5 M scores) 34 / 65; block 64, 32768 tokens
-// (1.05 M, fused) 70 / 75; segment 1024, block 128, 65536 tokens (1.05 M) 63 / 72; the general kernel with one CTA per SM: block 32, 32768 tokens
-// (2.1 M) 122 / 100; 8 / 8 heads, segment 128, block 32, 16384 tokens (0.5 M, counted as 2.1 M) 103 / 67.
+// Whether the two-kernel path is the faster one, by estimates of both (us).  The general kernel's work is its (CTA, key block) pairs per SM, which single heads
+// use no better than groups of four.  The two kernels start with some 36 us; the log-sum-exps take time for every wave of CTAs, by the key blocks that
+// each of them streams and by the share of its 128 rows that is in use; the visible blocks by their tiles per SM.  From 2.2 M scores on
+// two kernels are taken whatever the shape.  Fitted to 538 shapes (0.2 to 3.2 M scores, groups of 1 to 8 heads, segments of 128 to 1024, blocks of
+// 32 to 128, fused and not) with clustered keys as in attention, and with keys of which ten times as many come near a row's maximum: 0.8 and 2.0 %
+// slower on average than the better path of each.  A line at 1.5 M scores, those of groups of 2 heads counted twice and of single heads and
+// odd groups four times: 2.6 and 6.8 %, up to 1.4 and 1.9 times.
+// General kernel / two kernels, us, fused, clustered keys: 32 / 8 heads, segment 512, block 32, 15995 tokens 39.5 / 66.8, 27707 tokens 105.0 / 106.4, 33531
+// tokens 154.5 / 124.4; segment 1024, block 128, 84603 tokens 131.2 / 142.5; 24 / 8 heads, segment 512, block 64, 28603 tokens 112.4 / 96.5.
+constexpr long long kFastMinScores = 2200000;
 bool score_is_split(const cp_params& p, const Dims& m) {
-  const long long scores = (long long)m.B * m.Hq * m.n1 * m.n2 * (m.g % 4 == 0 ? 1 : (m.g % 2 == 0 ? 2 : 4));
-  return (p.dtype == CP_BF16 || p.dtype == CP_F16) && m.d == 128 &&
-         (scores >= kFastMinScores || (p.flags & CP_FLAG_FORCE_SPLIT_SCORE));
+  if ((p.dtype != CP_BF16 && p.dtype != CP_F16) || m.d != 128) return false;
+  if ((p.flags & CP_FLAG_FORCE_SPLIT_SCORE) || (long long)m.B * m.Hq * m.n1 * m.n2 >= kFastMinScores) return true;
+  const int U = score_heads(m), segs = lse_segments(m);
+  const long long groups = (long long)m.B * m.Hkv * (m.g / U);
+  const double per_sm = double(groups) * m.n1 * m.n2 / 148, waves = double((groups * ((m.n1 + segs - 1) / segs) + 147) / 148);
+  const double general = 16 + (0.019 + 0.0045 * U) * per_sm;
+  const double split = 36 + waves * (10 + m.n2 * (0.025 + 0.14 * segs * U / 64)) + 7.5 / 4096 * U * per_sm;
+  return general > split;
 }
 
 // K2 dispatcher.  16-bit inputs with head_dim 128 take the two-kernel path (log-sum-exps, then exact logits of
