@@ -63,6 +63,117 @@ def test_values_that_do_not_fit(dtype, where):
     check(Q, K, dtype, 128, 32, est_scale=0.0883 if where == "scale" else 1.0)
 
 
+def signed_bytes(x):
+    """The four signed bytes of integers of 31 bits, lowest first."""
+    out = []
+    for _ in range(4):
+        d = (x + 128) % 256 - 128
+        out.append(d)
+        x = (x - d) // 256
+    assert not x.any()
+    return out
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("shift,decisive", [(0, {0, 1, 2}), (8, {2, 3, 4}), (12, {2, 3, 4}), (18, {4, 5, 6})])
+def test_every_accumulator_decides(dtype, shift, decisive):
+    """Odd multiples of 2^(shift - 24) of both signs beside a 32 that meets a 0: the bytes that hold them carry the logits."""
+    Hq, Hkv, n1, r, blk = 8, 2, 40, 2, 16
+    rng = np.random.default_rng(shift)
+    bits = 8 if dtype == "bf16" else 11
+    odd = lambda *size: (2 * rng.integers(0, 2 ** (bits - 1), size) + 1) * rng.choice([-1, 1], size) * 2 ** shift
+    q, k = odd(1, Hq, n1, 128), odd(1, Hkv, n1 * r, 128)
+    q[..., 0], q[..., 1], k[..., 0], k[..., 1] = 0, 2 ** 29, 2 ** 29, 0
+    Q, K = (torch.from_numpy(x * 2.0 ** -24).to(DT[dtype]) for x in (q, k))
+    assert np.array_equal(Q.double().numpy() * 2 ** 24, q) and np.array_equal(K.double().numpy() * 2 ** 24, k)
+    est_scale = 2.0 ** (48 - 2 * (shift + bits) + 1)                           # logits of the order of ten
+    qd, kd = signed_bytes(q), signed_bytes(k.repeat(Hq // Hkv, axis=1))
+    acc = [sum(qd[i] @ kd[s - i].swapaxes(-1, -2) for i in range(max(0, s - 3), min(s, 3) + 1)) for s in range(7)]
+    part = [np.abs(a).max() * 2.0 ** (8 * s - 48) * est_scale for s, a in enumerate(acc)]
+    assert {s for s in range(7) if part[s] > 1e-5} >= decisive, part
+    check(Q.repeat_interleave(r * blk, 2), K.repeat_interleave(blk, 2), dtype, r * blk, blk, est_scale=est_scale)
+
+
+@pytest.mark.parametrize("power", [-64, 70])
+@pytest.mark.parametrize("which", ["Q", "K", "both"])
+def test_magnitudes_beyond_the_scales(power, which):
+    """bf16 rows or blocks whose exponent is out of range: marked, with logits of the usual size."""
+    Q, K, _ = make_uniform_qkv(1, 8, 2, 1500, 128, seed=9)
+    if which != "K":
+        Q = (Q.float() * 2.0 ** power).bfloat16()
+    if which != "Q":
+        K = (K.float() * 2.0 ** (-power if which == "both" else power)).bfloat16()
+    check(Q, K, "bf16", 128, 32, est_scale=0.125 * (1.0 if which == "both" else 2.0 ** -power))
+
+
+def maps(Q, K, seg, blk):
+    """The four logit maps of Algorithm 1; a NaN is left out of a maximum or minimum."""
+    rep = lambda X, size: [[f([X[:, :, i:i + size]], axis=3)[0] for i in range(0, X.shape[2], size)] for f in (np.fmax.reduce, np.fmin.reduce)]
+    q, k = [[np.stack(x, 2) for x in rep(X.double().numpy(), size)] for X, size in ((Q, seg), (K, blk))]
+    k = [x.repeat(Q.shape[1] // K.shape[1], axis=1).swapaxes(-1, -2) for x in k]
+    with np.errstate(invalid="ignore"):
+        return [a @ b for a in q for b in k]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("where", ["Q", "K", "future", "several"])
+@pytest.mark.parametrize("value", [float("inf"), float("-inf")])
+def test_infinities(dtype, where, value):
+    """A map of a row with an infinite logit has no log-sum-exp: the row's scores follow from its other maps.  Rows without one, and blocks that such
+    maps rule out, as ever."""
+    Q, K, _ = make_uniform_qkv(1, 8, 2, 2500, 128, dtype=dtype, seed=3)
+    if where in ("Q", "several"):
+        Q[0, 3, 700, 5] = Q[0, 1, 1300, 100] = value
+    if where in ("K", "several"):
+        K[0, 1, 333, 5] = value
+    if where == "future":
+        K[0, 1, 2499, 5] = value
+    prob = cp.Problem(1, 8, 2, 2500, 128, 128, 32, 4, DT[dtype], est_scale=0.25, flags=cp.FLAG_FORCE_SPLIT_SCORE)
+    ws = cp.alloc_workspace(prob)
+    S = cp.estimate(prob, Q.cuda(), K.cuda(), ws).cpu().numpy()
+    assert cp.device_status(ws) == 0
+    L = []
+    for l in maps(Q, K, 128, 32):
+        l = 0.25 * l
+        m = l.max(-1, keepdims=True)
+        with np.errstate(invalid="ignore"):
+            L.append(np.where(np.isfinite(m), l - m - np.log(np.exp(l - m).sum(-1, keepdims=True)), np.nan))
+    with np.errstate(invalid="ignore"):
+        pair = lambda a, b: np.where(np.isnan(a), b, np.where(np.isnan(b), a, np.logaddexp(a, b) - np.log(2.0)))
+    ref = np.fmax(pair(L[0], L[2]), pair(L[1], L[3]))
+    masked = oracle.estimation.causal_block_mask(20, 79, 128, 32)
+    assert any(np.isnan(x).any() for x in L) and np.isneginf(S[..., masked]).all()
+    assert np.isfinite(ref[..., ~masked]).all() and np.abs(S - ref)[..., ~masked].max() <= 1e-9
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("where", ["Q", "K", "tokens", "S_prev nan", "S_prev inf", "S_prev -inf"])
+def test_not_finite_as_in_the_general_kernel(dtype, where):
+    """Single NaN in Q or K (left out of the representatives) and S' that is not finite: both paths agree."""
+    Q, K, _ = make_uniform_qkv(1, 8, 2, 2500, 128, dtype=dtype, seed=4)
+    Q0, K0, _ = make_uniform_qkv(1, 8, 2, 2500, 128, dtype=dtype, seed=5)
+    if where == "Q":
+        Q[0, 3, 700, 5] = Q[0, 1, 1300:1310] = float("nan")
+    if where == "K":
+        K[0, 1, 333, 5] = K[0, 0, 2499, 7] = float("nan")
+    if where == "tokens":
+        K[0, :, 64:90] = Q[0, 2, 128:200] = float("nan")
+    out = []
+    for flags in (0, cp.FLAG_FORCE_SPLIT_SCORE):
+        prob = cp.Problem(1, 8, 2, 2500, 128, 128, 32, 4, DT[dtype], est_scale=0.25, flags=flags)
+        ws = cp.alloc_workspace(prob)
+        S_prev = cp.estimate(prob, Q0.cuda(), K0.cuda(), ws)
+        if where.startswith("S_prev"):
+            S_prev[0, 2, 10:14, 3:9] = float(where.split()[1])
+        S = cp.estimate(prob, Q.cuda(), K.cuda(), ws, S_prev=S_prev)
+        assert cp.device_status(ws) == 0
+        out.append(S.cpu().numpy())
+    a, b = out
+    assert all(np.array_equal(f(a), f(b)) for f in (np.isnan, np.isposinf, np.isneginf))
+    finite = np.isfinite(a)
+    assert np.abs(a[finite] - b[finite]).max() <= 1e-9
+
+
 @pytest.mark.parametrize("dtype,B,Hkv,g,n,seg,blk", [
     ("bf16", 1, 8, 4, 6000, 256, 16),          # parts that begin inside a row group, 375 blocks
     ("f16", 1, 2, 4, 8192, 128, 32),           # whole row groups of 16 segments
