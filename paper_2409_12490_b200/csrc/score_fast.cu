@@ -27,13 +27,14 @@
 //   warps 16-19 bytes of the next tile's key rows into shared memory
 //   warp 20     MMA issuer: 64 MMAs of 128 x 64 x 32 per tile, under the fp64 part of the epilogue
 //   warps 21-23 the masked part of the map: -inf
-// Bound by MMAs and fp64 operations, which do not run at the same time: a tile's combination takes 1900 cycles alone (50 fp64 operations
-// per score) and 6100 with the next tile's MMAs under way, which take 3400 to 4600 (6 KB of operands each from shared memory).  A tile
-// takes 10 to 13 thousand cycles, with 8 epilogue warps 14 thousand (latency).  Half tiles with accumulators of their own, so that half of the
-// warps combine while the others convert: slower (N = 32: 5 KB per MMA of half the work; 131072 tokens 665 -> 780 us).
+// No single unit bounds it (131072 tokens, segment 512, block 32; a tile takes some 10 thousand cycles): the byte MMAs and the fp64 operations hold the one
+// pipe that they share 40 % of the cycles (their sum: they take turns), the data stage of shared memory is busy 56 % (MMA operands, 6 KB each, 31 %), few
+// warps wait for it; they wait for tensor memory and for the fp64 pipe.  A tile's combination takes 1900 cycles alone (50 fp64 operations
+// per score) and 6100 with the next tile's MMAs under way, which take 3400 to 4600.  8 epilogue warps: 14 thousand cycles per tile
+// (latency).  Half tiles with accumulators of their own, so that half of the warps combine while the others convert: slower (N = 32: 5 KB per MMA of
+// half the work; 131072 tokens 665 -> 780 us).
 // Both kernels of the scores, this one with fp64 MMAs (m16n8k16, 8 to 12 warps each on its own tiles) -> now, us, in graphs, 32 / 8 heads:
-// 131072 tokens, segment 512, block 32, fused 982 -> 665 (641 with lse_sm100.cu as it is now); segment 1024, block 128 184 -> 153 (147.5);
-// 65536 tokens, segment 512, block 64 166 -> 161 (156).
+// 131072 tokens, segment 512, block 32, fused, fp16 960 -> 622; segment 1024, block 128 193 -> 151.
 #include "sm100_ptx.cuh"
 
 namespace cp {
