@@ -268,7 +268,7 @@ def everything(Q, K, seg, blk):
 
 
 # Both kernels of the scores, with / without: 183, 190 and 272 us against 176; with marked logits summed by single threads 225, 229 and 1641.
-# Times of a shared machine, hence the room.
+# Times vary from run to run, hence the room.
 @pytest.mark.parametrize("change,limit", [(one_row, 1.15), (some_blocks, 1.2), (everything, 2.5)])
 def test_values_that_do_not_fit_cost_little(change, limit):
     plain, marked = score_times("bf16", change)
